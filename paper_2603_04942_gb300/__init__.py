@@ -231,11 +231,10 @@ def lib():
     return load()
 
 
-PHASE_NAMES = ("tile start", "tile load", "look-ahead", "walk 2 and its scan", "trigger times",
-               "walk 4 (records)", "hash insert", "neighbour pass", "compression", "unions", "roots",
-               "member lists", "member-list walks (and the previous tile's copy-out)",
-               "staged stores", "labels and offsets", "tail", "CTA end",
-               "big ranges (batches: the sorted-window path)", "big ranges: the previous tile's copy-out",
+PHASE_NAMES = ("tile start", "packet loads", "records into slots", "pixel wraps", "trigger times",
+               "packets to records", "cell table ranks", "neighbour pass", "(unused)", "unions", "roots",
+               "member lists", "member-list walks", "records and label entries", "labels",
+               "tail", "CTA end", "big ranges (batches: the sorted-window path)", "(unused)",
                "label ranks (bitmap scan)", "big: range end, walk 2, triggers", "big: walk 4", "big: bins and sort",
                "big: neighbour pass", "big: compression and roots", "big: moments", "big: labels, records, outputs")
 

@@ -1,26 +1,25 @@
 // tpx_fused.cuh -- the fused single-pass TPX3 path for sm_103a.
 //
-// One persistent kernel reads the packet stream once.  Each CTA repeatedly
+// One persistent kernel reads the packet stream once, after the unwrap
+// pre-pass (tpx_prepass.cu), which reads it once before. Each CTA repeatedly
 // claims the next tile of T packets (dynamic, in stream order), and:
-//   1. loads the tile into shared memory; the exact state of the two ToA
-//      unwrap chains (pixels, TDCs; Sec. IV.A: a step down by more than the
-//      threshold adds a wrap, a step up by more removes one) at the tile start
-//      comes from the unwrap pre-pass, which scans the tiles' chain
-//      aggregates before the kernel starts (the chains are associative);
-//   2. owns the laser shots whose TDC packet lies in the tile, reading past
-//      the tile end up to the next TDC packet (its "range");
-//   3. unwraps every packet of the range, bins each pixel to the most recent
+//   1. owns the laser shots whose TDC packet lies in the tile: its range runs
+//      from the tile's first TDC packet to the first one past the tile, both
+//      known from the pre-pass's tile table, as is the state of the two ToA
+//      unwrap chains (pixels, TDCs; Sec. IV.A) where the range starts;
+//   2. reads the range into registers, bins each pixel to the most recent
 //      trigger in time, applies the <= tof_max background cut and the optional
 //      timewalk table (Sec. IV.B-C);
-//   4. hashes kept pixels by (shot, x, y) and visits each adjacent pair once
-//      under the box rule of Sec. V.A; a pair updates the local-maximum flags
-//      (Sec. V.B, equal ToT resolved towards the later pixel) and, in CC mode,
-//      a lock-free union-find whose root is the pair-wise minimum of the key
-//      (corrected time, stream position) -- so each component's root is its
-//      earliest pixel in sorted order without sorting the pixels;
-//   5. accumulates exact integer sums per cluster in shared memory (Sec. V.C)
-//      and writes per-packet labels and, after a second look-back over
-//      cluster counts, the cluster records in ascending label order.
+//   3. puts the kept pixels into the order of a table with one bit per cell
+//      (shot, y, x): the neighbours of a pixel are consecutive slots;
+//   4. visits each adjacent pair once under the box rule of Sec. V.A; a pair
+//      updates the local-maximum flags (Sec. V.B, equal ToT resolved towards
+//      the later pixel) and, in CC mode, joins two trees of a lock-free
+//      union-find;
+//   5. forms exact integer sums per cluster (Sec. V.C), stages the records in
+//      label order (the cluster's earliest pixel in (time, position) order),
+//      and writes per-packet labels; a warp of its own copies the records out
+//      to their offset, a decoupled look-back over the tiles' record counts.
 // Pixels whose trigger cannot be decided inside the range, and ranges that
 // exceed the on-chip capacities, raise a status bit instead (the kernel never
 // traps).  All device waits are bounded.
@@ -66,11 +65,19 @@ struct Ctl {                     // per-launch control block, cleared before eac
 struct GChain { long long n, first, last, sum; };
 struct GAgg { GChain pix, tdc; };            // 64 bytes
 
+// what the fused kernel plans a tile's range from: the tile's first TDC packet
+// (-1: none), and whether a pixel wrap step lies in the tile or between it and
+// the pixel before it
+struct TileInfo { int first_tdc, wrap; };
+
 // per-tile records: the unwrap pre-pass's tile aggregates and states, and
 // the record-count look-back chain
 struct TileScratch {
     GAgg *agg;               // [tiles] unwrap-chain aggregate of each tile
-    GAgg *pre;               // [tiles] unwrap state before each tile
+    GAgg *pre;               // [tiles] state before each tile: the TDC chain before the tile, the pixel
+                             // chain before the first packet the tile's range reads
+    GChain *head;            // [tiles] pixel chain from the tile's start to its first TDC packet
+    TileInfo *tinfo;         // [tiles]
     GAgg *blk;               // unwrap_prepass_scratch_bytes(tiles): block totals of the scan
     unsigned int *cflags;    // [tiles] cluster-count chain: (seq<<2)|1 count, |2 inclusive prefix
     long long *cagg;         // [tiles]

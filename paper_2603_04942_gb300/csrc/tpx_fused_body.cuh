@@ -1,18 +1,40 @@
 // tpx_fused_body.cuh -- the fused kernel, included once per tile geometry
 // by tpx_fused.cu inside a namespace that defines NT (threads per CTA),
-// T (packets per tile), C (range capacity), HB (hash buckets), MS (trigger
-// packets a range may hold) and MINB (CTAs per SM). No include guard: it
+// T (packets per tile), C (range capacity), TR (rows of the cell table), MS
+// (trigger packets a range may hold), MINB (CTAs per SM) and BIG_REGION (bytes
+// of shared scratch of the big-range path). No include guard: it
 // is meant to be included repeatedly.
-constexpr int NW = NT / 32;
+//
+// Bound by instruction issue and by the barriers between its phases, not by
+// bytes (18 B per packet, 5% of the copy bandwidth). Measured on 2.46e8 packets
+// of the large recipe, 2048-packet tiles: 61.9 -> 41.7 us per 10^6 packets,
+// 45.4 -> 29.5 warp instructions per packet, against the form with a chained
+// hash of the pixels in arrival order, a walk for the unwrap chains and the
+// copy-out as a phase of the workers.
+//
+// A CTA is NW worker warps, which cluster one tile's range after the other,
+// and one service warp, which claims and plans the next tile and copies the
+// finished tiles' records out meanwhile. The workers synchronise among
+// themselves (cta_sync); the two sides hand tiles over through counters in
+// shared memory.
+constexpr int NW = NT / 32 - 1;    // worker warps
+constexpr int NTW = 32 * NW;       // worker threads
 constexpr int MAXSEG = MS;         // TDC packets a range may hold (more: the call is redone)
 constexpr uint64_t INVALID = ~0ull;
 constexpr uint32_t EMPTY = 0xFFFFu;
 constexpr long long MAX_SPIN = 1LL << 22;   // bounded look-back waits (~0.5 s)
-constexpr int LA0 = T / 2;         // look-ahead window loaded with the tile
-static_assert(T + LA0 <= C, "the look-ahead window fits the range");
+constexpr long long MAX_TRIES = 1LL << 18;  // bounded look-back waits of the service warp (~0.5 s)
+constexpr long long MAX_HANDOVER = 1LL << 25;   // bounded waits between the two sides (seconds)
 
-static_assert(T % NT == 0 && C % NT == 0 && T <= C && C <= 16384, "tile geometry");
-static_assert(C < 0xFFFF && HB % 2 == 0 && (HB & (HB - 1)) == 0 && HB * 2 <= C * 4, "16-bit hash heads");
+static_assert(T <= C && C % 1024 == 0, "tile geometry");
+constexpr int KM = (C + NTW - 1) / NTW;   // packets of a range a worker thread holds
+constexpr int TB = 256 * TR;              // cell table: bits, words
+constexpr int TW = TB / 32;
+constexpr int OHB = C >= 8192 ? 2048 : 1024;   // buckets of the second hits of a table cell
+constexpr uint16_t NOLAB = 0xFFFFu, PEAK = 0x4000u;   // a position's label entry
+constexpr int QN = C / 2;          // pairs the union queue holds
+static_assert(C <= 0x4000 && (TR & (TR - 1)) == 0 && TR >= 256, "16-bit slots, positions and label entries");
+__device__ __forceinline__ void cta_sync() { asm volatile("bar.sync 1, %0;" ::"n"(NTW) : "memory"); }
 
 // ------------------------------------------------------------------ helpers
 // Checked build (-DTPX_CHECKED): every data-dependent shared-memory or global
@@ -47,8 +69,6 @@ __device__ unsigned long long g_phase[32];
 #define TPX_PH(k) do {} while (0)
 #endif
 
-__device__ __forceinline__ int pad(int p) { return p + (p >> 3); }   // conflict-free 8-wide walks
-
 // kept-pixel record: [63:40] tof+bias | [39:30] ToT | [29:16] segment | [15:8] y | [7:0] x;
 // the low 30 bits are the pixel's cell (segment, y, x)
 __device__ __forceinline__ uint64_t mkrec(uint32_t tofb, uint32_t seg, uint32_t tot, uint32_t x, uint32_t y) {
@@ -63,9 +83,12 @@ __device__ __forceinline__ uint32_t r_cell(uint64_t r) { return (uint32_t)r & 0x
 // |d| <= dt, for 0 <= dt < 2^31
 __device__ __forceinline__ bool within(int d, int dt) { return (uint32_t)d + (uint32_t)dt <= 2u * (uint32_t)dt; }
 
-__device__ __forceinline__ unsigned ld_acquire(const unsigned *p) {
+// The flags are polled with relaxed loads and a fence follows once they are
+// all there: an acquiring load empties the SM's L1, which the CTA's big-range
+// path reads through, at every poll (2.4x the time of an uneven batch).
+__device__ __forceinline__ unsigned ld_relaxed(const unsigned *p) {
     unsigned v;
-    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
     return v;
 }
 __device__ __forceinline__ void st_release(unsigned *p, unsigned v) {
@@ -86,66 +109,121 @@ __device__ __forceinline__ GAgg ld_agg(const GAgg *src) {
     return a;
 }
 
-// hash of a (segment, x, y) cell
-__device__ __forceinline__ uint32_t hcell(int seg, int x, int y) {
-    return (uint32_t)(x + 67 * y + 1543 * seg) & (HB - 1);
+// A (segment, y, x) cell's bit of the cell table: TR rows of 256 columns, the
+// rows of a shot shifted by its number, so that a row of cells is a run of bits
+// and the row above it the run 256 bits on. The kept pixels that find their
+// bit free take slots in the order of the bits (the table with the rank of
+// each word), so a pixel's right-hand neighbour is the next slot and the
+// neighbours in a row consecutive slots; a pixel that finds its bit taken (a
+// second hit of the cell, or another shot's cell) takes a slot after all of
+// them and a place in a chained hash.
+constexpr uint32_t HS = 101u << 8;
+__device__ __forceinline__ uint32_t tbit(uint64_t r) {
+    return (((uint32_t)r & 0xFFFFu) + HS * (uint32_t)r_seg(r)) & (TB - 1);
 }
+__device__ __forceinline__ uint32_t ohash(uint32_t bit) { return (bit ^ (bit >> 9)) & (OHB - 1); }
 
-// Union-find over a shared-memory parent array, addressed explicitly in the
-// shared window (32-bit addresses, ld/st.volatile.shared, atom.shared.cas).
-__device__ __forceinline__ uint32_t sh_ld(uint32_t a) {
-    uint32_t v;
-    asm volatile("ld.volatile.shared.u32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
+// Union-find over 16-bit parents addressed in the shared window (pb: the
+// array's shared address). Pointers set by the neighbour pass go forward in
+// (y, x); roots are linked the larger slot under the smaller.
+__device__ __forceinline__ uint32_t uf_ld(uint32_t pb, uint32_t x) {
+    unsigned short v;
+    asm volatile("ld.volatile.shared.u16 %0, [%1];" : "=h"(v) : "r"(pb + 2 * x) : "memory");
     return v;
 }
-__device__ __forceinline__ void sh_st(uint32_t a, uint32_t v) {
-    asm volatile("st.volatile.shared.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
+__device__ __forceinline__ void uf_st(uint32_t pb, uint32_t x, uint32_t v) {
+    asm volatile("st.volatile.shared.u16 [%0], %1;" ::"r"(pb + 2 * x), "h"((unsigned short)v) : "memory");
 }
-__device__ __forceinline__ uint32_t sh_cas(uint32_t a, uint32_t cmp, uint32_t v) {
-    uint32_t o;
-    asm volatile("atom.shared.cas.b32 %0, [%1], %2, %3;" : "=r"(o) : "r"(a), "r"(cmp), "r"(v) : "memory");
+__device__ __forceinline__ uint32_t uf_cas(uint32_t pb, uint32_t x, uint32_t cmp, uint32_t v) {
+    unsigned short o;
+    asm volatile("atom.shared.cas.b16 %0, [%1], %2, %3;"
+                 : "=h"(o) : "r"(pb + 2 * x), "h"((unsigned short)cmp), "h"((unsigned short)v) : "memory");
     return o;
 }
-__device__ __forceinline__ uint32_t find_ro(uint32_t pbase, uint32_t x) {
-    uint32_t p;
-    while ((p = sh_ld(pbase + 4 * x) & 0xFFFFu) != x) x = p;
+__device__ __forceinline__ uint32_t uf_find(uint32_t pb, uint32_t x) {
+    for (;;) {
+        const uint32_t px = uf_ld(pb, x);
+        if (px == x) return x;
+        const uint32_t g = uf_ld(pb, px);
+        if (g == px) return px;
+        uf_st(pb, x, g);   // path halving: g is an ancestor of x
+        x = g;
+    }
+}
+__device__ __forceinline__ uint32_t uf_root(uint32_t pb, uint32_t x) {   // changes nothing
+    uint32_t px;
+    while ((px = uf_ld(pb, x)) != x) x = px;
     return x;
+}
+// lock-free union: the larger root slot is linked under the smaller
+__device__ void uf_unite(uint32_t pb, uint32_t a, uint32_t b) {
+    for (;;) {
+        a = uf_find(pb, a);
+        b = uf_find(pb, b);
+        if (a == b) return;
+        const uint32_t lo = min(a, b), hi = max(a, b);
+        if (uf_cas(pb, hi, hi, lo) == hi) return;
+        a = lo;
+        b = hi;   // hi was linked meanwhile: find again
+    }
 }
 
 // --------------------------------------------------------------- smem layout
 struct __align__(16) Smem {
-    uint64_t buf[C + C / 8];                          // packets, then kept-pixel records
-    uint32_t parent[C];                               // union-find; then member links and
-                                                      // root positions (CC) / peak list (PAPER)
-    union { uint16_t head[HB]; uint32_t mhead[C]; } u1; // hash heads (16-bit positions), then
-                                                      // member-list heads
-    union { uint16_t next[C]; uint16_t rootof[C]; } u2;
-    uint8_t notpeak[C];
-    uint32_t lbits[C / 32];       // CC: the tile's label positions, one bit each
-    uint16_t lpre[C / 32];        // labels before each bitmap word
-    long long tdc_t[MAXSEG];      // unwrapped trigger times of the range
+    union {
+        struct {
+            uint64_t srec[C + 4];     // while the range is read: its TDC packets (all packets
+                                      // where a pixel wrap is near) by position; then the
+                                      // kept-pixel records by slot
+            uint16_t spos[C];         // wraps by position where a wrap is near; then the
+                                      // records' positions in the range
+            uint16_t par[C];          // union-find parents, then roots
+            union {
+                struct { uint32_t bits[TW]; uint16_t rank[TW], ohead[OHB]; } t;
+                uint32_t mhead[C];
+            } u1;                     // the cell table, then (CC) member-list heads and labels by root
+            union { uint32_t queue[QN]; uint16_t mnext[C]; uint16_t lab[C]; } u2;
+                                      // pairs left to unite, member links, labels by position
+            union { uint16_t onext[C]; uint16_t rootpos[C]; } u5;   // chains of second hits; CC: the roots
+            uint8_t notpeak[C];
+            union { uint32_t lbits[C / 32]; uint32_t tmask[C / 32]; uint32_t rwalk[C / 32]; } u3;
+                                      // TDC packets of each 32 positions; slots to walk again;
+                                      // then the label positions, one bit each
+            union { uint16_t lpre[C / 32]; uint16_t tpre[C / 32]; } u4;   // bits before each word
+        };
+        unsigned char big[BIG_REGION];   // the big-range path's shared scratch
+    };
+    long long tdc_t[MAXSEG + 1];  // unwrapped trigger times of the range, and a time past all
     uint16_t tdc_pos[MAXSEG];     // their positions
-    GAgg E;                       // unwrap state before the tile (from the pre-pass)
+    // the tile in work and the next one, planned by the service warp
+    struct Plan {
+        GAgg E;                   // unwrap state before the range (pixels) and the tile (TDCs)
+        long long tile;
+        int f, w0, len, term, slow;
+        unsigned status;
+    } plan[2];
     long long j0;                 // pixel wrap step from the last pixel before the range to its first
-    int warp_int[NW + 1];
+    int warp_int[NW + 2];
     unsigned long long cnt[C_NUM];   // this tile's counters
     unsigned long long acc[C_NUM];   // this CTA's counters, added to the call's at its end
-    long long next_tile;          // claimed while the current tile runs
-    long long tile;
-    long long clo;
-    long long tlo;                // trigger offset of a batch tile
-    // staged tiles awaiting their offsets: a ring, entry k staged in slot k
-    // (one entry for a single stream, RING in a batch)
+    long long clo;                // unstaged: the tile's record offset
+    // finished tiles awaiting their offsets: entry k of the CTA, staged in slot
+    // k % (1 for a single stream, RING in a batch). A tile with nothing to write
+    // (most tiles of a run whose shots span several) takes none.
     struct Pend {
         long long tile, ntr;      // the tile; its trigger total (single streams)
         int ncl, ntdc, run;       // its records and triggers; its run
         bool first, big;          // the run's first tile; records in the big-range slot
     } pend[4];
-    int pend_head, pend_count;
-    int first_tdc;
+    // the handover: tiles planned and finished, entries made and copied out
+    // (monotonic counts)
+    int planned, produced, entries, consumed;
     int first_pix;                // first pixel of the range
-    int la_first[3];              // first TDC packet past the tile (window, then rotating chunk slots)
-    int nroot;                    // CC: clusters of the tile (roots appended to the root list)
+    int ntdc;                     // TDC packets of the range
+    int nroot;                    // clusters of the tile
+    int nov;                      // kept pixels that found their table bit taken
+    int qn, rw;                   // pairs queued for a union; a slot has to be walked again
+    unsigned n_pre, n_bg, n_pk;   // dropped before a trigger, background, local maxima
     unsigned status;
 #ifdef TPX_PHASE_TIMING
     unsigned long long ph[32];
@@ -156,7 +234,7 @@ struct __align__(16) Smem {
 // reserved per CTA)
 static_assert(MINB * (sizeof(Smem) + 1024) <= 228 * 1024, "shared memory of the tile geometry");
 
-// a batch keeps up to RING staged tiles per CTA waiting for their offsets (a
+// a batch keeps up to RING finished tiles per CTA waiting for their offsets (a
 // tile behind a big range need not wait for it); a single stream keeps one
 constexpr int RING = kBatchRing;
 static_assert(RING >= 1 && RING <= 4, "the ring of staged tiles");
@@ -173,9 +251,10 @@ struct BrMom { unsigned long long s_tot, s_x, s_y, s_tt, best; unsigned n, npk; 
 static_assert(sizeof(BrMom) == 48, "moment record");
 // shared scratch: the tile arrays in front of the trigger tables
 constexpr int BR_REGION = (int)offsetof(Smem, tdc_t);
+static_assert(BR_REGION >= BIG_REGION, "the big-range scratch");
 // the neighbour pass reads the sorted records through shared memory, BR_CH
 // pixels at a time with the records before them that they can reach
-constexpr int BR_CH = 2 * NT;
+constexpr int BR_CH = 2 * NT;   // pixels of a step of the neighbour pass
 constexpr int BR_SB = 2 * BR_CH;
 constexpr int BR_FIXED = 4 * (BR_BINS + 4) + 4 * BR_LW + 2 * BR_LW + 4 * 5 * BR_S + 4 * 16 + 8 * BR_SB;
 // kept pixels: a 16-bit parent and a local-maximum bit each
@@ -183,7 +262,6 @@ constexpr int BR_N0 = ((BR_REGION - BR_FIXED) * 8 / 17) & ~63;
 constexpr int BR_N = BR_N0 < 65472 ? BR_N0 : 65472;
 static_assert(BR_N > C && BR_N % 64 == 0, "a big range holds more pixels than a tile");
 static_assert(2 * BR_N + BR_N / 8 + BR_FIXED <= BR_REGION, "big-range shared scratch");
-static_assert(BR_BINS % NT == 0 && BR_LW % NT == 0, "bins and label words split evenly over the CTA");
 // per-CTA global scratch: records by position, sorted records and their
 // positions, moments by root, and the staged cluster records (a big range
 // may hold up to one cluster per kept pixel)
@@ -207,7 +285,7 @@ __device__ unsigned block_scan_vadd2(Smem &S, unsigned v, unsigned *total) {
         if (lane >= o) incl = __vadd2(incl, u);
     }
     if (lane == 31) S.warp_int[w] = (int)incl;
-    __syncthreads();
+    cta_sync();
     if (w == 0) {
         const unsigned x = lane < NW ? (unsigned)S.warp_int[lane] : 0u;
         unsigned xi = x;
@@ -219,10 +297,10 @@ __device__ unsigned block_scan_vadd2(Smem &S, unsigned v, unsigned *total) {
         if (lane < NW) S.warp_int[lane] = (int)__vsub2(xi, x);
         if (lane == NW - 1) S.warp_int[NW] = (int)xi;
     }
-    __syncthreads();
+    cta_sync();
     const unsigned r = __vadd2((unsigned)S.warp_int[w], __vsub2(incl, v));
     *total = (unsigned)S.warp_int[NW];
-    __syncthreads();
+    cta_sync();
     return r;
 }
 
@@ -236,7 +314,7 @@ __device__ int block_scan_int(Smem &S, int v, int *total) {
         if (lane >= o) incl += u;
     }
     if (lane == 31) S.warp_int[w] = incl;
-    __syncthreads();
+    cta_sync();
     if (w == 0) {
         int x = lane < NW ? S.warp_int[lane] : 0;
         int xi = x;
@@ -248,10 +326,10 @@ __device__ int block_scan_int(Smem &S, int v, int *total) {
         if (lane < NW) S.warp_int[lane] = xi - x;
         if (lane == NW - 1) S.warp_int[NW] = xi;
     }
-    __syncthreads();
+    cta_sync();
     int r = S.warp_int[w] + incl - v;
     *total = S.warp_int[NW];
-    __syncthreads();
+    cta_sync();
     return r;
 }
 
@@ -293,7 +371,7 @@ __device__ __forceinline__ LbScan lb_scan(const unsigned *flags, long long hi, l
     for (int j = 0; j < LB; ++j) {
         const long long q = hi - LB * lane - j;
         if (q < lo) { rdy |= 1u << j; continue; }
-        const unsigned f = ld_acquire(&flags[q]);
+        const unsigned f = ld_relaxed(&flags[q]);
         if ((f >> 2) == seq && (f & 3u)) {
             rdy |= 1u << j;
             if ((f & 3u) == 2u) inc |= 1u << j;
@@ -330,6 +408,7 @@ __device__ longlong2 lookback_count_warp(const Params &p, long long tile, unsign
             }
             __nanosleep(64);
         }
+        __threadfence();
         long long v = 0, w = 0;
 #pragma unroll
         for (int j = 0; j < LBC; ++j) {
@@ -351,75 +430,96 @@ __device__ longlong2 lookback_count_warp(const Params &p, long long tile, unsign
     return acc;
 }
 
-// The CC union-find array holds one 32-bit word per position: the parent in
-// the lower half, in the upper half the pixel's second partner (NO_EXT: none;
-// REWALK: more than two, re-walked at the unions). Finds look at the lower
-// halves; writes keep the upper halves.
-constexpr uint32_t NO_EXT = 0xFFFFu, REWALK = 0xFFFEu;
-static_assert(C < (int)REWALK, "positions fit below the markers");
-static_assert((C / 32) % 32 == 0, "the label bitmap splits evenly over a warp");
+static_assert((C / 32) % 32 == 0, "the position bitmaps split evenly over a warp");
 
-__device__ __forceinline__ uint32_t find_hw(uint32_t pbase, uint32_t x) {
-    for (;;) {
-        const uint32_t w = sh_ld(pbase + 4 * x);
-        const uint32_t px = w & 0xFFFFu;
-        if (px == x) return x;
-        const uint32_t g = sh_ld(pbase + 4 * px) & 0xFFFFu;
-        if (g == px) return px;
-        sh_st(pbase + 4 * x, (w & 0xFFFF0000u) | g);   // path halving: g is an ancestor of x
-        x = g;
-    }
+// the slot of the table's first pixel at or after a bit
+__device__ __forceinline__ int rank_at(const Smem &S, uint32_t bit) {
+    return (int)S.u1.t.rank[bit >> 5] + __popc(S.u1.t.bits[bit >> 5] & ((1u << (bit & 31)) - 1u));
+}
+// the slots [*s0, *s1) of the table's pixels in the cells dlo..dhi columns from
+// the cell at `bit` (of column x), in the row dy above
+__device__ __forceinline__ void row_slots(const Smem &S, uint32_t bit, int dy, int dlo, int dhi, int *s0, int *s1) {
+    const uint32_t row = (bit + 256u * (uint32_t)dy) & (TB - 1);
+    *s0 = rank_at(S, row + dlo);
+    const uint32_t e = row + dhi;
+    *s1 = rank_at(S, e) + (int)((S.u1.t.bits[e >> 5] >> (e & 31)) & 1u);
 }
 
-// lock-free union: the larger root position is linked under the smaller
-__device__ void unite_hw(uint32_t pbase, uint32_t a, uint32_t b) {
-    for (;;) {
-        a = find_hw(pbase, a);
-        b = find_hw(pbase, b);
-        if (a == b) return;
-        const uint32_t lo = min(a, b), hi = max(a, b);
-        const uint32_t w = sh_ld(pbase + 4 * hi);
-        if ((w & 0xFFFFu) == hi && sh_cas(pbase + 4 * hi, w, (w & 0xFFFF0000u) | lo) == w) return;
-        a = lo;
-        b = hi;   // hi was linked meanwhile: find again
-    }
-}
-
-// a pixel with more than two partners: unite it with each partner in the
-// forward half of its box (Sec. V.A), found again in the cell hash
-template <int MODE>
-__device__ void rewalk_unite(const Smem &S, const Params &p, uint32_t pbase, int q) {
-    const uint64_t r = S.buf[pad(q)];
-    const int x = r_x(r), y = r_y(r), sg = r_seg(r), tb = r_tof(r);
-    for (int dx = 0; dx <= p.rx; ++dx) {
-        const int cx = x + dx;
-        if (cx > 255) break;
-        for (int dy = (dx == 0 ? 0 : -p.ry); dy <= p.ry; ++dy) {
-            const int cy = y + dy;
-            if (cy < 0 || cy > 255) continue;
-            for (uint32_t j = S.u1.head[hcell(sg, cx, cy)]; j != EMPTY; j = S.u2.next[j]) {
-                if (!TPX_IN(j, C)) break;
-                if (dx == 0 && dy == 0 && (int)j <= q) continue;
-                const uint64_t rj = S.buf[pad((int)j)];
-                if (r_x(rj) != cx || r_y(rj) != cy || r_seg(rj) != sg) continue;
-                const int d = r_tof(rj) - tb;
-                if (d < -p.dt || d > p.dt) continue;
-                unite_hw(pbase, (uint32_t)q, j);
-            }
+// Walks a table pixel's candidates again and unites it with each partner in
+// the forward half of its box (Sec. V.A).
+__device__ void rewalk_unite(const Smem &S, const Params &p, uint32_t pb, int i) {
+    const uint64_t r = S.srec[i];
+    const int x = r_x(r), y = r_y(r), tb = r_tof(r);
+    const uint32_t bit = tbit(r), cell = r_cell(r);
+    for (int dy = 0; dy <= p.ry && y + dy <= 255; ++dy) {
+        const int dlo = dy == 0 ? 0 : -min(p.rx, x), dhi = min(p.rx, 255 - x);
+        int j, s1;
+        row_slots(S, bit, dy, dlo, dhi, &j, &s1);
+        for (; j < s1; ++j) {
+            if (j == i || !TPX_IN(j, C)) continue;
+            const uint64_t rj = S.srec[j];
+            if (r_cell(rj) - (cell + (uint32_t)(256 * dy + dlo)) > (uint32_t)(dhi - dlo)) continue;
+            if (within(r_tof(rj) - tb, p.dt)) uf_unite(pb, (uint32_t)i, (uint32_t)j);
         }
     }
 }
 
+// An adjacent pair's local-maximum flags: equal ToT goes to the later pixel
+// (Sec. V.B).
+__device__ __forceinline__ bool dimmer(const Smem &S, int i, int tot, int j, int aj) {
+    return aj > tot || (aj == tot && S.spos[j] > S.spos[i]);
+}
+
+// A pair left to unite once the pointers stand; a full queue marks the pixel
+// for a second walk.
+__device__ __forceinline__ void queue_pair(Smem &S, int i, int j) {
+    const int at = atomicAdd(&S.qn, 1);
+    if (at < QN) S.u2.queue[at] = ((uint32_t)i << 16) | (uint32_t)j;
+    else { atomicOr(&S.u3.rwalk[i >> 5], 1u << (i & 31)); S.rw = 1; }
+}
+
+// One row (dy above) of the box of a pixel outside the table: its adjacent
+// pixels in the table, and among the others those after it.
+// CC: the pairs are queued, or united at once in a second walk.
+template <int MODE, bool UNITE>
+__device__ void overflow_row(Smem &S, const Params &p, uint32_t pb, int o, int dy, int nb) {
+    const int i = nb + o;
+    const uint64_t r = S.srec[i];
+    const int x = r_x(r), y = r_y(r), tb = r_tof(r), tot = r_tot(r);
+    if (y + dy < 0 || y + dy > 255) return;
+    const uint32_t bit = tbit(r), cell = r_cell(r);
+    const int dlo = -min(p.rx, x), dhi = min(p.rx, 255 - x);
+    const uint32_t c0 = cell + (uint32_t)(256 * dy + dlo);
+    auto visit = [&](int j) {
+        const uint64_t rj = S.srec[j];
+        if (r_cell(rj) - c0 > (uint32_t)(dhi - dlo) || !within(r_tof(rj) - tb, p.dt)) return;
+        S.notpeak[dimmer(S, i, tot, j, r_tot(rj)) ? i : j] = 1;
+        if (MODE != TPX_MODE_CC) return;
+        if (UNITE) uf_unite(pb, (uint32_t)i, (uint32_t)j); else queue_pair(S, i, j);
+    };
+    int j, s1;
+    row_slots(S, bit, dy, dlo, dhi, &j, &s1);
+    for (; j < s1; ++j)
+        if (TPX_IN(j, C)) visit(j);
+    const uint32_t row = (bit + 256u * (uint32_t)dy) & (TB - 1);
+    for (int dx = dlo; dx <= dhi; ++dx)
+        for (uint32_t q = S.u1.t.ohead[ohash(row + dx)]; q != EMPTY; q = S.u5.onext[q]) {
+            if (!TPX_IN(nb + q, C)) break;
+            // (cells of the same chain: visited for the cell they are in)
+            if ((int)q > o && r_cell(S.srec[nb + q]) == cell + (uint32_t)(256 * dy + dx)) visit(nb + (int)q);
+        }
+}
+
 // One warp resolves the record offset of tile tl holding nc records
 // (decoupled look-back over the counts), publishes its inclusive count and,
-// for the last tile, the call's totals; the offset is left in S.clo. In a
-// batch the chain also carries the tile's nt triggers (offset in S.tlo), and a
-// run's first tile records the run's record and trigger offsets.
+// for the last tile, the call's totals; the offsets come back in *O. In a
+// batch the chain also carries the tile's nt triggers, and a run's first tile
+// records the run's record and trigger offsets.
 // Without `block`, gives up (false, nothing published) when a predecessor's
 // count is not out yet.
 template <bool BATCH>
-__device__ bool resolve_offset(Smem &S, const Params &p, unsigned seq, long long tl, int nc, long long ntr, int nt,
-                               int run, bool run_first, bool block = true) {
+__device__ bool resolve_offset(const Params &p, unsigned seq, long long tl, int nc, long long ntr, int nt, int run,
+                               bool run_first, bool block, longlong2 *O) {
     unsigned st2 = 0;
     longlong2 Ow = make_longlong2(0, 0);
     bool ready = true;
@@ -431,9 +531,6 @@ __device__ bool resolve_offset(Smem &S, const Params &p, unsigned seq, long long
             if (BATCH) __stcg(&p.bt.tcpre[tl], Ow.y + (long long)nt);
             st_release(&p.ts.cflags[tl], (seq << 2) | 2u);
         }
-        S.clo = Ow.x;
-        S.tlo = Ow.y;
-        if (st2) atomicOr(&S.status, st2);
         if (BATCH && run_first) {
             p.bt.run_rec_off[run] = Ow.x;
             p.bt.run_trig_off[run] = Ow.y;
@@ -450,101 +547,103 @@ __device__ bool resolve_offset(Smem &S, const Params &p, unsigned seq, long long
             if (nt_all > p.trig_cap) atomicOr(&p.ctl->status, ST_TRIG_CAP);
         }
     }
+    *O = Ow;
     return true;
 }
 
-// Staged output: a tile's records (in label order) and, in a batch, its
-// trigger times wait in a staging slot of the CTA until a later tile of the
-// CTA (or the end of the kernel) resolves their offset, when the
-// predecessors' counts are long published; then one warp copies them out,
-// coalesced, eight loads in flight per lane. The staged tiles form a ring
-// (one entry for a single stream, RING in a batch): the oldest entries go out
-// in order while their offsets resolve; the warp waits for the oldest only
-// when the ring is full (the CTA needs the slot) or with `all` (the kernel's
-// end). Called by one whole warp.
+// Copies a finished tile's staged records (in label order) and, in a batch,
+// its trigger times to their offset, by the service warp: coalesced, eight
+// loads in flight per lane. False: a predecessor's count is not out yet (and
+// `block` not set); the caller tries again.
 template <bool BATCH>
-__device__ void flush_ring_warp(Smem &S, const Params &p, unsigned seq, bool all) {
+__device__ bool copy_out(Smem &S, const Params &p, unsigned seq, int slot, bool block) {
     constexpr int NP = BATCH ? RING : 1;
     const int lane = threadIdx.x & 31;
     constexpr int WPR = (int)(sizeof(tpx_record) / 8);
-    for (;;) {
-        const int cnt = S.pend_count;
-        if (cnt == 0) break;
-        const int slot = S.pend_head;
-        const long long pt = S.pend[slot].tile, ntr = S.pend[slot].ntr;
-        const int nc = S.pend[slot].ncl, nt = S.pend[slot].ntdc, run = S.pend[slot].run;
-        const bool first = S.pend[slot].first, big = S.pend[slot].big;
-        if (!resolve_offset<BATCH>(S, p, seq, pt, nc, ntr, nt, run, first, all || cnt == NP)) break;
-        __syncwarp();
-        const long long O = S.clo;
-        const long long keep = min((long long)nc, max(0LL, p.cl_cap - O));
-        const unsigned long long *src = reinterpret_cast<const unsigned long long *>(
-            (BATCH && big) ? br_stage(p, slot) : p.stage + ((long long)blockIdx.x * NP + slot) * C);
-        if (p.rec64) {   // 64-byte records: the first 8 words of each staged record
-            unsigned long long *d64 = reinterpret_cast<unsigned long long *>(p.clusters) + O * 8;
-            const long long nw = keep * 8;
-            for (long long w0 = lane; w0 < nw; w0 += 32 * 8) {
-                unsigned long long v[8];
-#pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    const long long w = w0 + 32 * u;
-                    v[u] = w < nw ? __ldcg(src + (w >> 3) * WPR + (w & 7)) : 0ull;
-                }
-#pragma unroll
-                for (int u = 0; u < 8; ++u)
-                    if (w0 + 32 * u < nw) d64[w0 + 32 * u] = v[u];
-            }
-        }
-        unsigned long long *dst = reinterpret_cast<unsigned long long *>(p.clusters + O);
-        const long long nw = p.rec64 ? 0 : keep * WPR;
+    const long long pt = S.pend[slot].tile, ntr = S.pend[slot].ntr;
+    const int nc = S.pend[slot].ncl, nt = S.pend[slot].ntdc, run = S.pend[slot].run;
+    const bool first = S.pend[slot].first, big = S.pend[slot].big;
+    longlong2 Ow;
+    if (!resolve_offset<BATCH>(p, seq, pt, nc, ntr, nt, run, first, block, &Ow)) return false;
+    const long long O = Ow.x;
+    const long long keep = min((long long)nc, max(0LL, p.cl_cap - O));
+    const unsigned long long *src = reinterpret_cast<const unsigned long long *>(
+        (BATCH && big) ? br_stage(p, slot) : p.stage + ((long long)blockIdx.x * NP + slot) * C);
+    if (p.rec64) {   // 64-byte records: the first 8 words of each staged record
+        unsigned long long *d64 = reinterpret_cast<unsigned long long *>(p.clusters) + O * 8;
+        const long long nw = keep * 8;
         for (long long w0 = lane; w0 < nw; w0 += 32 * 8) {
             unsigned long long v[8];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) v[u] = w0 + 32 * u < nw ? __ldcg(src + w0 + 32 * u) : 0ull;
+            for (int u = 0; u < 8; ++u) {
+                const long long w = w0 + 32 * u;
+                v[u] = w < nw ? __ldcg(src + (w >> 3) * WPR + (w & 7)) : 0ull;
+            }
 #pragma unroll
             for (int u = 0; u < 8; ++u)
-                if (w0 + 32 * u < nw) dst[w0 + 32 * u] = v[u];
+                if (w0 + 32 * u < nw) d64[w0 + 32 * u] = v[u];
         }
-        if (BATCH) {
-            const long long TO = S.tlo;
-            const long long tkeep = min((long long)nt, max(0LL, p.trig_cap - TO));
-            const long long *ts = p.bt.tstage + ((long long)blockIdx.x * NP + slot) * T;
-            for (long long i = lane; i < tkeep; i += 32) p.trig[TO + i] = __ldcg(ts + i);
-        }
-        __syncwarp();
-        if (lane == 0) {
-            S.pend_head = (slot + 1) % NP;
-            S.pend_count = cnt - 1;
-        }
-        __syncwarp();
     }
+    unsigned long long *dst = reinterpret_cast<unsigned long long *>(p.clusters + O);
+    const long long nw = p.rec64 ? 0 : keep * WPR;
+    for (long long w0 = lane; w0 < nw; w0 += 32 * 8) {
+        unsigned long long v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = w0 + 32 * u < nw ? __ldcg(src + w0 + 32 * u) : 0ull;
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            if (w0 + 32 * u < nw) dst[w0 + 32 * u] = v[u];
+    }
+    if (BATCH) {
+        const long long TO = Ow.y;
+        const long long tkeep = min((long long)nt, max(0LL, p.trig_cap - TO));
+        const long long *ts = p.bt.tstage + ((long long)blockIdx.x * NP + slot) * T;
+        for (long long i = lane; i < tkeep; i += 32) p.trig[TO + i] = __ldcg(ts + i);
+    }
+    __syncwarp();
+    return true;
 }
 
 // the exact integer moments of one cluster from its member list (Sec. V.C)
 // and its canonical label: the earliest member in (time, position) order
 struct Moments {
-    long long s_tot, s_x, s_y, s_tt;   // s_tt: sum of ToT x biased ToF
+    long long s_tt;                    // sum of ToT x biased ToF
+    uint32_t s_tot, s_x, s_y;          // a range's sums fit 32 bits (C x 1023 x 255 < 2^32)
     int n, npk;
+    int seg;                           // its shot, as a trigger index of the range
     uint32_t best_lo;                  // label position
     int tofb0;                         // its biased ToF
 };
+static_assert((unsigned long long)C * 1023 * 255 < (1ull << 32), "32-bit moment sums");
 
 __device__ __forceinline__ Moments walk_members(const Smem &S, const Params &p, uint32_t head) {
-    const uint16_t *mnext = reinterpret_cast<const uint16_t *>(S.parent);
     uint64_t best = ~0ull;
-    Moments m{0, 0, 0, 0, 0, 0, 0, 0};
-    for (uint32_t k = head; k != EMPTY; k = mnext[k]) {
-        if (!TPX_IN(k, C)) break;
-        const uint64_t rm = S.buf[pad((int)k)];
-        const long long tot = r_tot(rm);
-        const int tf = r_tof(rm);
-        best = min(best, ((uint64_t)tf << 16) | k);
+    Moments m{0, 0, 0, 0, 0, 0, 0, 0, 0};
+    // the next member's words are on their way while this one is added up
+    uint32_t k = head;
+    if (!TPX_IN(k, C)) return m;
+    uint64_t rm = S.srec[k];
+    uint32_t pos = S.spos[k], dimmed = S.notpeak[k];
+    m.seg = r_seg(rm);
+    for (;;) {
+        const uint32_t nx = S.u2.mnext[k];
+        const bool more = nx != EMPTY && TPX_IN(nx, C);
+        const uint32_t kn = more ? nx : k;
+        const uint64_t rn = S.srec[kn];
+        const uint32_t pn = S.spos[kn], dn = S.notpeak[kn];
+        const uint32_t tot = (uint32_t)r_tot(rm), tf = (uint32_t)r_tof(rm);
+        best = min(best, ((uint64_t)tf << 16) | pos);
         m.n += 1;
-        m.npk += (S.notpeak[k] & 1) ? 0 : 1;
+        m.npk += dimmed ? 0 : 1;
         m.s_tot += tot;
-        m.s_x += tot * r_x(rm);
-        m.s_y += tot * r_y(rm);
-        m.s_tt += tot * (long long)tf;
+        m.s_x += tot * (uint32_t)r_x(rm);
+        m.s_y += tot * (uint32_t)r_y(rm);
+        m.s_tt += (long long)((uint64_t)tot * tf);
+        if (!more) break;
+        k = nx;
+        rm = rn;
+        pos = pn;
+        dimmed = dn;
     }
     m.best_lo = (uint32_t)(best & 0xFFFFu);
     m.tofb0 = (int)(best >> 16);
@@ -552,20 +651,19 @@ __device__ __forceinline__ Moments walk_members(const Smem &S, const Params &p, 
 }
 
 // the record of a cluster whose label pixel lies at position best_lo of the
-// tile at stream position base
-__device__ __forceinline__ void put_record(tpx_record *dst, const Moments &m, const Smem &S, const Params &p,
-                                           long long base, long long shot0) {
-    const int seg = r_seg(S.buf[pad((int)m.best_lo)]);
+// range at stream position base
+__device__ __forceinline__ tpx_record make_record(const Moments &m, const Smem &S, const Params &p, long long base,
+                                                  long long shot0) {
     const long long tofc0 = (long long)m.tofb0 - kTofBias;
-    const long long s_t = m.s_tt - (long long)m.tofb0 * m.s_tot;
+    const long long s_t = m.s_tt - (long long)m.tofb0 * (long long)m.s_tot;
     tpx_record o;
     o.label = p.idx_base + base + m.best_lo;
-    o.shot = shot0 + seg;
-    o.t0 = S.tdc_t[seg] + tofc0;
+    o.shot = shot0 + m.seg;
+    o.t0 = S.tdc_t[m.seg] + tofc0;
     o.s_tot = m.s_tot; o.s_x = m.s_x; o.s_y = m.s_y; o.s_t = s_t;
     o.n = m.n; o.n_peaks = m.npk;
-    com_from_moments(m.s_x, m.s_y, s_t, m.s_tot, tofc0, &o.x, &o.y, &o.tof);
-    *dst = o;
+    com_from_moments(o.s_x, o.s_y, s_t, o.s_tot, tofc0, &o.x, &o.y, &o.tof);
+    return o;
 }
 
 // a record at position idx of the caller's buffer (88 bytes, or its first 64
@@ -583,7 +681,28 @@ __device__ __forceinline__ void out_record(const Params &p, long long idx, const
 
 // rank of label position lp among the tile's labels (after the bitmap scan)
 __device__ __forceinline__ int label_rank(const Smem &S, uint32_t lp) {
-    return (int)S.lpre[lp >> 5] + __popc(S.lbits[lp >> 5] & ((1u << (lp & 31)) - 1u));
+    return (int)S.u4.lpre[lp >> 5] + __popc(S.u3.lbits[lp >> 5] & ((1u << (lp & 31)) - 1u));
+}
+
+// the labels before each bitmap word, by one warp
+__device__ __forceinline__ void scan_label_bits(Smem &S) {
+    constexpr int WPL = C / 32 / 32;   // bitmap words per lane
+    const int lane = threadIdx.x & 31;
+    int c = 0;
+#pragma unroll
+    for (int k = 0; k < WPL; ++k) c += __popc(S.u3.lbits[lane * WPL + k]);
+    int incl = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int u = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += u;
+    }
+    int run = incl - c;
+#pragma unroll
+    for (int k = 0; k < WPL; ++k) {
+        S.u4.lpre[lane * WPL + k] = (uint16_t)run;
+        run += __popc(S.u3.lbits[lane * WPL + k]);
+    }
 }
 
 // ------------------------------------------------------------- big ranges
@@ -652,8 +771,8 @@ __device__ __forceinline__ void br_unite(uint32_t pb, unsigned a, unsigned b) {
     }
 }
 
-// The range of the tile at stream position `base` (first trigger packet at
-// f): its cluster count, or -1 with a status bit set when it goes back to
+// The range that starts at stream position `base` (first trigger packet at f,
+// the next one not before `from`): its cluster count, or -1 with a status bit set when it goes back to
 // the general path. Called by every thread of the CTA after the tile's
 // staging slot is free; writes the labels, local-maximum flags and staged
 // records, and replaces the tile's keep / drop counts by the whole range's.
@@ -668,8 +787,8 @@ __device__ __forceinline__ void br_unite(uint32_t pb, unsigned a, unsigned b) {
 #define BR_PH(k) do {} while (0)
 #endif
 template <bool BATCH>
-__device__ __noinline__ int big_range(Smem &S, const Params &p, long long base, long long rend, int f,
-                                      bool prev_global) {
+__device__ __noinline__ int big_range(Smem &S, const Params &p, long long base, long long rend, int f, int from,
+                                      bool prev_global, const GAgg &E, int slot) {
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
 #ifdef TPX_PHASE_TIMING
     long long br_t = clock64();
@@ -693,32 +812,31 @@ __device__ __noinline__ int big_range(Smem &S, const Params &p, long long base, 
     uint64_t *g_srec = g_rec + (BR_L + 1);
     uint16_t *g_spos = reinterpret_cast<uint16_t *>(g_srec + BR_N);
     BrMom *g_mom = reinterpret_cast<BrMom *>(g_spos + BR_N);
-    const GAgg E = S.E;
     const uint32_t pb = (uint32_t)__cvta_generic_to_shared(par);      // shared addresses
     const uint32_t nb_sh = (uint32_t)__cvta_generic_to_shared(npk);
     const int rx = p.rx, ry = p.ry, dtr = p.dt;
-    __syncthreads();
+    cta_sync();
     if (tid < 16) misc[tid] = tid < 4 ? INT_MAX : 0;
-    __syncthreads();
+    cta_sync();
 
-    // ---- the range end: the first TDC packet at or past C (the tile
-    // searched the positions below C); four packets per thread per step, the
+    // ---- the range end: the first TDC packet at or past `from` (the pre-pass
+    // found none in between); four packets per thread per step, the
     // steps' minima rotating over three slots as in the tile's look-ahead ----
     int L = 0;
     bool term = false;
     {
-        constexpr int STEP = 4 * NT;
-        long long q0 = C;
+        constexpr int STEP = 4 * NTW;
+        long long q0 = from;
         for (int k = 0;; ++k) {
             const long long lim = min((long long)BR_L, rend - base);
             if (q0 >= lim) { L = (int)lim; break; }
             if (tid == 0) misc[(k + 1) % 3] = INT_MAX;
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
-                const long long q = q0 + u * NT + tid;
+                const long long q = q0 + u * NTW + tid;
                 if (q < lim && (__ldcg(p.pk + base + q) >> 60) == 0x6u) atomicMin(&misc[k % 3], (int)q);
             }
-            __syncthreads();
+            cta_sync();
             const int lf = misc[k % 3];
             if (lf != INT_MAX) { L = lf + 1; term = true; break; }
             q0 += STEP;
@@ -728,7 +846,7 @@ __device__ __noinline__ int big_range(Smem &S, const Params &p, long long base, 
     if (!term && base + L < rend) { if (tid == 0) atomicOr(&S.status, ST_CAPACITY); return -1; }
 
     // ---- walk 2 over [0, L): wrap steps and TDC counts per contiguous chunk ----
-    const int kpd = (L + NT - 1) / NT;
+    const int kpd = (L + NTW - 1) / NTW;
     const int p0 = tid * kpd;
     int ntd = 0, jp = 0;
     {
@@ -777,8 +895,8 @@ __device__ __noinline__ int big_range(Smem &S, const Params &p, long long base, 
             ++li;
         }
     }
-    for (int s = tid; s < nseg; s += NT) { sg_n[s] = 0; sg_lo[s] = INT_MAX; sg_hi[s] = INT_MIN; }
-    __syncthreads();
+    for (int s = tid; s < nseg; s += NTW) { sg_n[s] = 0; sg_lo[s] = INT_MAX; sg_hi[s] = INT_MIN; }
+    cta_sync();
     // the trigger times (one warp, a scan of the TDC wrap steps)
     if (tid < 32) {
         bool has = E.tdc.n > 0;
@@ -809,7 +927,7 @@ __device__ __noinline__ int big_range(Smem &S, const Params &p, long long base, 
             has = true;
         }
     }
-    __syncthreads();
+    cta_sync();
 
     BR_PH(20);
     // ---- walk 4 over [0, L): shot, cut, timewalk, packed record per position
@@ -883,7 +1001,7 @@ __device__ __noinline__ int big_range(Smem &S, const Params &p, long long base, 
         }
         if (exc) atomicOr(&misc[7], (int)ST_EXCEPTION);
     }
-    __syncthreads();
+    cta_sync();
     const int N = misc[4];
     if (misc[7] || N > BR_N) {
         if (tid == 0) atomicOr(&S.status, misc[7] ? (unsigned)misc[7] : ST_CAPACITY);
@@ -929,30 +1047,30 @@ __device__ __noinline__ int big_range(Smem &S, const Params &p, long long base, 
             b0 += nb[k];
         }
     }
-    for (int b = tid; b < BR_BINS; b += NT) bins[b] = 0u;
-    __syncthreads();
+    for (int b = tid; b < BR_BINS; b += NTW) bins[b] = 0u;
+    cta_sync();
     auto bin_of = [&](uint64_t r) -> int {
         const int s = r_seg(r);
         return (sg_b0[s] + (r_tof(r) - sg_lo[s]) / sg_w[s]) * NS + r_x(r) / SW;
     };
     // ---- counting sort of the kept pixels by bin ----
-    for (int q = tid; q < L; q += NT) {
+    for (int q = tid; q < L; q += NTW) {
         const uint64_t r = g_rec[q];
         if (r != INVALID) atomicAdd(&bins[bin_of(r)], 1u);
     }
-    __syncthreads();
+    cta_sync();
     {
-        constexpr int BPT = BR_BINS / NT;   // bins per thread, contiguous
+        constexpr int BPT = (BR_BINS + NTW - 1) / NTW;   // bins per thread, contiguous
         unsigned c[BPT], s = 0;
 #pragma unroll
-        for (int k = 0; k < BPT; ++k) { c[k] = bins[tid * BPT + k]; s += c[k]; }
+        for (int k = 0; k < BPT; ++k) { c[k] = tid * BPT + k < BR_BINS ? bins[tid * BPT + k] : 0u; s += c[k]; }
         int total;
         unsigned run = (unsigned)block_scan_int(S, (int)s, &total);
 #pragma unroll
-        for (int k = 0; k < BPT; ++k) { bins[tid * BPT + k] = run; run += c[k]; }
+        for (int k = 0; k < BPT; ++k) { if (tid * BPT + k < BR_BINS) bins[tid * BPT + k] = run; run += c[k]; }
     }
-    __syncthreads();
-    for (int q = tid; q < L; q += NT) {
+    cta_sync();
+    for (int q = tid; q < L; q += NTW) {
         const uint64_t r = g_rec[q];
         if (r == INVALID) continue;
         const unsigned slot = atomicAdd(&bins[bin_of(r)], 1u);
@@ -961,10 +1079,10 @@ __device__ __noinline__ int big_range(Smem &S, const Params &p, long long base, 
         g_spos[slot] = (uint16_t)q;
     }
     // bins[b] is now the end of bin b (the start of bin b + 1)
-    for (int i = tid; i < N; i += NT) par[i] = (uint16_t)i;
-    for (int w = tid; w < BR_N / 32; w += NT) npk[w] = 0u;
-    for (int w = tid; w < BR_LW; w += NT) lbits[w] = 0u;
-    __syncthreads();
+    for (int i = tid; i < N; i += NTW) par[i] = (uint16_t)i;
+    for (int w = tid; w < BR_N / 32; w += NTW) npk[w] = 0u;
+    for (int w = tid; w < BR_LW; w += NTW) lbits[w] = 0u;
+    cta_sync();
 
     BR_PH(22);
     // ---- neighbour pass: every pixel of the sorted order is checked against
@@ -988,8 +1106,8 @@ __device__ __noinline__ int big_range(Smem &S, const Params &p, long long base, 
         const bool fits = e - lo <= BR_SB;
         if (tid == 0) misc[12] = 0;   // the chunk's task counter
         if (fits)
-            for (int j = lo + tid; j < e; j += NT) sbuf[j - lo] = g_srec[j];
-        __syncthreads();
+            for (int j = lo + tid; j < e; j += NTW) sbuf[j - lo] = g_srec[j];
+        cta_sync();
         auto rec_at = [&](int j) -> uint64_t { return fits ? sbuf[j - lo] : g_srec[j]; };
         // A warp takes 32 consecutive pixels at a time, the next task from the
         // chunk's counter (dense stretches take longer). A pixel's candidates
@@ -1053,16 +1171,16 @@ __device__ __noinline__ int big_range(Smem &S, const Params &p, long long base, 
                 br_unite(pb, (unsigned)ip, (unsigned)j);
             }
         }
-        __syncthreads();
+        cta_sync();
     }
     BR_PH(23);
     // compress: every pixel points to its root
-    for (int i = tid; i < N; i += NT) br_st(pb, (unsigned)i, br_find(pb, (unsigned)i));
-    __syncthreads();
+    for (int i = tid; i < N; i += NTW) br_st(pb, (unsigned)i, br_find(pb, (unsigned)i));
+    cta_sync();
     // roots: their moment records cleared, counted
     {
         int k = 0;
-        for (int i = tid; i < N; i += NT) {
+        for (int i = tid; i < N; i += NTW) {
             if (par[i] != i) continue;
             ++k;
             unsigned long long *m = reinterpret_cast<unsigned long long *>(&g_mom[i]);
@@ -1073,13 +1191,13 @@ __device__ __noinline__ int big_range(Smem &S, const Params &p, long long base, 
         k = (int)warp_sum((unsigned long long)k);
         if (lane == 0 && k) atomicAdd(&misc[8], k);
     }
-    __syncthreads();
+    cta_sync();
     const int K = misc[8];
 
     BR_PH(24);
     // ---- moments: a warp's lanes sharing a root add up among themselves, one
     // lane per root adds to its record ----
-    for (int i0 = wid * 32; i0 < N; i0 += NT) {
+    for (int i0 = wid * 32; i0 < N; i0 += NTW) {
         const int i = i0 + lane;
         const bool v = i < N;
         const unsigned r = v ? par[i] : 0xFFFFFFFFu;
@@ -1119,30 +1237,30 @@ __device__ __noinline__ int big_range(Smem &S, const Params &p, long long base, 
         }
         if (lane == 0 && c_pk) atomicAdd(&misc[9], (int)c_pk);
     }
-    __syncthreads();
+    cta_sync();
     BR_PH(25);
     // ---- the labels (each cluster's earliest pixel in (time, position)
     // order) marked in the bitmap, then their ranks ----
-    for (int i = tid; i < N; i += NT) {
+    for (int i = tid; i < N; i += NTW) {
         if (par[i] != i) continue;
         const unsigned lp = (unsigned)(__ldcg(&g_mom[i].best) & 0xFFFFu);
         atomicOr(&lbits[lp >> 5], 1u << (lp & 31));
     }
-    __syncthreads();
+    cta_sync();
     {
-        constexpr int WPT = BR_LW / NT;
+        constexpr int WPT = (BR_LW + NTW - 1) / NTW;
         unsigned c[WPT], s = 0;
 #pragma unroll
-        for (int k = 0; k < WPT; ++k) { c[k] = (unsigned)__popc(lbits[tid * WPT + k]); s += c[k]; }
+        for (int k = 0; k < WPT; ++k) { c[k] = tid * WPT + k < BR_LW ? (unsigned)__popc(lbits[tid * WPT + k]) : 0u; s += c[k]; }
         int total;
         unsigned run = (unsigned)block_scan_int(S, (int)s, &total);
 #pragma unroll
-        for (int k = 0; k < WPT; ++k) { lpre[tid * WPT + k] = (uint16_t)run; run += c[k]; }
+        for (int k = 0; k < WPT; ++k) { if (tid * WPT + k < BR_LW) lpre[tid * WPT + k] = (uint16_t)run; run += c[k]; }
     }
-    __syncthreads();
+    cta_sync();
     // ---- records, staged in label order ----
-    tpx_record *dst = br_stage(p, (S.pend_head + S.pend_count) % RING);   // the ring entry this tile takes
-    for (int i = tid; i < N; i += NT) {
+    tpx_record *dst = br_stage(p, slot);
+    for (int i = tid; i < N; i += NTW) {
         if (par[i] != i) continue;
         const unsigned long long *m = reinterpret_cast<const unsigned long long *>(&g_mom[i]);
         const long long s_tot = (long long)__ldcg(m), s_x = (long long)__ldcg(m + 1), s_y = (long long)__ldcg(m + 2);
@@ -1167,7 +1285,7 @@ __device__ __noinline__ int big_range(Smem &S, const Params &p, long long base, 
     }
     // ---- per-packet outputs over the range's label span ----
     if (p.labels || p.labels32 || p.is_peak) {
-        for (int i = tid; i < N; i += NT) {
+        for (int i = tid; i < N; i += NTW) {
             const long long q = g_spos[i];
             const unsigned lp = (unsigned)(__ldcg(&g_mom[par[i]].best) & 0xFFFFu);
             const uint8_t pk = ((npk[i >> 5] >> (i & 31)) & 1u) ? 0 : 1;
@@ -1177,14 +1295,14 @@ __device__ __noinline__ int big_range(Smem &S, const Params &p, long long base, 
             if (p.is_peak) p.is_peak[base + q] = pk;
         }
         const int W0 = prev_global ? f : 0, W1 = term ? L - 1 : L;
-        for (int q = W0 + tid; q < W1; q += NT) {
+        for (int q = W0 + tid; q < W1; q += NTW) {
             if (g_rec[q] != INVALID || !TPX_IN(base + q, rend)) continue;
             if (p.labels) p.labels[base + q] = -1LL;
             else if (p.labels32) p.labels32[base + q] = -1;
             if (p.is_peak) p.is_peak[base + q] = 0;
         }
     }
-    __syncthreads();
+    cta_sync();
     BR_PH(26);
     if (tid == 0) {
         S.cnt[C_KEPT] = (unsigned long long)misc[4];
@@ -1192,77 +1310,207 @@ __device__ __noinline__ int big_range(Smem &S, const Params &p, long long base, 
         S.cnt[C_DROP_BG] = (unsigned long long)misc[6];
         S.cnt[C_PEAKS] += (unsigned long long)misc[9];
     }
-    __syncthreads();
+    cta_sync();
     return K;
 }
 
 // ------------------------------------------------------------------- kernel
+// The service warp plans a tile's range and loads the unwrap state before it: the
+// tile's first TDC packet, the first one past the tile (the range's end) from
+// the pre-pass's tile table -- a range longer than the capacity needs no more
+// than the four tiles after its own -- and whether a pixel wrap is near.
+template <bool BATCH>
+__device__ void plan_tile(Smem::Plan &P, const Params &p, long long tile, bool bigr) {
+    const int lane = threadIdx.x & 31;
+    if (lane == 0) P.tile = tile;
+    if (tile >= p.n_tiles) return;
+    long long tile0 = 0, tile_end = p.n_tiles, base = tile * T, rend = p.n;
+    if (BATCH) {
+        const int run = p.bt.tile_run[tile];
+        tile0 = p.bt.run_tile0[run];
+        if (run + 1 < p.bt.n_runs) tile_end = p.bt.run_tile0[run + 1];
+        base = p.bt.run_off[run] + (tile - tile0) * T;
+        rend = p.bt.run_off[run + 1];
+    }
+    if (lane < 8)
+        reinterpret_cast<long long *>(&P.E)[lane] = __ldcg(reinterpret_cast<const long long *>(&p.ts.pre[tile]) + lane);
+    int f = -1;
+    unsigned wrap = 0;
+    if (lane <= 4 && tile + lane < tile_end) {
+        const int2 v = __ldcg(reinterpret_cast<const int2 *>(p.ts.tinfo) + tile + lane);
+        f = v.x;
+        wrap = (unsigned)v.y;
+    }
+    __syncwarp();
+    const unsigned has = __ballot_sync(0xffffffffu, f >= 0) & ~1u;
+    const int j = has ? __ffs(has) - 1 : 4;          // tiles the range reaches into
+    const int fj = __shfl_sync(0xffffffffu, f, j), f0 = __shfl_sync(0xffffffffu, f, 0);
+    const unsigned slow = __ballot_sync(0xffffffffu, wrap != 0 && lane <= j);
+    if (lane == 0) {
+        const long long trig_base = (!BATCH && p.E0) ? p.E0->tdc.n : 0;
+        const bool prev_global = P.E.tdc.n > trig_base;
+        const int cnt = (int)max(0LL, min((long long)T, rend - base));
+        const int w0 = prev_global && f0 >= 0 ? f0 : 0;
+        long long len = 0;
+        bool term = false, over = false;
+        if (f0 >= 0) {
+            // the capacity counts from the tile's first packet: a tile's
+            // range either always fits or never does, whatever precedes it
+            if (has) {
+                len = (long long)j * T + fj + 1;
+                term = true;
+            } else {
+                over = tile + 5 < tile_end;
+                len = over ? C : rend - base;
+            }
+            if (len > C) { over = true; len = C; term = false; }
+            len -= w0;
+        } else if (!prev_global) {
+            len = cnt;   // before the call's first trigger: nothing to cluster, labels of -1
+        }
+        P.f = f0;
+        P.w0 = w0;
+        P.len = (int)len;
+        P.term = term ? 1 : 0;
+        P.slow = slow != 0 ? 1 : 0;
+        P.status = over ? (bigr ? ST_BIG : ST_CAPACITY) : 0u;
+        // its packets start moving into L2 (one bulk prefetch, 16-byte granules)
+        if (p.l2_prefetch && len > 0) {
+            const uint64_t *a = p.pk + ((base + w0) & ~1LL);
+            const long long m = min(len + 1, p.n - ((base + w0) & ~1LL)) & ~1LL;
+            if (m > 0)
+                asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a), "r"((unsigned)(8 * m)) : "memory");
+        }
+    }
+}
+
+// The service warp: claims and plans the tile after the one in work, and
+// copies finished tiles' records out in order while the workers go on. A
+// predecessor's count that is not out yet is tried again later, so a tile
+// behind a slow one holds up neither the planning nor (while the ring has
+// room) the workers. On the large batch the copy of a tile takes about 9k
+// cycles, nearly all latency of the look-back and of the copies; as one of the
+// workers' phases it was 11% of the kernel.
+template <int MODE, bool BATCH>
+__device__ void service(Smem &S, const Params &p, unsigned seq, bool bigr) {
+    constexpr int NP = BATCH ? RING : 1;
+    const int lane = threadIdx.x & 31;
+    int planned = 0, consumed = 0, last = -1;
+    long long tries = 0, idle = 0;
+    for (;;) {
+        int produced = 0, entries = 0;
+        if (lane == 0) {
+            produced = *reinterpret_cast<volatile int *>(&S.produced);
+            __threadfence_block();
+            entries = *reinterpret_cast<volatile int *>(&S.entries);   // at least those of the tiles seen finished
+        }
+        produced = __shfl_sync(0xffffffffu, produced, 0);
+        entries = __shfl_sync(0xffffffffu, entries, 0);
+        bool did = false;
+        if (last < 0 && planned < produced + 2) {
+            unsigned claim = 0;
+            if (lane == 0) claim = atomicAdd(&p.ctl->tile_counter, 1u);
+            const long long tile = (long long)__shfl_sync(0xffffffffu, claim, 0);
+            plan_tile<BATCH>(S.plan[planned & 1], p, tile, bigr);
+            if (tile >= p.n_tiles) last = planned;
+            __syncwarp();
+            ++planned;
+            if (lane == 0) {
+                __threadfence_block();
+                *reinterpret_cast<volatile int *>(&S.planned) = planned;
+            }
+            did = true;
+        }
+        if (consumed < entries) {
+            __threadfence_block();
+            bool give_up = tries > 0 && timed_out(p);
+            if (tries > MAX_TRIES) {
+                if (lane == 0) atomicOr(&p.ctl->status, ST_DEVTIMEOUT);
+                __threadfence();
+                give_up = true;
+            }
+            give_up = __any_sync(0xffffffffu, give_up);
+            if (copy_out<BATCH>(S, p, seq, consumed % NP, give_up)) {
+                tries = 0;
+                ++consumed;
+                __syncwarp();
+                if (lane == 0) {
+                    __threadfence_block();
+                    *reinterpret_cast<volatile int *>(&S.consumed) = consumed;
+                }
+                did = true;
+            } else {
+                ++tries;
+            }
+        }
+        if (last >= 0 && produced == last && consumed == entries) break;
+        if (did) { idle = 0; continue; }
+        if (++idle > MAX_HANDOVER) {
+            if (lane == 0) atomicOr(&p.ctl->status, ST_DEVTIMEOUT);
+            break;
+        }
+        __nanosleep(BATCH && consumed < entries ? 1000 : 100);
+    }
+}
+
+// a worker thread waits until a handover count passes `than` (bounded)
+__device__ __forceinline__ bool wait_count(const int *count, int than, const Params &p) {
+    long long spins = 0;
+    while (*reinterpret_cast<const volatile int *>(count) <= than) {
+        if (++spins > MAX_HANDOVER) {
+            atomicOr(&p.ctl->status, ST_DEVTIMEOUT);
+            return false;
+        }
+        __nanosleep(40);
+    }
+    __threadfence_block();
+    return true;
+}
+
 template <int MODE, bool STAGED, bool BATCH>
 __global__ void __launch_bounds__(NT, MINB) fused_kernel(const Params p) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     Smem &S = *reinterpret_cast<Smem *>(smem_raw);
-    const int tid = threadIdx.x, lane = tid & 31;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const long long tp = p.thr_pix, tt = p.thr_tdc;
     const unsigned seq = p.seq & 0x3FFFFFFFu;
-    const uint32_t pbase = (uint32_t)__cvta_generic_to_shared(S.parent);
+    const uint32_t pb = (uint32_t)__cvta_generic_to_shared(S.par);
     // ranges past the capacity go through the big-range path (CC mode, batches)
     constexpr bool BIGR = BATCH && STAGED && MODE == TPX_MODE_CC;
-    constexpr int NP = BATCH ? RING : 1;   // staged tiles a CTA may hold
-    if (tid == 0) {
-        S.pend_head = 0;
-        S.pend_count = 0;
-        S.tile = atomicAdd(&p.ctl->tile_counter, 1u);
-        S.first_tdc = INT_MAX;
-        S.first_pix = INT_MAX;
-        S.nroot = 0;
-        S.status = 0;
-        S.la_first[0] = S.la_first[1] = S.la_first[2] = INT_MAX;
-    }
-    if (tid < C_NUM) S.cnt[tid] = 0;
-    if (tid < C_NUM) S.acc[tid] = 0;
+    constexpr int NP = BATCH ? RING : 1;   // finished tiles a CTA may hold
+    if (tid < C_NUM) { S.cnt[tid] = 0; S.acc[tid] = 0; }
+    if (tid == 0) S.planned = S.produced = S.entries = S.consumed = 0;
+    int ent = 0;   // entries this CTA has made
 #ifdef TPX_PHASE_TIMING
     if (tid < 32) S.ph[tid] = 0;
     long long ph_t = clock64();
 #endif
     __syncthreads();
-    // the unwrap state before the first tile, from the pre-pass
-    if (tid < 8 && S.tile < p.n_tiles)
-        reinterpret_cast<long long *>(&S.E)[tid] = __ldcg(reinterpret_cast<const long long *>(&p.ts.pre[S.tile]) + tid);
+    if (wid == NW) {
+        service<MODE, BATCH>(S, p, seq, BIGR && p.big);
+        return;
+    }
 
-    for (;;) {
-        // the tile's number, its unwrap state and the reset per-tile fields
-        // were written before this barrier (at the kernel's start or at the
-        // previous tile's tail)
-        __syncthreads();
-        const long long tile = S.tile;
-        // the next tile is claimed now; its number is needed only at the end
-        unsigned long long claim = 0;
-        if (tid == 0 && tile < p.n_tiles) {
-            claim = atomicAdd(&p.ctl->tile_counter, 1u);
-            // the claimed tile's packets (and its look-ahead window) start
-            // moving into L2 now, a tile ahead of their loads (one bulk
-            // prefetch; the start is 16-byte aligned, the size a multiple of 16)
-            if (!BATCH && p.l2_prefetch && claim < (unsigned long long)p.n_tiles) {
-                const long long b = (long long)claim * T;
-                const long long m = min((long long)(T + LA0), p.n - b) & ~1LL;
-                if (m > 0)
-                    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p.pk + b), "r"((unsigned)(8 * m))
-                                 : "memory");
-            }
+    for (int it = 0;; ++it) {
+        // the tile's plan; the per-tile fields start over
+        const Smem::Plan &P = S.plan[it & 1];
+        if (tid == 0) {
+            if (!wait_count(&S.planned, it, p)) S.plan[it & 1].tile = p.n_tiles;
+            S.status = P.status;
+            S.first_pix = INT_MAX;
+            S.nroot = S.nov = S.qn = S.rw = 0;
+            S.n_pre = S.n_bg = S.n_pk = 0;
         }
+        cta_sync();
+        const long long tile = P.tile;
         if (tile >= p.n_tiles) {
-            if (STAGED) {
-                if (tid < 32) flush_ring_warp<BATCH>(S, p, seq, true);
-                __syncthreads();
-                if (tid == 0 && S.status) atomicOr(&p.ctl->status, S.status);
-            }
             // this CTA's counters (packets of each class are counted by the
             // unwrap pre-pass)
             if (tid < C_NUM && tid != C_PIXELS && tid != C_TDCS && tid != C_CORRUPT && S.acc[tid])
                 atomicAdd(&p.ctl->counters[tid], S.acc[tid]);
 #ifdef TPX_PHASE_TIMING
             TPX_PH(16);
-            __syncthreads();
+            cta_sync();
             if (tid < 32 && S.ph[tid]) atomicAdd(&g_phase[tid], S.ph[tid]);
 #endif
             break;
@@ -1280,188 +1528,108 @@ __global__ void __launch_bounds__(NT, MINB) fused_kernel(const Params p) {
             base = tile * T;
         }
         const int cnt = (int)max(0LL, min((long long)T, rend - base));
-        TPX_PH(0);
-
-        // ---- load the tile and a first look-ahead window past it:
-        // coalesced 16-byte loads into the padded buffer; the tile's TDC
-        // packets are counted and its first one found on the way, and the
-        // first TDC packet of the window ----
-        const int lw = (int)max(0LL, min((long long)min(LA0, C - cnt), rend - base - cnt));   // window length
-        {
-            int my_first = INT_MAX, my_la = INT_MAX, c_tdc = 0;
-            const int ltot = cnt + lw;
-            if (BATCH && (base & 1)) {   // a run starting at an odd packet: 8-byte loads
-                for (int v = tid; v < ltot; v += NT) {
-                    const uint64_t w = __ldcg(p.pk + base + v);
-                    S.buf[pad(v)] = w;
-                    if ((w >> 60) == 0x6u) {
-                        if (v < cnt) { ++c_tdc; my_first = min(my_first, v); } else my_la = min(my_la, v);
-                    }
-                }
-            } else {
-                const ulonglong2 *src = reinterpret_cast<const ulonglong2 *>(p.pk + base);
-                const int npair = ltot >> 1;
-                for (int v = tid; v < npair; v += NT) {
-                    ulonglong2 w = __ldcg(src + v);
-                    S.buf[pad(2 * v)] = w.x;
-                    S.buf[pad(2 * v + 1)] = w.y;
-#pragma unroll
-                    for (int u = 0; u < 2; ++u) {
-                        const int q = 2 * v + u;
-                        if (((u ? w.y : w.x) >> 60) == 0x6u) {
-                            if (q < cnt) { ++c_tdc; my_first = min(my_first, q); } else my_la = min(my_la, q);
-                        }
-                    }
-                }
-                if ((ltot & 1) && tid == 0) {
-                    const uint64_t w = __ldcg(p.pk + base + ltot - 1);
-                    S.buf[pad(ltot - 1)] = w;
-                    if ((w >> 60) == 0x6u) {
-                        if (ltot - 1 < cnt) { ++c_tdc; my_first = min(my_first, ltot - 1); }
-                        else my_la = min(my_la, ltot - 1);
-                    }
-                }
-            }
-            for (int i = tid; i < HB / 2; i += NT) reinterpret_cast<uint32_t *>(S.u1.head)[i] = 0xFFFFFFFFu;
-            if (__any_sync(0xffffffffu, c_tdc != 0 || my_la != INT_MAX)) {
-                c_tdc = (int)warp_sum((unsigned long long)c_tdc);
-                my_first = __reduce_min_sync(0xffffffffu, (unsigned)my_first);
-                my_la = __reduce_min_sync(0xffffffffu, (unsigned)my_la);
-                if (lane == 0) {
-                    if (c_tdc) atomicAdd(&S.cnt[C_TDCS], (unsigned long long)c_tdc);
-                    if (my_first != INT_MAX) atomicMin(&S.first_tdc, my_first);
-                    if (my_la != INT_MAX) atomicMin(&S.la_first[0], my_la);
-                }
-            }
-        }
-        __syncthreads();
-
-        TPX_PH(1);
-        const int f = S.first_tdc;
-
-        // ---- look ahead past the window up to the next TDC packet, one
-        // barrier per chunk (the chunks' minima rotate over three slots: a
-        // slot is reset two chunks after it was read) ----
-        int L = f != INT_MAX ? cnt + lw : cnt;   // a tile without a TDC packet owns nothing
-        bool term = false;
-        if (f != INT_MAX) {
-            const int lf0 = S.la_first[0];
-            if (lf0 != INT_MAX) {
-                L = lf0 + 1;
-                term = true;
-            } else {
-                for (int k = 1; base + L < rend; ++k) {
-                    const int room = C - L;
-                    if (room <= 0) break;
-                    const int chunk = (int)min((long long)min(NT, room), rend - (base + L));
-                    const int slot = k % 3;
-                    if (tid == 0) S.la_first[(k + 1) % 3] = INT_MAX;
-                    if (tid < chunk) {
-                        const uint64_t w = __ldcg(p.pk + base + L + tid);
-                        if (TPX_IN(L + tid, C)) S.buf[pad(L + tid)] = w;
-                        if ((w >> 60) == 0x6u) atomicMin(&S.la_first[slot], tid);
-                    }
-                    __syncthreads();
-                    const int lf = S.la_first[slot];
-                    if (lf != INT_MAX) { L += lf + 1; term = true; break; }
-                    L += chunk;
-                }
-            }
-            // a range past the capacity: the big-range path, or its run goes back
-            if (!term && base + L < rend && tid == 0) atomicOr(&S.status, (BIGR && p.big) ? ST_BIG : ST_CAPACITY);
-        }
-
-        TPX_PH(2);
-        // ---- walk 2: wrap steps and TDC counts over [0, L) ----
-        // [0, L) is split evenly over all threads, in thread order (every
-        // later per-thread walk and scan uses the same contiguous chunks). A
-        // thread counts its TDC packets and the pixel wrap steps (Sec. IV.A)
-        // between consecutive pixels from its first pixel up to the first
-        // pixel after its chunk, so that one scan gives every chunk the wraps
-        // before its first pixel.
-        const int kpd = (L + NT - 1) / NT;
-        const int p0 = tid * kpd;
-        int ntd = 0, fpx = INT_MAX, jp = 0;
-        {
-            int lpx = -1;
-            long long lr = 0;
-            for (int j = 0; j < kpd; ++j) {
-                const int q = p0 + j;
-                if (q >= L) break;
-                const uint64_t w = S.buf[pad(q)];
-                const unsigned h = (unsigned)(w >> 60);
-                if (h == 0xBu) {
-                    const long long r = pix_raw(w);
-                    if (lpx >= 0) jp += (int)jump(r - lr, tp); else fpx = q;
-                    lpx = q;
-                    lr = r;
-                } else if (h == 0x6u) {
-                    ++ntd;
-                }
-            }
-            if (lpx >= 0) {   // the step to the next pixel after the chunk
-                for (int q = p0 + kpd; q < L; ++q) {
-                    const uint64_t w = S.buf[pad(q)];
-                    if ((w >> 60) == 0xBu) { jp += (int)jump(pix_raw(w) - lr, tp); break; }
-                }
-            }
-            const int fw = (int)__reduce_min_sync(0xffffffffu, (unsigned)fpx);
-            if (lane == 0 && fw != INT_MAX) atomicMin(&S.first_pix, fw);
-        }
-        // one scan of (TDC count, wrap steps) packed as two 16-bit halves
-        unsigned pk_tot;
-        const unsigned pk_ex = block_scan_vadd2(S, ((unsigned)ntd << 16) | ((unsigned)jp & 0xFFFFu), &pk_tot);
-        const int li0 = (int)(pk_ex >> 16);              // TDC packets before the chunk
-        const int ntdc = (int)(pk_tot >> 16);            // in [0, L)
-        const int jp_ex = (int)(short)(pk_ex & 0xFFFFu); // pixel wraps between the range's first pixel and the chunk
-        TPX_PH(3);
-        const GAgg E = S.E;
+        // the range: L packets from w0 on, its first TDC packet at R0 (both
+        // from w0), the TDC packet that ends it included when there is one
+        const int f = P.f, w0 = P.w0, L = P.len;
+        const bool term = P.term != 0, slow = P.slow != 0;
+        const long long gbase = base + w0;
+        const GAgg &E = P.E;
         // a call sees only its own triggers: "earlier" means earlier in this call
         const long long trig_base = (!BATCH && p.E0) ? p.E0->tdc.n : 0;
         const bool prev_global = E.tdc.n > trig_base;
-        const int nseg = min(ntdc, MAXSEG);
-        if (tid == 0) {
-            if (ntdc > MAXSEG) atomicOr(&S.status, ST_CAPACITY);
-            // the step into the range's first pixel, read while the buffer
-            // still holds packets (walk 4 overwrites them with records)
-            const int fp = S.first_pix;
-            S.j0 = (fp != INT_MAX && E.pix.n > 0) ? jump(pix_raw(S.buf[pad(fp)]) - E.pix.last, tp) : 0;
+        TPX_PH(0);
+
+        // ---- read the range, a packet per thread and step, into registers;
+        // the TDC packets of each 32 positions are kept as a mask, their
+        // words (near a pixel wrap all words) in shared memory ----
+        uint64_t w[KM];
+#pragma unroll
+        for (int j = 0; j < KM; ++j) {
+            const int r = j * NTW + tid;
+            w[j] = r < L ? __ldcg(p.pk + gbase + r) : 0ull;
         }
-        // ---- TDC packets of the range in stream order, then their unwrapped
-        // times (one warp, a scan of the wrap steps) ----
-        if (ntd) {
-            int li = li0;
-            for (int j = 0; j < kpd; ++j) {
-                const int q = p0 + j;
-                if (q >= L) break;
-                if ((S.buf[pad(q)] >> 60) != 0x6u) continue;
-                if (li < MAXSEG) S.tdc_pos[li] = (uint16_t)q;
-                ++li;
+        for (int i = tid; i < TW / 4; i += NTW) reinterpret_cast<uint4 *>(S.u1.t.bits)[i] = make_uint4(0, 0, 0, 0);
+        for (int i = tid; i < OHB / 2; i += NTW) reinterpret_cast<uint32_t *>(S.u1.t.ohead)[i] = 0xFFFFFFFFu;
+#pragma unroll
+        for (int j = 0; j < KM; ++j) {
+            if (j * NTW >= L) break;
+            const int r = j * NTW + tid;
+            const bool is_tdc = (w[j] >> 60) == 0x6u;
+            const unsigned m = __ballot_sync(0xffffffffu, is_tdc);
+            if (lane == 0 && r < L) S.u3.tmask[j * NW + wid] = m;
+            if ((is_tdc || slow) && r < L) S.srec[r] = w[j];
+        }
+        cta_sync();
+        TPX_PH(1);
+
+        // ---- the TDC packets before each 32 positions, the positions of all
+        // of them, and their unwrapped times (one warp, a scan of the wrap
+        // steps) ----
+        if (wid == 0) {
+            constexpr int GPL = C / 32 / 32;
+            const int G = (L + 31) >> 5;
+            int c = 0;
+#pragma unroll
+            for (int k = 0; k < GPL; ++k) {
+                const int g = lane * GPL + k;
+                c += g < G ? __popc(S.u3.tmask[g]) : 0;
             }
-        }
-        __syncthreads();
-        if (tid < 32) {
+            int incl = c;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int u = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += u;
+            }
+            const int ntdc = __shfl_sync(0xffffffffu, incl, 31);
+            int at = incl - c, mine = 0;
+#pragma unroll
+            for (int k = 0; k < GPL; ++k) {
+                const int g = lane * GPL + k;
+                if (g >= G) break;
+                S.u4.tpre[g] = (uint16_t)at;
+                for (unsigned m = S.u3.tmask[g]; m; m &= m - 1) {
+                    const int q = 32 * g + __ffs(m) - 1;
+                    if (at < MAXSEG) S.tdc_pos[at] = (uint16_t)q;
+                    mine += q < cnt - w0;
+                    ++at;
+                }
+            }
+            mine = (int)__reduce_add_sync(0xffffffffu, (unsigned)mine);
+            if (lane == 0) {
+                S.ntdc = ntdc;
+                S.cnt[C_TDCS] = (unsigned long long)mine;   // the tile's own
+                if (ntdc > MAXSEG) S.status |= ST_CAPACITY;
+                S.tdc_t[min(ntdc, MAXSEG)] = LLONG_MAX;
+            }
+            const int nseg = min(ntdc, MAXSEG);
+            __syncwarp();
             bool has = E.tdc.n > 0;
             long long last = E.tdc.last, ep = E.tdc.sum, t_last = 0;
             for (int i0 = 0; i0 < nseg; i0 += 32) {
                 const int i = i0 + lane;
                 long long r = 0;
-                if (i < nseg) r = tdc_raw(S.buf[pad((int)S.tdc_pos[i])]);
+                int q = 0;
+                if (i < nseg) {
+                    q = S.tdc_pos[i];
+                    r = tdc_raw(S.srec[q]);
+                }
                 const long long rp = __shfl_up_sync(0xffffffffu, r, 1);
                 int st = 0;
                 if (i < nseg && (lane > 0 || has)) st = (int)jump(r - (lane > 0 ? rp : last), tt);
                 int inc = st;
+                if (__any_sync(0xffffffffu, st != 0)) {
 #pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const int u = __shfl_up_sync(0xffffffffu, inc, o);
-                    if (lane >= o) inc += u;
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const int u = __shfl_up_sync(0xffffffffu, inc, o);
+                        if (lane >= o) inc += u;
+                    }
                 }
                 const long long t = r + (ep + inc) * kTdcPeriod;
                 const long long tp_ = __shfl_up_sync(0xffffffffu, t, 1);
                 if (i < nseg) {
                     S.tdc_t[i] = t;
                     if ((lane > 0 || i0 > 0) && t < (lane > 0 ? tp_ : t_last)) atomicOr(&p.ctl->status, ST_TRIG_ORDER);
-                    if (!BATCH && S.tdc_pos[i] < cnt) {   // a batch writes its triggers at the flush
+                    if (!BATCH && q < cnt - w0) {   // a batch writes its triggers at the flush
                         const long long g = E.tdc.n - trig_base + i;
                         if (g >= 0 && g < p.trig_cap) p.trig[g] = t; else atomicOr(&p.ctl->status, ST_TRIG_CAP);
                     }
@@ -1473,423 +1641,361 @@ __global__ void __launch_bounds__(NT, MINB) fused_kernel(const Params p) {
                 has = true;
             }
         }
-        __syncthreads();
-
         TPX_PH(4);
-        // ---- walk 4: pixels -> shot, cut, timewalk, packed record ----
-        {
-            // wraps at the chunk's first pixel: before the range, the step from
-            // the last pixel before it to the range's first pixel, the steps
-            // inside the range before the chunk
-            long long ep = E.pix.sum + S.j0 + jp_ex;
-            bool has = false;
+        if (slow) {
+            // a pixel wrap step (Sec. IV.A) lies in or near the range: the
+            // wraps of every position, over contiguous chunks of the packets.
+            // A thread counts the steps from its first pixel up to the first
+            // pixel after its chunk; one scan gives the wraps before each.
+            cta_sync();
+            const int kpd = (L + NTW - 1) / NTW;
+            const int p0 = tid * kpd;
+            int fpx = INT_MAX, jp = 0;
+            {
+                int lpx = -1;
+                long long lr = 0;
+                for (int q = p0; q < min(p0 + kpd, L); ++q) {
+                    const uint64_t v = S.srec[q];
+                    if ((v >> 60) != 0xBu) continue;
+                    const long long r = pix_raw(v);
+                    if (lpx >= 0) jp += (int)jump(r - lr, tp); else fpx = q;
+                    lpx = q;
+                    lr = r;
+                }
+                if (lpx >= 0) {   // the step to the next pixel after the chunk
+                    for (int q = p0 + kpd; q < L; ++q) {
+                        const uint64_t v = S.srec[q];
+                        if ((v >> 60) == 0xBu) { jp += (int)jump(pix_raw(v) - lr, tp); break; }
+                    }
+                }
+                const int fw = (int)__reduce_min_sync(0xffffffffu, (unsigned)fpx);
+                if (lane == 0 && fw != INT_MAX) atomicMin(&S.first_pix, fw);
+            }
+            int total;
+            const int jp_ex = block_scan_int(S, jp, &total);
+            if (tid == 0) {
+                const int fp = S.first_pix;
+                S.j0 = (fp != INT_MAX && E.pix.n > 0) ? jump(pix_raw(S.srec[fp]) - E.pix.last, tp) : 0;
+            }
+            cta_sync();
+            int d = (int)S.j0 + jp_ex;
+            bool any = false;
             long long last = 0;
-            int seg = li0 - 1;
+            for (int q = p0; q < min(p0 + kpd, L); ++q) {
+                const uint64_t v = S.srec[q];
+                if ((v >> 60) != 0xBu) continue;
+                const long long r = pix_raw(v);
+                if (any) d += (int)jump(r - last, tp);
+                any = true;
+                last = r;
+                S.spos[q] = (uint16_t)(int16_t)d;
+            }
+        }
+        cta_sync();
+
+        // a batch tile whose range the tiles cannot hold: its run is redone by
+        // the general path, so it clusters nothing (its counts still flow).
+        // A big range clusters nothing here either: its path runs below.
+        const bool big_tile = BIGR && (S.status & ST_BIG) && !(S.status & ST_CAPACITY);
+        const int nseg = min(S.ntdc, MAXSEG);
+        TPX_PH(3);
+        // ---- packets -> shot, cut, timewalk, packed record; each kept pixel
+        // takes its bit of the cell table, or a number among those that find
+        // it taken ----
+        uint32_t rk[(KM + 1) / 2];
+#pragma unroll
+        for (int j = 0; j < (KM + 1) / 2; ++j) rk[j] = 0u;
+        {
             const long long t_prev_global = E.tdc.last + E.tdc.sum * kTdcPeriod;
-            unsigned long long c_keep = 0, c_pre = 0, c_bg = 0;
+            const unsigned below = (1u << lane) - 1u;
+            unsigned c_pre = 0, c_bg = 0;
             bool exc = false;
-            for (int j = 0; j < kpd; ++j) {
-                const int q = p0 + j;
-                if (q >= L) break;
-                const uint64_t w = S.buf[pad(q)];
-                const unsigned h = (unsigned)(w >> 60);
+#pragma unroll
+            for (int j = 0; j < KM; ++j) {
+                if (j * NTW >= L || big_tile) { w[j] = INVALID; continue; }
+                const int r = j * NTW + tid;
+                const uint64_t v = w[j];
                 uint64_t rec = INVALID;
-                if (h == 0x6u) {
-                    ++seg;
-                } else if (h == 0xBu) {
-                    const long long r = pix_raw(w);
-                    if (has) ep += jump(r - last, tp);
-                    has = true;
-                    last = r;
-                    const long long t = r + ep * kPixPeriod;
+                if ((v >> 60) == 0xBu) {   // positions past the range hold zero
+                    const int g = j * NW + wid;
+                    const int seg = (int)S.u4.tpre[g] + __popc(S.u3.tmask[g] & below) - 1;
+                    long long ep = E.pix.sum;
+                    if (slow) ep += (int16_t)S.spos[r];
+                    const long long t = pix_raw(v) + ep * kPixPeriod;
                     if (seg < 0) {
                         if (!prev_global) ++c_pre;        // no trigger before it anywhere
                     } else if (seg < nseg) {
-                        const long long t_lo = S.tdc_t[seg];
-                        const bool has_hi = seg + 1 < nseg;
-                        int verdict;                      // 0 keep, 1 bg, 2 pre, 3 undecidable here
-                        if (has_hi && t >= S.tdc_t[seg + 1]) verdict = 3;
-                        else if (t >= t_lo) verdict = (t - t_lo > p.tof_max) ? 1 : 0;
-                        else {
+                        const long long t_lo = S.tdc_t[seg], d = t - t_lo;
+                        // the common case: at or after its trigger, before the next one, inside the cut
+                        if ((unsigned long long)d <= (unsigned long long)p.tof_max && t < S.tdc_t[seg + 1]) {
+                            const int tot = pix_tot(v);
+                            const int tofb = (int)d + kTofBias - (p.lut ? (int)p.lut[tot] : 0);
+                            rec = mkrec((uint32_t)tofb, (uint32_t)seg, (uint32_t)tot, (uint32_t)pix_x(v), (uint32_t)pix_y(v));
+                            const uint32_t b = tbit(rec), m = 1u << (b & 31);
+                            if (atomicOr(&S.u1.t.bits[b >> 5], m) & m)
+                                rk[j / 2] |= ((uint32_t)atomicAdd(&S.nov, 1) + 1u) << (16 * (j & 1));
+                        } else if (t >= S.tdc_t[seg + 1]) {
+                            exc = true;                   // after a trigger read out later
+                        } else if (d >= 0) {
+                            ++c_bg;
+                        } else {                          // read out late: an earlier shot's
                             const bool hp = seg > 0 || prev_global;
                             const long long tprev = seg > 0 ? S.tdc_t[seg - 1] : t_prev_global;
-                            if (!hp) verdict = 2;
-                            else if (t >= tprev) verdict = (t - tprev > p.tof_max) ? 1 : 3;
-                            else verdict = 3;
+                            if (!hp) ++c_pre;
+                            else if (t >= tprev && t - tprev > p.tof_max) ++c_bg;
+                            else exc = true;
                         }
-                        if (verdict == 0) {
-                            const int tot = pix_tot(w);
-                            const long long tc = t - (p.lut ? (long long)p.lut[tot] : 0LL);
-                            const long long tofb = tc - t_lo + kTofBias;
-                            rec = mkrec((uint32_t)tofb, (uint32_t)seg, (uint32_t)tot, (uint32_t)pix_x(w), (uint32_t)pix_y(w));
-                            ++c_keep;
-                        } else if (verdict == 1) ++c_bg;
-                        else if (verdict == 2) ++c_pre;
-                        else exc = true;
                     }
                 }
-                S.buf[pad(q)] = rec;
+                w[j] = rec;
             }
-            c_keep = warp_sum(c_keep); c_pre = warp_sum(c_pre); c_bg = warp_sum(c_bg);
-            if (lane == 0) {
-                atomicAdd(&S.cnt[C_KEPT], c_keep);
-                atomicAdd(&S.cnt[C_DROP_PRE], c_pre);
-                atomicAdd(&S.cnt[C_DROP_BG], c_bg);
+            if (__any_sync(0xffffffffu, (c_pre | c_bg) != 0)) {
+                c_pre = __reduce_add_sync(0xffffffffu, c_pre);
+                c_bg = __reduce_add_sync(0xffffffffu, c_bg);
+                if (lane == 0) { atomicAdd(&S.n_pre, c_pre); atomicAdd(&S.n_bg, c_bg); }
             }
             if (exc) atomicOr(&S.status, ST_EXCEPTION);
         }
-        __syncthreads();   // records written per contiguous chunk are read strided below
-
+        cta_sync();
         TPX_PH(5);
-        // a batch tile whose range the tiles cannot hold: its run is redone by
-        // the general path, so it clusters nothing (its counts still flow)
-        // (a big range clusters nothing here either: it has a path of its own)
-        const bool skip = BATCH && (S.status & (ST_CAPACITY | ST_EXCEPTION | ST_BIG)) != 0;
-        // a big range: its path runs before the previous tile is copied out
-        // (that copy may wait for other CTAs' big ranges)
-        const bool big_tile = BIGR && (S.status & ST_BIG) && !(S.status & (ST_CAPACITY | ST_EXCEPTION));
-        // the range this CTA owns: [R0, R1)
-        const int R0 = (f == INT_MAX || skip) ? 0 : f;
-        const int R1 = (f == INT_MAX || skip) ? 0 : (term ? L - 1 : L);
-        // label writes cover [W0, W1): the range, plus the packets before the
-        // tile's first trigger when no trigger precedes them anywhere
-        const int W0 = prev_global ? R0 : 0;
-        const int W1 = skip ? 0 : ((f == INT_MAX) ? (prev_global ? 0 : cnt) : R1);
 
-        // ---- hash insert ----
-        for (int q = R0 + tid; q < R1; q += NT) {
-            const uint64_t r = S.buf[pad(q)];
-            S.parent[q] = (NO_EXT << 16) | (uint32_t)q;
-            S.notpeak[q] = 0;
-            if (r != INVALID) {
-                const uint32_t b = hcell(r_seg(r), r_x(r), r_y(r));
-                // push q on the bucket's list (16-bit exchange as a CAS loop)
-                unsigned short old = S.u1.head[b], seen;
+        // ---- the rank of each table word: an exclusive scan of the bit counts ----
+        const bool skip = BATCH && (S.status & (ST_CAPACITY | ST_EXCEPTION | ST_BIG)) != 0;
+        int nb, nov = S.nov;   // kept pixels in the table, and outside it
+        {
+            constexpr int WPT = (TW + NTW - 1) / NTW;
+            int c[WPT], sum = 0;
+#pragma unroll
+            for (int k = 0; k < WPT; ++k) {
+                c[k] = tid * WPT + k < TW ? __popc(S.u1.t.bits[tid * WPT + k]) : 0;
+                sum += c[k];
+            }
+            int at = block_scan_int(S, sum, &nb);
+#pragma unroll
+            for (int k = 0; k < WPT; ++k) {
+                if (tid * WPT + k < TW) S.u1.t.rank[tid * WPT + k] = (uint16_t)at;
+                at += c[k];
+            }
+            for (int i = tid; i < C / 32; i += NTW) S.u3.rwalk[i] = 0u;
+        }
+        cta_sync();
+        TPX_PH(6);
+        // ---- the records into their slots ----
+#pragma unroll
+        for (int j = 0; j < KM; ++j) {
+            if (j * NTW >= L) break;
+            const uint64_t rec = w[j];
+            if (rec == INVALID) continue;
+            const uint32_t b = tbit(rec), o = (rk[j / 2] >> (16 * (j & 1))) & 0xFFFFu;
+            const int slot = o ? nb + (int)o - 1 : rank_at(S, b);
+            if (!TPX_IN(slot, C)) continue;
+            S.srec[slot] = rec;
+            S.spos[slot] = (uint16_t)(j * NTW + tid);
+            S.par[slot] = (uint16_t)slot;
+            S.notpeak[slot] = 0;
+            if (o) {   // push it on its chain (16-bit exchange as a CAS loop)
+                unsigned short *h = &S.u1.t.ohead[ohash(b)], old = *h, seen;
                 do {
                     seen = old;
-                    old = atomicCAS(&S.u1.head[b], seen, (unsigned short)q);
+                    old = atomicCAS(h, seen, (unsigned short)(o - 1));
                 } while (old != seen);
-                S.u2.next[q] = old;
+                S.u5.onext[o - 1] = old;
             }
         }
-        __syncthreads();
+        const int kept = nb + nov;
+        if (tid < 4) S.srec[kept + tid] = INVALID;   // the probes past the last slot find no cell
+        if (skip) nb = nov = 0;
+        const int n = nb + nov;
+        if (MODE == TPX_MODE_PAPER)   // no union queue: the label entries are free already
+            for (int i = tid; i < L; i += NTW) S.u2.lab[i] = NOLAB;
+        cta_sync();
+        TPX_PH(2);
 
-        TPX_PH(6);
-        // ---- neighbour pass: each adjacent pair once (Sec. V.A box rule) ----
-        // The warp walks 32 consecutive positions at a time; each lane gathers
-        // its pixel's partners in the forward half of the box -- a strict order
-        // of the pairs: a larger x, or the same x and a larger y, or the same
-        // cell and a later position -- and updates the local-maximum flags
-        // (Sec. V.B). CC mode: the pixel points to its first partner (a plain
-        // store: pointers only go forward, so they form a forest) and keeps its
-        // second partner in the upper half of its pointer word; a pixel with
-        // more partners marks its word for a re-walk.
-        {
-            for (int qb = R0 + (tid & ~31); qb < R1; qb += NT) {
-                const int q = qb + lane;
-                const uint64_t r = q < R1 ? S.buf[pad(q)] : INVALID;
-                if (r == INVALID) continue;
-                uint32_t e0 = (uint32_t)q, e1 = NO_EXT;
-                int ne = 0;
-                const int x = r_x(r), y = r_y(r), sg = r_seg(r), tb = r_tof(r), tot = r_tot(r);
-                const uint32_t hb = (uint32_t)(x + 67 * y + 1543 * sg);   // hcell of (x, y), unmasked
-                bool dim = false;
-                if (MODE == TPX_MODE_CC && p.rx == 1 && p.ry == 1) {
-                    // 8-neighbour box, its five forward cells unrolled. A diagonal
-                    // partner (dx = 1, dy = -1 or +1) is held back and needs no
-                    // union when the pixel's partner to the side (dx = 1, dy = 0),
-                    // or above it (dx = 0, dy = +1) for dy = +1, is adjacent to it
-                    // as well: that path of two axis-aligned pairs, which are never
-                    // held back, joins them
-                    uint32_t hold = 0xFFFFFFFFu;   // held partners: dy = -1 low half, dy = +1 high half
-                    int tA = 0, tB = 0, tE = INT_MIN, tN = INT_MIN;
-#pragma unroll
-                    for (int c = 0; c < 5; ++c) {
-                        const int dx = c < 2 ? 0 : 1;
-                        const int dy = c == 0 ? 0 : (c == 1 ? 1 : c - 3);
-                        if (x + dx > 255 || y + dy < 0 || y + dy > 255) continue;
-                        const uint32_t ck = r_cell(r) + (uint32_t)(256 * dy + dx);
-                        for (uint32_t j = S.u1.head[(hb + 67 * dy + dx) & (HB - 1)]; j != EMPTY; j = S.u2.next[j]) {
-                            if (!TPX_IN(j, C)) break;
-                            if (c == 0 && (int)j <= q) continue;
-                            const uint64_t rj = S.buf[pad((int)j)];
-                            if (r_cell(rj) != ck) continue;
-                            const int tjt = r_tof(rj);
-                            if (!within(tjt - tb, p.dt)) continue;
-                            const int tj = r_tot(rj);
-                            // local maxima: equal ToT goes to the later pixel (Sec. V.B)
-                            if (tj > tot || (tj == tot && (int)j > q)) dim = true;
-                            else S.notpeak[j] = 1;
-                            if (c == 3 && tE == INT_MIN) tE = tjt;
-                            if (c == 1 && tN == INT_MIN) tN = tjt;
-                            if (c == 2 || c == 4) {
-                                const int sh = c == 4 ? 16 : 0;
-                                if (((hold >> sh) & 0xFFFFu) == 0xFFFFu) {
-                                    hold = (hold & ~(0xFFFFu << sh)) | (j << sh);
-                                    if (c == 4) tB = tjt; else tA = tjt;
-                                    continue;
-                                }
-                            }
-                            if (ne == 0) e0 = j; else if (ne == 1) e1 = j;
-                            ++ne;
-                        }
+        // ---- neighbour pass: each adjacent pair of table pixels once (Sec. V.A
+        // box rule) ---- A lane's pixel looks at the next slot (its right-hand
+        // neighbour, if that is one) and at the slots of the row above, and
+        // sets the local-maximum flags (Sec. V.B). CC: the pixel points to one
+        // partner (a plain store: pointers only go forward in (y, x), so they
+        // form a forest) and queues the pairs that no path of other pairs
+        // joins.
+        for (int t0 = tid & ~31; t0 < nb; t0 += NTW) {
+            const int i = t0 + lane;
+            const bool live = i < nb;
+            const uint64_t r = live ? S.srec[i] : INVALID;
+            const int x = r_x(r), y = r_y(r), tb = r_tof(r), tot = r_tot(r);
+            const uint32_t cell = r_cell(r), b = tbit(r);
+            bool dim = false;
+            if (MODE == TPX_MODE_CC && p.rx == 1 && p.ry == 1) {
+                // 8-neighbour box: four probes, no loop. The row above has its
+                // (at most three) cells' pixels in consecutive slots from the
+                // rank of the first cell on.
+                int tmin = INT_MAX, tmax = INT_MIN;
+                auto probe = [&](int j, bool ok) -> bool {   // an adjacent pixel: its flags and time
+                    const uint64_t rj = S.srec[j];
+                    const int tj = r_tof(rj);
+                    ok = ok && within(tj - tb, p.dt);
+                    if (ok) {
+                        if (dimmer(S, i, tot, j, r_tot(rj))) dim = true; else S.notpeak[j] = 1;
+                        tmin = min(tmin, tj);
+                        tmax = max(tmax, tj);
                     }
-                    const uint32_t jA = hold & 0xFFFFu, jB = hold >> 16;
-                    const bool skipA = tE != INT_MIN && within(tE - tA, p.dt);
-                    const bool skipB = (tE != INT_MIN && within(tE - tB, p.dt)) || (tN != INT_MIN && within(tN - tB, p.dt));
-                    if (jA != 0xFFFFu && !skipA) { if (ne == 0) e0 = jA; else if (ne == 1) e1 = jA; ++ne; }
-                    if (jB != 0xFFFFu && !skipB) { if (ne == 0) e0 = jB; else if (ne == 1) e1 = jB; ++ne; }
-                } else {
-                    for (int dx = 0; dx <= p.rx; ++dx) {
-                        const int cx = x + dx;
-                        if (cx > 255) break;
-                        for (int dy = (dx == 0 ? 0 : -p.ry); dy <= p.ry; ++dy) {
-                            const int cy = y + dy;
-                            if (cy < 0 || cy > 255) continue;
-                            const uint32_t ck = r_cell(r) + (uint32_t)(256 * dy + dx);
-                            for (uint32_t j = S.u1.head[(hb + 67 * dy + dx) & (HB - 1)]; j != EMPTY; j = S.u2.next[j]) {
-                                if (!TPX_IN(j, C)) break;
-                                if (dx == 0 && dy == 0 && (int)j <= q) continue;
-                                const uint64_t rj = S.buf[pad((int)j)];
-                                if (r_cell(rj) != ck) continue;
-                                if (!within(r_tof(rj) - tb, p.dt)) continue;
-                                const int tj = r_tot(rj);
-                                // local maxima: equal ToT goes to the later pixel (Sec. V.B)
-                                if (tj > tot || (tj == tot && (int)j > q)) dim = true;
-                                else S.notpeak[j] = 1;
-                                if (MODE == TPX_MODE_CC) {
-                                    if (ne == 0) e0 = j; else if (ne == 1) e1 = j;
-                                    ++ne;
-                                }
-                            }
+                    return ok;
+                };
+                bool hE = live && i + 1 < nb && x < 255 && r_cell(S.srec[i + 1]) == cell + 1;
+                if (hE) hE = probe(i + 1, true);
+                int jL = -1, jM = -1, jR = -1;
+                if (live && y < 255) {
+                    const uint32_t l = x > 0 ? 1u : 0u, span = l + (x < 255 ? 1u : 0u);
+                    const int s0 = rank_at(S, (b + 256u) - ((b + 256u) & TB) - l);
+                    const uint32_t c0 = cell + 256u - l;
+#pragma unroll
+                    for (int k = 0; k < 3; ++k) {
+                        const int j = s0 + k;
+                        if (!TPX_IN(j, C + 4)) break;
+                        const uint32_t u = r_cell(S.srec[j]) - c0;
+                        if (probe(j, u <= span && j < nb)) {
+                            const uint32_t v = u + 1u - l;   // 0 left, 1 middle, 2 right
+                            if (v == 1) jM = j; else if (v == 0) jL = j; else jR = j;
                         }
                     }
                 }
-                if (dim) S.notpeak[q] = 1;
-                // with two partners the pointer takes the later-found one (the
-                // larger x when the two differ): pointers run along x first,
-                // which keeps the trees of a compact cloud shallow
-                if (MODE == TPX_MODE_CC)
-                    S.parent[q] = ne > 2 ? ((REWALK << 16) | e0) : ne == 2 ? ((e0 << 16) | e1) : ((NO_EXT << 16) | e0);
+                // Which pairs need a union of their own, when all partners lie
+                // within dt of each other (adjacent in time): the pair to the
+                // right always (pointer); a pixel above both this pixel and
+                // its right-hand neighbour is reached through the neighbour's
+                // pair with it (and so on to the right); a diagonal one through
+                // the pixel above when there is one. When they do not, every pair.
+                const bool close = tmax - tmin <= p.dt || tmin == INT_MAX;
+                int up = hE ? i + 1 : jM >= 0 ? jM : jR >= 0 ? jR : jL >= 0 ? jL : i;
+                if (close) {
+                    if (jL >= 0 && jM < 0 && up != jL) queue_pair(S, i, jL);
+                } else {
+                    if (jM >= 0 && up != jM) queue_pair(S, i, jM);
+                    if (jR >= 0 && up != jR) queue_pair(S, i, jR);
+                    if (jL >= 0 && up != jL) queue_pair(S, i, jL);
+                }
+                // along a row the pointer goes straight to the last slot of
+                // the run that this warp sees
+                const unsigned run = __ballot_sync(0xffffffffu, hE) & 0x7FFFFFFFu;
+                const int len = __ffs(~(run >> lane)) - 1;
+                if (len > 0) up = i + len;
+                // and from row to row where this warp's slots hold both (the
+                // 32 slots span a few rows): three doublings in registers, so
+                // that later finds take a hop or two
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    const int l = up - t0;
+                    const int v = __shfl_sync(0xffffffffu, up, l & 31);
+                    if ((unsigned)l < 32u) up = v;
+                }
+                if (live) S.par[i] = (uint16_t)up;
+            } else if (live) {
+                int up = i;
+                bool more = false;
+                for (int dy = 0; dy <= p.ry && y + dy <= 255; ++dy) {
+                    const int dlo = dy == 0 ? 0 : -min(p.rx, x), dhi = min(p.rx, 255 - x);
+                    const uint32_t c0 = cell + (uint32_t)(256 * dy + dlo);
+                    int j, s1;
+                    row_slots(S, b, dy, dlo, dhi, &j, &s1);
+                    for (; j < s1; ++j) {
+                        if (j == i || !TPX_IN(j, C)) continue;
+                        const uint64_t rj = S.srec[j];
+                        if (r_cell(rj) - c0 > (uint32_t)(dhi - dlo) || !within(r_tof(rj) - tb, p.dt)) continue;
+                        if (dimmer(S, i, tot, j, r_tot(rj))) dim = true; else S.notpeak[j] = 1;
+                        // CC: the pixel points to its first partner; any other is
+                        // united in a second walk
+                        if (up == i) up = j; else more = true;
+                    }
+                }
+                if (MODE == TPX_MODE_CC) {
+                    S.par[i] = (uint16_t)up;
+                    if (more) { atomicOr(&S.u3.rwalk[i >> 5], 1u << (i & 31)); S.rw = 1; }
+                }
             }
+            if (dim) S.notpeak[i] = 1;
         }
-        __syncthreads();
-
+        // pixels outside the table: each row of their boxes (dense lanes, the
+        // last warps first: they have the fewest slots above)
+        const int rows = 2 * p.ry + 1;
+        for (int t = NTW - 1 - tid; t < nov * rows; t += NTW)
+            overflow_row<MODE, false>(S, p, pb, t / rows, t % rows - p.ry, nb);
+        cta_sync();
         TPX_PH(7);
+
         int ncl = 0;
         if (MODE == TPX_MODE_CC) {
-            // compress: every pixel points to the root of its tree
-            for (int q = R0 + tid; q < R1; q += NT) {
-                const uint32_t w = sh_ld(pbase + 4 * q);
-                if ((w & 0xFFFFu) == (uint32_t)q) continue;
-                sh_st(pbase + 4 * q, (w & 0xFFFF0000u) | find_hw(pbase, w & 0xFFFFu));
+            // unions of the queued pairs; the slots marked for a second walk
+            // unite each of their partners in turn
+            const int nq = min(S.qn, QN);
+            for (int k = tid; k < nq; k += NTW) {
+                const uint32_t pr = S.u2.queue[k];
+                if (TPX_IN(pr >> 16, n) && TPX_IN(pr & 0xFFFFu, n)) uf_unite(pb, pr >> 16, pr & 0xFFFFu);
             }
-            __syncthreads();
-            TPX_PH(8);
-            // unions of the second partners, warp-synchronous: each trip
-            // advances every active lane by one find hop (path halving) or one
-            // link attempt, the larger root position linked under the smaller.
-            // A pixel marked for a re-walk unites each of its partners in turn.
-            for (int qb = R0 + (tid & ~31); qb < R1; qb += NT) {
-                const int q = qb + lane;
-                uint32_t b = q < R1 ? sh_ld(pbase + 4 * q) >> 16 : NO_EXT;
-                if (b == REWALK) {
-                    rewalk_unite<MODE>(S, p, pbase, q);
-                    b = NO_EXT;
+            if (S.rw)
+                for (int i = tid; i < n; i += NTW) {
+                    if (!((S.u3.rwalk[i >> 5] >> (i & 31)) & 1u)) continue;
+                    if (i < nb) rewalk_unite(S, p, pb, i);
+                    else
+                        for (int dy = -p.ry; dy <= p.ry; ++dy) overflow_row<MODE, true>(S, p, pb, i - nb, dy, nb);
                 }
-                __syncwarp();
-                uint32_t a = (uint32_t)q;
-                bool active = b != NO_EXT && TPX_IN(b, C);
-                while (__any_sync(0xffffffffu, active)) {
-                    if (active) {
-                        const uint32_t wa = sh_ld(pbase + 4 * a), wb = sh_ld(pbase + 4 * b);
-                        const uint32_t pa = wa & 0xFFFFu, pb = wb & 0xFFFFu;
-                        if (pa != a || pb != b) {
-                            if (pa != a) {
-                                const uint32_t ga = sh_ld(pbase + 4 * pa) & 0xFFFFu;
-                                if (ga != pa) sh_st(pbase + 4 * a, (wa & 0xFFFF0000u) | ga);
-                                a = ga;
-                            }
-                            if (pb != b) {
-                                const uint32_t gb = sh_ld(pbase + 4 * pb) & 0xFFFFu;
-                                if (gb != pb) sh_st(pbase + 4 * b, (wb & 0xFFFF0000u) | gb);
-                                b = gb;
-                            }
-                        } else if (a == b) {
-                            active = false;
-                        } else {
-                            const uint32_t lo = min(a, b), hi = max(a, b);
-                            const uint32_t wh = hi == a ? wa : wb;
-                            const uint32_t old = sh_cas(pbase + 4 * hi, wh, (wh & 0xFFFF0000u) | lo);
-                            if (old == wh) active = false;
-                            else { a = lo; b = old & 0xFFFFu; }   // hi was linked meanwhile: go on above it
-                        }
-                    }
-                }
-            }
-            __syncthreads();
+            cta_sync();
             TPX_PH(9);
-            // roots; the hash is free now: member-list heads, cleared
-            for (int q = R0 + tid; q < R1; q += NT) {
-                S.u1.mhead[q] = EMPTY;
-                if (S.buf[pad(q)] != INVALID) S.u2.rootof[q] = (uint16_t)find_ro(pbase, (uint32_t)q);
+            // roots (each slot's pointer is changed by its own thread alone);
+            // the cell table is free now: member-list heads, cleared
+            for (int i = tid; i < n; i += NTW) {
+                uf_st(pb, (uint32_t)i, uf_root(pb, (uint32_t)i));
+                S.u1.mhead[i] = EMPTY;
             }
-            __syncthreads();
+            for (int i = tid; i < C / 32; i += NTW) S.u3.lbits[i] = 0u;
+            cta_sync();
             TPX_PH(10);
-            // member lists: each kept pixel joins its root's list (the links
-            // take the first half of the union-find array); the roots are
-            // appended to the root list (its second half) in any order, and
-            // the label bitmap is cleared
-            uint16_t *mnext = reinterpret_cast<uint16_t *>(S.parent);
-            uint16_t *rootpos = reinterpret_cast<uint16_t *>(S.parent) + C;
-            for (int w = tid; w < C / 32; w += NT) S.lbits[w] = 0u;
-            for (int qb = R0 + (tid & ~31); qb < R1; qb += NT) {
-                const int q = qb + lane;
+            // member lists: each kept pixel joins its root's list; the roots
+            // are appended to the root list in any order
+            for (int t0 = tid & ~31; t0 < n; t0 += NTW) {
+                const int i = t0 + lane;
                 bool is_root = false;
-                if (q < R1 && S.buf[pad(q)] != INVALID) {
-                    const uint32_t rt = S.u2.rootof[q];
-                    if (TPX_IN(rt, C)) mnext[q] = (uint16_t)atomicExch(&S.u1.mhead[rt], (uint32_t)q);
-                    is_root = rt == (uint32_t)q;
+                if (i < n) {
+                    const uint32_t rt = S.par[i];
+                    if (TPX_IN(rt, n)) S.u2.mnext[i] = (uint16_t)atomicExch(&S.u1.mhead[rt], (uint32_t)i);
+                    is_root = rt == (uint32_t)i;
                 }
                 const unsigned m = __ballot_sync(0xffffffffu, is_root);
                 int at = 0;
                 if (lane == 0 && m) at = atomicAdd(&S.nroot, __popc(m));
                 at = __shfl_sync(0xffffffffu, at, 0) + __popc(m & ((1u << lane) - 1u));
-                if (is_root && TPX_IN(at, C)) rootpos[at] = (uint16_t)q;
+                if (is_root && TPX_IN(at, C)) S.u5.rootpos[at] = (uint16_t)i;
             }
-            __syncthreads();
-            TPX_PH(11);
+            cta_sync();
             ncl = S.nroot;
-            if (STAGED) {
-                // The last warp copies the previous tile's staged records out
-                // while the others walk this tile's member lists: one thread
-                // per cluster forms the exact integer moments (Sec. V.C) and
-                // finds the cluster's earliest pixel in (time, position) order
-                // -- its canonical label -- which is kept in the upper half of
-                // the list head and marked in the label bitmap. A thread keeps
-                // its first cluster's moments in registers until the labels'
-                // ranks are known; the records are staged in label order.
-                constexpr int NWALK = NT - 32;
-                Moments held{0, 0, 0, 0, 0, 0, 0, 0};
-                if (tid >= NWALK) {
-                    flush_ring_warp<BATCH>(S, p, seq, false);
-                } else {
-                    for (int i = tid; i < ncl; i += NWALK) {
-                        if (!TPX_IN(i, C)) break;
-                        const uint32_t rt = rootpos[i];
-                        if (!TPX_IN(rt, C)) continue;
-                        const uint32_t head = S.u1.mhead[rt] & 0xFFFFu;
-                        const Moments m = walk_members(S, p, head);
-                        if (!TPX_IN(m.best_lo, C)) continue;
-                        S.u1.mhead[rt] = (m.best_lo << 16) | head;
-                        atomicOr(&S.lbits[m.best_lo >> 5], 1u << (m.best_lo & 31));
-                        if (i == tid) held = m;
-                    }
-                }
-                __syncthreads();
-                TPX_PH(12);
-                // the labels' ranks: one warp scans the bitmap's counts
-                if (tid < 32) {
-                    constexpr int WPL = C / 32 / 32;   // bitmap words per lane
-                    int c = 0;
-#pragma unroll
-                    for (int k = 0; k < WPL; ++k) c += __popc(S.lbits[lane * WPL + k]);
-                    int incl = c;
-#pragma unroll
-                    for (int o = 1; o < 32; o <<= 1) {
-                        const int u = __shfl_up_sync(0xffffffffu, incl, o);
-                        if (lane >= o) incl += u;
-                    }
-                    int run = incl - c;
-#pragma unroll
-                    for (int k = 0; k < WPL; ++k) {
-                        S.lpre[lane * WPL + k] = (uint16_t)run;
-                        run += __popc(S.lbits[lane * WPL + k]);
-                    }
-                }
-                __syncthreads();
-                TPX_PH(19);
-                tpx_record *dst = p.stage + ((long long)blockIdx.x * NP + (S.pend_head + S.pend_count) % NP) * C;
-                if (tid < NWALK && tid < ncl && held.n > 0) {
-                    const int k = label_rank(S, held.best_lo);
-                    if (TPX_IN(k, C)) put_record(dst + k, held, S, p, base, E.tdc.n);
-                }
-                // clusters beyond one per walking thread: walked again
-                for (int i = tid + NWALK; tid < NWALK && i < ncl; i += NWALK) {
-                    if (!TPX_IN(i, C)) break;
-                    const uint32_t rt = rootpos[i];
-                    if (!TPX_IN(rt, C)) continue;
-                    const Moments m = walk_members(S, p, S.u1.mhead[rt] & 0xFFFFu);
-                    const int k = label_rank(S, m.best_lo);
-                    if (TPX_IN(k, C) && TPX_IN(m.best_lo, C)) put_record(dst + k, m, S, p, base, E.tdc.n);
-                }
-            } else {
-            // one thread per root walks its list for the cluster's earliest
-            // pixel in (time, position) order -- its canonical label -- keeps
-            // it in the upper half of the list head and flags it (bit 1 of
-            // notpeak)
-            for (int i = tid; i < ncl; i += NT) {
-                if (!TPX_IN(i, C)) break;
-                const uint32_t q = rootpos[i];
-                if (!TPX_IN(q, C)) continue;
-                const uint32_t head = S.u1.mhead[q] & 0xFFFFu;
-                uint64_t best = ~0ull;
-                for (uint32_t m = head; m != EMPTY; m = mnext[m]) {
-                    if (!TPX_IN(m, C)) break;
-                    best = min(best, ((uint64_t)r_tof(S.buf[pad((int)m)]) << 16) | m);
-                }
-                const uint32_t lp = (uint32_t)(best & 0xFFFFu);
-                S.u1.mhead[q] = (lp << 16) | head;
-                if (TPX_IN(lp, C)) S.notpeak[lp] |= 2;
-            }
-            __syncthreads();
-            // cluster ids in ascending label position
-            int c = 0;
-            for (int j = 0; j < kpd; ++j) {
-                const int q = p0 + j;
-                if (q >= R0 && q < R1 && (S.notpeak[q] & 2)) ++c;
-            }
-            int excl = block_scan_int(S, c, &ncl);
-            for (int j = 0; j < kpd; ++j) {
-                const int q = p0 + j;
-                if (q >= R0 && q < R1 && (S.notpeak[q] & 2)) {
-                    if (TPX_IN(excl, C)) rootpos[excl] = (uint16_t)q;
-                    ++excl;
-                }
-            }
-            }
         } else {
-            // PAPER mode: one record per local maximum (list kept in parent[])
+            // PAPER mode: one record per local maximum, marked by position
+            for (int i = tid; i < C / 32; i += NTW) S.u3.lbits[i] = 0u;
+            cta_sync();
             int c = 0;
-            for (int j = 0; j < kpd; ++j) {
-                const int q = p0 + j;
-                if (q >= R0 && q < R1 && S.buf[pad(q)] != INVALID && !S.notpeak[q]) ++c;
-            }
-            int excl = block_scan_int(S, c, &ncl);
-            for (int j = 0; j < kpd; ++j) {
-                const int q = p0 + j;
-                if (q >= R0 && q < R1 && S.buf[pad(q)] != INVALID && !S.notpeak[q]) {
-                    if (TPX_IN(excl, C)) S.parent[excl] = (uint32_t)q;
-                    ++excl;
+            for (int i = tid; i < n; i += NTW)
+                if (!S.notpeak[i]) {
+                    const uint32_t q = S.spos[i];
+                    atomicOr(&S.u3.lbits[q >> 5], 1u << (q & 31));
+                    ++c;
                 }
-            }
+            c = (int)__reduce_add_sync(0xffffffffu, (unsigned)c);
+            if (lane == 0 && c) atomicAdd(&S.nroot, c);
+            cta_sync();
+            ncl = S.nroot;
         }
         bool big_done = false;   // this tile's records wait in the big-range scratch
         if constexpr (BIGR) {
-            // a big range takes its own path once the staging slot is free
-            // (the previous tile's records were copied out above)
+            // a big range takes its own path, once its record slot is free
             if (big_tile) {
-                const int k = big_range<BATCH>(S, p, base, rend, f, prev_global);
+                if (tid == 0) wait_count(&S.consumed, ent - NP, p);
+                cta_sync();
+                const int k = big_range<BATCH>(S, p, gbase, rend, f - w0, C - w0, prev_global, E, ent % NP);
                 ncl = k > 0 ? k : 0;
                 big_done = k >= 0;
                 TPX_PH(17);
-                if (tid < 32) flush_ring_warp<BATCH>(S, p, seq, false);
-                __syncthreads();
-                TPX_PH(18);
             }
         }
-
-        TPX_PH(13);
+        TPX_PH(11);
         // ---- record offsets: publish this tile's count now, look back later ----
         if (tid == 0 && tile + 1 != p.hold) {
             if (tile > 0) {
@@ -1903,198 +2009,191 @@ __global__ void __launch_bounds__(NT, MINB) fused_kernel(const Params p) {
             }
         }
         const long long ntr_here = E.tdc.n - trig_base + (long long)S.cnt[C_TDCS];
-        // records go to the CTA's staging slot (STAGED) or straight to their
-        // offset after an inline look-back
-        auto record_target = [&](long long *lim) -> tpx_record * {
-            if (STAGED) {
-                if (tid < 32) flush_ring_warp<BATCH>(S, p, seq, false);
-                __syncthreads();   // the peak list is complete
-                *lim = C;
-                return p.stage + ((long long)blockIdx.x * NP + (S.pend_head + S.pend_count) % NP) * C;
-            }
-            if (tid < 32) resolve_offset<false>(S, p, seq, tile, ncl, ntr_here, 0, 0, false);
-            __syncthreads();
-            *lim = p.cl_cap - S.clo;
-            return p.clusters + S.clo;
+        // a tile with nothing to write (no records, no triggers; not a run's
+        // first tile nor the call's last) needs no offset: its count is
+        // published, and the successors' look-backs add it up
+        const bool any = STAGED && (ncl != 0 || S.cnt[C_TDCS] != 0 || (BATCH && tile == tile0) || tile == p.n_tiles - 1);
+        tpx_record *const stage = STAGED ? p.stage + ((long long)blockIdx.x * NP + ent % NP) * C : nullptr;
+        if (STAGED) {   // the slot's previous records are out (checked before the next barrier)
+            if (tid == 0) wait_count(&S.consumed, ent - NP, p);
+        } else if (wid == 0) {   // unstaged: the records' offset now, by an inline look-back
+            longlong2 O;
+            resolve_offset<false>(p, seq, tile, ncl, ntr_here, 0, 0, false, true, &O);
+            if (lane == 0) S.clo = O.x;
+        }
+        const int ncl_here = big_done ? 0 : ncl;   // records to form here
+        auto put = [&](int k, const tpx_record &o) {
+            if (STAGED) stage[k] = o;
+            else if (k < p.cl_cap - S.clo) out_record(p, S.clo + k, o);
         };
-
         if (MODE == TPX_MODE_CC) {
-            // Each kept pixel writes its label (the stream index of its
-            // cluster's earliest pixel); then one thread per cluster walks the
-            // member list and forms the exact integer moments in registers
-            // (Sec. V.C).
-            const uint16_t *mnext = reinterpret_cast<const uint16_t *>(S.parent);
-            const uint16_t *rootpos = mnext + C;
-            __syncthreads();
-            unsigned long long c_pk = 0;
-            for (int q = W0 + tid; q < W1; q += NT) {
-                const uint64_t r = S.buf[pad(q)];
-                bool kept = q >= R0 && r != INVALID;
-                uint32_t lp = 0;
-                uint8_t pk = 0;
-                if (kept && !TPX_IN(S.u2.rootof[q], C)) kept = false;
-                if (kept) {
-                    lp = S.u1.mhead[S.u2.rootof[q]] >> 16;
-                    pk = (S.notpeak[q] & 1) ? 0 : 1;
-                    c_pk += pk;
-                }
-                if (!TPX_IN(base + q, rend)) continue;
-                if (p.labels) p.labels[base + q] = kept ? p.idx_base + base + (long long)lp : -1LL;
-                else if (p.labels32) p.labels32[base + q] = kept ? (int)(p.idx_base - p.lab32_base + base + lp) : -1;
-                if (p.is_peak) p.is_peak[base + q] = pk;
+            // One thread per cluster walks its member list: the exact integer
+            // moments (Sec. V.C) and the cluster's earliest pixel in (time,
+            // position) order -- its canonical label -- which is kept in the
+            // upper half of the list head and marked in the label bitmap. A
+            // thread keeps its first cluster's moments in registers until the
+            // labels' ranks are known.
+            Moments held{0, 0, 0, 0, 0, 0, 0, 0, 0};
+            for (int k = tid; k < ncl_here; k += NTW) {
+                if (!TPX_IN(k, C)) break;
+                const uint32_t rt = S.u5.rootpos[k];
+                if (!TPX_IN(rt, C)) continue;
+                const uint32_t head = S.u1.mhead[rt] & 0xFFFFu;
+                const Moments m = walk_members(S, p, head);
+                if (!TPX_IN(m.best_lo, C)) continue;
+                S.u1.mhead[rt] = (m.best_lo << 16) | head;
+                atomicOr(&S.u3.lbits[m.best_lo >> 5], 1u << (m.best_lo & 31));
+                if (k == tid) held = m;
             }
-            c_pk = warp_sum(c_pk);
-            if (lane == 0) atomicAdd(&S.cnt[C_PEAKS], c_pk);
-            long long lim = 0;
-            tpx_record *dst = STAGED ? nullptr : record_target(&lim);
-            // records (unstaged: after the inline look-back, in label order):
-            // one thread per cluster walks its member list and forms the
-            // exact integer moments in registers (Sec. V.C)
-            for (int i = tid; !STAGED && i < ncl; i += NT) {
-                if (i >= lim) break;
-                const int q = rootpos[i];
-                if (!TPX_IN(q, C) || !TPX_IN(S.u2.rootof[q], C)) continue;
-                const uint64_t r = S.buf[pad(q)];
-                const int tofb0 = r_tof(r);
-                long long s_tot = 0, s_x = 0, s_y = 0, s_t = 0;
-                int n = 0, npk = 0;
-                for (uint32_t m = S.u1.mhead[S.u2.rootof[q]] & 0xFFFFu; m != EMPTY; m = mnext[m]) {
-                    if (!TPX_IN(m, C)) break;
-                    const uint64_t rm = S.buf[pad((int)m)];
-                    const long long tot = r_tot(rm);
-                    n += 1;
-                    npk += (S.notpeak[m] & 1) ? 0 : 1;
-                    s_tot += tot;
-                    s_x += tot * r_x(rm);
-                    s_y += tot * r_y(rm);
-                    s_t += tot * (long long)(r_tof(rm) - tofb0);
+            cta_sync();
+            TPX_PH(12);
+            // the labels' ranks: one warp scans the bitmap's counts; the
+            // others clear the label entries (they take the member links'
+            // place, unless more clusters than threads have to be walked again)
+            const bool many = ncl_here > NTW;
+            if (wid == 0) scan_label_bits(S);
+            else if (!many) for (int q = tid - 32; q < L; q += NTW - 32) S.u2.lab[q] = NOLAB;
+            cta_sync();
+            TPX_PH(19);
+            if (tid < ncl_here && held.n > 0) {
+                const int k = label_rank(S, held.best_lo);
+                if (TPX_IN(k, C)) put(k, make_record(held, S, p, gbase, E.tdc.n));
+            }
+            if (many) {
+                for (int i = tid + NTW; i < ncl_here; i += NTW) {
+                    if (!TPX_IN(i, C)) break;
+                    const uint32_t rt = S.u5.rootpos[i];
+                    if (!TPX_IN(rt, C)) continue;
+                    const Moments m = walk_members(S, p, S.u1.mhead[rt] & 0xFFFFu);
+                    const int k = label_rank(S, m.best_lo);
+                    if (TPX_IN(k, C)) put(k, make_record(m, S, p, gbase, E.tdc.n));
                 }
-                const int seg = r_seg(r);
-                const long long tofc0 = (long long)tofb0 - kTofBias;
-                tpx_record o;
-                o.label = p.idx_base + base + q;
-                o.shot = E.tdc.n + seg;
-                o.t0 = S.tdc_t[seg] + tofc0;
-                o.s_tot = s_tot; o.s_x = s_x; o.s_y = s_y; o.s_t = s_t;
-                o.n = n; o.n_peaks = npk;
-                com_from_moments(s_x, s_y, s_t, s_tot, tofc0, &o.x, &o.y, &o.tof);
-                out_record(p, S.clo + i, o);   // unstaged: straight to its offset
+                cta_sync();
+                for (int q = tid; q < L; q += NTW) S.u2.lab[q] = NOLAB;
+                cta_sync();
+            }
+            // the label position of each kept pixel, by position
+            if (!big_done) {
+                unsigned c = 0;
+                for (int i = tid; i < n; i += NTW) {
+                    const bool pk = !S.notpeak[i];
+                    if (!TPX_IN(S.par[i], C)) continue;
+                    S.u2.lab[S.spos[i]] = (uint16_t)((S.u1.mhead[S.par[i]] >> 16) | (pk ? PEAK : 0));
+                    c += pk;
+                }
+                c = __reduce_add_sync(0xffffffffu, c);
+                if (lane == 0 && c) atomicAdd(&S.n_pk, c);
             }
         } else {
-            unsigned long long c_pk = 0;
-            for (int q = W0 + tid; q < W1; q += NT) {
-                const uint64_t r = S.buf[pad(q)];
-                long long lab = -1;
-                uint8_t pk = 0;
-                if (q >= R0 && r != INVALID) {
-                    lab = p.idx_base + base + q;
-                    pk = S.notpeak[q] ? 0 : 1;
-                    c_pk += pk;
-                }
-                if (!TPX_IN(base + q, rend)) continue;
-                if (p.labels) p.labels[base + q] = lab;
-                else if (p.labels32) p.labels32[base + q] = lab < 0 ? -1 : (int)(lab - p.lab32_base);
-                if (p.is_peak) p.is_peak[base + q] = pk;
-            }
-            c_pk = warp_sum(c_pk);
-            if (lane == 0) atomicAdd(&S.cnt[C_PEAKS], c_pk);
-            long long lim = 0;
-            tpx_record *dst = record_target(&lim);
+            if (wid == 0) scan_label_bits(S);
+            cta_sync();
             // records: box neighbourhood sums of each local maximum (Sec. V.C)
-            for (int i = tid; i < ncl; i += NT) {
-                if (i >= lim) break;
-                const int q = (int)S.parent[i];
-                if (!TPX_IN(q, C)) continue;
-                const uint64_t r = S.buf[pad(q)];
-                const int x = r_x(r), y = r_y(r), sg = r_seg(r), tb = r_tof(r);
-                long long n = 0, s_tot = 0, s_x = 0, s_y = 0, a2 = 0;
-                int tmin = tb;
-                for (int dx = -p.rx; dx <= p.rx; ++dx) {
-                    const int cx = x + dx;
-                    if (cx < 0 || cx > 255) continue;
-                    for (int dy = -p.ry; dy <= p.ry; ++dy) {
-                        const int cy = y + dy;
-                        if (cy < 0 || cy > 255) continue;
-                        for (uint32_t j = S.u1.head[hcell(sg, cx, cy)]; j != EMPTY; j = S.u2.next[j]) {
-                            if (!TPX_IN(j, C)) break;
-                            const uint64_t rj = S.buf[pad((int)j)];
-                            if (r_x(rj) != cx || r_y(rj) != cy || r_seg(rj) != sg) continue;
-                            const int d = r_tof(rj) - tb;
-                            if (d < -p.dt || d > p.dt) continue;
-                            const long long tj = r_tot(rj);
-                            n += 1; s_tot += tj; s_x += tj * cx; s_y += tj * cy; a2 += tj * r_tof(rj);
-                            tmin = min(tmin, r_tof(rj));
+            unsigned c = 0;
+            for (int i = tid; i < n; i += NTW) {
+                const uint32_t q = S.spos[i];
+                const bool pk = !S.notpeak[i];
+                S.u2.lab[q] = (uint16_t)(q | (pk ? PEAK : 0));
+                if (!pk) continue;
+                ++c;
+                const uint64_t r = S.srec[i];
+                const int x = r_x(r), y = r_y(r), tb = r_tof(r);
+                const uint32_t bit = tbit(r), cell = r_cell(r);
+                Moments m{0, 0, 0, 0, 0, 1, r_seg(r), q, tb};
+                const int dlo = -min(p.rx, x), dhi = min(p.rx, 255 - x);
+                for (int dy = -min(p.ry, y); dy <= min(p.ry, 255 - y); ++dy) {
+                    const uint32_t c0 = cell + (uint32_t)(256 * dy + dlo);
+                    auto add = [&](int j) {
+                        const uint64_t rj = S.srec[j];
+                        const int tj = r_tof(rj);
+                        if (r_cell(rj) - c0 > (uint32_t)(dhi - dlo) || !within(tj - tb, p.dt)) return;
+                        const uint32_t aj = (uint32_t)r_tot(rj);
+                        m.n += 1;
+                        m.s_tot += aj;
+                        m.s_x += aj * (uint32_t)r_x(rj);
+                        m.s_y += aj * (uint32_t)r_y(rj);
+                        m.s_tt += (long long)((uint64_t)aj * (uint32_t)tj);
+                        m.tofb0 = min(m.tofb0, tj);
+                    };
+                    int j, s1;
+                    row_slots(S, bit, dy, dlo, dhi, &j, &s1);
+                    for (; j < s1; ++j)
+                        if (TPX_IN(j, C)) add(j);
+                    if (nov == 0) continue;
+                    const uint32_t row = (bit + 256u * (uint32_t)dy) & (TB - 1);
+                    for (int dx = dlo; dx <= dhi; ++dx)
+                        for (uint32_t o = S.u1.t.ohead[ohash(row + dx)]; o != EMPTY; o = S.u5.onext[o]) {
+                            if (!TPX_IN(nb + o, C)) break;
+                            if (r_cell(S.srec[nb + o]) == cell + (uint32_t)(256 * dy + dx)) add(nb + (int)o);
                         }
-                    }
                 }
-                const long long s_t = a2 - (long long)tmin * s_tot;
-                const long long tofc0 = (long long)tmin - kTofBias;
-                tpx_record o;
-                o.label = p.idx_base + base + q;
-                o.shot = E.tdc.n + sg;
-                o.t0 = S.tdc_t[sg] + tofc0;
-                o.s_tot = s_tot; o.s_x = s_x; o.s_y = s_y; o.s_t = s_t;
-                o.n = (int)n; o.n_peaks = 1;
-                com_from_moments(s_x, s_y, s_t, s_tot, tofc0, &o.x, &o.y, &o.tof);
-                if (STAGED) dst[i] = o;
-                else out_record(p, S.clo + i, o);
+                const int k = label_rank(S, q);
+                if (TPX_IN(k, C)) put(k, make_record(m, S, p, gbase, E.tdc.n));
+            }
+            c = __reduce_add_sync(0xffffffffu, c);
+            if (lane == 0 && c) atomicAdd(&S.n_pk, c);
+        }
+        cta_sync();
+        TPX_PH(13);
+        // ---- per-packet outputs over the range (and the packets before the
+        // call's first trigger) ----
+        {
+            const int W1 = skip ? 0 : (term ? L - 1 : L);
+            for (int q = tid; q < W1; q += NTW) {
+                if (!TPX_IN(gbase + q, rend)) continue;
+                const uint32_t v = S.u2.lab[q];
+                const bool k = v != NOLAB;
+                const long long lp = (long long)(v & (PEAK - 1));
+                if (p.labels) p.labels[gbase + q] = k ? p.idx_base + gbase + lp : -1LL;
+                else if (p.labels32) p.labels32[gbase + q] = k ? (int)(p.idx_base - p.lab32_base + gbase + lp) : -1;
+                if (p.is_peak) p.is_peak[gbase + q] = k && (v & PEAK) ? 1 : 0;
             }
         }
         TPX_PH(14);
         if (BATCH) {   // this tile's trigger times wait with its records
             const int nt = min((int)S.cnt[C_TDCS], MAXSEG);
-            long long *ts = p.bt.tstage + ((long long)blockIdx.x * NP + (S.pend_head + S.pend_count) % NP) * T;
-            for (int i = tid; i < nt; i += NT) ts[i] = S.tdc_t[i];
-            __syncthreads();   // every thread has its slot before the tile joins the ring
+            long long *ts = p.bt.tstage + ((long long)blockIdx.x * NP + ent % NP) * T;
+            for (int i = tid; i < nt; i += NTW) ts[i] = S.tdc_t[i];
         }
         if (tid == 0) {
+            S.cnt[C_PACKETS] = (unsigned long long)cnt;
             S.cnt[C_CLUSTERS] = (unsigned long long)ncl;
-            if (STAGED) {
-                // a tile with nothing to write (no records, no triggers; not
-                // a run's first tile nor the call's last) needs no offset: its
-                // count is published, and the successors' look-backs add it up
-                const bool first = tile == tile0;
-                if (ncl != 0 || S.cnt[C_TDCS] != 0 || (BATCH && first) || tile == p.n_tiles - 1) {
-                    const int e = (S.pend_head + S.pend_count) % NP;
-                    S.pend[e].tile = tile;
-                    S.pend[e].ncl = ncl;
-                    S.pend[e].ntr = ntr_here;
-                    S.pend[e].ntdc = (int)S.cnt[C_TDCS];
-                    S.pend[e].run = run;
-                    S.pend[e].first = first;
-                    S.pend[e].big = big_done;
-                    S.pend_count += 1;
-                }
+            if (!big_done) {   // a big range counted its own pixels
+                S.cnt[C_KEPT] = (unsigned long long)kept;
+                S.cnt[C_DROP_PRE] = S.n_pre;
+                S.cnt[C_DROP_BG] = S.n_bg;
+                S.cnt[C_PEAKS] = S.n_pk;
             }
         }
-        __syncthreads();
+        cta_sync();
         TPX_PH(15);
-        // the tile's counters join the CTA's, and the per-tile fields are
-        // reset for the next tile (which starts with a barrier)
-        if (tid < C_NUM) {
-            S.acc[tid] += tid == C_PACKETS ? (unsigned long long)cnt : S.cnt[tid];
-            S.cnt[tid] = 0;
-        }
-        // the next tile and its unwrap state, by warp 0 alone: no other warp
-        // reads S.tile or S.E before the next barrier
-        if (tid == 0) S.next_tile = (long long)claim;
-        __syncwarp();
-        if (tid < 8 && S.next_tile < p.n_tiles)
-            reinterpret_cast<long long *>(&S.E)[tid] =
-                __ldcg(reinterpret_cast<const long long *>(&p.ts.pre[S.next_tile]) + tid);
+        // the tile's counters join the CTA's; the tile goes to the service warp
         if (tid == 0) {
-            S.tile = S.next_tile;
             unsigned st = S.status & ~ST_BIG;
             if (BATCH && (st & (ST_CAPACITY | ST_EXCEPTION))) {   // only this run is redone
                 p.bt.run_failed[run] = 1u;
                 st = (st & ~(ST_CAPACITY | ST_EXCEPTION)) | ST_RUN_REDO;
             }
             if (st) atomicOr(&p.ctl->status, st);
-            S.status = 0;
-            S.first_tdc = INT_MAX;
-            S.first_pix = INT_MAX;
-            S.nroot = 0;
-            S.la_first[0] = S.la_first[1] = S.la_first[2] = INT_MAX;
+            if (any) {
+                Smem::Pend &e = S.pend[ent % NP];
+                e.tile = tile;
+                e.ncl = ncl;
+                e.ntr = ntr_here;
+                e.ntdc = (int)(ntr_here - (E.tdc.n - trig_base));
+                e.run = run;
+                e.first = tile == tile0;
+                e.big = big_done;
+            }
+            __threadfence_block();   // the staged records are this CTA's own
+            *reinterpret_cast<volatile int *>(&S.entries) = ent + (any ? 1 : 0);
+            __threadfence_block();
+            *reinterpret_cast<volatile int *>(&S.produced) = it + 1;
+        }
+        ent += any ? 1 : 0;
+        __syncwarp();
+        if (tid < C_NUM) {
+            S.acc[tid] += S.cnt[tid];
+            S.cnt[tid] = 0;
         }
     }
 }

@@ -18,7 +18,7 @@
 // TPX_EUNSUPPORTED and its outputs are incomplete.
 //
 // The array is a file-scope __device__ variable: every GPU that loads the
-// library holds it (about 2.4 MB) until the process exits, and all calls on a
+// library holds it (about 3.0 MB) until the process exits, and all calls on a
 // device share it. It keeps the contents of the last call; the per-call
 // control block is cleared before each launch, and the look-back flags carry
 // a per-device sequence number so stale flags from an earlier call never
@@ -51,6 +51,8 @@ struct NoAllocScratch {
     unsigned cflags[kMaxTiles];
     tpxk::GAgg agg[kMaxTiles];
     tpxk::GAgg pre[kMaxTiles];
+    tpxk::GChain head[kMaxTiles];
+    tpxk::TileInfo tinfo[kMaxTiles];
     long long cagg[kMaxTiles];
     long long cpre[kMaxTiles];
 };
@@ -157,6 +159,8 @@ extern "C" int tpx_process_noalloc(const tpx_config *cfg, void *cuda_stream, con
         p.ts.cflags = scr->cflags;
         p.ts.agg = scr->agg;
         p.ts.pre = scr->pre;
+        p.ts.head = scr->head;
+        p.ts.tinfo = scr->tinfo;
         p.ts.cagg = scr->cagg;
         p.ts.cpre = scr->cpre;
         p.ctl = &scr->ctl;

@@ -15,7 +15,13 @@
 //      1024 tiles, and each block's total;
 //   3. k_top_scan: one block scans the block totals, starting from the state
 //      before the call;
-//   4. k_apply: the state before each tile, and after the last one.
+//   4. k_apply: the state before each tile (its pixel chain carried on to the
+//      tile's first TDC packet, where the tile's range starts), and after the
+//      last one.
+// Beside the aggregates, k_tile_aggs leaves what the fused kernel plans its
+// ranges from (TileInfo): each tile's first TDC packet and whether a pixel wrap
+// lies in it, so that the fused kernel neither searches for the end of a range
+// nor follows the pixel chain inside it, save near a wrap.
 // In a batch of independent runs every run is a stream of its own: the scan is
 // segmented, restarting at each run's first tile.
 #include <cuda_runtime.h>
@@ -59,22 +65,25 @@ struct WarpChain {
     long long n;
     bool any;
 };
-__device__ __forceinline__ void warp_chain_step(WarpChain &c, bool h0, long long r0, bool h1, long long r1,
+// Returns whether this lane found a wrap step.
+__device__ __forceinline__ bool warp_chain_step(WarpChain &c, bool h0, long long r0, bool h1, long long r1,
                                                 long long thr, int lane) {
     const bool has = h0 || h1;
     const unsigned m = __ballot_sync(0xffffffffu, has);
-    if (!m) return;
+    if (!m) return false;
     const long long pf = h0 ? r0 : r1;       // first of the pair
     const long long pl = h1 ? r1 : r0;       // last of the pair
     long long s = (h0 && h1) ? jump(r1 - r0, thr) : 0;
+    bool found = s != 0;
     // the value before this pair: the last one of the nearest lower lane with
     // a value, else the chain's last value before this step
     const unsigned lower = m & ((1u << lane) - 1u);
     const int src = lower ? 31 - __clz(lower) : 0;
     const long long prev_lane = __shfl_sync(0xffffffffu, pl, src);
-    if (has) {
-        if (lower) s += jump(pf - prev_lane, thr);
-        else if (c.any) s += jump(pf - c.last, thr);
+    if (has && (lower || c.any)) {
+        const long long b = jump(pf - (lower ? prev_lane : c.last), thr);
+        s += b;
+        found |= b != 0;
     }
     c.sum += s;
     const int lo = __ffs(m) - 1, hi = 31 - __clz(m);
@@ -84,9 +93,15 @@ __device__ __forceinline__ void warp_chain_step(WarpChain &c, bool h0, long long
     c.last = step_last;
     c.any = true;
     c.n += __popc(m) + __popc(__ballot_sync(0xffffffffu, h0 && h1));
+    return found;
 }
 
-__global__ void __launch_bounds__(AW * 32) k_tile_aggs(const Params p, int T) {
+// Bound by the packet stream's bytes once the loads run ahead: KS steps of 64
+// packets are in flight per warp while the previous KS are combined. A step of
+// pixels only (the common one) takes a short path: the neighbour lane's last
+// value by one shuffle, the wrap test on both differences, nothing to rank.
+constexpr int KS = 4;
+__global__ void __launch_bounds__(AW * 32, 3) k_tile_aggs(const Params p, int T) {
     const int lane = threadIdx.x & 31;
     const long long warp = (long long)blockIdx.x * AW + (threadIdx.x >> 5);
     const long long nw = (long long)gridDim.x * AW;
@@ -94,46 +109,82 @@ __global__ void __launch_bounds__(AW * 32) k_tile_aggs(const Params p, int T) {
     unsigned long long c_pix = 0, c_tdc = 0, c_bad = 0;
     for (long long tile = warp; tile < p.n_tiles; tile += nw) {
         const TileSpan sp = tile_span(p, tile, T);
-        WarpChain cp{0, 0, 0, 0, false}, ct{0, 0, 0, 0, false};
+        WarpChain cp{0, 0, 0, 0, false}, ct{0, 0, 0, 0, false}, ch{0, 0, 0, 0, false};
+        int first_tdc = -1;
+        bool wraps = false;   // this lane saw a pixel wrap step
         const uint64_t *src = p.pk + sp.base;
         const bool vec = (sp.base & 1) == 0;
-        // the lane's two packets of step q0 (zero past the tile)
-        auto load2 = [&](int q0, uint64_t &a, uint64_t &b) {
-            const int q = q0 + 2 * lane;
-            a = 0;
-            b = 0;
-            if (vec && q + 1 < sp.cnt) {
-                const ulonglong2 v = __ldcs(reinterpret_cast<const ulonglong2 *>(src + q));
-                a = v.x;
-                b = v.y;
-            } else {
-                if (q < sp.cnt) a = __ldcs(src + q);
-                if (q + 1 < sp.cnt) b = __ldcs(src + q + 1);
+        // the lane's two packets of each step from q0 on (zero past the tile)
+        auto load = [&](int q0, uint64_t (&v)[2 * KS]) {
+#pragma unroll
+            for (int k = 0; k < KS; ++k) {
+                const int q = q0 + 64 * k + 2 * lane;
+                uint64_t a = 0, b = 0;
+                if (vec && q + 1 < sp.cnt) {
+                    const ulonglong2 u = __ldcs(reinterpret_cast<const ulonglong2 *>(src + q));
+                    a = u.x;
+                    b = u.y;
+                } else {
+                    if (q < sp.cnt) a = __ldcs(src + q);
+                    if (q + 1 < sp.cnt) b = __ldcs(src + q + 1);
+                }
+                v[2 * k] = a;
+                v[2 * k + 1] = b;
             }
         };
-        // one step ahead: the next 64 packets are in flight while these are combined
-        uint64_t nx0, nx1;
-        load2(0, nx0, nx1);
-        for (int q0 = 0; q0 < sp.cnt; q0 += 64) {
+        auto step = [&](int q0, uint64_t w0, uint64_t w1) {
             const int q = q0 + 2 * lane;
-            const uint64_t w0 = nx0, w1 = nx1;
-            if (q0 + 64 < sp.cnt) load2(q0 + 64, nx0, nx1);
-            const bool in0 = q < sp.cnt, in1 = q + 1 < sp.cnt;
             const unsigned h0 = (unsigned)(w0 >> 60), h1 = (unsigned)(w1 >> 60);
-            const bool p0 = in0 && h0 == 0xBu, p1 = in1 && h1 == 0xBu;
+            const bool p0 = h0 == 0xBu, p1 = h1 == 0xBu;   // zero past the tile: neither
+            if (__all_sync(0xffffffffu, p0 && p1)) {
+                const long long r0 = pix_raw(w0), r1 = pix_raw(w1);
+                long long prev = __shfl_up_sync(0xffffffffu, r1, 1);
+                if (lane == 0) prev = cp.any ? cp.last : r0;
+                const long long s = jump(r1 - r0, tp) + jump(r0 - prev, tp);
+                wraps |= jump(r1 - r0, tp) != 0 || jump(r0 - prev, tp) != 0;
+                cp.sum += s;
+                if (!cp.any) cp.first = __shfl_sync(0xffffffffu, r0, 0);
+                cp.last = __shfl_sync(0xffffffffu, r1, 31);
+                cp.any = true;
+                cp.n += 64;
+                c_pix += 2;
+                return;
+            }
+            const bool in0 = q < sp.cnt, in1 = q + 1 < sp.cnt;
             const bool t0 = in0 && h0 == 0x6u, t1 = in1 && h1 == 0x6u;
             c_pix += (unsigned)p0 + (unsigned)p1;
             c_tdc += (unsigned)t0 + (unsigned)t1;
             c_bad += (unsigned)(in0 && !p0 && !t0) + (unsigned)(in1 && !p1 && !t1);
-            warp_chain_step(cp, p0, p0 ? pix_raw(w0) : 0, p1, p1 ? pix_raw(w1) : 0, tp, lane);
-            if (__any_sync(0xffffffffu, t0 || t1))
-                warp_chain_step(ct, t0, t0 ? tdc_raw(w0) : 0, t1, t1 ? tdc_raw(w1) : 0, tt, lane);
-        }
-        long long sp_ = cp.sum, st_ = ct.sum;
+            const long long r0 = p0 ? pix_raw(w0) : 0, r1 = p1 ? pix_raw(w1) : 0;
+            const unsigned mt = __ballot_sync(0xffffffffu, t0 || t1);
+            if (mt && first_tdc < 0) {   // the pixel chain up to the tile's first TDC packet
+                const int fl = __ffs(mt) - 1;
+                first_tdc = __shfl_sync(0xffffffffu, t0 ? q : q + 1, fl);
+                ch = cp;
+                warp_chain_step(ch, p0 && q < first_tdc, r0, p1 && q + 1 < first_tdc, r1, tp, lane);
+            }
+            wraps |= warp_chain_step(cp, p0, r0, p1, r1, tp, lane);
+            if (mt) warp_chain_step(ct, t0, t0 ? tdc_raw(w0) : 0, t1, t1 ? tdc_raw(w1) : 0, tt, lane);
+        };
+        uint64_t cur[2 * KS], nxt[2 * KS];
+        load(0, nxt);
+        for (int q0 = 0; q0 < sp.cnt; q0 += 64 * KS) {
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            sp_ += __shfl_xor_sync(0xffffffffu, sp_, o);
-            st_ += __shfl_xor_sync(0xffffffffu, st_, o);
+            for (int k = 0; k < 2 * KS; ++k) cur[k] = nxt[k];
+            if (q0 + 64 * KS < sp.cnt) load(q0 + 64 * KS, nxt);
+#pragma unroll
+            for (int k = 0; k < KS; ++k)
+                if (q0 + 64 * k < sp.cnt) step(q0 + 64 * k, cur[2 * k], cur[2 * k + 1]);
+        }
+        long long sp_ = cp.sum, st_ = ct.sum, sh_ = ch.sum;
+        const bool any_wrap = __any_sync(0xffffffffu, wraps);
+        if (any_wrap || __any_sync(0xffffffffu, st_ != 0)) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                sp_ += __shfl_xor_sync(0xffffffffu, sp_, o);
+                st_ += __shfl_xor_sync(0xffffffffu, st_, o);
+                sh_ += __shfl_xor_sync(0xffffffffu, sh_, o);
+            }
         }
         if (lane == 0) {
             GAgg a;
@@ -142,6 +193,14 @@ __global__ void __launch_bounds__(AW * 32) k_tile_aggs(const Params p, int T) {
             if (!cp.any) a.pix = chain_id();
             if (!ct.any) a.tdc = chain_id();
             p.ts.agg[tile] = a;
+            GChain h;
+            h.n = ch.n; h.first = ch.first; h.last = ch.last; h.sum = sh_;
+            if (!ch.any) h = chain_id();
+            p.ts.head[tile] = h;
+            TileInfo ti;
+            ti.first_tdc = first_tdc;
+            ti.wrap = any_wrap ? 1 : 0;
+            p.ts.tinfo[tile] = ti;
         }
     }
     // packet-class counters of the call (Ctl is cleared before the launch)
@@ -271,9 +330,19 @@ __global__ void __launch_bounds__(256) k_apply(const Params p, const GAgg *bpre)
     if (p.bt.tile_run) fresh = p.bt.run_tile0[p.bt.tile_run[t]] >= bstart;
     else fresh = false;
     const GAgg loc = p.ts.pre[t];
-    const GAgg e = fresh ? loc : acomb(bpre[b], loc, tp, tt);
+    GAgg e = fresh ? loc : acomb(bpre[b], loc, tp, tt);
+    const GAgg g = p.ts.agg[t];
+    if (t == p.n_tiles - 1 && !p.bt.tile_run && p.state_out) *p.state_out = acomb(e, g, tp, tt);
+    TileInfo ti = p.ts.tinfo[t];
+    if (e.pix.n && g.pix.n && jump(g.pix.first - e.pix.last, tp) != 0) {   // the step into the tile's first pixel
+        ti.wrap = 1;
+        p.ts.tinfo[t] = ti;
+    }
+    // the range of a tile with triggers before it starts at its first TDC
+    // packet: the pixel chain goes on to there
+    const long long trig_base = (!p.bt.tile_run && p.E0) ? p.E0->tdc.n : 0;
+    if (e.tdc.n > trig_base && ti.first_tdc >= 0) e.pix = ccomb(e.pix, p.ts.head[t], tp);
     p.ts.pre[t] = e;
-    if (t == p.n_tiles - 1 && !p.bt.tile_run && p.state_out) *p.state_out = acomb(e, p.ts.agg[t], tp, tt);
 }
 
 }  // namespace

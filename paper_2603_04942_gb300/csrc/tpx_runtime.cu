@@ -62,6 +62,7 @@ int alloc_scratch(tpx_ctx *c, int64_t max_packets) {
     if (tiles < 1) tiles = 1;
     auto al = [](size_t b) { return (b + 255) & ~size_t(255); };
     const size_t b_flags = al(sizeof(unsigned) * tiles), b_agg = al(sizeof(tpxk::GAgg) * tiles),
+                 b_head = al(sizeof(tpxk::GChain) * tiles), b_info = al(sizeof(tpxk::TileInfo) * tiles),
                  b_cnt = al(sizeof(long long) * tiles), b_blk = al(tpxk::unwrap_prepass_scratch_bytes(tiles));
     // record staging of the fused kernel: one range's records per CTA
     size_t stage_records = 0;   // the largest grid of a call times its range capacity
@@ -74,7 +75,7 @@ int alloc_scratch(tpx_ctx *c, int64_t max_packets) {
     }
     c->stage_records = (int64_t)stage_records;
     const size_t b_stage = al(sizeof(tpx_record) * stage_records);
-    const size_t total = b_flags + b_blk + 2 * b_agg + 2 * b_cnt + b_stage;
+    const size_t total = b_flags + b_blk + 2 * b_agg + b_head + b_info + 2 * b_cnt + b_stage;
     void *mem = nullptr;
     if (cudaMalloc(&mem, total) != cudaSuccess) { cudaGetLastError(); return TPX_ENOMEM; }
     if (cudaMemset(mem, 0, total) != cudaSuccess) { cudaFree(mem); return TPX_ECUDA; }
@@ -83,6 +84,8 @@ int alloc_scratch(tpx_ctx *c, int64_t max_packets) {
     c->ts.cflags = reinterpret_cast<unsigned *>(p); p += b_flags;
     c->ts.agg = reinterpret_cast<tpxk::GAgg *>(p); p += b_agg;
     c->ts.pre = reinterpret_cast<tpxk::GAgg *>(p); p += b_agg;
+    c->ts.head = reinterpret_cast<tpxk::GChain *>(p); p += b_head;
+    c->ts.tinfo = reinterpret_cast<tpxk::TileInfo *>(p); p += b_info;
     c->ts.cagg = reinterpret_cast<long long *>(p); p += b_cnt;
     c->ts.cpre = reinterpret_cast<long long *>(p); p += b_cnt;
     c->stage = reinterpret_cast<tpx_record *>(p);
@@ -515,7 +518,8 @@ int tpx_process_batch(tpx_ctx *c, const uint64_t *d_packets, const int64_t *h_ru
     const size_t need_dev = al(4 * (size_t)n_tiles) + al(8 * (size_t)n_runs) + al(8 * (size_t)(n_runs + 1)) +
                             al(4 * (size_t)n_runs) + 4 * al(8 * (size_t)n_tiles) + al(8 * (size_t)(grid * T * RG)) +
                             al(tpxk::unwrap_prepass_scratch_bytes(n_tiles)) + al(4 * (size_t)n_tiles) +
-                            2 * al(sizeof(tpxk::GAgg) * (size_t)n_tiles) + al(big_bytes) + al(stage_bytes);
+                            2 * al(sizeof(tpxk::GAgg) * (size_t)n_tiles) + al(sizeof(tpxk::GChain) * (size_t)n_tiles) +
+                            al(sizeof(tpxk::TileInfo) * (size_t)n_tiles) + al(big_bytes) + al(stage_bytes);
     const size_t need_host = 8 * (size_t)(n_runs + 1) + 8 * (size_t)n_runs + 4 * (size_t)n_tiles + 64;
     // a call captured into a CUDA graph (relaxed capture mode) gets its own
     // device tables and pinned host tables, kept for the graph's replays
@@ -576,6 +580,8 @@ int tpx_process_batch(tpx_ctx *c, const uint64_t *d_packets, const int64_t *h_ru
     B.ts.cflags = reinterpret_cast<unsigned *>(take(4 * (size_t)n_tiles));
     B.ts.agg = reinterpret_cast<tpxk::GAgg *>(take(sizeof(tpxk::GAgg) * (size_t)n_tiles));
     B.ts.pre = reinterpret_cast<tpxk::GAgg *>(take(sizeof(tpxk::GAgg) * (size_t)n_tiles));
+    B.ts.head = reinterpret_cast<tpxk::GChain *>(take(sizeof(tpxk::GChain) * (size_t)n_tiles));
+    B.ts.tinfo = reinterpret_cast<tpxk::TileInfo *>(take(sizeof(tpxk::TileInfo) * (size_t)n_tiles));
     unsigned char *big = big_bytes ? reinterpret_cast<unsigned char *>(take(big_bytes)) : nullptr;
     tpx_record *bstage = reinterpret_cast<tpx_record *>(take(stage_bytes));
     bt.run_rec_off = reinterpret_cast<long long *>(d_run_clusters);
