@@ -26,6 +26,7 @@
 #include <cstdlib>
 #include <cstring>
 
+#include "tpx_mlp_train.cuh"
 #include "tpx.h"
 #include "tpx_common.cuh"
 #include "tpx_ctx.h"
@@ -631,6 +632,10 @@ int tpx_refiner_train_step(tpx_ctx *c, float *d_params, float *d_adam_m, float *
     const Layout L(hidden);
     const int h = hidden;
     cudaStream_t s = c->stream;
+    // widths that fit the fused step's shared memory (4096 rows, width 160: 2.58 ms with the GEMMs below)
+    if (h <= tpxt::kMaxHidden)
+        return ck(tpxt::train_step(s, d_params, d_adam_m, d_adam_v, d_grad, h, step, d_x, d_y, n, lr, offset_weight, d_work,
+                                   d_loss)) ? TPX_ECUDA : TPX_OK;
     float *a1 = d_work, *a2 = a1 + (long long)n * h, *out = a2 + (long long)n * h;
     float *dout = out + (long long)n * NOUT, *d2 = dout + (long long)n * NOUT, *d1 = d2 + (long long)n * h;
     int rc = forward(c, d_params, h, d_x, n, a1, a2, out);
