@@ -231,8 +231,8 @@ def lib():
     return load()
 
 
-PHASE_NAMES = ("tile start", "packet loads", "records into slots", "pixel wraps", "trigger times",
-               "packets to records", "cell table ranks", "neighbour pass", "(unused)", "unions", "roots",
+PHASE_NAMES = ("tile start", "tile load", "records into slots", "pixel wraps", "trigger times",
+               "walk 4 (records)", "cell table ranks", "neighbour pass", "(unused)", "unions", "roots",
                "member lists", "member-list walks", "records and label entries", "labels",
                "tail", "CTA end", "big ranges (batches: the sorted-window path)", "(unused)",
                "label ranks (bitmap scan)", "big: range end, walk 2, triggers", "big: walk 4", "big: bins and sort",
