@@ -1002,6 +1002,9 @@ int tpx_process_host(tpx_ctx *c, const uint64_t *h_packets, int64_t n, int64_t i
     rc = tpx_process(c, c->st_pk, n, idx_base, h_labels ? c->st_labels : nullptr, h_is_peak ? c->st_peak : nullptr,
                      c->st_cl, cl_cap, c->st_counts, c->st_trig, trig_cap, c->st_counts + 1);
     if (rc) return rc;
+    // a call that the fused kernel could not hold is redone here, before its
+    // outputs go down
+    const int rs = tpx_sync(c, nullptr);
     int64_t counts[2] = {0, 0};
     if (ckr(cudaMemcpyAsync(counts, c->st_counts, sizeof counts, cudaMemcpyDeviceToHost, s))) return TPX_ECUDA;
     if (h_labels && n &&
@@ -1018,9 +1021,10 @@ int tpx_process_host(tpx_ctx *c, const uint64_t *h_packets, int64_t n, int64_t i
         return TPX_ECUDA;
     if (ntr > 0 && cudaMemcpyAsync(h_trig, c->st_trig, sizeof(int64_t) * ntr, cudaMemcpyDeviceToHost, s) != cudaSuccess)
         return TPX_ECUDA;
+    if (ckr(cudaStreamSynchronize(s))) return TPX_ECUDA;
     *h_n_clusters = counts[0];
     *h_n_trig = counts[1];
-    return tpx_sync(c, nullptr);
+    return rs;
 }
 
 int tpx_debug_hold_tile(tpx_ctx *c, int64_t tile) {
