@@ -59,6 +59,8 @@ struct Ctl {                     // per-launch control block, cleared before eac
     unsigned int tile_counter;
     unsigned int status;
     unsigned long long counters[C_NUM];
+    unsigned int prepass_done;   // tiles whose aggregates are written (k_prepass_small)
+    unsigned int reserved;
 };
 
 // one unwrap chain over a stretch of the stream (64-bit form)

@@ -100,33 +100,28 @@ __device__ __forceinline__ bool warp_chain_step(WarpChain &c, bool h0, long long
 // packets are in flight per warp while the previous KS are combined. A step of
 // pixels only (the common one) takes a short path: the neighbour lane's last
 // value by one shuffle, the wrap test on both differences, nothing to rank.
-constexpr int KS = 4;
-__global__ void __launch_bounds__(AW * 32, 3) k_tile_aggs(const Params p, int T) {
-    const int lane = threadIdx.x & 31;
-    const long long warp = (long long)blockIdx.x * AW + (threadIdx.x >> 5);
-    const long long nw = (long long)gridDim.x * AW;
-    const long long tp = p.thr_pix, tt = p.thr_tdc;
-    unsigned long long c_pix = 0, c_tdc = 0, c_bad = 0;
-    for (long long tile = warp; tile < p.n_tiles; tile += nw) {
-        const TileSpan sp = tile_span(p, tile, T);
-        WarpChain cp{0, 0, 0, 0, false}, ct{0, 0, 0, 0, false}, ch{0, 0, 0, 0, false};
-        int first_tdc = -1;
-        bool wraps = false;   // this lane saw a pixel wrap step
-        const uint64_t *src = p.pk + sp.base;
-        const bool vec = (sp.base & 1) == 0;
-        // the lane's two packets of each step from q0 on (zero past the tile)
+template <int KS>
+struct WarpPart {
+    WarpChain cp{0, 0, 0, 0, false}, ct{0, 0, 0, 0, false}, ch{0, 0, 0, 0, false};
+    int first_tdc = -1;
+    bool wraps = false;   // some lane saw a pixel wrap step
+    unsigned long long c_pix = 0, c_tdc = 0, c_bad = 0;   // of this lane
+
+    // packets [qb, qe) of the tile at src (qb even); vec: src is 16-byte aligned
+    __device__ __forceinline__ void run(const uint64_t *src, bool vec, int qb, int qe, long long tp, long long tt, int lane) {
+        // the lane's two packets of each step from q0 on (zero past the end)
         auto load = [&](int q0, uint64_t (&v)[2 * KS]) {
 #pragma unroll
             for (int k = 0; k < KS; ++k) {
                 const int q = q0 + 64 * k + 2 * lane;
                 uint64_t a = 0, b = 0;
-                if (vec && q + 1 < sp.cnt) {
+                if (vec && q + 1 < qe) {
                     const ulonglong2 u = __ldcs(reinterpret_cast<const ulonglong2 *>(src + q));
                     a = u.x;
                     b = u.y;
                 } else {
-                    if (q < sp.cnt) a = __ldcs(src + q);
-                    if (q + 1 < sp.cnt) b = __ldcs(src + q + 1);
+                    if (q < qe) a = __ldcs(src + q);
+                    if (q + 1 < qe) b = __ldcs(src + q + 1);
                 }
                 v[2 * k] = a;
                 v[2 * k + 1] = b;
@@ -135,7 +130,7 @@ __global__ void __launch_bounds__(AW * 32, 3) k_tile_aggs(const Params p, int T)
         auto step = [&](int q0, uint64_t w0, uint64_t w1) {
             const int q = q0 + 2 * lane;
             const unsigned h0 = (unsigned)(w0 >> 60), h1 = (unsigned)(w1 >> 60);
-            const bool p0 = h0 == 0xBu, p1 = h1 == 0xBu;   // zero past the tile: neither
+            const bool p0 = h0 == 0xBu, p1 = h1 == 0xBu;   // zero past the end: neither
             if (__all_sync(0xffffffffu, p0 && p1)) {
                 const long long r0 = pix_raw(w0), r1 = pix_raw(w1);
                 long long prev = __shfl_up_sync(0xffffffffu, r1, 1);
@@ -150,14 +145,14 @@ __global__ void __launch_bounds__(AW * 32, 3) k_tile_aggs(const Params p, int T)
                 c_pix += 2;
                 return;
             }
-            const bool in0 = q < sp.cnt, in1 = q + 1 < sp.cnt;
+            const bool in0 = q < qe, in1 = q + 1 < qe;
             const bool t0 = in0 && h0 == 0x6u, t1 = in1 && h1 == 0x6u;
             c_pix += (unsigned)p0 + (unsigned)p1;
             c_tdc += (unsigned)t0 + (unsigned)t1;
             c_bad += (unsigned)(in0 && !p0 && !t0) + (unsigned)(in1 && !p1 && !t1);
             const long long r0 = p0 ? pix_raw(w0) : 0, r1 = p1 ? pix_raw(w1) : 0;
             const unsigned mt = __ballot_sync(0xffffffffu, t0 || t1);
-            if (mt && first_tdc < 0) {   // the pixel chain up to the tile's first TDC packet
+            if (mt && first_tdc < 0) {   // the pixel chain up to the first TDC packet
                 const int fl = __ffs(mt) - 1;
                 first_tdc = __shfl_sync(0xffffffffu, t0 ? q : q + 1, fl);
                 ch = cp;
@@ -167,18 +162,22 @@ __global__ void __launch_bounds__(AW * 32, 3) k_tile_aggs(const Params p, int T)
             if (mt) warp_chain_step(ct, t0, t0 ? tdc_raw(w0) : 0, t1, t1 ? tdc_raw(w1) : 0, tt, lane);
         };
         uint64_t cur[2 * KS], nxt[2 * KS];
-        load(0, nxt);
-        for (int q0 = 0; q0 < sp.cnt; q0 += 64 * KS) {
+        load(qb, nxt);
+        for (int q0 = qb; q0 < qe; q0 += 64 * KS) {
 #pragma unroll
             for (int k = 0; k < 2 * KS; ++k) cur[k] = nxt[k];
-            if (q0 + 64 * KS < sp.cnt) load(q0 + 64 * KS, nxt);
+            if (q0 + 64 * KS < qe) load(q0 + 64 * KS, nxt);
 #pragma unroll
             for (int k = 0; k < KS; ++k)
-                if (q0 + 64 * k < sp.cnt) step(q0 + 64 * k, cur[2 * k], cur[2 * k + 1]);
+                if (q0 + 64 * k < qe) step(q0 + 64 * k, cur[2 * k], cur[2 * k + 1]);
         }
+    }
+    // the part's aggregates, the same in every lane: both chains, and the pixel
+    // chain up to the first TDC packet; wraps: whether a pixel wrap lies inside
+    __device__ __forceinline__ void result(GAgg *a, GChain *h) {
         long long sp_ = cp.sum, st_ = ct.sum, sh_ = ch.sum;
-        const bool any_wrap = __any_sync(0xffffffffu, wraps);
-        if (any_wrap || __any_sync(0xffffffffu, st_ != 0)) {
+        wraps = __any_sync(0xffffffffu, wraps);
+        if (wraps || __any_sync(0xffffffffu, st_ != 0)) {
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) {
                 sp_ += __shfl_xor_sync(0xffffffffu, sp_, o);
@@ -186,35 +185,59 @@ __global__ void __launch_bounds__(AW * 32, 3) k_tile_aggs(const Params p, int T)
                 sh_ += __shfl_xor_sync(0xffffffffu, sh_, o);
             }
         }
+        a->pix.n = cp.n; a->pix.first = cp.first; a->pix.last = cp.last; a->pix.sum = sp_;
+        a->tdc.n = ct.n; a->tdc.first = ct.first; a->tdc.last = ct.last; a->tdc.sum = st_;
+        if (!cp.any) a->pix = chain_id();
+        if (!ct.any) a->tdc = chain_id();
+        h->n = ch.n; h->first = ch.first; h->last = ch.last; h->sum = sh_;
+        if (!ch.any) *h = chain_id();
+    }
+    // packet-class counters of the call (Ctl is cleared before the launch)
+    __device__ __forceinline__ void count(Ctl *ctl, int lane) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            c_pix += __shfl_xor_sync(0xffffffffu, c_pix, o);
+            c_tdc += __shfl_xor_sync(0xffffffffu, c_tdc, o);
+            c_bad += __shfl_xor_sync(0xffffffffu, c_bad, o);
+        }
         if (lane == 0) {
-            GAgg a;
-            a.pix.n = cp.n; a.pix.first = cp.first; a.pix.last = cp.last; a.pix.sum = sp_;
-            a.tdc.n = ct.n; a.tdc.first = ct.first; a.tdc.last = ct.last; a.tdc.sum = st_;
-            if (!cp.any) a.pix = chain_id();
-            if (!ct.any) a.tdc = chain_id();
+            if (c_pix) atomicAdd(&ctl->counters[C_PIXELS], c_pix);
+            if (c_tdc) atomicAdd(&ctl->counters[C_TDCS], c_tdc);
+            if (c_bad) atomicAdd(&ctl->counters[C_CORRUPT], c_bad);
+        }
+    }
+};
+
+__global__ void __launch_bounds__(AW * 32, 3) k_tile_aggs(const Params p, int T) {
+    const int lane = threadIdx.x & 31;
+    const long long warp = (long long)blockIdx.x * AW + (threadIdx.x >> 5);
+    const long long nw = (long long)gridDim.x * AW;
+    unsigned long long c_pix = 0, c_tdc = 0, c_bad = 0;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {   // the fused kernel's last tile writes them
+        *p.n_clusters = 0;
+        *p.n_trig = 0;
+    }
+    for (long long tile = warp; tile < p.n_tiles; tile += nw) {
+        const TileSpan sp = tile_span(p, tile, T);
+        WarpPart<4> w;
+        w.c_pix = c_pix; w.c_tdc = c_tdc; w.c_bad = c_bad;
+        w.run(p.pk + sp.base, (sp.base & 1) == 0, 0, sp.cnt, p.thr_pix, p.thr_tdc, lane);
+        c_pix = w.c_pix; c_tdc = w.c_tdc; c_bad = w.c_bad;
+        GAgg a;
+        GChain h;
+        w.result(&a, &h);
+        if (lane == 0) {
             p.ts.agg[tile] = a;
-            GChain h;
-            h.n = ch.n; h.first = ch.first; h.last = ch.last; h.sum = sh_;
-            if (!ch.any) h = chain_id();
             p.ts.head[tile] = h;
             TileInfo ti;
-            ti.first_tdc = first_tdc;
-            ti.wrap = any_wrap ? 1 : 0;
+            ti.first_tdc = w.first_tdc;
+            ti.wrap = w.wraps ? 1 : 0;
             p.ts.tinfo[tile] = ti;
         }
     }
-    // packet-class counters of the call (Ctl is cleared before the launch)
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        c_pix += __shfl_xor_sync(0xffffffffu, c_pix, o);
-        c_tdc += __shfl_xor_sync(0xffffffffu, c_tdc, o);
-        c_bad += __shfl_xor_sync(0xffffffffu, c_bad, o);
-    }
-    if (lane == 0) {
-        if (c_pix) atomicAdd(&p.ctl->counters[C_PIXELS], c_pix);
-        if (c_tdc) atomicAdd(&p.ctl->counters[C_TDCS], c_tdc);
-        if (c_bad) atomicAdd(&p.ctl->counters[C_CORRUPT], c_bad);
-    }
+    WarpPart<4> w;
+    w.c_pix = c_pix; w.c_tdc = c_tdc; w.c_bad = c_bad;
+    w.count(p.ctl, lane);
 }
 
 // segmented combine: a run start (flag) discards what came before it
@@ -345,6 +368,117 @@ __global__ void __launch_bounds__(256) k_apply(const Params p, const GAgg *bpre)
     p.ts.pre[t] = e;
 }
 
+// Up to SB tiles (4 M packets): the whole pre-pass in one launch. A call of a
+// few tiles is bound by latency, not by bytes: with a warp per tile the 4096
+// packets of a tile are 64 dependent steps of one warp, and three launches
+// follow (37 shots, 5 tiles: 30 + 6 + 6 + 4 us; the whole call 112 us, with
+// this kernel and two memsets and a copy fewer 69 us; 1000 shots, 117 tiles:
+// 125 -> 82 us). Here a CTA takes a tile, its 32 warps two steps each; the
+// parts are combined by one warp. The CTA that
+// finishes last (a counter in the control block) scans the aggregates of all
+// tiles and writes the states; nobody waits for anybody.
+__device__ __forceinline__ GChain ldcg_chain(const GChain *c) {   // written by another CTA: past L1
+    GChain r;
+    r.n = __ldcg(&c->n); r.first = __ldcg(&c->first); r.last = __ldcg(&c->last); r.sum = __ldcg(&c->sum);
+    return r;
+}
+__global__ void __launch_bounds__(SB, 1) k_prepass_small(const Params p, int T) {
+    __shared__ GAgg s_a[32];
+    __shared__ GChain s_h[32];
+    __shared__ int s_first[32];
+    __shared__ bool s_wrap[32];
+    __shared__ SAgg s_w[32];
+    __shared__ SAgg s_tot;
+    __shared__ bool s_last;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const long long tp = p.thr_pix, tt = p.thr_tdc;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {   // the fused kernel's last tile writes them
+        *p.n_clusters = 0;
+        *p.n_trig = 0;
+    }
+    {
+        const long long tile = blockIdx.x;
+        const TileSpan sp = tile_span(p, tile, T);
+        const int per = T / 32;   // 64 or 128 packets: one or two steps
+        const int qb = w * per, qe = min(sp.cnt, qb + per);
+        WarpPart<2> part;
+        if (qb < qe) part.run(p.pk + sp.base, (sp.base & 1) == 0, qb, qe, tp, tt, lane);
+        GAgg a;
+        GChain h;
+        part.result(&a, &h);
+        part.count(p.ctl, lane);
+        if (lane == 0) {
+            s_a[w] = a;
+            s_h[w] = h;
+            s_first[w] = part.first_tdc;
+            s_wrap[w] = part.wraps;
+        }
+        __syncthreads();
+        if (w == 0) {   // the 32 parts in order
+            const GAgg mine = s_a[lane];
+            const GAgg incl = warp_incl_scan(mine, lane, tp, tt);
+            GAgg before = shfl_up_agg(incl, 1);
+            if (lane == 0) before = agg_id();
+            const bool step = before.pix.n && mine.pix.n && jump(mine.pix.first - before.pix.last, tp) != 0;
+            const bool wrap = __any_sync(0xffffffffu, step || s_wrap[lane]);
+            const unsigned has = __ballot_sync(0xffffffffu, s_first[lane] >= 0);
+            const int fl = has ? __ffs(has) - 1 : 0;
+            if (lane == fl) {
+                TileInfo ti;
+                ti.first_tdc = has ? s_first[lane] : -1;
+                ti.wrap = wrap ? 1 : 0;
+                p.ts.tinfo[tile] = ti;
+                p.ts.head[tile] = has ? ccomb(before.pix, s_h[lane], tp) : chain_id();
+            }
+            if (lane == 31) p.ts.agg[tile] = incl;
+            __threadfence();
+            __syncwarp();
+            if (lane == 0) s_last = atomicAdd(&p.ctl->prepass_done, 1u) + 1u == gridDim.x;
+        }
+    }
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    // the state before every tile (as k_block_scan, k_top_scan and k_apply)
+    const long long t = threadIdx.x;
+    if (p.n_tiles <= 32 && w > 0) return;
+    SAgg v = sid();
+    if (t < p.n_tiles) {
+        v.a.pix = ldcg_chain(&p.ts.agg[t].pix);
+        v.a.tdc = ldcg_chain(&p.ts.agg[t].tdc);
+        v.f = run_starts_at(p, t);
+    }
+    SAgg ex;
+    if (p.n_tiles <= 32) {
+        SAgg incl = v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const SAgg u = shfl_up_sagg(incl, o);
+            if (lane >= o) incl = scomb(u, incl, tp, tt);
+        }
+        ex = shfl_up_sagg(incl, 1);
+        if (lane == 0) ex = sid();
+    } else {
+        ex = block_excl_sagg(v, s_w, &s_tot, tp, tt);
+    }
+    if (t >= p.n_tiles) return;
+    const bool one = !p.bt.tile_run;
+    GAgg e = v.f ? agg_id() : (one && p.E0) ? acomb(*p.E0, ex.a, tp, tt) : ex.a;
+    if (t == p.n_tiles - 1 && one && p.state_out) *p.state_out = acomb(e, v.a, tp, tt);
+    TileInfo ti;
+    ti.first_tdc = __ldcg(&p.ts.tinfo[t].first_tdc);
+    ti.wrap = __ldcg(&p.ts.tinfo[t].wrap);
+    if (e.pix.n && v.a.pix.n && jump(v.a.pix.first - e.pix.last, tp) != 0) {   // the step into the tile's first pixel
+        ti.wrap = 1;
+        p.ts.tinfo[t] = ti;
+    }
+    const long long trig_base = (one && p.E0) ? p.E0->tdc.n : 0;
+    if (e.tdc.n > trig_base && ti.first_tdc >= 0) {
+        e.pix = ccomb(e.pix, ldcg_chain(p.ts.head + t), tp);
+    }
+    p.ts.pre[t] = e;
+}
+
 }  // namespace
 
 size_t unwrap_prepass_scratch_bytes(long long n_tiles) {
@@ -354,6 +488,10 @@ size_t unwrap_prepass_scratch_bytes(long long n_tiles) {
 
 cudaError_t launch_unwrap_prepass(const Params &p, int T, int grid, cudaStream_t s) {
     if (p.n_tiles <= 0) return cudaSuccess;
+    if (p.n_tiles <= SB) {
+        k_prepass_small<<<(unsigned)p.n_tiles, SB, 0, s>>>(p, T);
+        return cudaGetLastError();
+    }
     const long long nb = (p.n_tiles + SB - 1) / SB;
     GAgg *bagg = p.ts.blk;
     int *bflag = reinterpret_cast<int *>(bagg + nb + 1);

@@ -116,6 +116,8 @@ int grow(Tp **ptr, int64_t *cap, int64_t want) {
 
 namespace {
 
+constexpr size_t kCtlBytes = sizeof(tpxk::Ctl) + sizeof(unsigned);
+
 // A call's failure bits (a range the tiles could not hold, a batch run to
 // redo) are resolved by the tpx_sync after it. When a new call starts before
 // that sync, the previous call's bits move to the sticky word, and tpx_sync
@@ -249,14 +251,16 @@ int tpx_create(tpx_ctx **out, const tpx_config *cfg, int64_t max_packets, void *
         delete c;
         return TPX_ECUDA;
     }
-    if (cudaMalloc(&c->ctl, sizeof(tpxk::Ctl)) != cudaSuccess) { delete c; return TPX_ENOMEM; }
-    if (cudaMallocHost(&c->h_ctl, sizeof(tpxk::Ctl)) != cudaSuccess) {
+    // the control block and, behind it, the sticky word: one copy brings both down
+    if (cudaMalloc(&c->ctl, kCtlBytes) != cudaSuccess) { delete c; return TPX_ENOMEM; }
+    if (cudaMallocHost(&c->h_ctl, kCtlBytes) != cudaSuccess) {
         cudaFree(c->ctl);
         delete c;
         return TPX_ENOMEM;
     }
-    std::memset(c->h_ctl, 0, sizeof(tpxk::Ctl));
-    cudaMemset(c->ctl, 0, sizeof(tpxk::Ctl));
+    std::memset(c->h_ctl, 0, kCtlBytes);
+    cudaMemset(c->ctl, 0, kCtlBytes);
+    c->d_sticky = reinterpret_cast<unsigned *>(c->ctl + 1);
     if (cudaMalloc(&c->d_state, 2 * sizeof(tpxk::GAgg)) != cudaSuccess) {
         cudaFree(c->ctl);
         cudaFreeHost(c->h_ctl);
@@ -264,11 +268,6 @@ int tpx_create(tpx_ctx **out, const tpx_config *cfg, int64_t max_packets, void *
         return TPX_ENOMEM;
     }
     cudaMemset(c->d_state, 0, 2 * sizeof(tpxk::GAgg));   // all zero = the start of a stream
-    if (cudaMalloc(&c->d_sticky, sizeof(unsigned)) != cudaSuccess || cudaMemset(c->d_sticky, 0, sizeof(unsigned)) != cudaSuccess) {
-        cudaGetLastError();
-        tpx_destroy(c);
-        return TPX_ENOMEM;
-    }
     c->synced = true;
     for (auto &smp : c->tune.ring)
         if (cudaEventCreate(&smp.a) != cudaSuccess || cudaEventCreate(&smp.b) != cudaSuccess) {
@@ -312,7 +311,6 @@ int tpx_destroy(tpx_ctx *c) {
     if (c->st_counts) cudaFree(c->st_counts);
     if (c->g_mem) cudaFree(c->g_mem);
     if (c->d_state) cudaFree(c->d_state);
-    if (c->d_sticky) cudaFree(c->d_sticky);
     for (auto &smp : c->tune.ring) {
         if (smp.a) cudaEventDestroy(smp.a);
         if (smp.b) cudaEventDestroy(smp.b);
@@ -386,9 +384,9 @@ int tpx_process(tpx_ctx *c, const uint64_t *d_packets, int64_t n, int64_t idx_ba
     c->last.E0 = E0;
     c->last.state_out = state_out;
     if (ckr(cudaMemsetAsync(c->ctl, 0, sizeof(tpxk::Ctl), c->stream))) return TPX_ECUDA;
-    if (ckr(cudaMemsetAsync(d_n_clusters, 0, sizeof(int64_t), c->stream))) return TPX_ECUDA;
-    if (ckr(cudaMemsetAsync(d_n_trig, 0, sizeof(int64_t), c->stream))) return TPX_ECUDA;
     if (n == 0) {   // the state passes through unchanged
+        if (ckr(cudaMemsetAsync(d_n_clusters, 0, sizeof(int64_t), c->stream))) return TPX_ECUDA;
+        if (ckr(cudaMemsetAsync(d_n_trig, 0, sizeof(int64_t), c->stream))) return TPX_ECUDA;
         if (E0) return cudaMemcpyAsync(state_out, E0, sizeof(tpxk::GAgg), cudaMemcpyDeviceToDevice, c->stream)
                        == cudaSuccess ? TPX_OK : TPX_ECUDA;
         return cudaMemsetAsync(state_out, 0, sizeof(tpxk::GAgg), c->stream) == cudaSuccess ? TPX_OK : TPX_ECUDA;
@@ -699,13 +697,11 @@ int tpx_sync(tpx_ctx *c, tpx_counters *out) {
     int64_t redone = c->redone_early;
     c->redone_early = 0;
     c->synced = true;
-    unsigned sticky = 0;
-    if (ckr(cudaMemcpyAsync(&sticky, c->d_sticky, 4, cudaMemcpyDeviceToHost, c->stream)) ||
-        ckr(cudaMemsetAsync(c->d_sticky, 0, 4, c->stream)))
-        return TPX_ECUDA;
-    if (cudaMemcpyAsync(c->h_ctl, c->ctl, sizeof(tpxk::Ctl), cudaMemcpyDeviceToHost, c->stream) != cudaSuccess)
+    if (cudaMemcpyAsync(c->h_ctl, c->ctl, kCtlBytes, cudaMemcpyDeviceToHost, c->stream) != cudaSuccess)
         return TPX_ECUDA;
     if (ckr(cudaStreamSynchronize(c->stream))) return TPX_ECUDA;
+    const unsigned sticky = *reinterpret_cast<const unsigned *>(c->h_ctl + 1);
+    if (sticky && ckr(cudaMemsetAsync(c->d_sticky, 0, 4, c->stream))) return TPX_ECUDA;
     // a checked build's index violation stays reported even when the call is redone
     const unsigned bounds = c->h_ctl->status & tpxk::ST_BOUNDS;
     if ((c->h_ctl->status & (tpxk::ST_CAPACITY | tpxk::ST_EXCEPTION)) && !(c->h_ctl->status & tpxk::ST_DEVTIMEOUT) &&
