@@ -18,6 +18,7 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <atomic>
 
 #include <cmath>
@@ -53,75 +54,329 @@ inline unsigned grid_for(long long n, int bt = 256) {
 }
 
 // ---------------------------------------------------------------- patches
-__global__ void k_sel_flags(const tpx_record *cl, long long ncl, int min_px, unsigned *f) {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < ncl; i += (long long)gridDim.x * blockDim.x)
-        f[i] = cl[i].n > min_px ? 1u : 0u;
-}
-// exclusive scan in three steps: per-block sums, one block over them, add
-constexpr int SB = 1024;
-__global__ void k_scan_local(const unsigned *in, unsigned *out, long long n, unsigned *bsum) {
-    __shared__ unsigned s[SB];
-    const long long i = blockIdx.x * (long long)SB + threadIdx.x;
-    const unsigned v = i < n ? in[i] : 0u;
-    s[threadIdx.x] = v;
-    __syncthreads();
-    for (int o = 1; o < SB; o <<= 1) {
-        const unsigned u = threadIdx.x >= o ? s[threadIdx.x - o] : 0u;
-        __syncthreads();
-        s[threadIdx.x] += u;
-        __syncthreads();
+// Which clusters get a patch: counted per block of SELB records, then every
+// block places its own behind those of the blocks before it.
+constexpr int SELT = 256, SELW = SELT / 32, SELR = 2, SELB = SELT * SELR;
+constexpr int PT = 2048, PH = 1024, PTH = 512;   // packets of a tile, of its margins; threads of k_patch_tiles
+struct TileSel { unsigned first_inv, count; };   // the selected clusters whose root lies in a tile: 2^32 - 1 - the first, how many
+struct SelRoot { long long root, raw0; unsigned n; short cx, cy; };   // what k_patch_tiles needs of a selected cluster, in one load
+struct PatchInfo {               // read back once per call
+    unsigned long long n_sel;    // selected clusters
+    unsigned n_inc;              // patches the tiles could not complete (listed)
+    unsigned n_far;              // of those, the ones that the wider search could not either
+    unsigned odd;                // labels not strictly ascending, or outside the packets, or a centre off the sensor: no tiles
+    unsigned reserved;
+};
+__device__ __forceinline__ unsigned sel_flags(const tpx_record *cl, long long ncl, int min_px, unsigned (&m)[SELR],
+                                              unsigned *s_c, unsigned *total) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    unsigned c = 0;
+#pragma unroll
+    for (int j = 0; j < SELR; ++j) {
+        const long long i = blockIdx.x * (long long)SELB + w * (32 * SELR) + 32 * j + lane;
+        m[j] = __ballot_sync(0xffffffffu, i < ncl && cl[i].n > min_px);
+        c += __popc(m[j]);
     }
-    if (i < n) out[i] = s[threadIdx.x] - v;
-    if (threadIdx.x == SB - 1) bsum[blockIdx.x] = s[SB - 1];
-}
-// exclusive scan of the block sums by one block, SB at a time
-__global__ void k_scan_sums(unsigned *bsum, long long nb, long long *total) {
-    __shared__ unsigned s[SB];
-    __shared__ unsigned carry;
-    if (threadIdx.x == 0) carry = 0;
+    if (lane == 0) s_c[w] = c;
     __syncthreads();
-    for (long long b0 = 0; b0 < nb; b0 += SB) {
+    unsigned before = 0, all = 0;
+#pragma unroll
+    for (int k = 0; k < SELW; ++k) {
+        before += k < w ? s_c[k] : 0u;
+        all += s_c[k];
+    }
+    *total = all;
+    return before;
+}
+__global__ void __launch_bounds__(SELT) k_sel_count(const tpx_record *cl, long long ncl, int min_px, unsigned *bcnt) {
+    __shared__ unsigned s_c[SELW];
+    unsigned m[SELR], total;
+    (void)sel_flags(cl, ncl, min_px, m, s_c, &total);
+    if (threadIdx.x == 0) bcnt[blockIdx.x] = total;
+}
+// every block's first slot, beyond kResumBlocks blocks (one block)
+constexpr long long kResumBlocks = 4096;
+__global__ void __launch_bounds__(1024) k_sel_scan(unsigned *bcnt, long long nb) {
+    __shared__ unsigned s[1024];
+    unsigned carry = 0;
+    for (long long b0 = 0; b0 < nb; b0 += 1024) {
         const long long b = b0 + threadIdx.x;
-        const unsigned v = b < nb ? bsum[b] : 0u;
+        const unsigned v = b < nb ? bcnt[b] : 0u;
         s[threadIdx.x] = v;
         __syncthreads();
-        for (int o = 1; o < SB; o <<= 1) {
+        for (int o = 1; o < 1024; o <<= 1) {
             const unsigned u = threadIdx.x >= o ? s[threadIdx.x - o] : 0u;
             __syncthreads();
             s[threadIdx.x] += u;
             __syncthreads();
         }
-        if (b < nb) bsum[b] = carry + s[threadIdx.x] - v;
-        __syncthreads();
-        if (threadIdx.x == SB - 1) carry += s[SB - 1];
+        if (b < nb) bcnt[b] = carry + s[threadIdx.x] - v;
+        carry += s[1023];
         __syncthreads();
     }
-    if (threadIdx.x == 0) *total = carry;
 }
-__global__ void k_scan_add(unsigned *out, long long n, const unsigned *bsum) {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        out[i] += bsum[i / SB];
-}
-__global__ void k_select(const uint64_t *pk, const tpx_record *cl, long long ncl, const unsigned *f, const unsigned *off,
-                         long long cap, long long base, long long n, long long *sel, int *centre, int *slot_of_root) {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < ncl; i += (long long)gridDim.x * blockDim.x) {
-        if (!f[i]) continue;
-        const long long s = off[i];
+__global__ void __launch_bounds__(SELT) k_select(const uint64_t *pk, const tpx_record *cl, long long ncl, int min_px,
+                                                 const unsigned *bcnt, long long nb, long long cap, long long base,
+                                                 long long n, long long *sel, int *centre, long long *n_patches,
+                                                 TileSel *tiles, SelRoot *roots, PatchInfo *info) {
+    __shared__ unsigned s_c[SELW];
+    __shared__ unsigned s_sum[SELW];
+    unsigned m[SELR], total;
+    unsigned o = sel_flags(cl, ncl, min_px, m, s_c, &total);
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    unsigned first = 0;
+    if (nb > kResumBlocks) first = bcnt[blockIdx.x];
+    else {
+        unsigned v = 0;
+        for (unsigned k = threadIdx.x; k < blockIdx.x; k += SELT) v += bcnt[k];
+        v = __reduce_add_sync(0xffffffffu, v);
+        if (lane == 0) s_sum[w] = v;
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < SELW; ++k) first += s_sum[k];
+    }
+#pragma unroll
+    for (int j = 0; j < SELR; ++j) {
+        const long long i = blockIdx.x * (long long)SELB + w * (32 * SELR) + 32 * j + lane;
+        const long long s = (long long)first + o + __popc(m[j] & ((1u << lane) - 1u));
+        o += __popc(m[j]);
+        if (i < ncl && i > 0 && cl[i - 1].label >= cl[i].label) info->odd = 1u;
+        if (!((m[j] >> lane) & 1u)) continue;
+        const tpx_record &c = cl[i];
+        const long long r = c.label - base;
+        if (r < 0 || r >= n) info->odd = 1u;
         if (s >= cap) continue;
         sel[s] = i;
-        const long long r = cl[i].label - base;
-        const tpx_record &c = cl[i];
+        if (r >= 0 && r < n) {
+            atomicMax(&tiles[r / PT].first_inv, 0xFFFFFFFFu - (unsigned)s);
+            atomicAdd(&tiles[r / PT].count, 1u);
+        }
         int cx = 0, cy = 0;
         if (c.s_tot > 0) {   // the centroid rounded half up, exactly: floor((2 s_x + s_tot) / (2 s_tot))
-            cx = (int)((2 * c.s_x + c.s_tot) / (2 * c.s_tot));
-            cy = (int)((2 * c.s_y + c.s_tot) / (2 * c.s_tot));
+            const long long d = 2 * c.s_tot, nx = 2 * c.s_x + c.s_tot, ny = 2 * c.s_y + c.s_tot;
+            if (((unsigned long long)nx | (unsigned long long)ny | (unsigned long long)d) >> 32) {
+                cx = (int)(nx / d);
+                cy = (int)(ny / d);
+            } else {   // the usual cluster: 32-bit divisions
+                cx = (int)((unsigned)nx / (unsigned)d);
+                cy = (int)((unsigned)ny / (unsigned)d);
+            }
         } else if (r >= 0 && r < n) {   // no charge: the earliest pixel
             cx = pix_x(pk[r]);
             cy = pix_y(pk[r]);
         }
         centre[2 * s] = cx;
         centre[2 * s + 1] = cy;
-        if (r >= 0 && r < n) slot_of_root[r] = (int)s;   // else not a record of these packets: an empty patch
+        if ((unsigned)cx > 255u || (unsigned)cy > 255u) info->odd = 1u;
+        SelRoot v;
+        v.root = r;
+        v.raw0 = r >= 0 && r < n ? pix_raw(pk[r]) : 0;
+        v.n = (unsigned)c.n;
+        v.cx = (short)cx;   // within the sensor: a centroid
+        v.cy = (short)cy;
+        roots[s] = v;
+    }
+    if (blockIdx.x == nb - 1 && threadIdx.x == 0) {
+        *n_patches = (long long)first + total;
+        info->n_sel = (unsigned long long)first + total;
+    }
+}
+
+// a pixel's two patch values. Channel 0: ToT / 1023 rounded to bf16; channel 1:
+// ToA relative to the cluster's earliest pixel, in units of 32 ticks (50 ns),
+// clamped to [-8, 8], rounded to fp16 (exact: multiples of 1/32 below 8); both
+// are exact in bf16 as well
+__device__ __forceinline__ float patch_tot(int tot) { return __bfloat162float(__float2bfloat16_rn((float)tot / 1023.f)); }
+// (the ticks already clamped to 256 = 8 units either way)
+__device__ __forceinline__ float patch_rel(int ticks) { return __half2float(__float2half_rn((float)ticks / 32.f)); }
+// elements e and e + 1 of a patch row
+// (one store where the caller's buffer is aligned to the pair)
+__device__ __forceinline__ void put_pair(float *row, int e, float a, float b) {
+    if (reinterpret_cast<uintptr_t>(row) & 7) {
+        row[e] = a;
+        row[e + 1] = b;
+    } else {
+        *reinterpret_cast<float2 *>(row + e) = make_float2(a, b);
+    }
+}
+__device__ __forceinline__ void put_pair(uint16_t *row, int e, float a, float b) {
+    const __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
+    if (reinterpret_cast<uintptr_t>(row) & 3) {
+        reinterpret_cast<__nv_bfloat16 *>(row)[e] = v.x;
+        reinterpret_cast<__nv_bfloat16 *>(row)[e + 1] = v.y;
+    } else {
+        *reinterpret_cast<__nv_bfloat162 *>(row + e) = v;
+    }
+}
+
+// A cluster's packets lie close to one another in the stream (within its shot's
+// readout), so a CTA takes the clusters whose earliest pixel is among PT
+// packets, with their cells in shared memory, and looks for their members
+// there and in PH packets on either side; a patch whose members all turned up
+// (the record's count) is written at once, the others are listed for the
+// kernels below. A cell's word holds all that its values follow from: ToT, the
+// packet's place in the window (the brighter pixel wins, ties go to the later)
+// and the clamped time, never zero. Bound by latency, so every thread's loads
+// of a step are in flight together; the bytes are the labels (twice, mostly
+// from L2) and the patches. Before, every cell had an 8-byte key in global
+// memory, cleared, updated and read back: 300 us of the 460 of a call of
+// 440,000 patches; now 134 of 300.
+constexpr int PMAX = 96;                         // clusters a pass holds (2048 packets of 24-pixel clusters: 85)
+constexpr int PWIN = PT + 2 * PH, PU = PWIN / PTH;
+static_assert(PWIN <= 4096, "the window position has 12 bits");
+constexpr int kRelMax = 256;                     // 8 units of 32 ticks
+__device__ __forceinline__ int rel_ticks(long long raw, long long raw0) {
+    long long d = (raw - raw0) & (kPixPeriod - 1);
+    if (d >= kPixPeriod / 2) d -= kPixPeriod;   // the signed difference, wrap-safe
+    return (int)min((long long)kRelMax, max(-(long long)kRelMax, d));
+}
+__device__ __forceinline__ unsigned cell_word(int tot, unsigned at, int rel) {
+    return ((unsigned)tot << 22) | (at << 10) | (unsigned)(rel + kRelMax + 1);
+}
+template <typename OutT>
+__device__ __forceinline__ void write_patch(OutT *row, const unsigned *key, int lane) {
+#pragma unroll
+    for (int e = 2 * lane; e < NIN; e += 64) {
+        float v[2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const bool t = e + u < PC;
+            const unsigned x = key[t ? e + u : e + u - PC];
+            v[u] = x == 0u ? 0.f : t ? patch_tot((int)(x >> 22)) : patch_rel((int)(x & 1023u) - kRelMax - 1);
+        }
+        put_pair(row, e, v[0], v[1]);
+    }
+}
+template <typename OutT>
+__global__ void __launch_bounds__(PTH, 3) k_patch_tiles(const uint64_t *pk, long long n, long long base,
+                                                        const long long *labels, const SelRoot *roots,
+                                                        const TileSel *tiles, OutT *patch, unsigned *inc,
+                                                        PatchInfo *info) {
+    __shared__ unsigned s_key[PMAX * PC];
+    __shared__ __align__(4) unsigned char s_slot[PT];   // of each packet of the tile: its cluster's place in this pass + 1
+    __shared__ int s_c[PMAX];                           // the centre, x | y << 16
+    __shared__ unsigned s_cnt[PMAX], s_n[PMAX];
+    __shared__ long long s_raw0[PMAX];
+    static_assert(PMAX < 255 && sizeof(s_key) + PT + 24 * PMAX < 48 * 1024, "shared memory of a pass");
+    const long long a = blockIdx.x * (long long)PT, w0 = a - PH;
+    const int tile_n = (int)min((long long)PT, n - a);
+    int L[PU];                                   // the window's labels: root - a where the root is in this tile, else -1
+#pragma unroll
+    for (int u = 0; u < PU; ++u) {
+        const long long q = w0 + u * PTH + threadIdx.x;
+        const long long lab = q >= 0 && q < n ? labels[q] : -1ll;
+        const long long r = lab - base - a;
+        L[u] = lab >= 0 && r >= 0 && r < tile_n ? (int)r : -1;
+    }
+    // the selected clusters of the tile: labels ascend, so they are consecutive
+    const TileSel ts = tiles[blockIdx.x];
+    if (!ts.count || info->odd) return;
+    const long long s0 = 0xFFFFFFFFu - ts.first_inv, s1 = s0 + ts.count;
+    for (long long p0 = s0; p0 < s1; p0 += PMAX) {
+        const int m = (int)min((long long)PMAX, s1 - p0);
+        SelRoot v;
+        if (threadIdx.x < m) v = roots[p0 + threadIdx.x];
+        __syncthreads();
+        for (int k = threadIdx.x; k < PT / 4; k += PTH) reinterpret_cast<unsigned *>(s_slot)[k] = 0u;
+        for (int k = threadIdx.x; k < m * PC; k += PTH) s_key[k] = 0u;
+        __syncthreads();
+        if (threadIdx.x < m) {
+            s_slot[v.root - a] = (unsigned char)(threadIdx.x + 1);
+            s_n[threadIdx.x] = v.n;
+            s_raw0[threadIdx.x] = v.raw0;
+            s_c[threadIdx.x] = (int)(unsigned short)v.cx | ((int)v.cy << 16);
+            s_cnt[threadIdx.x] = 0u;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int h = 0; h < PU; h += PU / 2) {   // half of the window's packets in flight together
+            int k[PU / 2];
+            uint64_t w[PU / 2];
+#pragma unroll
+            for (int u = 0; u < PU / 2; ++u) {
+                k[u] = L[h + u] >= 0 ? (int)s_slot[L[h + u]] - 1 : -1;
+                w[u] = k[u] >= 0 ? pk[w0 + (h + u) * PTH + threadIdx.x] : 0ull;
+            }
+#pragma unroll
+            for (int u = 0; u < PU / 2; ++u) {
+                if (k[u] < 0) continue;
+                atomicAdd(&s_cnt[k[u]], 1u);
+                const int c = s_c[k[u]];
+                const int dx = pix_x(w[u]) - (c & 0xFFFF) + PS / 2, dy = pix_y(w[u]) - (c >> 16) + PS / 2;
+                if (dx < 0 || dx >= PS || dy < 0 || dy >= PS) continue;
+                atomicMax(&s_key[k[u] * PC + dy * PS + dx],
+                          cell_word(pix_tot(w[u]), (unsigned)((h + u) * PTH + threadIdx.x), rel_ticks(pix_raw(w[u]), s_raw0[k[u]])));
+            }
+        }
+        __syncthreads();
+        const int lane = threadIdx.x & 31;
+        for (int j = threadIdx.x >> 5; j < m; j += PTH / 32) {
+            if (s_cnt[j] != s_n[j]) {
+                if (lane == 0) inc[atomicAdd(&info->n_inc, 1u)] = (unsigned)(p0 + j);
+                continue;
+            }
+            write_patch(patch + (p0 + j) * (long long)NIN, s_key + j * PC, lane);
+        }
+    }
+}
+
+// The listed patches with a wider search, a CTA each: PW packets on either side
+// of the root. (50 particles a shot: a shot's readout is longer than PH.) What
+// is still incomplete goes on to the second list.
+constexpr int PW = 16384, PWT = 256;
+template <typename OutT>
+__global__ void __launch_bounds__(PWT) k_patch_wide(const uint64_t *pk, long long n, long long base, const long long *labels,
+                                                    const tpx_record *cl, const long long *sel, const int *centre,
+                                                    const unsigned *inc, OutT *patch, unsigned *far, PatchInfo *info) {
+    __shared__ unsigned long long s_key[PC];     // ToT + 1, place in the window, time (as cell_word, more bits)
+    __shared__ unsigned s_word[PC];
+    __shared__ unsigned s_cnt;
+    const unsigned ni = info->n_inc;
+    for (unsigned j = blockIdx.x; j < ni; j += gridDim.x) {
+        const long long s = inc[j];
+        const tpx_record &c = cl[sel[s]];
+        const long long root = c.label - base, w0 = max(0ll, root - PW), w1 = min(n, root + PW);
+        const long long raw0 = pix_raw(pk[root]);
+        const int cx = centre[2 * s], cy = centre[2 * s + 1];
+        __syncthreads();
+        if (threadIdx.x < PC) s_key[threadIdx.x] = 0ull;
+        if (threadIdx.x == 0) s_cnt = 0u;
+        __syncthreads();
+#pragma unroll 8
+        for (long long q = w0 + threadIdx.x; q < w1; q += PWT) {
+            if (labels[q] != c.label) continue;
+            atomicAdd(&s_cnt, 1u);
+            const uint64_t w = pk[q];
+            const int dx = pix_x(w) - cx + PS / 2, dy = pix_y(w) - cy + PS / 2;
+            if (dx < 0 || dx >= PS || dy < 0 || dy >= PS) continue;
+            atomicMax(&s_key[dy * PS + dx], ((unsigned long long)pix_tot(w) << 42) | ((unsigned long long)(q - w0) << 10) |
+                                                (unsigned long long)(rel_ticks(pix_raw(w), raw0) + kRelMax + 1));
+        }
+        __syncthreads();
+        if (s_cnt != (unsigned)c.n) {
+            if (threadIdx.x == 0) far[atomicAdd(&info->n_far, 1u)] = (unsigned)s;
+            continue;
+        }
+        if (threadIdx.x < PC) {
+            const unsigned long long x = s_key[threadIdx.x];
+            s_word[threadIdx.x] = (unsigned)(x >> 42 << 22) | (unsigned)(x & 1023u);
+        }
+        __syncthreads();
+        if (threadIdx.x < 32) write_patch(patch + s * (long long)NIN, s_word, (int)threadIdx.x);
+    }
+}
+
+// ---- patches the tiles could not complete: member packets anywhere ----
+// the list of all patches (odd calls)
+__global__ void k_list_all(unsigned *inc, long long ns) {
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < ns; i += (long long)gridDim.x * blockDim.x) inc[i] = (unsigned)i;
+}
+// the listed patch of each root packet
+__global__ void k_roots(const tpx_record *cl, const long long *sel, const unsigned *inc, long long ni, long long base,
+                        long long n, int *slot_of_root) {
+    for (long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x; j < ni; j += (long long)gridDim.x * blockDim.x) {
+        const long long r = cl[sel[inc[j]]].label - base;
+        if (r >= 0 && r < n) slot_of_root[r] = (int)j;   // else not a record of these packets: an empty patch
     }
 }
 __global__ void k_fill_i32(int *p, long long n, int v) {
@@ -129,47 +384,39 @@ __global__ void k_fill_i32(int *p, long long n, int v) {
 }
 // the brighter pixel of a shared cell wins (ties: the later one)
 __global__ void k_patch_keys(const uint64_t *pk, long long n, long long base, const long long *labels,
-                             const int *slot_of_root, const int *centre, unsigned long long *key) {
+                             const int *slot_of_root, const unsigned *inc, const int *centre, unsigned long long *key) {
     for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < n; q += (long long)gridDim.x * blockDim.x) {
         const long long L = labels[q] - base;
         if (labels[q] < 0 || L < 0 || L >= n) continue;
-        const int s = slot_of_root[L];
-        if (s < 0) continue;
+        const int j = slot_of_root[L];
+        if (j < 0) continue;
+        const long long s = inc[j];
         const uint64_t w = pk[q];
         const int dx = pix_x(w) - centre[2 * s] + PS / 2, dy = pix_y(w) - centre[2 * s + 1] + PS / 2;
         if (dx < 0 || dx >= PS || dy < 0 || dy >= PS) continue;
         const unsigned long long k = ((unsigned long long)(pix_tot(w) + 1) << 40) | (unsigned long long)q;
-        atomicMax(&key[(long long)s * PC + dy * PS + dx], k);
+        atomicMax(&key[(long long)j * PC + dy * PS + dx], k);
     }
 }
-// channel 0: ToT / 1023 rounded to bf16; channel 1: ToA relative to the
-// cluster's earliest pixel, in units of 32 ticks (50 ns), clamped to [-8, 8],
-// rounded to fp16 (exact: multiples of 1/32 below 8); empty cells 0
+// empty cells 0
 template <typename OutT>
 __global__ void k_patch_fill(const uint64_t *pk, long long base, const tpx_record *cl, const long long *sel,
-                             const unsigned long long *key, long long ns, OutT *patch) {
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < ns * PC; c += (long long)gridDim.x * blockDim.x) {
-        const long long s = c / PC;
-        const int cell = (int)(c % PC);
-        float tot = 0.f, rel = 0.f;
-        const unsigned long long k = key[c];
-        if (k) {
+                             const unsigned *inc, const unsigned long long *key, long long ni, OutT *patch) {
+    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < ni * PC; c += (long long)gridDim.x * blockDim.x) {
+        const long long j = c / PC, s = inc[j];
+        const int e = 2 * (int)(c - j * PC);   // elements e, e + 1 of the row
+        float v[2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const bool t = e + u < PC;
+            const unsigned long long k = key[j * PC + (t ? e + u : e + u - PC)];
+            v[u] = 0.f;
+            if (k == 0) continue;
             const long long q = (long long)(k & ((1ull << 40) - 1));
-            const uint64_t w = pk[q];
-            const uint64_t w0 = pk[cl[sel[s]].label - base];   // in range: the key came from this cluster
-            long long d = (pix_raw(w) - pix_raw(w0)) & (kPixPeriod - 1);
-            if (d >= kPixPeriod / 2) d -= kPixPeriod;   // the signed difference, wrap-safe
-            // the patch precisions: ToT in bf16, relative ToA in fp16 (held widened to fp32)
-            tot = __bfloat162float(__float2bfloat16_rn((float)pix_tot(w) / 1023.f));
-            rel = __half2float(__float2half_rn(fminf(8.f, fmaxf(-8.f, (float)d / 32.f))));
+            // the root packet is in range: the key came from this cluster
+            v[u] = t ? patch_tot(pix_tot(pk[q])) : patch_rel(rel_ticks(pix_raw(pk[q]), pix_raw(pk[cl[sel[s]].label - base])));
         }
-        if (sizeof(OutT) == 4) {
-            patch[s * NIN + cell] = tot;
-            patch[s * NIN + PC + cell] = rel;
-        } else {   // exact in bf16 as well
-            reinterpret_cast<__nv_bfloat16 *>(patch)[s * NIN + cell] = __float2bfloat16_rn(tot);
-            reinterpret_cast<__nv_bfloat16 *>(patch)[s * NIN + PC + cell] = __float2bfloat16_rn(rel);
-        }
+        put_pair(patch + s * NIN, e, v[0], v[1]);
     }
 }
 
@@ -547,36 +794,50 @@ static int refine_patches(tpx_ctx *c, const uint64_t *d_packets, int64_t n, int6
     cudaStream_t s = c->stream;
     if (ck(cudaMemsetAsync(d_n_patches, 0, 8, s))) return TPX_ECUDA;
     if (n_clusters == 0 || n == 0) return TPX_OK;
-    // scratch: flags, offsets, block sums, slot of each root packet, cell keys
-    const long long nb = (n_clusters + SB - 1) / SB;
+    // scratch: block counts, the list of incomplete patches; for those the
+    // patch of each root packet and the cell keys
+    const long long nb = (n_clusters + SELB - 1) / SELB;
     auto al = [](size_t b) { return (b + 255) & ~size_t(255); };
-    const size_t need = 2 * al(4 * (size_t)n_clusters) + al(4 * (size_t)nb) + al(4 * (size_t)n) +
+    const long long nt = (n + PT - 1) / PT;
+    const size_t b_info = al(sizeof(PatchInfo)) + al(sizeof(TileSel) * (size_t)nt);
+    const size_t need = b_info + al(4 * (size_t)nb) + 2 * al(4 * (size_t)capacity + 4) +
+                        al(sizeof(SelRoot) * (size_t)capacity) + al(4 * (size_t)n) +
                         al(8 * (size_t)capacity * PC + 8);
     int rc = tpxg::reserve(c, need);
     if (rc) return rc;
     char *m = static_cast<char *>(c->g_mem);
-    unsigned *f = reinterpret_cast<unsigned *>(m); m += al(4 * (size_t)n_clusters);
-    unsigned *off = reinterpret_cast<unsigned *>(m); m += al(4 * (size_t)n_clusters);
-    unsigned *bsum = reinterpret_cast<unsigned *>(m); m += al(4 * (size_t)nb);
+    PatchInfo *info = reinterpret_cast<PatchInfo *>(m); m += al(sizeof(PatchInfo));
+    TileSel *tiles = reinterpret_cast<TileSel *>(m); m += al(sizeof(TileSel) * (size_t)nt);
+    unsigned *bcnt = reinterpret_cast<unsigned *>(m); m += al(4 * (size_t)nb);
+    unsigned *inc = reinterpret_cast<unsigned *>(m); m += al(4 * (size_t)capacity + 4);
+    unsigned *far = reinterpret_cast<unsigned *>(m); m += al(4 * (size_t)capacity + 4);
+    SelRoot *roots = reinterpret_cast<SelRoot *>(m); m += al(sizeof(SelRoot) * (size_t)capacity);
     int *slot = reinterpret_cast<int *>(m); m += al(4 * (size_t)n);
     unsigned long long *key = reinterpret_cast<unsigned long long *>(m);
-    k_sel_flags<<<grid_for(n_clusters), 256, 0, s>>>(d_clusters, n_clusters, min_pixels, f);
-    k_scan_local<<<(unsigned)nb, SB, 0, s>>>(f, off, n_clusters, bsum);
-    k_scan_sums<<<1, SB, 0, s>>>(bsum, nb, reinterpret_cast<long long *>(d_n_patches));
-    k_scan_add<<<grid_for(n_clusters), 256, 0, s>>>(off, n_clusters, bsum);
-    k_fill_i32<<<grid_for(n), 256, 0, s>>>(slot, n, -1);
-    long long np = 0;
-    if (ck(cudaMemcpyAsync(&np, d_n_patches, 8, cudaMemcpyDeviceToHost, s)) || ck(cudaStreamSynchronize(s)))
-        return TPX_ECUDA;
-    const long long ns = np < capacity ? np : capacity;
-    k_select<<<grid_for(n_clusters), 256, 0, s>>>(d_packets, d_clusters, n_clusters, f, off, capacity, base, n,
-                                                  reinterpret_cast<long long *>(d_sel), d_centre, slot);
-    if (ns == 0) return ck(cudaGetLastError()) ? TPX_ECUDA : TPX_OK;
-    if (ck(cudaMemsetAsync(key, 0, 8 * (size_t)ns * PC, s))) return TPX_ECUDA;
-    k_patch_keys<<<grid_for(n), 256, 0, s>>>(d_packets, n, base, reinterpret_cast<const long long *>(d_labels), slot,
-                                             d_centre, key);
-    k_patch_fill<OutT><<<grid_for(ns * PC), 256, 0, s>>>(d_packets, base, d_clusters,
-                                                         reinterpret_cast<const long long *>(d_sel), key, ns, d_patches);
+    const long long *lab = reinterpret_cast<const long long *>(d_labels);
+    long long *sel = reinterpret_cast<long long *>(d_sel);
+    if (ck(cudaMemsetAsync(info, 0, b_info, s))) return TPX_ECUDA;
+    k_sel_count<<<(unsigned)nb, SELT, 0, s>>>(d_clusters, n_clusters, min_pixels, bcnt);
+    if (nb > kResumBlocks) k_sel_scan<<<1, 1024, 0, s>>>(bcnt, nb);
+    k_select<<<(unsigned)nb, SELT, 0, s>>>(d_packets, d_clusters, n_clusters, min_pixels, bcnt, nb, capacity, base, n, sel,
+                                           d_centre, reinterpret_cast<long long *>(d_n_patches), tiles, roots, info);
+    if (capacity > 0) {
+        k_patch_tiles<OutT><<<(unsigned)nt, PTH, 0, s>>>(d_packets, n, base, lab, roots, tiles, d_patches, inc, info);
+        k_patch_wide<OutT><<<c->num_sms * 4, PWT, 0, s>>>(d_packets, n, base, lab, d_clusters, sel, d_centre, inc, d_patches,
+                                                          far, info);
+    }
+    PatchInfo h{};
+    if (ck(cudaMemcpyAsync(&h, info, sizeof h, cudaMemcpyDeviceToHost, s)) || ck(cudaStreamSynchronize(s))) return TPX_ECUDA;
+    const long long np = (long long)h.n_sel, ns = np < capacity ? np : capacity;
+    const long long ni = h.odd ? ns : (long long)h.n_far;
+    if (ni > 0) {
+        if (h.odd) k_list_all<<<grid_for(ns), 256, 0, s>>>(far, ns);
+        k_fill_i32<<<grid_for(n), 256, 0, s>>>(slot, n, -1);
+        k_roots<<<grid_for(ni), 256, 0, s>>>(d_clusters, sel, far, ni, base, n, slot);
+        if (ck(cudaMemsetAsync(key, 0, 8 * (size_t)ni * PC, s))) return TPX_ECUDA;
+        k_patch_keys<<<grid_for(n), 256, 0, s>>>(d_packets, n, base, lab, slot, far, d_centre, key);
+        k_patch_fill<OutT><<<grid_for(ni * PC), 256, 0, s>>>(d_packets, base, d_clusters, sel, far, key, ni, d_patches);
+    }
     if (ck(cudaGetLastError())) return TPX_ECUDA;
     return np > capacity ? TPX_EOVERFLOW : TPX_OK;
 }
