@@ -566,7 +566,7 @@ __global__ void k_decide(const float *out, const tpx_record *cl, const long long
 
 // ---------------------------------------------------------------- bf16 inference
 // The whole network in one persistent kernel on the tensor cores
-// (mma.sync m16n8k16, bf16 operands, fp32 accumulation). Each warp owns 16
+// (mma.sync m16n8k16, bf16 operands, fp32 accumulation). Each warp owns 16 MT
 // patches and carries them through the three layers: the fp32 accumulator
 // fragment of one layer, after bias and ReLU, is exactly the bf16 A-operand
 // fragment of the next (row g = lane / 4 and column pair 2 (lane % 4) of
@@ -641,18 +641,42 @@ __device__ __forceinline__ void to_frags(const float (&acc)[NT][4], uint32_t (&a
         a[s][3] = pack_bf16(fmaxf(acc[2 * s + 1][2], 0.f), fmaxf(acc[2 * s + 1][3], 0.f));
     }
 }
+// the weight fragments of two n-tiles for one k-step: b[0], b[1] of the first,
+// b[2], b[3] of the second
+__device__ __forceinline__ void load_b2(uint32_t addr, uint32_t (&b)[4]) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(b[0]), "=r"(b[1]), "=r"(b[2]), "=r"(b[3]) : "r"(addr));
+}
 
-template <int H>
+// What bounds it: reading the weights from shared memory (every warp reads all
+// of them for its rows) and the latency of the patch loads. With MT = 2 a
+// weight fragment serves 32 rows; layer 2 runs in two halves of its outputs,
+// each at once taken into layer 3, so that the accumulators fit the registers;
+// a CTA's next rows are prefetched into L2 a tile ahead. 1,000,003 rows of width
+// 160: 326 -> 272 us (2.9 cycles per m16n8k16 and SM). Every accumulator sees
+// the same products in the same order as with MT = 1, so the outputs are equal.
+template <int H, int MT>
 __global__ void __launch_bounds__(256, 1) k_mlp_bf16(const float *__restrict__ x, long long n,
                                                       const uint16_t *__restrict__ wt, const float *__restrict__ bias,
                                                       float *__restrict__ out) {
     using G = MlpGeo<H>;
-    constexpr int NT = G::NT, S2 = G::S2;
+    constexpr int NT = G::NT, S2 = G::S2, NH = NT / 2, ROWS = 128 * MT, K1 = K1P / 16;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     uint16_t *W1s = reinterpret_cast<uint16_t *>(smem_raw);
     uint16_t *W2s = W1s + H * S1;
     uint16_t *W3s = W2s + H * S2;
     float *Bs = reinterpret_cast<float *>(W3s + 8 * S2);
+    const long long n_tiles = (n + ROWS - 1) / ROWS;
+    // the whole 16-byte words of tile t's rows, into L2
+    auto prefetch = [&](long long t) {
+        if (threadIdx.x != 0 || t >= n_tiles) return;
+        const char *a = reinterpret_cast<const char *>(x + t * ROWS * NIN);
+        const char *b = reinterpret_cast<const char *>(x + min(n, (t + 1) * (long long)ROWS) * NIN);
+        a += (16 - (reinterpret_cast<uintptr_t>(a) & 15)) & 15;
+        const long long bytes = (b - a) & ~15ll;
+        if (bytes > 0) asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a), "r"((unsigned)bytes) : "memory");
+    };
+    prefetch(blockIdx.x);
     // weights into shared memory, 16 bytes at a time (rows are 16-byte multiples)
     for (int i = threadIdx.x; i < H * (K1P / 8); i += blockDim.x) {
         const int r = i / (K1P / 8), c = i % (K1P / 8);
@@ -671,69 +695,114 @@ __global__ void __launch_bounds__(256, 1) k_mlp_bf16(const float *__restrict__ x
 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int g = lane >> 2, t = lane & 3;
-    const long long n_tiles = (n + 127) / 128;
+    // the lane's row for ldmatrix: n = lane % 8 (+ 8 for the second n-tile), k = 8 for odd groups of 8 lanes
+    const int br = (lane & 7) + ((lane >> 4) << 3), bk = ((lane >> 3) & 1) * 8;
+    const uint32_t w1a = (uint32_t)__cvta_generic_to_shared(W1s + br * S1 + bk);
+    const uint32_t w2a = (uint32_t)__cvta_generic_to_shared(W2s + br * S2 + bk);
     for (long long tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
-        const long long r0 = tile * 128 + warp * 16 + g, r1 = r0 + 8;
-        const float *x0 = x + r0 * NIN, *x1 = x + r1 * NIN;
-        const bool v0 = r0 < n, v1 = r1 < n;
-        // layer 1: acc = b1 + x W1
-        float acc[NT][4];
+        prefetch(tile + gridDim.x);
+        const long long r0 = tile * ROWS + warp * (16 * MT) + g;   // rows r0 + 16 m and r0 + 16 m + 8
+        const float *xr[MT];
+        bool v0[MT], v1[MT];
 #pragma unroll
-        for (int j = 0; j < NT; ++j) {
-            acc[j][0] = acc[j][2] = Bs[8 * j + 2 * t];
-            acc[j][1] = acc[j][3] = Bs[8 * j + 2 * t + 1];
+        for (int m = 0; m < MT; ++m) {
+            xr[m] = x + (r0 + 16 * m) * NIN + 2 * t;
+            v0[m] = r0 + 16 * m < n;
+            v1[m] = r0 + 16 * m + 8 < n;
         }
-        float2 p[4], q[4];
-        auto load = [&](int s, float2 (&f)[4]) {
-            const int k0 = 16 * s + 2 * t, k1 = k0 + 8;
-            const float2 z = make_float2(0.f, 0.f);
-            f[0] = v0 && k0 < NIN ? *reinterpret_cast<const float2 *>(x0 + k0) : z;
-            f[1] = v1 && k0 < NIN ? *reinterpret_cast<const float2 *>(x1 + k0) : z;
-            f[2] = v0 && k1 < NIN ? *reinterpret_cast<const float2 *>(x0 + k1) : z;
-            f[3] = v1 && k1 < NIN ? *reinterpret_cast<const float2 *>(x1 + k1) : z;
-        };
-        load(0, p);
+        uint32_t af[MT][NT / 2][4];
+        {   // layer 1: acc = b1 + x W1
+            float acc[MT][NT][4];
 #pragma unroll
-        for (int s = 0; s < K1P / 16; ++s) {
-            if (s + 1 < K1P / 16) load(s + 1, q);
-            const uint32_t a[4] = {pack_bf16(p[0].x, p[0].y), pack_bf16(p[1].x, p[1].y), pack_bf16(p[2].x, p[2].y),
-                                   pack_bf16(p[3].x, p[3].y)};
+            for (int j = 0; j < NT; ++j)
 #pragma unroll
-            for (int j = 0; j < NT; ++j) {
-                const uint16_t *w = W1s + (8 * j + g) * S1 + 16 * s + 2 * t;
-                mma_bf16(acc[j], a, *reinterpret_cast<const uint32_t *>(w), *reinterpret_cast<const uint32_t *>(w + 8));
+                for (int m = 0; m < MT; ++m) {
+                    acc[m][j][0] = acc[m][j][2] = Bs[8 * j + 2 * t];
+                    acc[m][j][1] = acc[m][j][3] = Bs[8 * j + 2 * t + 1];
+                }
+            float2 p[2][MT][4];
+            auto load = [&](int s, float2 (&f)[MT][4]) {
+                const float2 z = make_float2(0.f, 0.f);
+                const bool a = 16 * s + 2 * t < NIN, b = 16 * s + 2 * t + 8 < NIN;
+#pragma unroll
+                for (int m = 0; m < MT; ++m) {
+                    const float *x0 = xr[m] + 16 * s, *x1 = x0 + 8 * NIN;
+                    f[m][0] = v0[m] && a ? *reinterpret_cast<const float2 *>(x0) : z;
+                    f[m][1] = v1[m] && a ? *reinterpret_cast<const float2 *>(x1) : z;
+                    f[m][2] = v0[m] && b ? *reinterpret_cast<const float2 *>(x0 + 8) : z;
+                    f[m][3] = v1[m] && b ? *reinterpret_cast<const float2 *>(x1 + 8) : z;
+                }
+            };
+            load(0, p[0]);
+#pragma unroll
+            for (int s = 0; s < K1; ++s) {
+                if (s + 1 < K1) load(s + 1, p[(s + 1) & 1]);
+                uint32_t a[MT][4];
+#pragma unroll
+                for (int m = 0; m < MT; ++m)
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) a[m][u] = pack_bf16(p[s & 1][m][u].x, p[s & 1][m][u].y);
+#pragma unroll
+                for (int j = 0; j < NT; j += 2) {
+                    uint32_t b[4];
+                    load_b2(w1a + (uint32_t)(8 * j * S1 + 16 * s) * 2, b);
+#pragma unroll
+                    for (int m = 0; m < MT; ++m) mma_bf16(acc[m][j], a[m], b[0], b[1]);
+#pragma unroll
+                    for (int m = 0; m < MT; ++m) mma_bf16(acc[m][j + 1], a[m], b[2], b[3]);
+                }
             }
 #pragma unroll
-            for (int u = 0; u < 4; ++u) p[u] = q[u];
+            for (int m = 0; m < MT; ++m) to_frags<NT>(acc[m], af[m]);
         }
-        uint32_t af[NT / 2][4];
-        to_frags<NT>(acc, af);
-        // layer 2
+        // layer 2, a half of its outputs at a time, and layer 3 (6 outputs in one n-tile of 8) over that half
+        float o[MT][4];
 #pragma unroll
-        for (int j = 0; j < NT; ++j) {
-            acc[j][0] = acc[j][2] = Bs[H + 8 * j + 2 * t];
-            acc[j][1] = acc[j][3] = Bs[H + 8 * j + 2 * t + 1];
+        for (int m = 0; m < MT; ++m) {
+            o[m][0] = o[m][2] = Bs[2 * H + 2 * t];
+            o[m][1] = o[m][3] = Bs[2 * H + 2 * t + 1];
         }
 #pragma unroll
-        for (int s = 0; s < G::KS; ++s)
+        for (int half = 0; half < 2; ++half) {
+            float acc[MT][NH][4];
 #pragma unroll
-            for (int j = 0; j < NT; ++j) {
-                const uint16_t *w = W2s + (8 * j + g) * S2 + 16 * s + 2 * t;
-                mma_bf16(acc[j], af[s], *reinterpret_cast<const uint32_t *>(w), *reinterpret_cast<const uint32_t *>(w + 8));
+            for (int j = 0; j < NH; ++j)
+#pragma unroll
+                for (int m = 0; m < MT; ++m) {
+                    acc[m][j][0] = acc[m][j][2] = Bs[H + 8 * (half * NH + j) + 2 * t];
+                    acc[m][j][1] = acc[m][j][3] = Bs[H + 8 * (half * NH + j) + 2 * t + 1];
+                }
+#pragma unroll
+            for (int s = 0; s < G::KS; ++s)
+#pragma unroll
+                for (int j = 0; j < NH; j += 2) {
+                    uint32_t b[4];
+                    load_b2(w2a + (uint32_t)(8 * (half * NH + j) * S2 + 16 * s) * 2, b);
+#pragma unroll
+                    for (int m = 0; m < MT; ++m) mma_bf16(acc[m][j], af[m][s], b[0], b[1]);
+#pragma unroll
+                    for (int m = 0; m < MT; ++m) mma_bf16(acc[m][j + 1], af[m][s], b[2], b[3]);
+                }
+#pragma unroll
+            for (int i = 0; i < NH / 2; ++i) {
+                const uint16_t *w = W3s + g * S2 + 16 * (half * (NH / 2) + i) + 2 * t;
+                const uint32_t b0 = *reinterpret_cast<const uint32_t *>(w), b1 = *reinterpret_cast<const uint32_t *>(w + 8);
+#pragma unroll
+                for (int m = 0; m < MT; ++m) {
+                    const float (&c0)[4] = acc[m][2 * i], (&c1)[4] = acc[m][2 * i + 1];
+                    const uint32_t a[4] = {pack_bf16(fmaxf(c0[0], 0.f), fmaxf(c0[1], 0.f)), pack_bf16(fmaxf(c0[2], 0.f), fmaxf(c0[3], 0.f)),
+                                           pack_bf16(fmaxf(c1[0], 0.f), fmaxf(c1[1], 0.f)), pack_bf16(fmaxf(c1[2], 0.f), fmaxf(c1[3], 0.f))};
+                    mma_bf16(o[m], a, b0, b1);
+                }
             }
-        to_frags<NT>(acc, af);
-        // layer 3 (6 outputs in one n-tile of 8)
-        float o[4];
-        o[0] = o[2] = Bs[2 * H + 2 * t];
-        o[1] = o[3] = Bs[2 * H + 2 * t + 1];
-#pragma unroll
-        for (int s = 0; s < G::KS; ++s) {
-            const uint16_t *w = W3s + g * S2 + 16 * s + 2 * t;
-            mma_bf16(o, af[s], *reinterpret_cast<const uint32_t *>(w), *reinterpret_cast<const uint32_t *>(w + 8));
         }
         if (t < 3) {
-            if (v0) *reinterpret_cast<float2 *>(out + r0 * NOUT + 2 * t) = make_float2(o[0], o[1]);
-            if (v1) *reinterpret_cast<float2 *>(out + r1 * NOUT + 2 * t) = make_float2(o[2], o[3]);
+#pragma unroll
+            for (int m = 0; m < MT; ++m) {
+                float *q = out + (r0 + 16 * m) * NOUT + 2 * t;
+                if (v0[m]) *reinterpret_cast<float2 *>(q) = make_float2(o[m][0], o[m][1]);
+                if (v1[m]) *reinterpret_cast<float2 *>(q + 8 * NOUT) = make_float2(o[m][2], o[m][3]);
+            }
         }
     }
 }
@@ -747,15 +816,17 @@ int infer_h(tpx_ctx *c, const void *packed, const float *x, long long n, float *
     if (ck(cudaGetDevice(&dev)) || ck(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev))) return TPX_ECUDA;
     const bool known = dev >= 0 && dev < 64;
     if (!known || !attr[dev].load(std::memory_order_acquire)) {
-        if (ck(cudaFuncSetAttribute(k_mlp_bf16<H>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::smem)))
+        if (ck(cudaFuncSetAttribute(k_mlp_bf16<H, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::smem)) ||
+            ck(cudaFuncSetAttribute(k_mlp_bf16<H, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::smem)))
             return TPX_ECUDA;
         if (known) attr[dev].store(true, std::memory_order_release);
     }
-    const long long tiles = (n + 127) / 128;
-    const unsigned grid = (unsigned)(tiles < sms ? tiles : sms);
     const uint16_t *wt = static_cast<const uint16_t *>(packed);
     const float *bias = reinterpret_cast<const float *>(static_cast<const char *>(packed) + packed_bias_off(G::wend));
-    k_mlp_bf16<H><<<grid, 256, G::smem, c->stream>>>(x, n, wt, bias, out);
+    // one tile of 128 rows per SM is the shortest way for few rows; beyond that 256 rows a tile
+    const long long tiles = (n + 127) / 128;
+    if (tiles <= sms) k_mlp_bf16<H, 1><<<(unsigned)tiles, 256, G::smem, c->stream>>>(x, n, wt, bias, out);
+    else k_mlp_bf16<H, 2><<<(unsigned)std::min<long long>((n + 255) / 256, sms), 256, G::smem, c->stream>>>(x, n, wt, bias, out);
     return ck(cudaGetLastError()) ? TPX_ECUDA : TPX_OK;
 }
 template <int H>
