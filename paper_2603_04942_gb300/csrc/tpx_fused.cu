@@ -17,6 +17,7 @@ constexpr int kAttrDevices = 64;   // devices whose kernel attributes are rememb
 // 1024-thread CTAs, one per SM, 4096-packet tiles, 8192-position ranges
 namespace geo_t4096 {
 constexpr int NT = 1024, T = 4096, C = 8192, TR = 512, MS = T + 16, MINB = 1, BIG_REGION = 165376;
+constexpr bool STAGED_ONLY = false;
 #include "tpx_fused_body.cuh"
 }  // namespace geo_t4096
 
@@ -24,10 +25,21 @@ constexpr int NT = 1024, T = 4096, C = 8192, TR = 512, MS = T + 16, MINB = 1, BI
 // shot of up to 3072 packets fits, wherever its trigger falls in the tile)
 namespace geo_t2048 {
 constexpr int NT = 512, T = 2048, C = 5120, TR = 256, MS = T / 4 + 16, MINB = 2, BIG_REGION = 103360;
+constexpr bool STAGED_ONLY = false;
 #include "tpx_fused_body.cuh"
 }  // namespace geo_t2048
 
-int fused_tile_packets(int geo) { return geo == GEO_T2048 ? geo_t2048::T : geo_t4096::T; }
+// for calls of few packets: the 4096 geometry with a quarter of a tile per CTA,
+// while the tiles are no more than the SMs. Such a call is one tile's latency,
+// and that grows with the tile's packets per thread (37 shots, 17,723 packets:
+// 5 tiles of 4096 took 37 us, 18 tiles of 1024 take 23: the call 69 -> 57 us).
+namespace geo_small {
+constexpr int NT = 1024, T = 1024, C = 8192, TR = 512, MS = 4096 + 16, MINB = 1, BIG_REGION = 165376;
+constexpr bool STAGED_ONLY = true;
+#include "tpx_fused_body.cuh"
+}  // namespace geo_small
+
+int fused_tile_packets(int geo) { return geo == GEO_T2048 ? geo_t2048::T : geo == GEO_SMALL ? geo_small::T : geo_t4096::T; }
 int fused_threads(int geo) { return geo == GEO_T2048 ? geo_t2048::NT : geo_t4096::NT; }
 int fused_range_capacity(int geo) { return geo == GEO_T2048 ? geo_t2048::C : geo_t4096::C; }
 int fused_ctas_per_sm(int geo) { return geo == GEO_T2048 ? geo_t2048::MINB : geo_t4096::MINB; }
@@ -38,7 +50,8 @@ cudaError_t launch_fused(const Params &p, int mode, int geo, int grid, cudaStrea
     cudaError_t e = launch_unwrap_prepass(p, fused_tile_packets(geo), grid, s);
     if (e == cudaSuccess && mid) e = cudaEventRecord(mid, s);
     if (e != cudaSuccess) return e;
-    return geo == GEO_T2048 ? geo_t2048::launch(p, mode, grid, s) : geo_t4096::launch(p, mode, grid, s);
+    return geo == GEO_T2048 ? geo_t2048::launch(p, mode, grid, s) : geo == GEO_SMALL ? geo_small::launch(p, mode, grid, s)
+                                                                                    : geo_t4096::launch(p, mode, grid, s);
 }
 
 }  // namespace tpxk

@@ -141,7 +141,7 @@ struct Params {
 // launch entry points (defined in tpx_fused.cu)
 namespace tpxk {
 // tile geometries of the fused kernel
-enum : int { GEO_T4096 = 1, GEO_T2048 = 2 };
+enum : int { GEO_T4096 = 1, GEO_T2048 = 2, GEO_SMALL = 3 };   // the last for small calls only (tpx_process)
 int fused_tile_packets(int geo);
 int fused_smem_bytes(int geo);
 int fused_threads(int geo);

@@ -27,6 +27,8 @@ constexpr long long MAX_TRIES = 1LL << 18;  // bounded look-back waits of the se
 constexpr long long MAX_HANDOVER = 1LL << 25;   // bounded waits between the two sides (seconds)
 
 static_assert(T <= C && C % 1024 == 0, "tile geometry");
+constexpr int LOOK = C / T > 4 ? C / T : 4;   // tiles after its own that a range within the capacity can reach into
+static_assert(C % T == 0 || LOOK * T >= C, "tiles of a range");
 constexpr int KM = (C + NTW - 1) / NTW;   // packets of a range a worker thread holds
 constexpr int TB = 256 * TR;              // cell table: bits, words
 constexpr int TW = TB / 32;
@@ -1317,8 +1319,8 @@ __device__ __noinline__ int big_range(Smem &S, const Params &p, long long base, 
 // ------------------------------------------------------------------- kernel
 // The service warp plans a tile's range and loads the unwrap state before it: the
 // tile's first TDC packet, the first one past the tile (the range's end) from
-// the pre-pass's tile table -- a range longer than the capacity needs no more
-// than the four tiles after its own -- and whether a pixel wrap is near.
+// the pre-pass's tile table -- a range within the capacity reaches no further
+// than LOOK tiles after its own -- and whether a pixel wrap is near.
 template <bool BATCH>
 __device__ void plan_tile(Smem::Plan &P, const Params &p, long long tile, bool bigr) {
     const int lane = threadIdx.x & 31;
@@ -1336,14 +1338,14 @@ __device__ void plan_tile(Smem::Plan &P, const Params &p, long long tile, bool b
         reinterpret_cast<long long *>(&P.E)[lane] = __ldcg(reinterpret_cast<const long long *>(&p.ts.pre[tile]) + lane);
     int f = -1;
     unsigned wrap = 0;
-    if (lane <= 4 && tile + lane < tile_end) {
+    if (lane <= LOOK && tile + lane < tile_end) {
         const int2 v = __ldcg(reinterpret_cast<const int2 *>(p.ts.tinfo) + tile + lane);
         f = v.x;
         wrap = (unsigned)v.y;
     }
     __syncwarp();
     const unsigned has = __ballot_sync(0xffffffffu, f >= 0) & ~1u;
-    const int j = has ? __ffs(has) - 1 : 4;          // tiles the range reaches into
+    const int j = has ? __ffs(has) - 1 : LOOK;       // tiles the range reaches into
     const int fj = __shfl_sync(0xffffffffu, f, j), f0 = __shfl_sync(0xffffffffu, f, 0);
     const unsigned slow = __ballot_sync(0xffffffffu, wrap != 0 && lane <= j);
     if (lane == 0) {
@@ -1360,7 +1362,7 @@ __device__ void plan_tile(Smem::Plan &P, const Params &p, long long tile, bool b
                 len = (long long)j * T + fj + 1;
                 term = true;
             } else {
-                over = tile + 5 < tile_end;
+                over = tile + LOOK + 1 < tile_end;
                 len = over ? C : rend - base;
             }
             if (len > C) { over = true; len = C; term = false; }
@@ -2221,9 +2223,11 @@ cudaError_t launch_one(const Params &p, int grid, cudaStream_t s) {
 
 cudaError_t launch(const Params &p, int mode, int grid, cudaStream_t s) {
     const bool cc = mode == TPX_MODE_CC;
-    if (p.bt.tile_run)   // a batch always stages its output
-        return cc ? launch_one<TPX_MODE_CC, true, true>(p, grid, s) : launch_one<TPX_MODE_PAPER, true, true>(p, grid, s);
-    if (p.stage)
-        return cc ? launch_one<TPX_MODE_CC, true, false>(p, grid, s) : launch_one<TPX_MODE_PAPER, true, false>(p, grid, s);
-    return cc ? launch_one<TPX_MODE_CC, false, false>(p, grid, s) : launch_one<TPX_MODE_PAPER, false, false>(p, grid, s);
+    if constexpr (!STAGED_ONLY) {
+        if (p.bt.tile_run)   // a batch always stages its output
+            return cc ? launch_one<TPX_MODE_CC, true, true>(p, grid, s) : launch_one<TPX_MODE_PAPER, true, true>(p, grid, s);
+        if (!p.stage)
+            return cc ? launch_one<TPX_MODE_CC, false, false>(p, grid, s) : launch_one<TPX_MODE_PAPER, false, false>(p, grid, s);
+    }
+    return cc ? launch_one<TPX_MODE_CC, true, false>(p, grid, s) : launch_one<TPX_MODE_PAPER, true, false>(p, grid, s);
 }

@@ -60,13 +60,17 @@ int alloc_scratch(tpx_ctx *c, int64_t max_packets) {
     const int64_t T = tpxk::fused_tile_packets(tpxk::GEO_T2048);
     int64_t tiles = (max_packets + T - 1) / T;
     if (tiles < 1) tiles = 1;
+    max_packets = tiles * T;
+    // the small tiles are used up to one per SM
+    const int64_t Ts = tpxk::fused_tile_packets(tpxk::GEO_SMALL);
+    tiles = std::max(tiles, std::min<int64_t>((max_packets + Ts - 1) / Ts, c->num_sms));
     auto al = [](size_t b) { return (b + 255) & ~size_t(255); };
     const size_t b_flags = al(sizeof(unsigned) * tiles), b_agg = al(sizeof(tpxk::GAgg) * tiles),
                  b_head = al(sizeof(tpxk::GChain) * tiles), b_info = al(sizeof(tpxk::TileInfo) * tiles),
                  b_cnt = al(sizeof(long long) * tiles), b_blk = al(tpxk::unwrap_prepass_scratch_bytes(tiles));
     // record staging of the fused kernel: one range's records per CTA
     size_t stage_records = 0;   // the largest grid of a call times its range capacity
-    for (int geo : {(int)tpxk::GEO_T4096, (int)tpxk::GEO_T2048}) {
+    for (int geo : {(int)tpxk::GEO_T4096, (int)tpxk::GEO_T2048, (int)tpxk::GEO_SMALL}) {
         const int64_t tg = (max_packets + tpxk::fused_tile_packets(geo) - 1) / tpxk::fused_tile_packets(geo);
         int64_t ctas = (int64_t)c->num_sms * tpxk::fused_ctas_per_sm(geo);
         if (tg < ctas) ctas = tg < 1 ? 1 : tg;
@@ -91,7 +95,7 @@ int alloc_scratch(tpx_ctx *c, int64_t max_packets) {
     c->stage = reinterpret_cast<tpx_record *>(p);
     c->scratch = mem;
     c->max_tiles = tiles;
-    c->max_packets = tiles * T;
+    c->max_packets = max_packets;
     c->seq = 0;   // fresh flags: any sequence number is new
     return TPX_OK;
 }
@@ -137,13 +141,14 @@ int begin_call(tpx_ctx *c) {
 }
 
 // ---- tile-geometry autotuner ----
-constexpr int64_t kTuneMinPackets = 1LL << 20;   // smaller calls run untimed on the 4096 tiles
+constexpr int64_t kTuneMinPackets = 1LL << 20;   // smaller calls run untimed: on small tiles while there is an SM for each, then on the 4096 tiles
 constexpr double kTunePenalty = 1e30;            // a sample whose call had to be redone
 
 int tune_pick(const tpx_ctx *c, int64_t n) {
     if (c->cfg.tile_geometry != TPX_TILE_DEFAULT) return c->geo;
     if (c->tune.fixed) return c->tune.fixed;
-    if (n < kTuneMinPackets) return tpxk::GEO_T4096;
+    if (n < kTuneMinPackets)
+        return n <= (int64_t)c->num_sms * tpxk::fused_tile_packets(tpxk::GEO_SMALL) ? tpxk::GEO_SMALL : tpxk::GEO_T4096;
     // alternate, the smaller tiles first
     return c->tune.issued[tpxk::GEO_T2048 - 1] <= c->tune.issued[tpxk::GEO_T4096 - 1] ? tpxk::GEO_T2048 : tpxk::GEO_T4096;
 }
