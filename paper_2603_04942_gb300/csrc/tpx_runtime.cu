@@ -764,7 +764,10 @@ int tpx_sync(tpx_ctx *c, tpx_counters *out) {
 namespace {
 
 constexpr int64_t kPipeMinPackets = 1LL << 24;     // below this one call does it
-constexpr int64_t kPipePiecePackets = 1LL << 23;   // smallest piece
+// smallest piece: the first piece's copy up and the last one's copies down are
+// all that nothing overlaps (1.9e7 packets in 2 pieces 1.82 ms, in 4 1.62 ms), and
+// up to 1024 tiles the pre-pass is one launch
+constexpr int64_t kPipePiecePackets = 1LL << 22;
 
 int pipe_init(tpx_ctx *c) {
     auto &P = c->pipe;
