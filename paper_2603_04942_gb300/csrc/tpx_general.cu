@@ -36,6 +36,7 @@
 #include "tpx_common.cuh"
 #include "tpx_ctx.h"
 #include "tpx_fused.cuh"
+#include "tpx_unwrap.cuh"
 
 namespace tpxg {
 
@@ -148,26 +149,71 @@ __device__ __forceinline__ void strip_of(long long items, long long *b, long lon
     *e = min(items, *b + per);
 }
 
-// ------------------------------------------------------------ decode kernels
-__global__ void __launch_bounds__(GT) k_tile_agg(const uint64_t *pk, long long n, long long tp, long long tt,
-                                                 GAgg *tagg, long long *tcnt) {
-    __shared__ GAgg s_w[GW];
-    __shared__ GAgg s_tot;
-    const long long tile = blockIdx.x, base = tile * GTILE;
-    GAgg a = agg_id();
-    long long ntdc = 0;
-    for (int j = 0; j < GK; ++j) {
-        const long long q = base + threadIdx.x * GK + j;
-        if (q >= n) break;
-        const uint64_t w = pk[q];
-        const unsigned h = (unsigned)(w >> 60);
-        if (h == 0xBu) chain_push(a.pix, pix_raw(w), tp);
-        else if (h == 0x6u) { chain_push(a.tdc, tdc_raw(w), tt); ++ntdc; }
+// the block's flags: a warp takes 32 * GK consecutive items, 32 per ballot;
+// returns the slot of the warp's first flagged item within the block
+template <class F>
+__device__ __forceinline__ unsigned block_flags(long long n, F flag, unsigned (&m)[GK], unsigned *s_c, unsigned *total) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const long long base = blockIdx.x * (long long)GTILE + w * (32 * GK) + lane;
+    unsigned f = 0, c = 0;
+#pragma unroll
+    for (int j = 0; j < GK; ++j) {   // no ballot yet: the loads of all rounds are in flight together
+        const long long i = base + 32 * j;
+        if (i < n && flag(i, j)) f |= 1u << j;
     }
-    (void)block_scan_agg_g(a, s_w, &s_tot, tp, tt);
-    if (threadIdx.x == 0) {
-        tagg[tile] = s_tot;
-        tcnt[tile] = s_tot.tdc.n;
+#pragma unroll
+    for (int j = 0; j < GK; ++j) {
+        m[j] = __ballot_sync(0xffffffffu, (f >> j) & 1u);
+        c += __popc(m[j]);
+    }
+    if (lane == 0) s_c[w] = c;
+    __syncthreads();
+    unsigned before = 0, all = 0;
+#pragma unroll
+    for (int k = 0; k < GW; ++k) {
+        before += k < w ? s_c[k] : 0u;
+        all += s_c[k];
+    }
+    *total = all;
+    return before;
+}
+
+// ------------------------------------------------------------ decode kernels
+// a tile's chain aggregates, its triggers, and whether a wrap step of either
+// stream lies inside it: a warp per 512 packets, its loads ahead of its steps
+__global__ void __launch_bounds__(GT) k_tile_agg(const uint64_t *pk, long long n, long long tp, long long tt,
+                                                 GAgg *tagg, long long *tcnt, unsigned char *twrap) {
+    __shared__ GAgg s_a[32];
+    __shared__ bool s_wrap[GW];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const long long tile = blockIdx.x, base = tile * GTILE;
+    const int cnt = (int)min((long long)GTILE, n - base), per = GTILE / GW;
+    const int qb = w * per, qe = min(cnt, qb + per);
+    WarpPart<4> part;
+    if (qb < qe) part.run(pk + base, (reinterpret_cast<uintptr_t>(pk) & 15) == 0, qb, qe, tp, tt, lane);
+    GAgg a;
+    GChain head;
+    part.result(&a, &head);
+    if (lane == 0) {
+        s_a[w] = a;
+        s_wrap[w] = part.wraps;
+    }
+    __syncthreads();
+    if (w == 0) {
+        const GAgg mine = lane < GW ? s_a[lane] : agg_id();
+        const GAgg incl = warp_incl_scan(mine, lane, tp, tt);
+        const bool wrap = __any_sync(0xffffffffu, lane < GW && s_wrap[lane]);
+        if (lane == 31) {   // sums of opposite wraps cancel: `wraps` and the parts' steps tell of each
+            tagg[tile] = incl;
+            tcnt[tile] = incl.tdc.n;
+        }
+        GAgg before = shfl_up_agg(incl, 1);
+        if (lane == 0) before = agg_id();
+        const bool step = (before.pix.n && mine.pix.n && jump(mine.pix.first - before.pix.last, tp) != 0) ||
+                          (before.tdc.n && mine.tdc.n && jump(mine.tdc.first - before.tdc.last, tt) != 0) ||
+                          mine.tdc.sum != 0;
+        const bool any = __any_sync(0xffffffffu, step);
+        if (lane == 0) twrap[tile] = wrap || any;
     }
 }
 
@@ -203,12 +249,50 @@ __global__ void __launch_bounds__(PT) k_tile_prefix(const GAgg *tagg, GAgg *tpre
     }
 }
 
-__global__ void __launch_bounds__(GT) k_unwrap(const uint64_t *pk, long long n, const GAgg *tpre, const long long *toff,
+// A tile without a wrap step (nearly all) adds one constant per stream: warps
+// read and write 512 consecutive packets each, bound by the bytes. The others
+// follow the chains packet by packet.
+__global__ void __launch_bounds__(GT) k_unwrap(const uint64_t *pk, long long n, const GAgg *tagg, const GAgg *tpre,
+                                               const unsigned char *twrap, const long long *toff,
                                                long long tp, long long tt, long long *t_all, long long *trig,
                                                long long trig_cap, unsigned *status, long long *trig_pos) {
     __shared__ GAgg s_w[GW];
     __shared__ GAgg s_tot;
+    __shared__ unsigned s_c[GW];
     const long long tile = blockIdx.x, base = tile * GTILE;
+    const GAgg before = tpre[tile], own = tagg[tile];
+    const bool wraps = twrap[tile] || (before.pix.n && own.pix.n && jump(own.pix.first - before.pix.last, tp) != 0) ||
+                       (before.tdc.n && own.tdc.n && jump(own.tdc.first - before.tdc.last, tt) != 0);
+    if (!wraps) {
+        const int lane = threadIdx.x & 31;
+        const long long q0 = base + (threadIdx.x >> 5) * (32 * GK) + lane;
+        const long long dp = before.pix.sum * kPixPeriod, dd = before.tdc.sum * kTdcPeriod;
+        uint64_t v[GK];
+#pragma unroll
+        for (int j = 0; j < GK; ++j) v[j] = q0 + 32 * j < n ? pk[q0 + 32 * j] : 0;
+        unsigned m[GK], total;
+        unsigned o = block_flags(n, [&](long long, int j) { return (unsigned)(v[j] >> 60) == 0x6u; }, m, s_c, &total);
+#pragma unroll
+        for (int j = 0; j < GK; ++j) {
+            const long long q = q0 + 32 * j;
+            const unsigned h = (unsigned)(v[j] >> 60);
+            long long t = 0;
+            if (h == 0xBu) t = pix_raw(v[j]) + dp;
+            else if (h == 0x6u) {
+                t = tdc_raw(v[j]) + dd;
+                const long long ti = toff[tile] + o + __popc(m[j] & ((1u << lane) - 1u));
+                if (ti < trig_cap) {
+                    trig[ti] = t;
+                    if (trig_pos) trig_pos[ti] = q;
+                } else {
+                    atomicOr(status, ST_TRIG_CAP);
+                }
+            }
+            o += __popc(m[j]);
+            if (q < n) t_all[q] = t;
+        }
+        return;
+    }
     const long long q0 = base + threadIdx.x * GK;
     GAgg a = agg_id();
     for (int j = 0; j < GK; ++j) {
@@ -277,51 +361,63 @@ __device__ __forceinline__ long long shot_of(const long long *trig, long long nt
     return lo - 1;
 }
 
-// 0 keep, 1 background, 2 before any trigger, 3 not a pixel
-__device__ __forceinline__ int bin_pixel(uint64_t w, long long t, const long long *trig, long long ntr,
-                                         long long tof_max, long long *shot, long long *tof) {
-    if ((w >> 60) != 0xBu) return 3;
-    const long long s = shot_of(trig, ntr, t);
-    if (s < 0) return 2;
-    const long long f = t - trig[s];
-    if (f > tof_max) return 1;
-    *shot = s;
-    *tof = f;
-    return 0;
-}
-
-// per tile: kept pixels and the drop counters (packets read warp-strided)
+// per tile: kept pixels and the drop counters; per packet: its shot, or -1 when
+// it is not a kept pixel. A thread's packets follow one another in time, so the
+// shot of the one before is tried first; a search over the triggers for the rest.
 __global__ void __launch_bounds__(GT) k_bin(const uint64_t *pk, long long n, const long long *t_all, const long long *trig,
-                                            const long long *n_trig, long long trig_cap, long long tof_max,
+                                            const long long *n_trig, long long trig_cap, long long tof_max, int *shot,
                                             long long *tile_kept, unsigned long long *counters) {
-    __shared__ long long s_w[GW];
-    __shared__ long long s_tot;
+    __shared__ unsigned s_c[6];
     const long long tile = blockIdx.x, base = tile * GTILE;
     const long long ntr = usable_triggers(n_trig, trig_cap);
-    long long keep = 0, bg = 0, pre = 0, pix = 0, tdc = 0, bad = 0;
-    for (int j = 0; j < GK && ntr >= 0; ++j) {
-        const long long q = base + j * GT + threadIdx.x;
-        if (q >= n) break;
-        const uint64_t w = pk[q];
-        const unsigned h = (unsigned)(w >> 60);
-        if (h == 0x6u) { ++tdc; continue; }
-        if (h != 0xBu) { ++bad; continue; }
-        ++pix;
-        long long s, f;
-        const int v = bin_pixel(w, t_all[q], trig, ntr, tof_max, &s, &f);
-        keep += v == 0;
-        bg += v == 1;
-        pre += v == 2;
+    if (threadIdx.x < 6) s_c[threadIdx.x] = 0;
+    __syncthreads();
+    unsigned keep = 0, bg = 0, pre = 0, pix = 0, tdc = 0, bad = 0;
+    long long s = -1, from = 1, to = 0;   // the last pixel's shot and its times [from, to)
+    constexpr int B = 8;   // packets whose loads are in flight together
+    for (int j0 = 0; j0 < GK && ntr >= 0; j0 += B) {
+        unsigned h[B];
+        long long t[B];
+#pragma unroll
+        for (int j = 0; j < B; ++j) {
+            const long long q = base + (j0 + j) * GT + threadIdx.x;
+            h[j] = q < n ? (unsigned)(pk[q] >> 60) : 0x100u;
+            t[j] = q < n ? t_all[q] : 0;
+        }
+#pragma unroll
+        for (int j = 0; j < B; ++j) {
+            if (h[j] == 0x100u) break;
+            int out = -1;
+            if (h[j] == 0xBu) {
+                ++pix;
+                if (t[j] < from || t[j] >= to) {
+                    s = shot_of(trig, ntr, t[j]);
+                    from = s >= 0 ? trig[s] : LLONG_MIN;
+                    to = s + 1 < ntr ? trig[s + 1] : LLONG_MAX;
+                }
+                if (s < 0) ++pre;
+                else if (t[j] - from > tof_max) ++bg;
+                else {
+                    ++keep;
+                    out = (int)s;
+                }
+            } else if (h[j] == 0x6u) ++tdc;
+            else ++bad;
+            shot[base + (j0 + j) * GT + threadIdx.x] = out;
+        }
     }
-    const long long vals[6] = {keep, bg, pre, pix, tdc, bad};
-    const int idx[6] = {C_KEPT, C_DROP_BG, C_DROP_PRE, C_PIXELS, C_TDCS, C_CORRUPT};
+    const unsigned vals[6] = {keep, bg, pre, pix, tdc, bad};
+#pragma unroll
     for (int k = 0; k < 6; ++k) {
-        unsigned long long v = (unsigned long long)vals[k];
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-        if ((threadIdx.x & 31) == 0 && v) atomicAdd(&counters[idx[k]], v);
+        const unsigned v = __reduce_add_sync(0xffffffffu, vals[k]);
+        if ((threadIdx.x & 31) == 0 && v) atomicAdd(&s_c[k], v);
     }
-    (void)block_scan_ll(keep, s_w, &s_tot);
-    if (threadIdx.x == 0) tile_kept[tile] = s_tot;
+    __syncthreads();
+    if (threadIdx.x < 6) {
+        const int idx[6] = {C_KEPT, C_DROP_BG, C_DROP_PRE, C_PIXELS, C_TDCS, C_CORRUPT};
+        if (s_c[threadIdx.x]) atomicAdd(&counters[idx[threadIdx.x]], (unsigned long long)s_c[threadIdx.x]);
+        if (threadIdx.x == 0) tile_kept[tile] = s_c[0];
+    }
 }
 
 // exclusive prefix of per-tile counts (one block)
@@ -344,48 +440,37 @@ __global__ void __launch_bounds__(PT) k_count_prefix(const long long *cnt, long 
     }
 }
 
-// kept pixels in stream order: per round of GT consecutive packets, a ballot
-// and the warp counts give every kept pixel its slot (coalesced writes)
+// kept pixels in stream order (a warp takes 512 consecutive packets, so its
+// writes are runs)
 __global__ void __launch_bounds__(GT) k_compact(const uint64_t *pk, long long n, long long idx_base, const long long *t_all,
                                                 const long long *trig, const long long *n_trig, long long trig_cap,
-                                                long long tof_max, const int16_t *lut, const long long *tile_off,
+                                                const int *shot, const int16_t *lut, const long long *tile_off,
                                                 tpx_hits hits, long long cap, unsigned *status, const GAgg *E0) {
-    __shared__ unsigned s_wc[GW];
+    __shared__ unsigned s_c[GW];
     const long long trig_base = E0 ? E0->tdc.n : 0;
-    const long long ntr = usable_triggers(n_trig, trig_cap);
-    if (ntr < 0) return;
-    const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
-    const long long tile = blockIdx.x, base = tile * GTILE;
-    long long o = tile_off[tile];
-    for (int j = 0; j < GK; ++j) {
-        if (base + j * GT >= n) break;                  // uniform over the block
-        const long long q = base + j * GT + threadIdx.x;
-        uint64_t w = 0;
-        long long s = 0, f = 0;
-        bool keep = false;
-        if (q < n) {
-            w = pk[q];
-            keep = bin_pixel(w, t_all[q], trig, ntr, tof_max, &s, &f) == 0;
-        }
-        const unsigned bal = __ballot_sync(0xffffffffu, keep);
-        if (lane == 0) s_wc[wi] = __popc(bal);
-        __syncthreads();
-        unsigned before = 0, total = 0;
+    if (usable_triggers(n_trig, trig_cap) < 0) return;
+    const int lane = threadIdx.x & 31;
+    const long long tile = blockIdx.x;
+    const long long q0 = tile * GTILE + (threadIdx.x >> 5) * (32 * GK) + lane;
+    int sh[GK];
 #pragma unroll
-        for (int k = 0; k < GW; ++k) {
-            const unsigned c = s_wc[k];
-            before += k < wi ? c : 0u;
-            total += c;
-        }
-        if (keep) {
-            const long long slot = o + before + __popc(bal & ((1u << lane) - 1u));
+    for (int j = 0; j < GK; ++j) sh[j] = q0 + 32 * j < n ? shot[q0 + 32 * j] : -1;
+    unsigned m[GK], total;
+    const unsigned before = block_flags(n, [&](long long, int j) { return sh[j] >= 0; }, m, s_c, &total);
+    long long o = tile_off[tile] + before;
+#pragma unroll
+    for (int j = 0; j < GK; ++j) {
+        if (sh[j] >= 0) {
+            const long long q = q0 + 32 * j, slot = o + __popc(m[j] & ((1u << lane) - 1u));
             if (slot < cap) {
+                const uint64_t w = pk[q];
+                const long long t = t_all[q];
                 const int tot = pix_tot(w);
                 const long long corr = lut ? (long long)lut[tot] : 0LL;
                 hits.index[slot] = idx_base + q;
-                hits.shot[slot] = s + trig_base;
-                hits.t[slot] = t_all[q] - corr;
-                hits.tof[slot] = (int32_t)(f - corr);
+                hits.shot[slot] = sh[j] + trig_base;
+                hits.t[slot] = t - corr;
+                hits.tof[slot] = (int32_t)(t - trig[sh[j]] - corr);
                 hits.x[slot] = (uint8_t)pix_x(w);
                 hits.y[slot] = (uint8_t)pix_y(w);
                 hits.tot[slot] = (uint16_t)tot;
@@ -393,76 +478,155 @@ __global__ void __launch_bounds__(GT) k_compact(const uint64_t *pk, long long n,
                 atomicOr(status, ST_CLUSTER_CAP);
             }
         }
-        o += total;
-        __syncthreads();
+        o += __popc(m[j]);
     }
 }
 
 // ------------------------------------------------------------ radix sort
-// stable LSD sort of (key, value) pairs on 8-bit digits
-__global__ void __launch_bounds__(GT) k_sort_hist(const unsigned long long *keys, long long n, int shift, unsigned *hist,
-                                                  long long tiles) {
-    __shared__ unsigned h[256];
-    h[threadIdx.x] = 0;
+// Stable LSD sort of (key, value) pairs on 8-bit digits, in tiles of 4096 keys;
+// per digit: each tile's histogram (the first digit's is taken while the keys
+// are made), a scan of them over the tiles, and the placing. A CTA ranks its
+// tile in registers (a warp's 32 keys by eight ballots, its own counters in
+// shared memory), puts it in digit order in shared memory and writes runs. Keys
+// of 32 bits where (shot, ToF) fits them.
+// What bounds it: instruction issue (the ranking) on large inputs, the launches
+// on small ones. Measured per digit of 6.0e6 / 1.2e6 hits: 109 / 45 us with a
+// scatter of 16 rounds, each waiting for the one before, and three scan
+// launches; 60 / 19 us with one launch whose tiles look back for the counts
+// before them (their polling took two thirds of the issue slots); now 58 / 17.
+template <class K>
+__device__ __forceinline__ unsigned digit_of(K key, int shift) { return (unsigned)(key >> shift) & 255u; }
+// one count in shared memory; a warp whose keys share the digit, as those of
+// the upper digits do, adds once. act: the lanes that call.
+__device__ __forceinline__ void count_digit(unsigned *h, unsigned d, unsigned act) {
+    int same = 0;
+    __match_all_sync(act, d, &same);
+    if (!same) atomicAdd(&h[d], 1u);
+    else if ((int)(threadIdx.x & 31) == __ffs(act) - 1) atomicAdd(&h[d], (unsigned)__popc(act));
+}
+template <class K>
+__global__ void __launch_bounds__(GT) k_digit_hist(const K *keys, long long n, int shift, unsigned *hist) {
+    __shared__ unsigned s_h[256];
+    s_h[threadIdx.x] = 0;
+    const long long base = blockIdx.x * (long long)GTILE + threadIdx.x;
+    K k[GK];
+#pragma unroll
+    for (int j = 0; j < GK; ++j) k[j] = base + j * GT < n ? keys[base + j * GT] : K(0);
     __syncthreads();
-    const long long base = blockIdx.x * (long long)GTILE;
+#pragma unroll
     for (int j = 0; j < GK; ++j) {
-        const long long i = base + j * GT + threadIdx.x;
-        if (i < n) atomicAdd(&h[(keys[i] >> shift) & 255], 1u);
+        const bool ok = base + j * GT < n;
+        const unsigned act = __ballot_sync(0xffffffffu, ok);
+        if (ok) count_digit(s_h, digit_of(k[j], shift), act);
     }
     __syncthreads();
-    hist[(long long)threadIdx.x * tiles + blockIdx.x] = h[threadIdx.x];
+    hist[blockIdx.x * 256ll + threadIdx.x] = s_h[threadIdx.x];
 }
-
-__global__ void __launch_bounds__(GT) k_sort_scatter(const unsigned long long *kin, const unsigned *vin, long long n,
-                                                     int shift, const unsigned *offs, long long tiles,
-                                                     unsigned long long *kout, unsigned *vout) {
-    __shared__ unsigned run[256];       // running count per digit in this tile
-    __shared__ unsigned wcnt[GW][256];  // per-warp counts of the current round
+// per digit the exclusive prefix over the tiles, in place, and the total: a CTA
+// takes 32 digits, each of its warps a stretch of the tiles
+__global__ void __launch_bounds__(PT) k_digit_scan(unsigned *hist, long long tiles, unsigned *total) {
+    __shared__ unsigned s_sum[32][33];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    run[threadIdx.x] = offs[(long long)threadIdx.x * tiles + blockIdx.x];
-    const long long base = blockIdx.x * (long long)GTILE;
-    for (int j = 0; j < GK; ++j) {
-        for (int k = 0; k < GW; ++k) wcnt[k][threadIdx.x] = 0;
-        __syncthreads();
-        const long long i = base + j * GT + threadIdx.x;
-        const bool ok = i < n;
-        const unsigned long long key = ok ? kin[i] : 0ull;
-        const unsigned d = ok ? (unsigned)((key >> shift) & 255) : 256u + lane;   // unique dummy for idle lanes
-        const unsigned peers = __match_any_sync(0xffffffffu, d);
-        const unsigned before = __popc(peers & ((1u << lane) - 1u));
-        if (ok && before == 0) wcnt[w][d] = __popc(peers);
-        __syncthreads();
-        unsigned pos = 0;
-        if (ok) {
-            unsigned acc = 0;
-            for (int k = 0; k < w; ++k) acc += wcnt[k][d];
-            pos = run[d] + acc + before;
-            kout[pos] = key;
-            vout[pos] = vin[i];
+    const long long per = (tiles + 31) / 32, t0 = min(tiles, w * per), t1 = min(tiles, t0 + per);
+    unsigned *h = hist + blockIdx.x * 32 + lane;
+    unsigned sum = 0;
+#pragma unroll 8
+    for (long long t = t0; t < t1; ++t) sum += h[t * 256];
+    s_sum[w][lane] = sum;
+    __syncthreads();
+    unsigned run = 0, all = 0;
+#pragma unroll
+    for (int k = 0; k < 32; ++k) {
+        const unsigned v = s_sum[k][lane];
+        run += k < w ? v : 0u;
+        all += v;
+    }
+    if (w == 0) total[blockIdx.x * 32 + lane] = all;
+    for (long long t = t0; t < t1; t += 8) {
+        unsigned v[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) v[k] = t + k < t1 ? h[(t + k) * 256] : 0u;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            if (t + k < t1) h[(t + k) * 256] = run;
+            run += v[k];
         }
-        __syncthreads();
-        // advance the running counts by this round's totals
-        unsigned tot = 0;
-        for (int k = 0; k < GW; ++k) tot += wcnt[k][threadIdx.x];
-        run[threadIdx.x] += tot;
-        __syncthreads();
     }
 }
-
-// exclusive scan of unsigned counts (serial over block sums; general path only)
-__global__ void __launch_bounds__(GT) k_scan_blocks(const unsigned *in, unsigned *out, long long n, unsigned *bsum) {
+template <class K>
+__global__ void __launch_bounds__(GT, sizeof(K) == 4 ? 4 : 3) k_digit_place(const K *kin, const unsigned *vin, long long n,
+                                                                           int shift, const unsigned *offs,
+                                                                           const unsigned *total, K *kout, unsigned *vout) {
+    extern __shared__ __align__(16) unsigned char s_buf[];   // the tile in digit order: keys, values
+    __shared__ unsigned s_wh[GW][256];      // per warp: digit counts, then the warp's first slot of each digit
+    __shared__ unsigned s_off[256];         // output position of a digit's run minus its slot in the tile
     __shared__ long long s_w[GW];
     __shared__ long long s_tot;
-    const long long base = blockIdx.x * (long long)GTILE + threadIdx.x * GK;
-    long long mine = 0;
-    for (int j = 0; j < GK; ++j)
-        if (base + j < n) mine += in[base + j];
-    long long o = block_scan_ll(mine, s_w, &s_tot);
-    for (int j = 0; j < GK; ++j)
-        if (base + j < n) { out[base + j] = (unsigned)o; o += in[base + j]; }
-    if (threadIdx.x == 0) bsum[blockIdx.x] = (unsigned)s_tot;
+    K *bk = reinterpret_cast<K *>(s_buf);
+    unsigned *bv = reinterpret_cast<unsigned *>(s_buf + GTILE * sizeof(K));
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    const long long base = blockIdx.x * (long long)GTILE;
+    const int valid = (int)min((long long)GTILE, n - base);
+    const int i0 = w * (32 * GK) + lane;
+    K key[GK];
+    unsigned pos[GK];
+#pragma unroll
+    for (int j = 0; j < GK; ++j) key[j] = i0 + 32 * j < valid ? kin[base + i0 + 32 * j] : ~K(0);   // past the end: behind every key
+    const unsigned before = offs[blockIdx.x * 256ll + t], all = total[t];   // thread t: digit t
+#pragma unroll
+    for (int k = 0; k < GW; ++k) s_wh[k][t] = 0;
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < GK; ++j) {
+        const unsigned d = digit_of(key[j], shift);
+        unsigned peers = 0xffffffffu;
+#pragma unroll
+        for (int b = 0; b < 8; ++b) {
+            const unsigned m = __ballot_sync(0xffffffffu, (d >> b) & 1u);
+            peers &= ((d >> b) & 1u) ? m : ~m;
+        }
+        const int leader = __ffs(peers) - 1;
+        unsigned old = 0;
+        if (lane == leader) {
+            old = s_wh[w][d];
+            s_wh[w][d] = old + __popc(peers);
+        }
+        pos[j] = __shfl_sync(0xffffffffu, old, leader) + __popc(peers & ((1u << lane) - 1u));
+        __syncwarp();
+    }
+    __syncthreads();
+    unsigned cnt = 0;
+#pragma unroll
+    for (int k = 0; k < GW; ++k) {
+        const unsigned x = s_wh[k][t];
+        s_wh[k][t] = cnt;
+        cnt += x;
+    }
+    // the digits' starts in the whole output and in the tile, one scan
+    const long long both = block_scan_ll(((long long)all << 16) | cnt, s_w, &s_tot);
+    const unsigned lstart = (unsigned)(both & 0xFFFF);
+    s_off[t] = (unsigned)(both >> 16) + before - lstart;
+#pragma unroll
+    for (int k = 0; k < GW; ++k) s_wh[k][t] += lstart;
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < GK; ++j) {
+        const int i = i0 + 32 * j;
+        const unsigned q = pos[j] + s_wh[w][digit_of(key[j], shift)];
+        bk[q] = key[j];
+        bv[q] = i < valid ? (vin ? vin[base + i] : (unsigned)(base + i)) : 0u;
+    }
+    __syncthreads();
+#pragma unroll 4
+    for (int i = t; i < valid; i += GT) {
+        const K k = bk[i];
+        const unsigned g = s_off[digit_of(k, shift)] + i;
+        kout[g] = k;
+        vout[g] = bv[i];
+    }
 }
+
+// exclusive scan of block counts in place (one block)
 __global__ void __launch_bounds__(PT) k_scan_bsum(unsigned *bsum, long long nb) {
     __shared__ long long s_c[32];
     __shared__ long long s_tot;
@@ -477,22 +641,43 @@ __global__ void __launch_bounds__(PT) k_scan_bsum(unsigned *bsum, long long nb) 
         o += x;
     }
 }
-__global__ void k_scan_add(unsigned *out, long long n, const unsigned *bsum) {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        out[i] += bsum[i / GTILE];
-}
-
 // ------------------------------------------------------------ cluster kernels
-// sort key: (shot relative to the call's first shot) << 24 | corrected ToF + bias
-__global__ void k_make_keys(tpx_hits h, long long n, const unsigned long long *shot_min, unsigned long long *keys,
-                            unsigned *vals) {
+// sort key: (shot relative to the call's first shot) << 24 | corrected ToF + bias;
+// beside it each hit's pixel and ToT in one word, and the tiles' histograms of
+// the first digit
+template <class K>
+__global__ void __launch_bounds__(GT) k_make_keys(tpx_hits h, long long n, const unsigned long long *shot_min, K *keys,
+                                                  unsigned *pxt, unsigned *hist) {
+    __shared__ unsigned s_h[256];
+    s_h[threadIdx.x] = 0;
     const unsigned long long m = *shot_min;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        keys[i] = (((unsigned long long)h.shot[i] - m) << 24) | (unsigned long long)(h.tof[i] + kBias);
-        vals[i] = (unsigned)i;
+    const long long base = blockIdx.x * (long long)GTILE + threadIdx.x;
+    __syncthreads();
+#pragma unroll
+    for (int j0 = 0; j0 < GK; j0 += 4) {
+        K key[4];
+        unsigned px[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const long long i = base + (j0 + j) * GT;
+            if (i >= n) continue;
+            key[j] = (K)((((unsigned long long)h.shot[i] - m) << 24) | (unsigned long long)(h.tof[i] + kBias));
+            px[j] = (unsigned)h.x[i] | ((unsigned)h.y[i] << 8) | ((unsigned)h.tot[i] << 16);
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const long long i = base + (j0 + j) * GT;
+            if (i >= n) continue;
+            keys[i] = key[j];
+            pxt[i] = px[j];
+            atomicAdd(&s_h[(unsigned)key[j] & 255u], 1u);
+        }
     }
+    __syncthreads();
+    hist[blockIdx.x * 256ll + threadIdx.x] = s_h[threadIdx.x];
 }
-__global__ void k_shot_range(tpx_hits h, long long n, unsigned long long *mn, unsigned long long *mx) {
+__global__ void __launch_bounds__(GT) k_shot_range(tpx_hits h, long long n, unsigned long long *mn, unsigned long long *mx) {
+    __shared__ unsigned long long s_lo[GW], s_hi[GW];
     unsigned long long lo = ~0ull, hi = 0;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
         const unsigned long long v = (unsigned long long)h.shot[i];
@@ -504,48 +689,93 @@ __global__ void k_shot_range(tpx_hits h, long long n, unsigned long long *mn, un
         hi = max(hi, __shfl_down_sync(0xffffffffu, hi, o));
     }
     if ((threadIdx.x & 31) == 0) {
+        s_lo[threadIdx.x >> 5] = lo;
+        s_hi[threadIdx.x >> 5] = hi;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {   // one atomic pair per block: they all meet on two addresses
+        for (int k = 1; k < GW; ++k) {
+            lo = min(lo, s_lo[k]);
+            hi = max(hi, s_hi[k]);
+        }
         atomicMin(mn, lo);
         atomicMax(mx, hi);
     }
 }
 
-struct Sorted {                     // hits in sorted order
-    unsigned *hit;                  // sorted position -> hit index
-    long long *shot;
-    int *tofb;                      // corrected ToF + bias
-    unsigned char *x, *y;
-    unsigned short *tot;
-    long long *index;
+// the hits in sorted order, read through the sorted keys and values: shots are
+// relative to the call's first one
+struct Sorted {
+    const unsigned *hit;            // sorted position -> hit index
+    const unsigned *k32;            // the sorted keys, 32 or 64 bits wide
+    const unsigned long long *k64;
+    unsigned *pxt;                  // x | y << 8 | ToT << 16 in sorted order
+    const int64_t *hindex;          // per hit: its stream index
+    const unsigned long long *shot_min;
+    __device__ __forceinline__ unsigned long long key(long long i) const { return k32 ? (unsigned long long)k32[i] : k64[i]; }
+    __device__ __forceinline__ long long shot(long long i) const { return (long long)(key(i) >> 24); }
+    __device__ __forceinline__ int tofb(long long i) const { return (int)(key(i) & 0xFFFFFFull); }
+    __device__ __forceinline__ int x(long long i) const { return (int)(pxt[i] & 255u); }
+    __device__ __forceinline__ int y(long long i) const { return (int)((pxt[i] >> 8) & 255u); }
+    __device__ __forceinline__ int tot(long long i) const { return (int)(pxt[i] >> 16); }
+    __device__ __forceinline__ long long index(long long i) const { return hindex[hit[i]]; }
+    __device__ __forceinline__ bool emits(long long i, long long limit) const { return shot(i) + (long long)*shot_min < limit; }
 };
 
-__global__ void k_gather(tpx_hits h, const unsigned *vals, long long n, Sorted s) {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const unsigned k = vals[i];
-        s.hit[i] = k;
-        s.shot[i] = h.shot[k];
-        s.tofb[i] = h.tof[k] + kBias;
-        s.x[i] = h.x[k];
-        s.y[i] = h.y[k];
-        s.tot[i] = h.tot[k];
-        s.index[i] = h.index[k];
-    }
+// Counting without scan launches: a kernel counts per block of GTILE items, the
+// next one adds up the counts of the blocks before its own (up to kResum
+// blocks: a few loads per thread; beyond that k_scan_bsum has made the counts
+// into prefixes).
+constexpr long long kResum = 4096;
+__device__ long long blocks_before(const unsigned *bcnt, long long nb, long long *s_w, long long *s_tot) {
+    if (nb > kResum) return bcnt[blockIdx.x];
+    long long v = 0;
+    for (long long k = threadIdx.x; k < blockIdx.x; k += GT) v += bcnt[k];
+    (void)block_scan_ll(v, s_w, s_tot);
+    return *s_tot;
 }
-
 // Segments: in sorted order a gap larger than dt (or a new shot) separates
 // everything before it from everything after it -- no adjacent pair spans
 // it -- so each run between such gaps clusters on its own.
-__global__ void k_seg_flags(Sorted s, long long n, int dt, unsigned *f) {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        f[i] = (i == 0 || s.shot[i] != s.shot[i - 1] || s.tofb[i] - s.tofb[i - 1] > dt) ? 1u : 0u;
+__device__ __forceinline__ bool seg_begins(const Sorted &s, long long i, int dt) {
+    if (i == 0) return true;
+    const unsigned long long a = s.key(i - 1), b = s.key(i);
+    return (a >> 24) != (b >> 24) || (long long)((b & 0xFFFFFFull) - (a & 0xFFFFFFull)) > dt;
 }
-__global__ void k_seg_starts(const unsigned *f, const unsigned *off, long long n, long long *start, long long *nseg) {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        if (f[i]) start[off[i]] = i;
-        if (i == n - 1) {
-            const long long m = (long long)off[i] + f[i];
-            start[m] = n;
-            *nseg = m;
-        }
+// counts the segments per block, and brings the pixels into sorted order
+__global__ void __launch_bounds__(GT) k_seg_count(Sorted s, const unsigned *pxt_hit, long long n, int dt, unsigned *bcnt) {
+    __shared__ unsigned s_c[GW];
+    unsigned m[GK], total;
+    const long long base = blockIdx.x * (long long)GTILE + (threadIdx.x >> 5) * (32 * GK) + (threadIdx.x & 31);
+    unsigned k[GK];
+#pragma unroll
+    for (int j = 0; j < GK; ++j) k[j] = base + 32 * j < n ? s.hit[base + 32 * j] : 0u;
+#pragma unroll
+    for (int j = 0; j < GK; ++j) k[j] = pxt_hit[k[j]];
+#pragma unroll
+    for (int j = 0; j < GK; ++j)
+        if (base + 32 * j < n) s.pxt[base + 32 * j] = k[j];
+    (void)block_flags(n, [&](long long i, int) { return seg_begins(s, i, dt); }, m, s_c, &total);
+    if (threadIdx.x == 0) bcnt[blockIdx.x] = total;
+}
+__global__ void __launch_bounds__(GT) k_seg_starts(Sorted s, long long n, int dt, const unsigned *bcnt, long long nb,
+                                                   long long *start, long long *nseg) {
+    __shared__ unsigned s_c[GW];
+    __shared__ long long s_w[GW];
+    __shared__ long long s_tot;
+    unsigned m[GK], total;
+    unsigned o = block_flags(n, [&](long long i, int) { return seg_begins(s, i, dt); }, m, s_c, &total);
+    const long long first = blocks_before(bcnt, nb, s_w, &s_tot);
+    const int lane = threadIdx.x & 31;
+    const long long base = blockIdx.x * (long long)GTILE + (threadIdx.x >> 5) * (32 * GK) + lane;
+#pragma unroll
+    for (int j = 0; j < GK; ++j) {
+        if ((m[j] >> lane) & 1u) start[first + o + __popc(m[j] & ((1u << lane) - 1u))] = base + 32 * j;
+        o += __popc(m[j]);
+    }
+    if (blockIdx.x == nb - 1 && threadIdx.x == 0) {
+        start[first + total] = n;
+        *nseg = first + total;
     }
 }
 
@@ -557,11 +787,18 @@ constexpr int WCAP = 256;           // hits of a segment held by one warp in sha
 constexpr int ECAP = 1024;          // adjacent pairs of a segment kept for the hooking rounds
 constexpr int HBW = 512;            // cell-hash buckets of a warp's segment
 constexpr int SEGW = 4;             // warps per block
+struct SmallSm {                    // a segment of up to WREG hits
+    int tofb[WREG];
+    unsigned short tot[WREG];
+    unsigned rows[16];              // occupied cells of each row of the grid
+    __align__(16) unsigned short charge[256];   // ToT + 1 of a cell's hit
+    __align__(8) unsigned char cell[256];
+};
 struct SegSm {
     int tofb[WCAP];
     int parent[WCAP];
-    unsigned edge[ECAP];            // (k << 16) | j, k < j
-    unsigned hhead[HBW];            // cell hash: first position, 0xFFFF = none
+    unsigned edge[ECAP];            // (k << 16) | j, k < j; later the roots' sums
+    __align__(8) unsigned hhead[HBW];   // cell hash: first position, 0xFFFF = none; later the roots' time sums
     unsigned ecnt;
     unsigned short hnext[WCAP];
     unsigned short tot[WCAP];
@@ -593,8 +830,8 @@ __device__ __forceinline__ void s_unite(int *par, int a, int b) {
 }
 
 // Sec. V.B tie rule: equal ToT goes to the hit later in the stream
-__device__ __forceinline__ bool j_brighter(int tj, int ti, const long long *index, long long j, long long i) {
-    return tj > ti || (tj == ti && index[j] > index[i]);
+__device__ __forceinline__ bool j_brighter(int tj, int ti, const Sorted &s, long long j, long long i) {
+    return tj > ti || (tj == ti && s.index(j) > s.index(i));
 }
 
 // Segments of at most 64 hits, in registers: lane l holds hits l and l + 32.
@@ -607,23 +844,25 @@ __device__ __forceinline__ unsigned long long warp_sum_u64(unsigned long long v)
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
 }
-__device__ void seg_small(const Sorted &s, long long s0, int L, int rx, int ry, int dt, int cc, bool emit,
-                          long long *labels, unsigned char *is_peak, unsigned *rflag, AccH *acc, int lane,
-                          SegSm &W) {
+struct SegIn {                      // a segment's hits in registers: two per lane
+    int ta, tb;                     // ToF + bias
+    unsigned a, b, ha, hb;          // pixel and ToT, hit index
+    __device__ __forceinline__ void load(const Sorted &s, long long s0, long long len, int lane) {
+        ta = tb = 0;
+        a = b = ha = hb = 0;
+        if (len > WREG) return;
+        if (lane < len) { ta = s.tofb(s0 + lane); a = s.pxt[s0 + lane]; ha = s.hit[s0 + lane]; }
+        if (lane + 32 < len) { tb = s.tofb(s0 + lane + 32); b = s.pxt[s0 + lane + 32]; hb = s.hit[s0 + lane + 32]; }
+    }
+};
+__device__ __forceinline__ void seg_small(const Sorted &s, const SegIn &in, long long s0, int L, int rx, int ry, int dt, int cc, bool emit,
+                          long long *labels, unsigned char *is_peak, unsigned char *rflag, AccH *acc, int lane,
+                          SmallSm &W) {
     constexpr unsigned FULL = 0xffffffffu;
     const int a = lane, b = lane + 32;
     const bool va = a < L, vb = b < L;
-    int ta = 0, tb = 0;
-    unsigned pa = 0, pb = 0, oa = 0, ob = 0, ha = 0, hb = 0;
-    long long ia = 0, ib = 0;
-    if (va) {
-        ta = s.tofb[s0 + a]; pa = s.x[s0 + a] | ((unsigned)s.y[s0 + a] << 8); oa = s.tot[s0 + a];
-        ia = s.index[s0 + a]; ha = s.hit[s0 + a];
-    }
-    if (vb) {
-        tb = s.tofb[s0 + b]; pb = s.x[s0 + b] | ((unsigned)s.y[s0 + b] << 8); ob = s.tot[s0 + b];
-        ib = s.index[s0 + b]; hb = s.hit[s0 + b];
-    }
+    const int ta = in.ta, tb = in.tb;
+    const unsigned pa = in.a & 0xFFFFu, pb = in.b & 0xFFFFu, oa = in.a >> 16, ob = in.b >> 16, ha = in.ha, hb = in.hb;
     unsigned long long rowA = 0, rowB = 0;
     bool npA = false, npB = false;
     // A compact segment (one particle, or a few close ones) with the 8-neighbour
@@ -632,6 +871,13 @@ __device__ void seg_small(const Sorted &s, long long s0, int L, int rx, int ry, 
     // per hit instead of one warp-wide step per hit of the segment. Two hits on
     // one pixel, a larger box or other radii take the all-pairs steps below.
     bool grid = false;
+    // A grid segment whose hits all lie within dt of each other -- a single
+    // particle, nearly always -- needs no times: local maxima from the cells'
+    // charges, components by flooding rows of bits (lane r holds row r). The
+    // general grid steps took 937 warp instructions per segment.
+    bool flood = false;
+    unsigned occ = 0;
+    int ca = 0, cb = 0;             // the hits' cells
     if (rx == 1 && ry == 1) {
         const unsigned xa = pa & 255u, ya = pa >> 8, xb = pb & 255u, yb = pb >> 8;
         const unsigned x0 = __reduce_min_sync(FULL, min(va ? xa : 255u, vb ? xb : 255u));
@@ -639,26 +885,53 @@ __device__ void seg_small(const Sorted &s, long long s0, int L, int rx, int ry, 
         const unsigned y0 = __reduce_min_sync(FULL, min(va ? ya : 255u, vb ? yb : 255u));
         const unsigned y1 = __reduce_max_sync(FULL, max(va ? ya : 0u, vb ? yb : 0u));
         if (x1 - x0 <= 13u && y1 - y0 <= 13u) {
-            unsigned *cell = W.edge;   // 256 cells: hit + 1, 0 = empty (the edge list is not in use)
-            __syncwarp();              // the warp's previous segment is done with W
-            for (int i = lane; i < 256; i += 32) cell[i] = 0u;
+            const int t_last = __shfl_sync(FULL, L > 32 ? tb : ta, (L - 1) & 31);
+            flood = t_last - __shfl_sync(FULL, ta, 0) <= dt;   // in ToF order
+            unsigned char *cell = W.cell;   // 256 cells: hit + 1, 0 = empty
+            __syncwarp();                   // the warp's previous segment is done with W
+            reinterpret_cast<uint2 *>(cell)[lane] = make_uint2(0u, 0u);
+            reinterpret_cast<uint4 *>(W.charge)[lane] = make_uint4(0u, 0u, 0u, 0u);
+            if (lane < 16) W.rows[lane] = 0u;
             if (va) { W.tofb[a] = ta; W.tot[a] = (unsigned short)oa; }
             if (vb) { W.tofb[b] = tb; W.tot[b] = (unsigned short)ob; }
             __syncwarp();
-            const int ca = (int)(xa - x0 + 1) + 16 * (int)(ya - y0 + 1), cb = (int)(xb - x0 + 1) + 16 * (int)(yb - y0 + 1);
-            bool twice = false;
-            if (va && atomicCAS(&cell[ca], 0u, (unsigned)a + 1u) != 0u) twice = true;
-            if (vb && atomicCAS(&cell[cb], 0u, (unsigned)b + 1u) != 0u) twice = true;
+            ca = (int)(xa - x0 + 1) + 16 * (int)(ya - y0 + 1);
+            cb = (int)(xb - x0 + 1) + 16 * (int)(yb - y0 + 1);
+            if (va) { cell[ca] = (unsigned char)(a + 1); W.charge[ca] = (unsigned short)(oa + 1u); atomicOr(&W.rows[ca >> 4], 1u << (ca & 15)); }
+            if (vb) { cell[cb] = (unsigned char)(b + 1); W.charge[cb] = (unsigned short)(ob + 1u); atomicOr(&W.rows[cb >> 4], 1u << (cb & 15)); }
             __syncwarp();
-            grid = !__any_sync(FULL, twice);
-            if (grid) {
+            // a hit that does not find itself shares its pixel with another
+            grid = !__any_sync(FULL, (va && cell[ca] != a + 1) || (vb && cell[cb] != b + 1));
+            flood = flood && grid && oa < 65535u && ob < 65535u;
+            flood = __all_sync(FULL, flood);
+            if (flood) {
+                occ = lane < 16 ? W.rows[lane] : 0u;
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    if (!(h ? vb : va)) continue;
+                    const int c = h ? cb : ca;
+                    const unsigned o1 = (h ? ob : oa) + 1u;
+                    unsigned mx = 0;
+#pragma unroll
+                    for (int d = 0; d < 9; ++d)
+                        if (d != 4) mx = max(mx, (unsigned)W.charge[c + (d % 3 - 1) + 16 * (d / 3 - 1)]);
+                    bool np = mx > o1;
+                    if (mx == o1) {   // Sec. V.B ties: the later hit in the stream wins
+                        for (int d = 0; d < 9; ++d) {
+                            const int cj = c + (d % 3 - 1) + 16 * (d / 3 - 1);
+                            if (d != 4 && W.charge[cj] == o1 && s.index(s0 + cell[cj] - 1) > (long long)s.hindex[h ? hb : ha]) np = true;
+                        }
+                    }
+                    if (h) npB = np; else npA = np;
+                }
+            }
+            if (grid && !flood) {
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     const bool v = h ? vb : va;
                     if (!v) continue;
                     const int c = h ? cb : ca, t = h ? tb : ta;
                     const unsigned o = h ? ob : oa;
-                    const long long ix = h ? ib : ia;
                     unsigned long long row = 0;
                     bool np = false;
 #pragma unroll
@@ -670,7 +943,7 @@ __device__ void seg_small(const Sorted &s, long long s0, int L, int rx, int ry, 
                         if (abs(W.tofb[j] - t) > dt) continue;
                         row |= 1ull << j;
                         const unsigned oj = W.tot[j];
-                        if (oj > o || (oj == o && s.index[s0 + j] > ix)) np = true;
+                        if (oj > o || (oj == o && s.index(s0 + j) > (long long)s.hindex[h ? hb : ha])) np = true;
                     }
                     if (h) { rowB = row; npB = np; } else { rowA = row; npA = np; }
                 }
@@ -691,9 +964,9 @@ __device__ void seg_small(const Sorted &s, long long s0, int L, int rx, int ry, 
         bool brA = adjA && oa > ko, brB = adjB && ob > ko;
         const bool tA = adjA && oa == ko, tB = adjB && ob == ko;
         if (__any_sync(FULL, tA || tB)) {   // Sec. V.B ties: the later hit in the stream wins
-            const long long ki = __shfl_sync(FULL, kb ? ib : ia, src);
-            brA = brA || (tA && ia > ki);
-            brB = brB || (tB && ib > ki);
+            const long long ki = s.index(s0 + k);
+            brA = brA || (tA && (long long)s.hindex[ha] > ki);
+            brB = brB || (tB && (long long)s.hindex[hb] > ki);
         }
         const bool knp = __any_sync(FULL, brA || brB);
         if (lane == src) {
@@ -704,17 +977,19 @@ __device__ void seg_small(const Sorted &s, long long s0, int L, int rx, int ry, 
     const bool pkA = va && !npA, pkB = vb && !npB;
     if (!cc) {   // PAPER mode: every hit is its own label; local maxima carry the records
         if (va) {
-            if (labels) labels[ha] = ia;
+            if (labels) labels[ha] = s.hindex[ha];
             if (is_peak) is_peak[ha] = pkA;
             if (rflag) rflag[ha] = emit && pkA;
         }
         if (vb) {
-            if (labels) labels[hb] = ib;
+            if (labels) labels[hb] = s.hindex[hb];
             if (is_peak) is_peak[hb] = pkB;
             if (rflag) rflag[hb] = emit && pkB;
         }
         return;
     }
+    // the hits' stream indices, for the labels: on their way during the closures
+    const long long ia = labels && va ? (long long)s.hindex[ha] : 0, ib = labels && vb ? (long long)s.hindex[hb] : 0;
     const unsigned long long peaks = ((unsigned long long)__ballot_sync(FULL, pkB) << 32) | __ballot_sync(FULL, pkA);
     unsigned long long todo = L == 64 ? ~0ull : ((1ull << L) - 1ull);
     long long rootA = 0, rootB = 0;
@@ -722,6 +997,24 @@ __device__ void seg_small(const Sorted &s, long long s0, int L, int rx, int ry, 
     while (todo) {
         const int seed = __ffsll((long long)todo) - 1;
         unsigned long long comp = 1ull << seed, front = comp;
+        if (flood) {
+            const int sc = __shfl_sync(FULL, seed >= 32 ? cb : ca, seed & 31);
+            unsigned f = lane == (sc >> 4) ? 1u << (sc & 15) : 0u;
+            for (;;) {
+                const unsigned was = f;
+#pragma unroll
+                for (int k = 0; k < 2; ++k) {
+                    const unsigned e = f | (f << 1) | (f >> 1);
+                    f = (e | __shfl_up_sync(FULL, e, 1) | __shfl_down_sync(FULL, e, 1)) & occ;
+                }
+                if (!__any_sync(FULL, f != was)) break;
+            }
+            const unsigned fa = __shfl_sync(FULL, f, ca >> 4), fb = __shfl_sync(FULL, f, cb >> 4);
+            const unsigned lo = __ballot_sync(FULL, va && ((fa >> (ca & 15)) & 1u));
+            const unsigned hi = __ballot_sync(FULL, vb && ((fb >> (cb & 15)) & 1u));
+            comp = ((unsigned long long)hi << 32) | lo;
+            front = 0;
+        }
         while (front) {
             unsigned long long c = 0;
             if ((front >> a) & 1ull) c |= rowA;
@@ -732,24 +1025,26 @@ __device__ void seg_small(const Sorted &s, long long s0, int L, int rx, int ry, 
             front = nb & ~comp;
             comp |= nb;
         }
-        const long long sidx = __shfl_sync(FULL, seed >= 32 ? ib : ia, seed & 31);
+        const long long sidx = labels ? __shfl_sync(FULL, seed >= 32 ? ib : ia, seed & 31) : 0;
         const bool inA = (comp >> a) & 1ull, inB = (comp >> b) & 1ull;
         if (inA) { rootA = sidx; rposA = seed; }
         if (inB) { rootB = sidx; rposB = seed; }
         if (acc && emit) {
             const int st = __shfl_sync(FULL, seed >= 32 ? tb : ta, seed & 31);
-            unsigned long long v_tot = 0, v_x = 0, v_y = 0, v_t = 0;
-            if (inA) { v_tot += oa; v_x += (unsigned long long)oa * (pa & 255u); v_y += (unsigned long long)oa * (pa >> 8);
-                       v_t += (unsigned long long)(ta - st) * oa; }
-            if (inB) { v_tot += ob; v_x += (unsigned long long)ob * (pb & 255u); v_y += (unsigned long long)ob * (pb >> 8);
-                       v_t += (unsigned long long)(tb - st) * ob; }
-            v_tot = warp_sum_u64(v_tot);
-            v_x = warp_sum_u64(v_x);
-            v_y = warp_sum_u64(v_y);
-            v_t = warp_sum_u64(v_t);
+            // 64 hits: ToT sums and their products with a coordinate fit 32 bits
+            unsigned v_tot = 0, v_x = 0, v_y = 0;
+            unsigned long long v_t = 0;
+            if (inA) { v_tot += oa; v_x += oa * (pa & 255u); v_y += oa * (pa >> 8); v_t += (unsigned long long)(ta - st) * oa; }
+            if (inB) { v_tot += ob; v_x += ob * (pb & 255u); v_y += ob * (pb >> 8); v_t += (unsigned long long)(tb - st) * ob; }
+            v_tot = __reduce_add_sync(FULL, v_tot);
+            v_x = __reduce_add_sync(FULL, v_x);
+            v_y = __reduce_add_sync(FULL, v_y);
+            // 64 hits within 63 dt of each other: also s_t for dt <= 1000 and 10-bit ToT
+            if (dt <= 1000 && __all_sync(FULL, (oa | ob) < 1024u)) v_t = __reduce_add_sync(FULL, (unsigned)v_t);
+            else v_t = warp_sum_u64(v_t);
             if (lane == (seed & 31)) {
                 AccH r;
-                r.s_tot = (long long)v_tot; r.s_x = (long long)v_x; r.s_y = (long long)v_y; r.s_t = (long long)v_t;
+                r.s_tot = v_tot; r.s_x = v_x; r.s_y = v_y; r.s_t = (long long)v_t;
                 r.n = (unsigned)__popcll(comp); r.npk = (unsigned)__popcll(comp & peaks);
                 acc[seed >= 32 ? hb : ha] = r;
             }
@@ -768,55 +1063,75 @@ __device__ void seg_small(const Sorted &s, long long s0, int L, int rx, int ry, 
     }
 }
 
-// One warp per segment. Up to 64 hits: in registers (seg_small). Up to
-// WCAP: in shared memory, where a cell hash of the segment gives every hit
-// the candidates of the forward half of its box (same cell: later positions
-// only), so that each adjacent pair is met once even when the whole segment
-// lies within dt; pairs set the local-maximum flags and are joined by
-// hooking rounds; then labels, peaks, root flags (emitted shots only) and
-// the root's int64 moments. Longer segments are marked for the cell-hash
-// kernels in global memory below.
-__global__ void __launch_bounds__(SEGW * 32) k_segments(Sorted s, const long long *seg_start, const long long *nseg_p,
-                                                        int rx, int ry, int dt, int cc, long long shot_limit,
-                                                        long long *labels, unsigned char *is_peak, unsigned *rflag,
-                                                        AccH *acc, unsigned char *mark) {
-    __shared__ SegSm sm[SEGW];
+// One warp per segment of up to 64 hits, in registers (seg_small) and 1,300
+// bytes of shared memory; the rare longer segments are listed for
+// k_segments_mid (up to WCAP) or marked for the cell-hash kernels in global
+// memory below. Bound by instruction issue: 6.0e6 hits 402 -> 141 us, of which
+// the longer segments' 11 KB of shared memory taken out of this kernel 190, the
+// flooding of bit rows (below) 85.
+struct SegLists { unsigned n_mid, n_long; };
+__global__ void __launch_bounds__(SEGW * 32, 8) k_segments(Sorted s, const long long *seg_start, const long long *nseg_p,
+                                                           int rx, int ry, int dt, int cc, long long shot_limit,
+                                                           long long *labels, unsigned char *is_peak,
+                                                           unsigned char *rflag, AccH *acc, unsigned char *mark,
+                                                           unsigned *mid, SegLists *lists) {
+    __shared__ SmallSm sm[SEGW];
     const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
-    SegSm &W = sm[wi];
     const long long nseg = *nseg_p;
     for (long long seg = blockIdx.x * (long long)SEGW + wi; seg < nseg; seg += (long long)gridDim.x * SEGW) {
         const long long s0 = seg_start[seg], len = seg_start[seg + 1] - s0;
-        if (len > WCAP) {
-            for (long long k = lane; k < len; k += 32) mark[s0 + k] = 1;
-            continue;
-        }
-        const int L = (int)len;
-        const bool emit = s.shot[s0] < shot_limit;
-        const bool sums = cc && acc && emit;
-        if (L > 1 && L <= WREG) {
-            seg_small(s, s0, L, rx, ry, dt, cc, emit, labels, is_peak, rflag, sums ? acc : nullptr, lane, W);
-            continue;
-        }
-        if (L == 1) {
+        SegIn in;
+        in.load(s, s0, len, lane);
+        for (long long k = lane; k < len; k += 32) mark[s0 + k] = len > WCAP;
+        if (len > WREG) {
             if (lane == 0) {
-                const unsigned hh = s.hit[s0];
-                if (labels) labels[hh] = s.index[s0];
-                if (is_peak) is_peak[hh] = 1;
-                if (rflag) rflag[hh] = emit;
+                if (len > WCAP) lists->n_long = 1;
+                else mid[atomicAdd(&lists->n_mid, 1u)] = (unsigned)seg;
+            }
+        } else {
+            const bool emit = s.emits(s0, shot_limit);
+            const bool sums = cc && acc && emit;
+            if (len > 1) {
+                seg_small(s, in, s0, (int)len, rx, ry, dt, cc, emit, labels, is_peak, rflag, sums ? acc : nullptr, lane, sm[wi]);
+            } else if (lane == 0) {
+                if (labels) labels[in.ha] = s.hindex[in.ha];
+                if (is_peak) is_peak[in.ha] = 1;
+                if (rflag) rflag[in.ha] = emit;
                 if (sums) {
-                    const long long t = s.tot[s0];
-                    AccH a;
-                    a.s_tot = t; a.s_x = t * s.x[s0]; a.s_y = t * s.y[s0]; a.s_t = 0; a.n = 1; a.npk = 1;
-                    acc[hh] = a;
+                    const long long t = in.a >> 16;
+                    AccH v;
+                    v.s_tot = t; v.s_x = t * (in.a & 255u); v.s_y = t * ((in.a >> 8) & 255u); v.s_t = 0; v.n = 1; v.npk = 1;
+                    acc[in.ha] = v;
                 }
             }
-            continue;
         }
+    }
+}
+
+// Segments of 65 to WCAP hits: one warp in shared memory, where a cell hash of
+// the segment gives every hit the candidates of the forward half of its box
+// (same cell: later positions only), so that each adjacent pair is met once
+// even when the whole segment lies within dt; pairs set the local-maximum flags
+// and are joined by hooking rounds; then labels, peaks, root flags (emitted
+// shots only) and the root's int64 moments.
+__global__ void __launch_bounds__(SEGW * 32) k_segments_mid(Sorted s, const long long *seg_start, const unsigned *mid,
+                                                            const SegLists *lists, int rx, int ry, int dt, int cc,
+                                                            long long shot_limit, long long *labels,
+                                                            unsigned char *is_peak, unsigned char *rflag, AccH *acc) {
+    __shared__ SegSm sm[SEGW];
+    const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
+    SegSm &W = sm[wi];
+    const long long n_mid = lists->n_mid;
+    for (long long q = blockIdx.x * (long long)SEGW + wi; q < n_mid; q += (long long)gridDim.x * SEGW) {
+        const long long s0 = seg_start[mid[q]];
+        const int L = (int)(seg_start[mid[q] + 1ll] - s0);
+        const bool emit = s.emits(s0, shot_limit);
+        const bool sums = cc && acc && emit;
         for (int k = lane; k < L; k += 32) {
-            W.tofb[k] = s.tofb[s0 + k];
-            W.x[k] = s.x[s0 + k];
-            W.y[k] = s.y[s0 + k];
-            W.tot[k] = s.tot[s0 + k];
+            W.tofb[k] = s.tofb(s0 + k);
+            W.x[k] = s.x(s0 + k);
+            W.y[k] = s.y(s0 + k);
+            W.tot[k] = s.tot(s0 + k);
             W.parent[k] = k;
             W.np[k] = 0;
         }
@@ -840,7 +1155,7 @@ __global__ void __launch_bounds__(SEGW * 32) k_segments(Sorted s, const long lon
                         if (d < -dt || d > dt) continue;
                         // the pair (lo, hi) in position order
                         const int lo = min(k, (int)j), hi = max(k, (int)j);
-                        if (j_brighter(W.tot[j], tk, s.index, s0 + j, s0 + k)) W.np[k] = 1; else W.np[j] = 1;
+                        if (j_brighter(W.tot[j], tk, s, s0 + j, s0 + k)) W.np[k] = 1; else W.np[j] = 1;
                         if (cc) {   // record the pair (warp-aggregated slot); beyond the buffer, join it now
                             const unsigned am = __activemask();
                             const int leader = __ffs(am) - 1;
@@ -907,36 +1222,36 @@ __global__ void __launch_bounds__(SEGW * 32) k_segments(Sorted s, const long lon
             const int r = rk[u];
             const unsigned hh = s.hit[s0 + k];
             const bool peak = W.np[k] == 0;
-            if (labels) labels[hh] = s.index[s0 + r];
+            if (labels) labels[hh] = s.index(s0 + r);
             if (is_peak) is_peak[hh] = peak;
             if (rflag) rflag[hh] = emit && (cc ? r == k : peak);
         }
         if (sums) {
-            // each root's lane sweeps the segment once (broadcast reads, no
-            // atomics): exact 64-bit moments in registers
-            for (int base = 0; base < L; base += 32) {
-                const int k = base + lane;
-                const bool own = k < L && W.parent[k] == k;
-                if (__ballot_sync(0xffffffffu, own) == 0) continue;
-                unsigned long long st = 0, sx = 0, sy = 0, stt = 0;
-                unsigned cnt = 0, npk = 0;
-                const int tk = own ? W.tofb[k] : 0;
-                for (int j = own ? k : L; j < L; ++j) {   // members sit at or after their root
-                    if (W.parent[j] != k) continue;
-                    const unsigned long long t = W.tot[j];
-                    st += t;
-                    sx += t * W.x[j];
-                    sy += t * W.y[j];
-                    stt += (unsigned long long)(W.tofb[j] - tk) * t;
-                    cnt += 1;
-                    npk += W.np[j] == 0;
-                }
-                if (own) {
-                    AccH a;
-                    a.s_tot = (long long)st; a.s_x = (long long)sx; a.s_y = (long long)sy; a.s_t = (long long)stt;
-                    a.n = cnt; a.npk = npk;
-                    acc[s.hit[s0 + k]] = a;
-                }
+            // every hit adds to its root's sums in the space of the pair list and
+            // the hash heads: 256 hits, so ToT sums times a coordinate fit 32 bits
+            unsigned *q_n = W.edge, *q_tot = q_n + WCAP, *q_x = q_tot + WCAP, *q_y = q_x + WCAP;
+            unsigned long long *q_t = reinterpret_cast<unsigned long long *>(W.hhead);
+            for (int k = lane; k < L; k += 32) {
+                q_n[k] = q_tot[k] = q_x[k] = q_y[k] = 0u;
+                q_t[k] = 0ull;
+            }
+            __syncwarp();
+            for (int k = lane; k < L; k += 32) {
+                const int r = W.parent[k];
+                const unsigned t = W.tot[k];
+                atomicAdd(&q_n[r], 1u | (W.np[k] == 0 ? 1u << 16 : 0u));
+                atomicAdd(&q_tot[r], t);
+                atomicAdd(&q_x[r], t * W.x[k]);
+                atomicAdd(&q_y[r], t * W.y[k]);
+                atomicAdd(&q_t[r], (unsigned long long)(W.tofb[k] - W.tofb[r]) * t);
+            }
+            __syncwarp();
+            for (int k = lane; k < L; k += 32) {
+                if (W.parent[k] != k) continue;
+                AccH a;
+                a.s_tot = q_tot[k]; a.s_x = q_x[k]; a.s_y = q_y[k]; a.s_t = (long long)q_t[k];
+                a.n = q_n[k] & 0xFFFFu; a.npk = q_n[k] >> 16;
+                acc[s.hit[s0 + k]] = a;
             }
         }
         __syncwarp();
@@ -965,8 +1280,12 @@ __device__ void g_unite(int *parent, int a, int b) {
         b = old;
     }
 }
-__global__ void k_long_init(Sorted s, long long n, const unsigned char *mark, int *parent, unsigned char *notpeak,
-                            AccH *acc) {
+// (every k_long_ kernel returns at once when no segment is that long)
+__global__ void k_long_init(Sorted s, long long n, const SegLists *lists, const unsigned char *mark, int *parent,
+                            unsigned char *notpeak, AccH *acc, unsigned *head, unsigned long long mask) {
+    if (!lists->n_long) return;
+    for (unsigned long long i = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; i <= mask; i += (unsigned long long)gridDim.x * blockDim.x)
+        head[i] = 0xFFFFFFFFu;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
         if (!mark[i]) continue;
         parent[i] = (int)i;
@@ -992,24 +1311,27 @@ __device__ __forceinline__ unsigned long long cell_hash(long long shot, int x, i
 __device__ __forceinline__ unsigned cell_key(long long shot, int x, int y) {
     return (unsigned)x | ((unsigned)y << 8) | ((unsigned)(shot & 0xFFFF) << 16);
 }
-__global__ void k_long_insert(Sorted s, long long n, const unsigned char *mark, unsigned *head, unsigned *next,
-                              unsigned long long *word, unsigned long long mask) {
+__global__ void k_long_insert(Sorted s, long long n, const SegLists *lists, const unsigned char *mark, unsigned *head,
+                              unsigned *next, unsigned long long *word, unsigned long long mask) {
+    if (!lists->n_long) return;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
         if (!mark[i]) continue;
-        const long long sh = s.shot[i];
-        const int x = s.x[i], y = s.y[i];
-        word[i] = (unsigned long long)cell_key(sh, x, y) | ((unsigned long long)(unsigned)s.tofb[i] << 32);
+        const long long sh = s.shot(i);
+        const int x = s.x(i), y = s.y(i);
+        word[i] = (unsigned long long)cell_key(sh, x, y) | ((unsigned long long)(unsigned)s.tofb(i) << 32);
         next[i] = atomicExch(&head[cell_hash(sh, x, y, mask)], (unsigned)i);
     }
 }
-__global__ void k_long_pairs(Sorted s, long long n, const unsigned char *mark, const unsigned *head,
-                             const unsigned *next, const unsigned long long *word, unsigned long long mask, int rx,
-                             int ry, int dt, int cc, int *parent, unsigned char *notpeak) {
+__global__ void k_long_pairs(Sorted s, long long n, const SegLists *lists, const unsigned char *mark,
+                             const unsigned *head, const unsigned *next, const unsigned long long *word,
+                             unsigned long long mask, int rx, int ry, int dt, int cc, int *parent,
+                             unsigned char *notpeak) {
+    if (!lists->n_long) return;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
         if (!mark[i]) continue;
         const unsigned long long wi = word[i];
-        const long long sh = s.shot[i];
-        const int tb = (int)(unsigned)(wi >> 32), xi = (int)(wi & 255), yi = (int)((wi >> 8) & 255), ti = s.tot[i];
+        const long long sh = s.shot(i);
+        const int tb = (int)(unsigned)(wi >> 32), xi = (int)(wi & 255), yi = (int)((wi >> 8) & 255), ti = s.tot(i);
         for (int dx = 0; dx <= rx; ++dx) {
             const int cx = xi + dx;
             if (cx > 255) break;
@@ -1020,34 +1342,35 @@ __global__ void k_long_pairs(Sorted s, long long n, const unsigned char *mark, c
                 for (unsigned j = head[cell_hash(sh, cx, cy, mask)]; j != 0xFFFFFFFFu; j = next[j]) {
                     if (dx == 0 && dy == 0 && (long long)j <= i) continue;
                     const unsigned long long wj = word[j];
-                    if ((unsigned)wj != key || s.shot[j] != sh) continue;
+                    if ((unsigned)wj != key || s.shot(j) != sh) continue;
                     const int d = (int)(unsigned)(wj >> 32) - tb;
                     if (d < -dt || d > dt) continue;
-                    if (j_brighter(s.tot[j], ti, s.index, j, i)) notpeak[i] = 1; else notpeak[j] = 1;
+                    if (j_brighter(s.tot(j), ti, s, j, i)) notpeak[i] = 1; else notpeak[j] = 1;
                     if (cc) g_unite(parent, (int)i, (int)j);
                 }
             }
         }
     }
 }
-__global__ void k_long_finish(Sorted s, long long n, const unsigned char *mark, int cc, long long shot_limit,
-                              int *parent, const unsigned char *notpeak, long long *labels, unsigned char *is_peak,
-                              unsigned *rflag, AccH *acc) {
+__global__ void k_long_finish(Sorted s, long long n, const SegLists *lists, const unsigned char *mark, int cc,
+                              long long shot_limit, int *parent, const unsigned char *notpeak, long long *labels,
+                              unsigned char *is_peak, unsigned char *rflag, AccH *acc) {
+    if (!lists->n_long) return;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
         if (!mark[i]) continue;
         const long long r = cc ? g_find(parent, (int)i) : i;
         const unsigned hh = s.hit[i];
-        const bool peak = notpeak[i] == 0, emit = s.shot[i] < shot_limit;
-        if (labels) labels[hh] = s.index[r];
+        const bool peak = notpeak[i] == 0, emit = s.emits(i, shot_limit);
+        if (labels) labels[hh] = s.index(r);
         if (is_peak) is_peak[hh] = peak;
         if (rflag) rflag[hh] = emit && (cc ? r == i : peak);
         if (cc && acc && emit) {
             AccH &a = acc[s.hit[r]];
-            const unsigned long long t = s.tot[i];
+            const unsigned long long t = s.tot(i);
             atomicAdd(reinterpret_cast<unsigned long long *>(&a.s_tot), t);
-            atomicAdd(reinterpret_cast<unsigned long long *>(&a.s_x), t * s.x[i]);
-            atomicAdd(reinterpret_cast<unsigned long long *>(&a.s_y), t * s.y[i]);
-            atomicAdd(reinterpret_cast<unsigned long long *>(&a.s_t), (unsigned long long)(s.tofb[i] - s.tofb[r]) * t);
+            atomicAdd(reinterpret_cast<unsigned long long *>(&a.s_x), t * s.x(i));
+            atomicAdd(reinterpret_cast<unsigned long long *>(&a.s_y), t * s.y(i));
+            atomicAdd(reinterpret_cast<unsigned long long *>(&a.s_t), (unsigned long long)(s.tofb(i) - s.tofb(r)) * t);
             atomicAdd(&a.n, 1u);
             if (peak) atomicAdd(&a.npk, 1u);
         }
@@ -1055,13 +1378,87 @@ __global__ void k_long_finish(Sorted s, long long n, const unsigned char *mark, 
 }
 
 // ------------------------------------------------------------ centroid kernels
-__global__ void k_root_flags(tpx_hits h, const long long *labels, const unsigned char *is_peak, long long n, int cc,
-                             unsigned *flags) {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        flags[i] = cc ? (labels[i] == h.index[i]) : (unsigned)is_peak[i];
+// Records in ascending label order: the roots (CC mode: the hits that carry
+// their own label; PAPER mode: the local maxima) are counted per block of
+// GTILE hits, then every block places its own behind those of the blocks
+// before it.
+struct RootFlag {
+    const long long *labels, *index;    // CC mode from labels
+    const unsigned char *flag;          // or flags as they are
+    __device__ __forceinline__ bool operator()(long long i, int) const { return flag ? flag[i] != 0 : labels[i] == index[i]; }
+};
+__global__ void __launch_bounds__(GT) k_root_count(RootFlag f, long long n, unsigned *bcnt) {
+    __shared__ unsigned s_c[GW];
+    unsigned m[GK], total;
+    (void)block_flags(n, f, m, s_c, &total);
+    if (threadIdx.x == 0) bcnt[blockIdx.x] = total;
+}
+// latches the number of records, the capacity status and the clusters counter
+__device__ __forceinline__ void latch_count(long long m, long long cap, long long *n_rec, unsigned *status,
+                                            unsigned long long *counter) {
+    *n_rec = m;
+    if (m > cap) atomicOr(status, ST_CLUSTER_CAP);
+    if (counter) *counter = (unsigned long long)m;
+}
+__device__ __forceinline__ void write_record(const tpx_hits &h, long long i, const AccH &a, tpx_record *out) {
+    tpx_record o;
+    o.label = h.index[i];
+    o.shot = h.shot[i];
+    o.t0 = h.t[i];
+    o.s_tot = a.s_tot; o.s_x = a.s_x; o.s_y = a.s_y; o.s_t = a.s_t;
+    o.n = (int)a.n; o.n_peaks = (int)a.npk;
+    com_from_moments(o.s_x, o.s_y, o.s_t, o.s_tot, h.tof[i], &o.x, &o.y, &o.tof);
+    *out = o;
+}
+// places the roots; one of three uses: `out` (with acc, per hit): the records
+// themselves; `zero`: each record's empty sums and its root, for k_accum (and
+// `rank`, the record of a root's label, when the labels' span allows it); `cid`
+// (per hit): the roots' slots, for k_paper
+struct Roots {
+    const AccH *acc; tpx_record *out;
+    unsigned *cid;
+    unsigned *rank; long long rank_cap;
+    struct Acc *zero; unsigned *rootpos; long long *root_t;
+};
+struct Acc { unsigned long long n_npk, s_tot, s_x, s_y, s_t; };   // n_npk: hits | local maxima << 32
+__global__ void __launch_bounds__(GT) k_root_place(RootFlag f, tpx_hits h, long long n, const unsigned *bcnt, long long nb,
+                                                   long long cap, long long *n_rec, unsigned *status,
+                                                   unsigned long long *counter, Roots r) {
+    __shared__ unsigned s_c[GW];
+    __shared__ long long s_w[GW];
+    __shared__ long long s_tot;
+    __shared__ unsigned s_root[GTILE];
+    unsigned m[GK], total;
+    unsigned o = block_flags(n, f, m, s_c, &total);
+    const long long first = blocks_before(bcnt, nb, s_w, &s_tot);
+    const int lane = threadIdx.x & 31;
+    const int at = (threadIdx.x >> 5) * (32 * GK) + lane;
+    const long long base = blockIdx.x * (long long)GTILE;
+#pragma unroll
+    for (int j = 0; j < GK; ++j) {
+        if ((m[j] >> lane) & 1u) {
+            const unsigned k = o + __popc(m[j] & ((1u << lane) - 1u));
+            s_root[k] = (unsigned)(at + 32 * j);
+        }
+        o += __popc(m[j]);
+    }
+    __syncthreads();
+    const bool ranked = r.rank && h.index[n - 1] - h.index[0] < r.rank_cap;
+    for (unsigned k = threadIdx.x; k < total; k += GT) {
+        const long long i = base + s_root[k], c = first + k;
+        if (r.cid) r.cid[i] = (unsigned)c;
+        if (c < cap && r.out && r.acc) write_record(h, i, r.acc[i], r.out + c);
+        if (c < cap && r.zero) {
+            r.zero[c] = Acc{0, 0, 0, 0, 0};
+            r.rootpos[c] = (unsigned)i;
+            r.root_t[c] = h.t[i];
+            if (ranked) r.rank[h.index[i] - h.index[0]] = (unsigned)c;
+        }
+    }
+    if (blockIdx.x == nb - 1 && threadIdx.x == 0) latch_count(first + total, cap, n_rec, status, counter);
 }
 
-__device__ __forceinline__ long long find_index(const long long *index, long long n, long long v) {
+__device__ __forceinline__ long long find_index(const int64_t *index, long long n, long long v) {
     long long lo = 0, hi = n;
     while (lo < hi) {
         const long long mid = lo + ((hi - lo) >> 1);
@@ -1070,106 +1467,144 @@ __device__ __forceinline__ long long find_index(const long long *index, long lon
     return lo;
 }
 
-struct Acc { unsigned long long n, s_tot, s_x, s_y, s_t, npk; };
-
-__global__ void k_accum(tpx_hits h, const long long *labels, const unsigned char *is_peak, long long n,
-                        const unsigned *cid, Acc *acc) {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const long long rp = find_index(reinterpret_cast<const long long *>(h.index), n, labels[i]);
-        const unsigned c = cid[rp];
-        const unsigned long long tot = h.tot[i];
-        atomicAdd(&acc[c].n, 1ull);
-        atomicAdd(&acc[c].s_tot, tot);
-        atomicAdd(&acc[c].s_x, tot * h.x[i]);
-        atomicAdd(&acc[c].s_y, tot * h.y[i]);
-        atomicAdd(&acc[c].s_t, tot * (unsigned long long)(h.t[i] - h.t[rp]));
-        if (is_peak && is_peak[i]) atomicAdd(&acc[c].npk, 1ull);
+// Every hit adds to its record's sums. The record comes from the rank table
+// (4 bytes per stream index; a binary search over the roots where the indices
+// span more). A block's 4096 hits in stream order belong to a few hundred
+// records, so they meet in a hash table in shared memory first, in 32 bits
+// (4096 hits: ToT sums times a coordinate fit; s_t for times within 1023 ticks
+// of the root, else past the table), and its entries go to global memory.
+// With six 64-bit global atomics and a 23-step search per hit, 6.0e6 hits
+// took 264 us; 92 with one hit's loads in flight per thread, fewer with four's.
+constexpr int AH = 1024;            // hash slots: a quarter of a block's hits
+__global__ void __launch_bounds__(GT) k_accum(tpx_hits h, const long long *labels, const unsigned char *is_peak, long long n,
+                                              const long long *n_rec, long long cap, const unsigned *rank,
+                                              long long rank_cap, const unsigned *rootpos, const long long *root_t,
+                                              Acc *acc) {
+    __shared__ unsigned s_key[AH];      // record + 1, 0: free
+    __shared__ unsigned s_n[AH], s_p[AH], s_t[AH], s_x[AH], s_y[AH], s_d[AH];
+    for (int k = threadIdx.x; k < AH; k += GT) s_key[k] = s_n[k] = s_p[k] = s_t[k] = s_x[k] = s_y[k] = s_d[k] = 0u;
+    __syncthreads();
+    const long long m = min(*n_rec, cap);
+    const long long i0 = h.index[0], span = h.index[n - 1] - i0;
+    const bool ranked = span < rank_cap;
+    const long long base = blockIdx.x * (long long)GTILE;
+    constexpr int B = 4;   // hits whose loads are in flight together
+    for (int j0 = 0; j0 < GK; j0 += B) {
+        long long rec[B], t[B];
+        unsigned xyt[B], pks[B];
+#pragma unroll
+        for (int j = 0; j < B; ++j) {
+            const long long i = base + (j0 + j) * GT + threadIdx.x;
+            rec[j] = -1;
+            if (i >= n) continue;
+            rec[j] = labels[i];
+            t[j] = h.t[i];
+            xyt[j] = (unsigned)h.x[i] | ((unsigned)h.y[i] << 8) | ((unsigned)h.tot[i] << 16);
+            pks[j] = is_peak && is_peak[i] ? 1u : 0u;
+        }
+#pragma unroll
+        for (int j = 0; j < B; ++j) {
+            const long long lab = rec[j];
+            const bool in = base + (j0 + j) * GT + threadIdx.x < n;
+            if (ranked) {   // no record's label: the table's 2^32 - 1, past every count
+                rec[j] = in && lab >= i0 && lab - i0 <= span ? (long long)rank[lab - i0] : -1;
+            } else {
+                long long lo = 0, hi = in ? m : 0;   // the record whose root carries the label
+                while (lo < hi) {
+                    const long long mid = lo + ((hi - lo) >> 1);
+                    if (h.index[rootpos[mid]] < lab) lo = mid + 1; else hi = mid;
+                }
+                rec[j] = in && lo < m && h.index[rootpos[lo]] == lab ? lo : -1;
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < B; ++j)
+            if (rec[j] >= 0 && rec[j] < m) t[j] -= root_t[rec[j]];
+#pragma unroll
+        for (int j = 0; j < B; ++j) {
+            const long long c = rec[j], d = t[j];
+            if (c < 0 || c >= m) continue;   // past the capacity, or no record's label
+            const unsigned tot = xyt[j] >> 16, x = xyt[j] & 255u, y = (xyt[j] >> 8) & 255u, pk = pks[j];
+            unsigned slot = (unsigned)c * 2654435761u >> 22;   // AH = 2^10 slots
+            int probe = tot < 1024u ? 0 : 8;   // larger ones (not from packets) could overflow the table's sums
+            for (; probe < 8; ++probe, slot = (slot + 1) & (AH - 1)) {
+                const unsigned k = atomicCAS(&s_key[slot], 0u, (unsigned)c + 1u);
+                if (k == 0u || k == (unsigned)c + 1u) break;
+            }
+            if (probe < 8) {
+                atomicAdd(&s_n[slot], 1u);
+                if (pk) atomicAdd(&s_p[slot], 1u);
+                atomicAdd(&s_t[slot], tot);
+                atomicAdd(&s_x[slot], tot * x);
+                atomicAdd(&s_y[slot], tot * y);
+                if (d >= 0 && d < 1024) atomicAdd(&s_d[slot], tot * (unsigned)d);
+                else atomicAdd(&acc[c].s_t, tot * (unsigned long long)d);
+            } else {
+                atomicAdd(&acc[c].n_npk, 1ull | ((unsigned long long)pk << 32));
+                atomicAdd(&acc[c].s_tot, (unsigned long long)tot);
+                atomicAdd(&acc[c].s_x, (unsigned long long)tot * x);
+                atomicAdd(&acc[c].s_y, (unsigned long long)tot * y);
+                atomicAdd(&acc[c].s_t, tot * (unsigned long long)d);
+            }
+        }
+    }
+    __syncthreads();
+    for (int k = threadIdx.x; k < AH; k += GT) {
+        if (!s_key[k]) continue;
+        Acc &a = acc[s_key[k] - 1u];
+        atomicAdd(&a.n_npk, s_n[k] | ((unsigned long long)s_p[k] << 32));
+        atomicAdd(&a.s_tot, (unsigned long long)s_t[k]);
+        atomicAdd(&a.s_x, (unsigned long long)s_x[k]);
+        atomicAdd(&a.s_y, (unsigned long long)s_y[k]);
+        if (s_d[k]) atomicAdd(&a.s_t, (unsigned long long)s_d[k]);
     }
 }
 
-__global__ void k_final(tpx_hits h, long long n, const unsigned *flags, const unsigned *cid, const Acc *acc,
-                        tpx_record *out, long long cap) {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        if (!flags[i]) continue;
-        const long long c = cid[i];
-        if (c >= cap) continue;
+__global__ void k_final(tpx_hits h, const long long *n_rec, long long cap, const unsigned *rootpos, const Acc *acc,
+                        tpx_record *out) {
+    const long long m = min(*n_rec, cap);
+    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < m; c += (long long)gridDim.x * blockDim.x) {
         const Acc a = acc[c];
-        tpx_record o;
-        o.label = h.index[i];
-        o.shot = h.shot[i];
-        o.t0 = h.t[i];
-        o.s_tot = (long long)a.s_tot; o.s_x = (long long)a.s_x; o.s_y = (long long)a.s_y; o.s_t = (long long)a.s_t;
-        o.n = (int)a.n; o.n_peaks = (int)a.npk;
-        com_from_moments(o.s_x, o.s_y, o.s_t, o.s_tot, h.tof[i], &o.x, &o.y, &o.tof);
-        out[c] = o;
+        AccH v;
+        v.s_tot = (long long)a.s_tot; v.s_x = (long long)a.s_x; v.s_y = (long long)a.s_y; v.s_t = (long long)a.s_t;
+        v.n = (unsigned)a.n_npk; v.npk = (unsigned)(a.n_npk >> 32);
+        write_record(h, rootpos[c], v, out + c);
     }
 }
 
 // PAPER mode: each local maximum sums its box neighbourhood (both directions
 // in sorted order, within dt)
-__global__ void k_paper(Sorted s, long long n, int rx, int ry, int dt, const unsigned *flag_hit,
+__global__ void k_paper(Sorted s, long long n, int rx, int ry, int dt, const unsigned char *flag_hit,
                         const unsigned *cid_hit, tpx_hits h, tpx_record *out, long long cap) {
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
         const unsigned hi = s.hit[i];
         if (!flag_hit[hi]) continue;
         const long long c = cid_hit[hi];
         if (c >= cap) continue;
-        const long long sh = s.shot[i];
-        const int tb = s.tofb[i], xi = s.x[i], yi = s.y[i];
+        const long long sh = s.shot(i);
+        const int tb = s.tofb(i), xi = s.x(i), yi = s.y(i);
         long long m = 0, st = 0, sx = 0, sy = 0, a2 = 0;
         int tmin = tb;
         for (int dir = -1; dir <= 1; dir += 2) {
             for (long long j = (dir < 0 ? i : i + 1); j >= 0 && j < n; j += dir) {
-                if (s.shot[j] != sh) break;
-                const int d = s.tofb[j] - tb;
+                if (s.shot(j) != sh) break;
+                const int d = s.tofb(j) - tb;
                 if (d > dt || d < -dt) break;
-                const int dx = (int)s.x[j] - xi, dy = (int)s.y[j] - yi;
+                const int dx = (int)s.x(j) - xi, dy = (int)s.y(j) - yi;
                 if (dx < -rx || dx > rx || dy < -ry || dy > ry) continue;
-                const long long tj = s.tot[j];
-                m += 1; st += tj; sx += tj * s.x[j]; sy += tj * s.y[j]; a2 += tj * s.tofb[j];
-                tmin = min(tmin, s.tofb[j]);
+                const long long tj = s.tot(j);
+                m += 1; st += tj; sx += tj * s.x(j); sy += tj * s.y(j); a2 += tj * s.tofb(j);
+                tmin = min(tmin, s.tofb(j));
             }
         }
         tpx_record o;
-        o.label = s.index[i];
-        o.shot = sh;
+        o.label = s.index(i);
+        o.shot = h.shot[hi];
         const long long tofc0 = (long long)tmin - kBias;
         o.t0 = h.t[hi] - h.tof[hi] + tofc0;
         o.s_tot = st; o.s_x = sx; o.s_y = sy; o.s_t = a2 - (long long)tmin * st;
         o.n = (int)m; o.n_peaks = 1;
         com_from_moments(sx, sy, o.s_t, st, tofc0, &o.x, &o.y, &o.tof);
-        out[c] = o;
-    }
-}
-
-// number of records; latches the capacity status and the clusters counter
-__global__ void k_count_from_scan(const unsigned *flags, const unsigned *cid, long long n, long long *out,
-                                  long long cap, unsigned *status, unsigned long long *counter) {
-    const long long m = n ? (long long)cid[n - 1] + flags[n - 1] : 0;
-    *out = m;
-    if (m > cap) atomicOr(status, ST_CLUSTER_CAP);
-    if (counter) *counter = (unsigned long long)m;
-}
-
-// position of every record's root hit, in record (label) order
-__global__ void k_root_list(const unsigned *rflag, const unsigned *cid, long long n, long long cap, unsigned *rootpos) {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        if (rflag[i] && cid[i] < cap) rootpos[cid[i]] = (unsigned)i;
-}
-// CC records from the per-root moments, one thread per record
-__global__ void k_records(tpx_hits h, const long long *n_rec, long long cap, const unsigned *rootpos, const AccH *acc,
-                          tpx_record *out) {
-    const long long m = min(*n_rec, cap);
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < m; c += (long long)gridDim.x * blockDim.x) {
-        const long long i = rootpos[c];
-        const AccH a = acc[i];
-        tpx_record o;
-        o.label = h.index[i];
-        o.shot = h.shot[i];
-        o.t0 = h.t[i];
-        o.s_tot = a.s_tot; o.s_x = a.s_x; o.s_y = a.s_y; o.s_t = a.s_t;
-        o.n = (int)a.n; o.n_peaks = (int)a.npk;
-        com_from_moments(o.s_x, o.s_y, o.s_t, o.s_tot, h.tof[i], &o.x, &o.y, &o.tof);
         out[c] = o;
     }
 }
@@ -1213,35 +1648,55 @@ int reserve(tpx_ctx *c, size_t bytes) {
     return TPX_OK;
 }
 
-// exclusive scan of n unsigned counts into out (a.used advanced for temporaries)
-int scan_u32(Arena &a, const unsigned *in, unsigned *out, long long n, cudaStream_t s) {
-    const long long nb = (n + GTILE - 1) / GTILE;
-    unsigned *bsum = a.take<unsigned>(nb);
-    k_scan_blocks<<<(unsigned)(nb > 0 ? nb : 1), GT, 0, s>>>(in, out, n, bsum);
-    k_scan_bsum<<<1, PT, 0, s>>>(bsum, nb);
-    k_scan_add<<<grid_for(n), GT, 0, s>>>(out, n, bsum);
+// counts per block of GTILE items -> what the placing kernel expects
+int block_prefix(unsigned *bcnt, long long nb, cudaStream_t s) {
+    if (nb > kResum) k_scan_bsum<<<1, PT, 0, s>>>(bcnt, nb);
     return ck(cudaGetLastError());
 }
+inline long long blocks_of(long long n) { return (n + GTILE - 1) / GTILE; }
 
 size_t sort_bytes(long long n) {
-    const long long tiles = (n + GTILE - 1) / GTILE;
-    return 2 * sz(n, 8) + 2 * sz(n, 4) + 2 * sz(256 * tiles, 4) + sz((256 * tiles + GTILE - 1) / GTILE + 1, 4) +
-           sz(2, 8) + 4096;
+    return 2 * sz(n, 8) + 2 * sz(n, 4) + 2 * sz(n, 4) + sz(256 * blocks_of(n), 4) + sz(256, 4) + sz(2, 8) + 4096;
 }
 
-// sort the hits by (shot, corrected ToF); returns the sorted values buffer.
-// shot_span >= 0 bounds max shot - min shot (no host round trip); < 0 reads it.
-int sort_hits(tpx_ctx *c, Arena &a, const tpx_hits &h, long long n, long long shot_span, unsigned **vals_out) {
+// sorts the hits by (shot, corrected ToF); k_seg_count then brings their pixels
+// into that order. shot_span >= 0 bounds max shot - min shot (no host round
+// trip); < 0 reads it. *pxt_hit: the pixels in hit order.
+template <class K>
+int sort_keys(tpx_ctx *c, Arena &a, const tpx_hits &h, long long n, int bits, const unsigned long long *mm,
+              unsigned *pxt_hit, const K **keys_out, const unsigned **vals_out) {
     cudaStream_t s = c->stream;
-    const long long tiles = (n + GTILE - 1) / GTILE;
-    unsigned long long *k0 = a.take<unsigned long long>(n), *k1 = a.take<unsigned long long>(n);
+    const unsigned tiles = (unsigned)blocks_of(n);
+    K *k0 = reinterpret_cast<K *>(a.take<unsigned long long>(n)), *k1 = reinterpret_cast<K *>(a.take<unsigned long long>(n));
     unsigned *v0 = a.take<unsigned>(n), *v1 = a.take<unsigned>(n);
-    unsigned *hist = a.take<unsigned>(256 * tiles), *offs = a.take<unsigned>(256 * tiles);
+    unsigned *hist = a.take<unsigned>(256ll * tiles), *total = a.take<unsigned>(256);
+    constexpr int smem = GTILE * (int)(sizeof(K) + sizeof(unsigned));
+    if (ck(cudaFuncSetAttribute(k_digit_place<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem))) return TPX_ECUDA;
+    k_make_keys<K><<<tiles, GT, 0, s>>>(h, n, mm, k0, pxt_hit, hist);
+    const unsigned *vin = nullptr;   // the first digit's values are the positions themselves
+    for (int shift = 0; shift < bits; shift += 8) {
+        if (shift > 0) k_digit_hist<K><<<tiles, GT, 0, s>>>(k0, n, shift, hist);
+        k_digit_scan<<<256 / 32, PT, 0, s>>>(hist, tiles, total);
+        k_digit_place<K><<<tiles, GT, smem, s>>>(k0, vin, n, shift, hist, total, k1, v0);
+        vin = v0;
+        std::swap(k0, k1);
+        std::swap(v0, v1);
+    }
+    *keys_out = k0;
+    *vals_out = vin;
+    return ck(cudaGetLastError());
+}
+int sort_hits(tpx_ctx *c, Arena &a, const tpx_hits &h, long long n, long long shot_span, Sorted *so, unsigned **pxt_hit) {
+    cudaStream_t s = c->stream;
     unsigned long long *mm = a.take<unsigned long long>(2);   // min, max shot
-    const unsigned long long init[2] = {~0ull, 0ull};
-    if (ck(cudaMemcpyAsync(mm, init, sizeof init, cudaMemcpyHostToDevice, s))) return TPX_ECUDA;
-    k_shot_range<<<grid_for(n), GT, 0, s>>>(h, n, mm, mm + 1);
-    k_make_keys<<<grid_for(n), GT, 0, s>>>(h, n, mm, k0, v0);
+    so->pxt = a.take<unsigned>(n);
+    *pxt_hit = a.take<unsigned>(n);
+    so->hindex = h.index;
+    so->shot_min = mm;
+    so->k32 = nullptr;
+    so->k64 = nullptr;
+    if (ck(cudaMemsetAsync(mm, 0xFF, 8, s)) || ck(cudaMemsetAsync(mm + 1, 0, 8, s))) return TPX_ECUDA;
+    k_shot_range<<<(unsigned)std::min<long long>((n + 4 * GT - 1) / (4 * GT), (long long)c->num_sms * 4), GT, 0, s>>>(h, n, mm, mm + 1);
     unsigned long long span = (unsigned long long)shot_span;
     if (shot_span < 0) {
         unsigned long long hm[2] = {0, 0};
@@ -1251,24 +1706,13 @@ int sort_hits(tpx_ctx *c, Arena &a, const tpx_hits &h, long long n, long long sh
     }
     int bits = 24;
     while (bits < 64 && (span >> (bits - 24)) != 0) ++bits;
-    const size_t mark = a.used;
-    for (int shift = 0; shift < bits; shift += 8) {
-        a.used = mark;
-        k_sort_hist<<<(unsigned)tiles, GT, 0, s>>>(k0, n, shift, hist, tiles);
-        int rc = scan_u32(a, hist, offs, 256 * tiles, s);
-        if (rc) return rc;
-        k_sort_scatter<<<(unsigned)tiles, GT, 0, s>>>(k0, v0, n, shift, offs, tiles, k1, v1);
-        unsigned long long *tk = k0; k0 = k1; k1 = tk;
-        unsigned *tv = v0; v0 = v1; v1 = tv;
-    }
-    a.used = mark;
-    *vals_out = v0;
-    return ck(cudaGetLastError());
+    return bits <= 32 ? sort_keys<unsigned>(c, a, h, n, bits, mm, *pxt_hit, &so->k32, &so->hit)
+                      : sort_keys<unsigned long long>(c, a, h, n, bits, mm, *pxt_hit, &so->k64, &so->hit);
 }
 
 size_t decode_bytes(long long n) {
     const long long tiles = (n + GTILE - 1) / GTILE;
-    return sz(tiles, sizeof(GAgg)) * 2 + sz(tiles + 1, 8) * 4 + sz(n, 8) + 4096;
+    return sz(tiles, sizeof(GAgg)) * 2 + sz(tiles + 1, 8) * 4 + sz(tiles, 1) + sz(n, 8) + sz(n, 4) + 4096;
 }
 
 int decode_impl(tpx_ctx *c, const uint64_t *pk, int64_t n, int64_t base, const tpx_hits &h, int64_t cap,
@@ -1282,7 +1726,9 @@ int decode_impl(tpx_ctx *c, const uint64_t *pk, int64_t n, int64_t base, const t
     GAgg *tagg = a.take<GAgg>(tiles), *tpre = a.take<GAgg>(tiles);
     long long *tcnt = a.take<long long>(tiles + 1), *toff = a.take<long long>(tiles + 1);
     long long *tkept = a.take<long long>(tiles + 1), *tkoff = a.take<long long>(tiles + 1);
+    unsigned char *twrap = a.take<unsigned char>(tiles);
     long long *t_all = a.take<long long>(n);
+    int *shot = a.take<int>(n);
     if (t_all_out) *t_all_out = t_all;
     if (clear_ctl && cudaMemsetAsync(c->ctl, 0, sizeof(Ctl), s) != cudaSuccess) return TPX_ECUDA;
     if (cudaMemsetAsync(d_n_hits, 0, 8, s) != cudaSuccess || cudaMemsetAsync(d_n_trig, 0, 8, s) != cudaSuccess)
@@ -1295,15 +1741,16 @@ int decode_impl(tpx_ctx *c, const uint64_t *pk, int64_t n, int64_t base, const t
     const long long tp = c->cfg.wrap_thr_pix_ticks, tt = c->cfg.wrap_thr_tdc_ticks;
     long long *ntr = reinterpret_cast<long long *>(d_n_trig);
     long long *tr = reinterpret_cast<long long *>(trig);
-    k_tile_agg<<<(unsigned)tiles, GT, 0, s>>>(pk, n, tp, tt, tagg, tcnt);
+    k_tile_agg<<<(unsigned)tiles, GT, 0, s>>>(pk, n, tp, tt, tagg, tcnt, twrap);
     k_tile_prefix<<<1, PT, 0, s>>>(tagg, tpre, tcnt, toff, tiles, tp, tt, ntr, E0, state_out);
-    k_unwrap<<<(unsigned)tiles, GT, 0, s>>>(pk, n, tpre, toff, tp, tt, t_all, tr, trig_cap, &c->ctl->status, trig_pos);
+    k_unwrap<<<(unsigned)tiles, GT, 0, s>>>(pk, n, tagg, tpre, twrap, toff, tp, tt, t_all, tr, trig_cap, &c->ctl->status,
+                                            trig_pos);
     k_check_trig<<<152, GT, 0, s>>>(tr, ntr, trig_cap, &c->ctl->status);
-    k_bin<<<(unsigned)tiles, GT, 0, s>>>(pk, n, t_all, tr, ntr, trig_cap, c->cfg.tof_max_ticks, tkept,
+    k_bin<<<(unsigned)tiles, GT, 0, s>>>(pk, n, t_all, tr, ntr, trig_cap, c->cfg.tof_max_ticks, shot, tkept,
                                          c->ctl->counters);
     k_count_prefix<<<1, PT, 0, s>>>(tkept, tkoff, tiles, reinterpret_cast<long long *>(d_n_hits));
-    k_compact<<<(unsigned)tiles, GT, 0, s>>>(pk, n, base, t_all, tr, ntr, trig_cap, c->cfg.tof_max_ticks,
-                                             c->cfg.d_timewalk_lut, tkoff, h, cap, &c->ctl->status, E0);
+    k_compact<<<(unsigned)tiles, GT, 0, s>>>(pk, n, base, t_all, tr, ntr, trig_cap, shot, c->cfg.d_timewalk_lut, tkoff, h,
+                                             cap, &c->ctl->status, E0);
     const unsigned long long np = (unsigned long long)n;
     if (cudaMemcpyAsync(&c->ctl->counters[C_PACKETS], &np, 8, cudaMemcpyHostToDevice, s) != cudaSuccess)
         return TPX_ECUDA;
@@ -1311,10 +1758,10 @@ int decode_impl(tpx_ctx *c, const uint64_t *pk, int64_t n, int64_t base, const t
 }
 
 size_t cluster_bytes(long long n) {
-    return sort_bytes(n) + sz(n, 4) + sz(n, 8) * 2 + sz(n, 4) + sz(n, 2) + 2 * sz(n, 1)   // sorted hits
-           + 2 * sz(n, 4) + sz(n + 1, 8) + sz(1, 8)                                     // segments
+    return sort_bytes(n) + sz(n, 4)                                                     // sorted pixels
+           + sz(blocks_of(n), 4) + sz(n + 1, 8) + sz(1, 8) + sz(n, 4) + sz(1, 8)         // segments
            + 2 * sz(n, 1) + sz(n, 4)                                                    // long segments
-           + 2 * sz(n, 4) + sz(n, sizeof(AccH)) + sz((n + GTILE - 1) / GTILE + 1, 4)    // records
+           + sz(n, 1) + sz(n, 4) + sz(n, sizeof(AccH))                                  // records
            + sz(4 * n + 2, 4) + sz(n, 4) + sz(n, 8)                                    // long-segment hash
            + 8192;
 }
@@ -1332,61 +1779,50 @@ int cluster_all(tpx_ctx *c, const tpx_hits &h, int64_t n, int64_t *labels, uint8
     int rc = reserve(c, cluster_bytes(n));
     if (rc) return rc;
     Arena a{static_cast<char *>(c->g_mem), 0, c->g_bytes};
-    Sorted so;
-    so.hit = a.take<unsigned>(n);
-    so.shot = a.take<long long>(n);
-    so.index = a.take<long long>(n);
-    so.tofb = a.take<int>(n);
-    so.tot = a.take<unsigned short>(n);
-    so.x = a.take<unsigned char>(n);
-    so.y = a.take<unsigned char>(n);
-    unsigned *segf = a.take<unsigned>(n), *sego = a.take<unsigned>(n);
+    const long long nb = blocks_of(n);
+    unsigned *bcnt = a.take<unsigned>(nb), *mid = a.take<unsigned>(n);
     long long *seg_start = a.take<long long>(n + 1), *nseg = a.take<long long>(1);
-    unsigned char *mark = a.take<unsigned char>(n), *notpeak = a.take<unsigned char>(n);
+    SegLists *lists = a.take<SegLists>(1);
+    unsigned char *mark = a.take<unsigned char>(n), *notpeak = a.take<unsigned char>(n), *rflag = a.take<unsigned char>(n);
     int *parent = a.take<int>(n);
-    unsigned *rflag = a.take<unsigned>(n), *cid = a.take<unsigned>(n);
+    unsigned *cid = a.take<unsigned>(n);
     AccH *acc = a.take<AccH>(n);
     unsigned long long lmask = 1;   // the long segments' cell hash: >= 2n buckets
     while (lmask + 1 < 2ull * (unsigned long long)n) lmask = 2 * lmask + 1;
     unsigned *lhead = a.take<unsigned>((long long)lmask + 1), *lnext = a.take<unsigned>(n);
     unsigned long long *lword = a.take<unsigned long long>(n);
-    const size_t mark_used = a.used;
-    unsigned *vals = nullptr;
-    rc = sort_hits(c, a, h, n, shot_span, &vals);
+    Sorted so;
+    unsigned *pxt_hit = nullptr;
+    rc = sort_hits(c, a, h, n, shot_span, &so, &pxt_hit);
     if (rc) return rc;
-    k_gather<<<grid_for(n), GT, 0, s>>>(h, vals, n, so);
-    a.used = mark_used;   // the sort's scratch is free again
     const int dt = c->cfg.dt_ticks;
-    k_seg_flags<<<grid_for(n), GT, 0, s>>>(so, n, dt, segf);
-    rc = scan_u32(a, segf, sego, n, s);
+    if (ck(cudaMemsetAsync(lists, 0, sizeof(SegLists), s))) return TPX_ECUDA;
+    k_seg_count<<<(unsigned)nb, GT, 0, s>>>(so, pxt_hit, n, dt, bcnt);
+    rc = block_prefix(bcnt, nb, s);
     if (rc) return rc;
-    k_seg_starts<<<grid_for(n), GT, 0, s>>>(segf, sego, n, seg_start, nseg);
-    if (ck(cudaMemsetAsync(mark, 0, (size_t)n, s))) return TPX_ECUDA;
+    k_seg_starts<<<(unsigned)nb, GT, 0, s>>>(so, n, dt, bcnt, nb, seg_start, nseg);
     long long *lab = reinterpret_cast<long long *>(labels);
-    unsigned *rf = out ? rflag : nullptr;
+    unsigned char *rf = out ? rflag : nullptr;
     AccH *ac = (out && cc) ? acc : nullptr;
-    int seg_blocks = c->num_sms * 8;
-    if ((long long)seg_blocks * SEGW > n) seg_blocks = (int)((n + SEGW - 1) / SEGW);
-    k_segments<<<seg_blocks, SEGW * 32, 0, s>>>(so, seg_start, nseg, c->cfg.rx, c->cfg.ry, dt, cc, shot_limit, lab,
-                                                is_peak, rf, ac, mark);
-    k_long_init<<<grid_for(n), GT, 0, s>>>(so, n, mark, parent, notpeak, ac);
-    if (ck(cudaMemsetAsync(lhead, 0xFF, sizeof(unsigned) * (size_t)(lmask + 1), s))) return TPX_ECUDA;
-    k_long_insert<<<grid_for(n), GT, 0, s>>>(so, n, mark, lhead, lnext, lword, lmask);
-    k_long_pairs<<<grid_for(n), GT, 0, s>>>(so, n, mark, lhead, lnext, lword, lmask, c->cfg.rx, c->cfg.ry, dt, cc,
+    const long long seg_max = (n + SEGW - 1) / SEGW;   // more blocks than that have no segment
+    k_segments<<<(unsigned)std::min<long long>(seg_max, (long long)c->num_sms * 16), SEGW * 32, 0, s>>>(
+        so, seg_start, nseg, c->cfg.rx, c->cfg.ry, dt, cc, shot_limit, lab, is_peak, rf, ac, mark, mid, lists);
+    k_segments_mid<<<(unsigned)std::min<long long>(seg_max, (long long)c->num_sms * 4), SEGW * 32, 0, s>>>(
+        so, seg_start, mid, lists, c->cfg.rx, c->cfg.ry, dt, cc, shot_limit, lab, is_peak, rf, ac);
+    k_long_init<<<grid_for(n), GT, 0, s>>>(so, n, lists, mark, parent, notpeak, ac, lhead, lmask);
+    k_long_insert<<<grid_for(n), GT, 0, s>>>(so, n, lists, mark, lhead, lnext, lword, lmask);
+    k_long_pairs<<<grid_for(n), GT, 0, s>>>(so, n, lists, mark, lhead, lnext, lword, lmask, c->cfg.rx, c->cfg.ry, dt, cc,
                                             parent, notpeak);
-    k_long_finish<<<grid_for(n), GT, 0, s>>>(so, n, mark, cc, shot_limit, parent, notpeak, lab, is_peak, rf, ac);
+    k_long_finish<<<grid_for(n), GT, 0, s>>>(so, n, lists, mark, cc, shot_limit, parent, notpeak, lab, is_peak, rf, ac);
     if (!out) return ck(cudaGetLastError());
-    rc = scan_u32(a, rflag, cid, n, s);
+    const RootFlag f{nullptr, nullptr, rflag};
+    k_root_count<<<(unsigned)nb, GT, 0, s>>>(f, n, bcnt);
+    rc = block_prefix(bcnt, nb, s);
     if (rc) return rc;
-    k_count_from_scan<<<1, 1, 0, s>>>(rflag, cid, n, reinterpret_cast<long long *>(d_n_clusters), cap,
-                                      &c->ctl->status, &c->ctl->counters[C_CLUSTERS]);
-    if (cc) {
-        unsigned *rootpos = segf;   // free again: the segments are done
-        k_root_list<<<grid_for(n), GT, 0, s>>>(rflag, cid, n, cap, rootpos);
-        k_records<<<grid_for(n / 16 + 1), GT, 0, s>>>(h, reinterpret_cast<const long long *>(d_n_clusters), cap, rootpos,
-                                                     acc, out);
-    } else
-        k_paper<<<grid_for(n), GT, 0, s>>>(so, n, c->cfg.rx, c->cfg.ry, dt, rflag, cid, h, out, cap);
+    const Roots roots{acc, cc ? out : nullptr, cc ? nullptr : cid, nullptr, 0, nullptr, nullptr, nullptr};
+    k_root_place<<<(unsigned)nb, GT, 0, s>>>(f, h, n, bcnt, nb, cap, reinterpret_cast<long long *>(d_n_clusters),
+                                             &c->ctl->status, &c->ctl->counters[C_CLUSTERS], roots);
+    if (!cc) k_paper<<<grid_for(n), GT, 0, s>>>(so, n, c->cfg.rx, c->cfg.ry, dt, rflag, cid, h, out, cap);
     return ck(cudaGetLastError());
 }
 
@@ -1401,37 +1837,41 @@ int centroid_impl(tpx_ctx *c, const tpx_hits &h, const int64_t *labels, const ui
     if (n <= 0) return TPX_OK;
     const int cc = c->cfg.mode == TPX_MODE_CC;
     if (!cc && !is_peak) return TPX_EINVAL;
-    const size_t need = 2 * sz(n, 4) + sz(n, sizeof(Acc)) + sort_bytes(n) + sz(n, 4) + sz(n, 8) * 2 + sz(n, 4) +
-                        sz(n, 2) + 3 * sz(n, 1) + 4096;
+    const long long nb = blocks_of(n);
+    const long long recs = std::min<long long>(n, cap), rank_cap = 2 * n + 65536;
+    const size_t need = sz(nb, 4) + (cc ? sz(rank_cap, 4) + sz(recs, sizeof(Acc)) + sz(recs, 4) + sz(recs, 8)
+                                        : sz(n, 4) + sz(n, 4) + sort_bytes(n)) + 8192;
     int rc = reserve(c, need);
     if (rc) return rc;
     Arena a{static_cast<char *>(c->g_mem), 0, c->g_bytes};
-    unsigned *flags = a.take<unsigned>(n), *cid = a.take<unsigned>(n);
-    Acc *acc = a.take<Acc>(n);
+    unsigned *bcnt = a.take<unsigned>(nb);
     const long long *lab = reinterpret_cast<const long long *>(labels);
-    k_root_flags<<<grid_for(n), GT, 0, s>>>(h, lab, is_peak, n, cc, flags);
-    rc = scan_u32(a, flags, cid, n, s);
+    long long *nrec = reinterpret_cast<long long *>(d_n_clusters);
+    const RootFlag f{cc ? lab : nullptr, reinterpret_cast<const long long *>(h.index), cc ? nullptr : is_peak};
+    k_root_count<<<(unsigned)nb, GT, 0, s>>>(f, n, bcnt);
+    rc = block_prefix(bcnt, nb, s);
     if (rc) return rc;
-    k_count_from_scan<<<1, 1, 0, s>>>(flags, cid, n, reinterpret_cast<long long *>(d_n_clusters), cap,
-                                      &c->ctl->status, &c->ctl->counters[C_CLUSTERS]);
     if (cc) {
-        if (ck(cudaMemsetAsync(acc, 0, sizeof(Acc) * (size_t)n, s))) return TPX_ECUDA;
-        k_accum<<<grid_for(n), GT, 0, s>>>(h, lab, is_peak, n, cid, acc);
-        k_final<<<grid_for(n), GT, 0, s>>>(h, n, flags, cid, acc, out, cap);
+        unsigned *rank = a.take<unsigned>(rank_cap), *rootpos = a.take<unsigned>(recs);
+        Acc *acc = a.take<Acc>(recs);
+        long long *root_t = a.take<long long>(recs);
+        if (ck(cudaMemsetAsync(rank, 0xFF, 4 * (size_t)rank_cap, s))) return TPX_ECUDA;
+        const Roots roots{nullptr, nullptr, nullptr, rank, rank_cap, acc, rootpos, root_t};
+        k_root_place<<<(unsigned)nb, GT, 0, s>>>(f, h, n, bcnt, nb, cap, nrec, &c->ctl->status,
+                                                 &c->ctl->counters[C_CLUSTERS], roots);
+        k_accum<<<(unsigned)nb, GT, 0, s>>>(h, lab, is_peak, n, nrec, cap, rank, rank_cap, rootpos, root_t, acc);
+        k_final<<<grid_for(recs / 8 + 1), GT, 0, s>>>(h, nrec, cap, rootpos, acc, out);
     } else {
+        unsigned *cid = a.take<unsigned>(n);
+        const Roots roots{nullptr, nullptr, cid, nullptr, 0, nullptr, nullptr, nullptr};
+        k_root_place<<<(unsigned)nb, GT, 0, s>>>(f, h, n, bcnt, nb, cap, nrec, &c->ctl->status,
+                                                 &c->ctl->counters[C_CLUSTERS], roots);
         Sorted so;
-        so.hit = a.take<unsigned>(n);
-        so.shot = a.take<long long>(n);
-        so.index = a.take<long long>(n);
-        so.tofb = a.take<int>(n);
-        so.tot = a.take<unsigned short>(n);
-        so.x = a.take<unsigned char>(n);
-        so.y = a.take<unsigned char>(n);
-        unsigned *vals = nullptr;
-        rc = sort_hits(c, a, h, n, -1, &vals);
+        unsigned *pxt_hit = nullptr;
+        rc = sort_hits(c, a, h, n, -1, &so, &pxt_hit);
         if (rc) return rc;
-        k_gather<<<grid_for(n), GT, 0, s>>>(h, vals, n, so);
-        k_paper<<<grid_for(n), GT, 0, s>>>(so, n, c->cfg.rx, c->cfg.ry, c->cfg.dt_ticks, flags, cid, h, out, cap);
+        k_seg_count<<<(unsigned)nb, GT, 0, s>>>(so, pxt_hit, n, c->cfg.dt_ticks, bcnt);   // brings the pixels into order
+        k_paper<<<grid_for(n), GT, 0, s>>>(so, n, c->cfg.rx, c->cfg.ry, c->cfg.dt_ticks, is_peak, cid, h, out, cap);
     }
     return ck(cudaGetLastError());
 }
@@ -1894,19 +2334,20 @@ extern "C" int tpx_summarize(tpx_ctx *c, const uint64_t *pk, int64_t n, tpx_chai
     using namespace tpxg;
     cudaStream_t s = c->stream;
     const long long tiles = (n + GTILE - 1) / GTILE;
-    const size_t need = sz(tiles, sizeof(tpxk::GAgg)) * 2 + sz(tiles + 1, 8) * 2 + sz(1, sizeof(tpxk::GAgg)) + 4096;
+    const size_t need = sz(tiles, sizeof(tpxk::GAgg)) * 2 + sz(tiles + 1, 8) * 2 + sz(1, sizeof(tpxk::GAgg)) + sz(tiles, 1) + 4096;
     int rc = reserve(c, need);
     if (rc) return rc;
     Arena a{static_cast<char *>(c->g_mem), 0, c->g_bytes};
     tpxk::GAgg *tagg = a.take<tpxk::GAgg>(tiles), *tpre = a.take<tpxk::GAgg>(tiles);
     long long *tcnt = a.take<long long>(tiles + 1), *toff = a.take<long long>(tiles + 1);
     tpxk::GAgg *res = a.take<tpxk::GAgg>(1);
+    unsigned char *twrap = a.take<unsigned char>(tiles);
     long long *ntr = toff + tiles;
     tpxk::GAgg h;
     std::memset(&h, 0, sizeof h);
     if (n > 0) {
         const long long tp = c->cfg.wrap_thr_pix_ticks, tt = c->cfg.wrap_thr_tdc_ticks;
-        k_tile_agg<<<(unsigned)tiles, GT, 0, s>>>(pk, n, tp, tt, tagg, tcnt);
+        k_tile_agg<<<(unsigned)tiles, GT, 0, s>>>(pk, n, tp, tt, tagg, tcnt, twrap);
         k_tile_prefix<<<1, PT, 0, s>>>(tagg, tpre, tcnt, toff, tiles, tp, tt, ntr, nullptr, res);
         if (ck(cudaMemcpyAsync(&h, res, sizeof h, cudaMemcpyDeviceToHost, s))) return TPX_ECUDA;
     }

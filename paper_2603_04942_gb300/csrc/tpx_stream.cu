@@ -131,7 +131,19 @@ __global__ void k_probe(const uint64_t *pk, long long p, Probe *pr) {
         np += __shfl_down_sync(0xffffffffu, np, o);
         nt += __shfl_down_sync(0xffffffffu, nt, o);
     }
+    __shared__ unsigned long long s_v[BT / 32][4];
     if ((threadIdx.x & 31) == 0) {
+        unsigned long long *v = s_v[threadIdx.x >> 5];
+        v[0] = lp; v[1] = lt; v[2] = np; v[3] = nt;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {   // one set of atomics per block: they all meet on four addresses
+        for (int k = 1; k < BT / 32; ++k) {
+            lp = max(lp, s_v[k][0]);
+            lt = max(lt, s_v[k][1]);
+            np += s_v[k][2];
+            nt += s_v[k][3];
+        }
         if (lp) atomicMax(&pr->last_pix, lp);
         if (lt) atomicMax(&pr->last_tdc, lt);
         if (np) atomicAdd(&pr->n_pix, np);
@@ -233,7 +245,7 @@ int process_job(tpx_stream *S, Slot *sl, const uint64_t *h_chunk, int64_t n, boo
         if (cks(cudaMemcpyAsync(S->st[2], S->st[1], sizeof(GAgg), cudaMemcpyDeviceToDevice, s))) return TPX_ECUDA;
     } else if (p > 0) {
         if (cks(cudaMemsetAsync(S->d_probe, 0, sizeof(Probe), s))) return TPX_ECUDA;
-        k_probe<<<gridn(p), BT, 0, s>>>(pk, p, S->d_probe);
+        k_probe<<<gridn((p + 7) / 8), BT, 0, s>>>(pk, p, S->d_probe);
         k_state_at<<<1, 1, 0, s>>>(pk, t_all, S->d_probe, S->st[0], S->st[2]);
     } else {
         if (cks(cudaMemcpyAsync(S->st[2], S->st[0], sizeof(GAgg), cudaMemcpyDeviceToDevice, s))) return TPX_ECUDA;
