@@ -730,8 +730,9 @@ class Stream:
         n = r.n_clusters
         cl = np.zeros(0, CLUSTER_DTYPE)
         if n:
-            buf = (ctypes.c_char * (n * CLUSTER_DTYPE.itemsize)).from_address(r.clusters)
-            cl = np.frombuffer(bytes(buf), CLUSTER_DTYPE).copy()
+            # the slot's buffer is reused: one copy out of it (two cost 0.3 ms on 2.5 MB)
+            cl = np.empty(n, CLUSTER_DTYPE)
+            ctypes.memmove(cl.ctypes.data, r.clusters, n * CLUSTER_DTYPE.itemsize)
         tr = np.zeros(0, np.int64)
         if r.n_shots:
             tr = np.array((ctypes.c_int64 * r.n_shots).from_address(r.trig_t), dtype=np.int64)
