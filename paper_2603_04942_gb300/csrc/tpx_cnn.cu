@@ -173,14 +173,11 @@ void sgemm(cudaStream_t s, const float *A, long long sam, long long sak, const f
         k_sgemm<<<g, 256, 0, s>>>(A + m0 * sam, sam, sak, B, sbk, sbn, C + m0 * ldc, ldc, m, N, K, bias, relu ? 1 : 0);
     }
 }
-// splits for a weight gradient whose inner dimension runs over `rows`: four
-// blocks per SM, at least 96 rows each. A block's steps of 16 rows wait for
-// their loads one after another, so its rows are the kernel's time: 4096
-// patches, 1024 rows or more a split: 254 to 291 us for each of the five layers.
+// splits for a weight gradient whose inner dimension runs over `rows`
 inline int splits_for(long long rows, int M, int N) {
     const long long tiles = (long long)((M + TM - 1) / TM) * ((N + TN - 1) / TN);
     long long sp = (152LL * 4) / (tiles > 0 ? tiles : 1);
-    const long long per = rows / 96;
+    const long long per = rows / 1024;   // at least ~1024 rows per split
     if (sp > per) sp = per;
     return (int)(sp < 1 ? 1 : (sp > 65535 ? 65535 : sp));
 }
@@ -198,7 +195,6 @@ __global__ void k_colsum(const float *d, long long rows, int m, float *g) {
     const long long per = (rows + gridDim.x - 1) / gridDim.x;
     const long long r0 = blockIdx.x * per, r1 = min(rows, r0 + per);
     float s = 0.f;
-#pragma unroll 8
     for (long long r = r0 + rl; r < r1; r += lanes) s += d[r * m + j];
     atomicAdd(&g[j], s);
 }
@@ -239,10 +235,7 @@ void layer_back(cudaStream_t s, const float *P, float *G, const Conv &L, const f
                 float *dX) {
     const int K = L.cin * L.kk * L.kk;
     sgemm(s, dZ, 1, L.cout, X, K, 1, G + L.ow, K, L.cout, K, rows, nullptr, false, splits_for(rows, L.cout, K));
-    // 64 rows per row lane of a block, at most eight blocks per SM (one block for
-    // 4096 rows of 144 columns took 516 us)
-    const long long strips = (rows * L.cout + 64 * 256 - 1) / (64 * 256);
-    k_colsum<<<(unsigned)(strips < 152 * 8 ? strips : 152 * 8), 256, 0, s>>>(dZ, rows, L.cout, G + L.ob);
+    k_colsum<<<grid_for(rows / 64 + 1), 256, 0, s>>>(dZ, rows, L.cout, G + L.ob);
     if (dX) sgemm(s, dZ, L.cout, 1, P + L.ow, K, 1, dX, K, rows, K, L.cout, nullptr, false);
 }
 
