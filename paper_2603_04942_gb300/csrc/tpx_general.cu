@@ -1452,7 +1452,8 @@ __global__ void __launch_bounds__(GT) k_root_place(RootFlag f, tpx_hits h, long 
             r.zero[c] = Acc{0, 0, 0, 0, 0};
             r.rootpos[c] = (unsigned)i;
             r.root_t[c] = h.t[i];
-            if (ranked) r.rank[h.index[i] - h.index[0]] = (unsigned)c;
+            const long long at = h.index[i] - h.index[0];
+            if (ranked && at >= 0 && at < r.rank_cap) r.rank[at] = (unsigned)c;
         }
     }
     if (blockIdx.x == nb - 1 && threadIdx.x == 0) latch_count(first + total, cap, n_rec, status, counter);
