@@ -254,11 +254,11 @@ static_assert(sizeof(BrMom) == 48, "moment record");
 // shared scratch: the tile arrays in front of the trigger tables
 constexpr int BR_REGION = (int)offsetof(Smem, tdc_t);
 static_assert(BR_REGION >= BIG_REGION, "the big-range scratch");
-// the neighbour pass reads the sorted records through shared memory, BR_CH
-// pixels at a time with the records before them that they can reach
-constexpr int BR_CH = 2 * NT;   // pixels of a step of the neighbour pass
-constexpr int BR_SB = 2 * BR_CH;
-constexpr int BR_FIXED = 4 * (BR_BINS + 4) + 4 * BR_LW + 2 * BR_LW + 4 * 5 * BR_S + 4 * 16 + 8 * BR_SB;
+// the neighbour pass chains the pixels by cell: heads in place of the sort's
+// bins, and the chains of the first BR_NX pixels in shared memory (the others'
+// in the scratch)
+constexpr int BR_NX = 16 * NT;
+constexpr int BR_FIXED = 4 * (BR_BINS + 4) + 4 * BR_LW + 2 * BR_LW + 4 * 5 * BR_S + 4 * 16 + 2 * BR_NX;
 // kept pixels: a 16-bit parent and a local-maximum bit each
 constexpr int BR_N0 = ((BR_REGION - BR_FIXED) * 8 / 17) & ~63;
 constexpr int BR_N = BR_N0 < 65472 ? BR_N0 : 65472;
@@ -711,14 +711,14 @@ __device__ __forceinline__ void scan_label_bits(Smem &S) {
 // A range longer than the range capacity C (in CC mode: a shot of more pixels
 // than a tile holds) stays in the launch. The CTA decodes the whole range
 // into its own global scratch (the tile's unwrap, binning and cut, Sec.
-// IV.A-C), sorts the kept pixels by (shot, time bin, 8-column x stripe)
-// with bins at least dt + 1 ticks wide, and compares each pixel with the
-// pixels of the keys before its own that can hold a neighbour: the previous
-// bin's three stripes around its own, its own bin's stripe to the left, and
-// its own key up to itself. Two adjacent pixels (Sec. V.A: same shot, box
-// neighbours, |dt| within the radius) lie in the same or consecutive bins
-// and stripes, so every adjacent pair is seen once, as in the tile's
-// neighbour pass. Union-find over the sorted order runs in shared
+// IV.A-C), sorts the kept pixels by (shot, time bin, 8-column x stripe), so
+// that a cluster's pixels lie together, and chains them by cell in a hash. Each
+// pixel walks the chains of the forward half of its box (in its own cell only
+// the pixels before it in the sorted order), so every adjacent pair (Sec. V.A:
+// same shot, box neighbours, |dt| within the radius) is seen once. (Comparing
+// each pixel with all of the time bins and stripes around it cost 134 of the
+// path's 179 warp instructions per packet.) Union-find over the sorted order
+// runs in shared
 // memory (16-bit parents, roots linked by a hashed priority). The
 // exact integer moments of each cluster (Sec. V.C) are gathered with
 // warp-aggregated atomics, and the records are staged in label order in the
@@ -805,15 +805,18 @@ __device__ __noinline__ int big_range(Smem &S, const Params &p, long long base, 
     int *sg_n = reinterpret_cast<int *>(lpre + BR_LW);
     int *sg_lo = sg_n + BR_S, *sg_hi = sg_lo + BR_S, *sg_b0 = sg_hi + BR_S, *sg_w = sg_b0 + BR_S;
     // misc: [0..2] range-end slots, [3] first pixel, [4] kept, [5] dropped
-    // before a trigger, [6] background, [7] failure bits, [8] clusters, [9]
-    // peaks, [12] the neighbour pass's task counter
+    // before a trigger, [6] background, [7] failure bits, [8] clusters, [9] peaks
     int *misc = sg_w + BR_S;
-    uint64_t *sbuf = reinterpret_cast<uint64_t *>(misc + 16);   // [BR_SB] staged sorted records
+    uint16_t *nx_sh = reinterpret_cast<uint16_t *>(misc + 16);   // [BR_NX] the cell chains
     unsigned char *G = p.big + (size_t)blockIdx.x * BR_STRIDE;
     uint64_t *g_rec = reinterpret_cast<uint64_t *>(G);
     uint64_t *g_srec = g_rec + (BR_L + 1);
     uint16_t *g_spos = reinterpret_cast<uint16_t *>(g_srec + BR_N);
     BrMom *g_mom = reinterpret_cast<BrMom *>(g_spos + BR_N);
+    // before the moments: up to three further neighbours per pixel, and the
+    // cell chains past BR_NX
+    uint64_t *g_more = reinterpret_cast<uint64_t *>(g_mom);
+    uint16_t *nx_g = reinterpret_cast<uint16_t *>(g_more + BR_N);
     const uint32_t pb = (uint32_t)__cvta_generic_to_shared(par);      // shared addresses
     const uint32_t nb_sh = (uint32_t)__cvta_generic_to_shared(npk);
     const int rx = p.rx, ry = p.ry, dtr = p.dt;
@@ -854,18 +857,21 @@ __device__ __noinline__ int big_range(Smem &S, const Params &p, long long base, 
     {
         int lpx = -1, fpx = INT_MAX;
         long long lr = 0;
-        for (int j = 0; j < kpd; ++j) {
-            const int q = p0 + j;
-            if (q >= L) break;
-            const uint64_t w = __ldg(p.pk + base + q);
-            const unsigned h = (unsigned)(w >> 60);
-            if (h == 0xBu) {
-                const long long r = pix_raw(w);
-                if (lpx >= 0) jp += (int)jump(r - lr, tp); else fpx = q;
-                lpx = q;
-                lr = r;
-            } else if (h == 0x6u) {
-                ++ntd;
+        for (int j0 = 0; j0 < kpd; j0 += 8) {   // eight loads in flight
+            uint64_t w8[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) w8[u] = j0 + u < kpd && p0 + j0 + u < L ? __ldg(p.pk + base + p0 + j0 + u) : 0ull;
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const unsigned h = (unsigned)(w8[u] >> 60);
+                if (h == 0xBu) {
+                    const long long r = pix_raw(w8[u]);
+                    if (lpx >= 0) jp += (int)jump(r - lr, tp); else fpx = p0 + j0 + u;
+                    lpx = p0 + j0 + u;
+                    lr = r;
+                } else if (h == 0x6u) {
+                    ++ntd;
+                }
             }
         }
         if (lpx >= 0) {
@@ -943,10 +949,16 @@ __device__ __noinline__ int big_range(Smem &S, const Params &p, long long base, 
         int c_keep = 0, c_pre = 0, c_bg = 0;
         bool exc = false;
         int cs = -1, cn = 0, clo = INT_MAX, chi = INT_MIN;   // the current shot's running stats
+        uint64_t w4[4];
         for (int j = 0; j < kpd; ++j) {
             const int q = p0 + j;
             if (q >= L) break;
-            const uint64_t w = __ldg(p.pk + base + q);
+            if ((j & 3) == 0) {   // four loads in flight
+#pragma unroll
+                for (int u = 0; u < 4; ++u) w4[u] = q + u < L ? __ldg(p.pk + base + q + u) : 0ull;
+            }
+            const uint64_t w = w4[0];
+            w4[0] = w4[1]; w4[1] = w4[2]; w4[2] = w4[3];
             const unsigned h = (unsigned)(w >> 60);
             uint64_t rec = INVALID;
             if (h == 0x6u) {
@@ -1056,9 +1068,13 @@ __device__ __noinline__ int big_range(Smem &S, const Params &p, long long base, 
         return (sg_b0[s] + (r_tof(r) - sg_lo[s]) / sg_w[s]) * NS + r_x(r) / SW;
     };
     // ---- counting sort of the kept pixels by bin ----
-    for (int q = tid; q < L; q += NTW) {
-        const uint64_t r = g_rec[q];
-        if (r != INVALID) atomicAdd(&bins[bin_of(r)], 1u);
+    for (int q0 = tid; q0 < L; q0 += 4 * NTW) {   // (here and below: four positions' loads in flight)
+        uint64_t r[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) r[u] = q0 + u * NTW < L ? g_rec[q0 + u * NTW] : INVALID;
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (r[u] != INVALID) atomicAdd(&bins[bin_of(r[u])], 1u);
     }
     cta_sync();
     {
@@ -1072,109 +1088,169 @@ __device__ __noinline__ int big_range(Smem &S, const Params &p, long long base, 
         for (int k = 0; k < BPT; ++k) { if (tid * BPT + k < BR_BINS) bins[tid * BPT + k] = run; run += c[k]; }
     }
     cta_sync();
-    for (int q = tid; q < L; q += NTW) {
-        const uint64_t r = g_rec[q];
-        if (r == INVALID) continue;
-        const unsigned slot = atomicAdd(&bins[bin_of(r)], 1u);
-        if (!TPX_IN(slot, N)) continue;
-        g_srec[slot] = r;
-        g_spos[slot] = (uint16_t)q;
+    for (int q0 = tid; q0 < L; q0 += 4 * NTW) {
+        uint64_t r[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) r[u] = q0 + u * NTW < L ? g_rec[q0 + u * NTW] : INVALID;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            if (r[u] == INVALID) continue;
+            const unsigned slot = atomicAdd(&bins[bin_of(r[u])], 1u);
+            if (!TPX_IN(slot, N)) continue;
+            g_srec[slot] = r[u];
+            g_spos[slot] = (uint16_t)(q0 + u * NTW);
+        }
     }
-    // bins[b] is now the end of bin b (the start of bin b + 1)
     for (int i = tid; i < N; i += NTW) par[i] = (uint16_t)i;
     for (int w = tid; w < BR_N / 32; w += NTW) npk[w] = 0u;
-    for (int w = tid; w < BR_LW; w += NTW) lbits[w] = 0u;
+    // the neighbour pass's flags, a byte each in what the parents leave free:
+    // plain stores (as bits, 32 lanes of one cluster met in the same word's
+    // atomics: a third of the path's cycles)
+    uint8_t *lost = 3 * N + 3 <= 2 * BR_N ? reinterpret_cast<uint8_t *>(par + N) : nullptr;
+    if (lost)
+        for (int i = tid; i < N; i += NTW) lost[i] = 0;
+    // Behind them, and on in the label bitmap's place, a byte hashed from each
+    // pixel's cell, as far as that goes (18,592 pixels with 4096-packet tiles):
+    // the other cells of a bucket cost no read of their record, which come from
+    // L2 (14% hits in L1)
+    constexpr int TAG2 = 6 * BR_LW;                              // bytes of lbits and lpre
+    const int tag1 = lost ? 2 * (BR_N - N) - N : 0;
+    uint8_t *tags1 = reinterpret_cast<uint8_t *>(par + N) + N, *tags2 = reinterpret_cast<uint8_t *>(lbits);
+    auto tag_of = [&](uint32_t cell) -> unsigned { return (cell * 0x85EBCA6Bu) >> 24; };
+    cta_sync();
+    // ---- the cell chains: the last pixel of a bucket first ----
+    constexpr unsigned NONE = 0xFFFFu;
+    auto bucket = [&](uint32_t cell) -> unsigned { return __umulhi(cell * 0x9E3779B1u, (unsigned)BR_BINS); };
+    for (int b = tid; b < BR_BINS; b += NTW) bins[b] = NONE;
+    cta_sync();
+    for (int i = tid; i < N; i += NTW) {
+        const uint32_t cell = r_cell(g_srec[i]);
+        const unsigned prev = atomicExch(&bins[bucket(cell)], (unsigned)i);
+        if (i < BR_NX) nx_sh[i] = (uint16_t)prev; else nx_g[i] = (uint16_t)prev;
+        if (i < tag1) tags1[i] = (uint8_t)tag_of(cell);
+        else if (i - tag1 < TAG2) tags2[i - tag1] = (uint8_t)tag_of(cell);
+    }
     cta_sync();
 
     BR_PH(22);
-    // ---- neighbour pass: every pixel of the sorted order is checked against
-    // the keys that can hold its earlier neighbours (the box rule, Sec. V.A);
-    // an adjacent pair clears the loser's local-maximum flag (Sec. V.B: the
-    // larger ToT wins, equal ToT goes to the later pixel) and unites. The
-    // sorted records are read through shared memory: BR_CH pixels at a time,
-    // staged with the records before them from the start of the first one's
-    // previous time bin (or straight from the scratch when those do not fit) ----
-    auto kstart = [&](int k) -> int { return k > 0 ? (int)bins[k - 1] : 0; };   // a key's first slot
-    for (int a = 0; a < N; a += BR_CH) {
-        const int e = min(N, a + BR_CH);
-        int lo;
-        {
-            const uint64_t ra = g_srec[a];
-            const int s = r_seg(ra);
-            const int tbin = sg_b0[s] + (r_tof(ra) - sg_lo[s]) / sg_w[s];
-            const int k0 = (tbin > sg_b0[s] ? tbin - 1 : tbin) * NS;
-            lo = k0 > 0 ? (int)bins[k0 - 1] : 0;
+    // ---- neighbour pass: every pixel against the chains of the cells that can
+    // hold its neighbours (the box rule, Sec. V.A); an adjacent pair clears the
+    // loser's local-maximum flag (Sec. V.B: the larger ToT wins, equal ToT goes
+    // to the later pixel). A pixel points to the first neighbour it finds: its
+    // own entry only, and pointers go forward in a strict order (cell, then
+    // slot), so they form a forest without a single compare-and-swap. The next
+    // three neighbours are kept aside. Consecutive slots are mostly one
+    // cluster, so a warp's chains are near each other and its records in L1 ----
+    // the first pixel from j on along its chain that may be of the cell (own:
+    // only those before pixel i), NONE at the end
+    auto next_of = [&](int i, uint32_t cell, unsigned j, bool own) -> unsigned {
+        const unsigned tag = tag_of(cell);
+        while (j != NONE) {
+            if (!TPX_IN(j, N)) return NONE;
+            const int k = (int)j - tag1;
+            const unsigned t = k < 0 ? tags1[j] : k < TAG2 ? tags2[k] : tag;
+            if (t == tag && !(own && j >= (unsigned)i)) return j;
+            j = j < (unsigned)BR_NX ? nx_sh[j] : nx_g[j];
         }
-        const bool fits = e - lo <= BR_SB;
-        if (tid == 0) misc[12] = 0;   // the chunk's task counter
-        if (fits)
-            for (int j = lo + tid; j < e; j += NTW) sbuf[j - lo] = g_srec[j];
-        cta_sync();
-        auto rec_at = [&](int j) -> uint64_t { return fits ? sbuf[j - lo] : g_srec[j]; };
-        // A warp takes 32 consecutive pixels at a time, the next task from the
-        // chunk's counter (dense stretches take longer). A pixel's candidates
-        // are two runs of consecutive slots: the previous bin's stripes around
-        // its own (consecutive keys), and its own bin's left stripe with its
-        // own key up to itself. The warp spreads all its (pixel, candidate)
-        // pairs evenly over its lanes: a prefix of the pixels' candidate
-        // counts, and each lane finds the pixel of its pair by a search over
-        // the lanes.
-        const int ntask = (e - a + 31) >> 5;
-        for (;;) {
-            int task = 0;
-            if (lane == 0) task = atomicAdd(&misc[12], 1);
-            task = __shfl_sync(0xffffffffu, task, 0);
-            if (task >= ntask) break;
-            const int i0 = a + 32 * task;
-            const int i = i0 + lane;
-            int a0 = 0, la = 0, b0 = 0, lb = 0;
-            if (i < e) {
-                const uint64_t ri = rec_at(i);
-                const int s = r_seg(ri);
-                const int tbin = sg_b0[s] + (r_tof(ri) - sg_lo[s]) / sg_w[s];
-                const int st = r_x(ri) / SW;
-                if (tbin > sg_b0[s]) {
-                    a0 = kstart((tbin - 1) * NS + max(st - 1, 0));
-                    la = (int)bins[(tbin - 1) * NS + min(st + 1, NS - 1)] - a0;
-                }
-                b0 = kstart(tbin * NS + max(st - 1, 0));
-                lb = i - b0;
+        return NONE;
+    };
+    auto link = [&](unsigned j) -> unsigned { return j < (unsigned)BR_NX ? nx_sh[j] : nx_g[j]; };
+    // every neighbour of pixel i among the forward half of its box
+    auto walk_all = [&](int i, uint64_t ri, auto pair) {
+        const int x = r_x(ri), y = r_y(ri), tb = r_tof(ri);
+        const uint32_t seg = r_cell(ri) & ~0xFFFFu;
+        auto cell_at = [&](int cx, int cy) -> uint32_t { return seg | ((uint32_t)cy << 8) | (uint32_t)cx; };
+        auto first_of = [&](int cx, int cy, bool own) -> unsigned {
+            if (cx > 255 || cy < 0 || cy > 255) return NONE;
+            return next_of(i, cell_at(cx, cy), bins[bucket(cell_at(cx, cy))], own);
+        };
+        // the chain from its first candidate j on, whose record is r
+        auto walk = [&](uint32_t cell, unsigned j, uint64_t r, bool own) {
+            while (j != NONE) {
+                if (r_cell(r) == cell && within(r_tof(r) - tb, dtr)) pair(j, r);
+                j = next_of(i, cell, link(j), own);
+                if (j != NONE) r = g_srec[j];
             }
-            const int n = la + lb;
-            int incl = n;
+        };
+        if (rx == 1 && ry == 1) {   // the five cells' first candidates, then their records together
+            unsigned j[5];
+            uint64_t r[5];
+            j[0] = first_of(x, y, true);
+            j[1] = first_of(x, y + 1, false);
+            j[2] = first_of(x + 1, y, false);
+            j[3] = first_of(x + 1, y - 1, false);
+            j[4] = first_of(x + 1, y + 1, false);
 #pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int u = __shfl_up_sync(0xffffffffu, incl, o);
-                if (lane >= o) incl += u;
-            }
-            const int off = incl - n;
-            const int W = __shfl_sync(0xffffffffu, incl, 31);
-            for (int wb = 0; wb < W; wb += 32) {
-                const int w = wb + lane;
-                int q = 0;   // the last lane whose pairs start at or before w
-#pragma unroll
-                for (int step = 16; step > 0; step >>= 1) {
-                    const int o = __shfl_sync(0xffffffffu, off, q + step);
-                    if (o <= w) q += step;
+            for (int k = 0; k < 5; ++k) r[k] = j[k] != NONE ? g_srec[j[k]] : 0ull;
+            walk(cell_at(x, y), j[0], r[0], true);
+            walk(cell_at(x, y + 1), j[1], r[1], false);
+            walk(cell_at(x + 1, y), j[2], r[2], false);
+            walk(cell_at(x + 1, y - 1), j[3], r[3], false);
+            walk(cell_at(x + 1, y + 1), j[4], r[4], false);
+        } else {
+            for (int dx = 0; dx <= rx; ++dx)
+                for (int dy = dx == 0 ? 0 : -ry; dy <= ry; ++dy) {
+                    const bool own = dx == 0 && dy == 0;
+                    const unsigned j = first_of(x + dx, y + dy, own);
+                    if (j != NONE) walk(cell_at(x + dx, y + dy), j, g_srec[j], own);
                 }
-                const int qa0 = __shfl_sync(0xffffffffu, a0, q), qla = __shfl_sync(0xffffffffu, la, q);
-                const int qb0 = __shfl_sync(0xffffffffu, b0, q), qoff = __shfl_sync(0xffffffffu, off, q);
-                if (w >= W) continue;
-                const int c = w - qoff;
-                const int ip = i0 + q;
-                const int j = c < qla ? qa0 + c : qb0 + (c - qla);
-                const uint64_t rp = rec_at(ip), rj = rec_at(j);
-                const int dx = r_x(rj) - r_x(rp), dy = r_y(rj) - r_y(rp);
-                if (dx < -rx || dx > rx || dy < -ry || dy > ry || !within(r_tof(rj) - r_tof(rp), dtr)) continue;
-                const int tj = r_tot(rj), tp = r_tot(rp);
-                const bool j_wins = tj > tp || (tj == tp && g_spos[j] > g_spos[ip]);
-                const int loser = j_wins ? ip : j;
-                br_or(nb_sh + 4 * (loser >> 5), 1u << (loser & 31));
-                br_unite(pb, (unsigned)ip, (unsigned)j);
-            }
         }
-        cta_sync();
+    };
+    for (int i0 = wid * 32; i0 < N; i0 += NTW) {
+        const int i = i0 + lane;
+        bool own_lost = false;
+        if (i < N) {
+            const uint64_t ri = g_srec[i];
+            const int ti = r_tot(ri);
+            unsigned n = 0;
+            uint64_t more = 0;
+            walk_all(i, ri, [&](unsigned j, uint64_t rj) {
+                const int tj = r_tot(rj);
+                const bool j_wins = tj > ti || (tj == ti && g_spos[j] > g_spos[i]);
+                if (j_wins) own_lost = true;
+                else if (lost) lost[j] = 1;
+                else br_or(nb_sh + 4 * (j >> 5), 1u << (j & 31));
+                if (n == 0) br_st(pb, (unsigned)i, j);
+                else if (n <= 3) more |= (uint64_t)j << (16 * (n - 1));
+                n = min(n + 1, 5u);
+            });
+            g_more[i] = more | ((uint64_t)n << 48);
+        }
+        const unsigned w = __ballot_sync(0xffffffffu, own_lost);   // 32 consecutive slots: one word
+        if (lane == 0 && w) br_or(nb_sh + 4 * (i0 >> 5), w);
     }
+    cta_sync();
+    // every pixel to its root, then the pairs that the pointers left out: the
+    // two ends have one root already, nearly always (with a union for each of
+    // the 4 pairs per pixel, lanes of one cluster met in the same
+    // compare-and-swaps and flag words: this pass took 1.1e6 cycles of the
+    // path's 1.5e6 per shot of 15,500 pixels, now 0.33e6 of 0.73e6; 600 such
+    // shots 4.1 -> 2.35 ms)
+    for (int i = tid; i < N; i += NTW) {
+        unsigned r = br_ld(pb, (unsigned)i);
+        for (unsigned up = br_ld(pb, r); up != r; up = br_ld(pb, r)) r = up;
+        br_st(pb, (unsigned)i, r);
+    }
+    if (lost)
+        for (int i0 = wid * 32; i0 < N; i0 += NTW) {
+            const unsigned w = __ballot_sync(0xffffffffu, i0 + lane < N && lost[i0 + lane]);
+            if (lane == 0 && w) br_or(nb_sh + 4 * (i0 >> 5), w);
+        }
+    cta_sync();
+    for (int i = tid; i < N; i += NTW) {
+        const uint64_t more = g_more[i];
+        const unsigned n = (unsigned)(more >> 48);
+        auto join = [&](unsigned j) {
+            if (TPX_IN(j, N) && br_ld(pb, (unsigned)i) != br_ld(pb, j)) br_unite(pb, (unsigned)i, j);
+        };
+        if (n <= 4) {
+            for (unsigned k = 1; k < n; ++k) join((unsigned)(more >> (16 * (k - 1))) & 0xFFFFu);
+        } else {
+            walk_all(i, g_srec[i], [&](unsigned j, uint64_t) { join(j); });
+        }
+    }
+    cta_sync();
+    for (int w = tid; w < BR_LW; w += NTW) lbits[w] = 0u;
     BR_PH(23);
     // compress: every pixel points to its root
     for (int i = tid; i < N; i += NTW) br_st(pb, (unsigned)i, br_find(pb, (unsigned)i));
@@ -1287,21 +1363,40 @@ __device__ __noinline__ int big_range(Smem &S, const Params &p, long long base, 
     }
     // ---- per-packet outputs over the range's label span ----
     if (p.labels || p.labels32 || p.is_peak) {
-        for (int i = tid; i < N; i += NTW) {
-            const long long q = g_spos[i];
-            const unsigned lp = (unsigned)(__ldcg(&g_mom[par[i]].best) & 0xFFFFu);
-            const uint8_t pk = ((npk[i >> 5] >> (i & 31)) & 1u) ? 0 : 1;
-            if (!TPX_IN(base + q, rend)) continue;
-            if (p.labels) p.labels[base + q] = p.idx_base + base + lp;
-            else if (p.labels32) p.labels32[base + q] = (int)(p.idx_base - p.lab32_base + base + lp);
-            if (p.is_peak) p.is_peak[base + q] = pk;
+        for (int i0 = tid; i0 < N; i0 += 4 * NTW) {
+            unsigned q4[4], lp4[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int i = i0 + u * NTW;
+                q4[u] = i < N ? g_spos[i] : 0u;
+                lp4[u] = i < N ? (unsigned)(__ldcg(&g_mom[par[i]].best) & 0xFFFFu) : 0u;
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int i = i0 + u * NTW;
+                if (i >= N) break;
+                const long long q = q4[u];
+                const unsigned lp = lp4[u];
+                const uint8_t pk = ((npk[i >> 5] >> (i & 31)) & 1u) ? 0 : 1;
+                if (!TPX_IN(base + q, rend)) continue;
+                if (p.labels) p.labels[base + q] = p.idx_base + base + lp;
+                else if (p.labels32) p.labels32[base + q] = (int)(p.idx_base - p.lab32_base + base + lp);
+                if (p.is_peak) p.is_peak[base + q] = pk;
+            }
         }
         const int W0 = prev_global ? f : 0, W1 = term ? L - 1 : L;
-        for (int q = W0 + tid; q < W1; q += NTW) {
-            if (g_rec[q] != INVALID || !TPX_IN(base + q, rend)) continue;
-            if (p.labels) p.labels[base + q] = -1LL;
-            else if (p.labels32) p.labels32[base + q] = -1;
-            if (p.is_peak) p.is_peak[base + q] = 0;
+        for (int q0 = W0 + tid; q0 < W1; q0 += 4 * NTW) {
+            uint64_t r[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) r[u] = q0 + u * NTW < W1 ? g_rec[q0 + u * NTW] : 0ull;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int q = q0 + u * NTW;
+                if (q >= W1 || r[u] != INVALID || !TPX_IN(base + q, rend)) continue;
+                if (p.labels) p.labels[base + q] = -1LL;
+                else if (p.labels32) p.labels32[base + q] = -1;
+                if (p.is_peak) p.is_peak[base + q] = 0;
+            }
         }
     }
     cta_sync();
