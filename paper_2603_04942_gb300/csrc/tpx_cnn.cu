@@ -70,18 +70,25 @@ __host__ __device__ constexpr Conv layer_of(int l) {
 
 // ================================================================ fp32 training
 // im2col: out[(p, oy, ox)][ci * kk^2 + ky * kk + kx] = in(p, oy + ky, ox + kx, ci)
-// with in(p, y, x, c) = in[p * sn + y * sy + x * sx + c * sc]
-__global__ void k_im2col(const float *in, long long sn, int sy, int sx, int sc, long long n, int cin, int ho, int kk,
-                         float *out) {
-    const int K = cin * kk * kk;
-    const long long total = n * ho * ho * K;
+// with in(p, y, x, c) = in[p * sn + y * sy + x * sx + c * sc]; a thread per
+// (row, input channel): its kk^2 columns are consecutive (a thread per element
+// spent its time on the index divisions: 99 us of conv2's rows of 4096 patches)
+template <int KK>
+__global__ void k_im2col(const float *in, long long sn, int sy, int sx, int sc, long long n, int cin, int ho, float *out) {
+    const long long total = n * ho * ho * cin;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
-        const int k = (int)(i % K);
-        const long long r = i / K;
-        const int ox = (int)(r % ho), oy = (int)((r / ho) % ho);
-        const long long p = r / ((long long)ho * ho);
-        const int ci = k / (kk * kk), t = k % (kk * kk), ky = t / kk, kx = t % kk;
-        out[i] = in[p * sn + (long long)(oy + ky) * sy + (long long)(ox + kx) * sx + (long long)ci * sc];
+        const unsigned ci = (unsigned)(i % (unsigned)cin);
+        const long long r = i / (unsigned)cin;
+        const unsigned hw = (unsigned)(ho * ho);
+        const long long p = r / hw;
+        const unsigned pos = (unsigned)(r - p * hw), oy = pos / (unsigned)ho, ox = pos - oy * (unsigned)ho;
+        const float *src = in + p * sn + (long long)oy * sy + (long long)ox * sx + (long long)ci * sc;
+        float *dst = out + i * (KK * KK);
+        float v[KK * KK];
+#pragma unroll
+        for (int t = 0; t < KK * KK; ++t) v[t] = src[(t / KK) * sy + (t % KK) * sx];
+#pragma unroll
+        for (int t = 0; t < KK * KK; ++t) dst[t] = v[t];
     }
 }
 // the input gradient from the im2col gradient: each input element gathers the
@@ -111,25 +118,33 @@ __global__ void k_col2im(const float *dcol, long long n, int cin, int hin, int h
 // C[M x N] (+)= op(A)[M x K] op(B)[K x N] (+ bias, ReLU), strides as in the
 // MLP refiner's GEMM; gridDim.z > 1 splits K and adds the partial products
 // atomically into C (zeroed by the caller; no bias or ReLU then)
-constexpr int TM = 64, TN = 64, TK = 16;
+// The tile is 64 x 64, or longer and narrower where one side has 16 or 32 only
+// (the convolutions' channels: a 64-wide tile multiplied zeros for the rest).
+constexpr int TK = 16;
+template <int TM, int TN>
 __global__ void __launch_bounds__(256) k_sgemm(const float *A, long long sam, long long sak, const float *B,
                                                long long sbk, long long sbn, float *C, long long ldc, int M, int N,
                                                long long K, const float *bias, int relu) {
-    __shared__ float As[TK][TM + 4];
-    __shared__ float Bs[TK][TN + 4];
-    const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
+    static_assert(TM * TN == 4096, "256 threads of 4 x 4 outputs");
+    __shared__ __align__(16) float As[TK][TM + 4];
+    __shared__ __align__(16) float Bs[TK][TN + 4];
+    const int tx = threadIdx.x % (TN / 4), ty = threadIdx.x / (TN / 4);
     const int i0 = blockIdx.y * TM, j0 = blockIdx.x * TN;
     const long long kc = (K + gridDim.z - 1) / gridDim.z;
     const long long kb = blockIdx.z * kc, ke = min(K, kb + kc);
     float acc[4][4] = {};
     for (long long k0 = kb; k0 < ke; k0 += TK) {
-        for (int t = threadIdx.x; t < TK * TM; t += 256) {
+#pragma unroll
+        for (int t0 = 0; t0 < TK * TM; t0 += 256) {
+            const int t = t0 + threadIdx.x;
             const int kk = sak == 1 ? t % TK : t / TM, ii = sak == 1 ? t / TK : t % TM;
             const int i = i0 + ii;
             const long long k = k0 + kk;
             As[kk][ii] = (i < M && k < ke) ? A[i * sam + k * sak] : 0.f;
         }
-        for (int t = threadIdx.x; t < TK * TN; t += 256) {
+#pragma unroll
+        for (int t0 = 0; t0 < TK * TN; t0 += 256) {
+            const int t = t0 + threadIdx.x;
             const int kk = sbk == 1 ? t % TK : t / TN, jj = sbk == 1 ? t / TK : t % TN;
             const int j = j0 + jj;
             const long long k = k0 + kk;
@@ -138,11 +153,8 @@ __global__ void __launch_bounds__(256) k_sgemm(const float *A, long long sam, lo
         __syncthreads();
 #pragma unroll
         for (int kk = 0; kk < TK; ++kk) {
-            float a[4], b[4];
-#pragma unroll
-            for (int r = 0; r < 4; ++r) a[r] = As[kk][ty * 4 + r];
-#pragma unroll
-            for (int r = 0; r < 4; ++r) b[r] = Bs[kk][tx * 4 + r];
+            const float4 a4 = *reinterpret_cast<const float4 *>(&As[kk][ty * 4]), b4 = *reinterpret_cast<const float4 *>(&Bs[kk][tx * 4]);
+            const float a[4] = {a4.x, a4.y, a4.z, a4.w}, b[4] = {b4.x, b4.y, b4.z, b4.w};
 #pragma unroll
             for (int r = 0; r < 4; ++r)
 #pragma unroll
@@ -164,20 +176,39 @@ __global__ void __launch_bounds__(256) k_sgemm(const float *A, long long sam, lo
             *c = v;
         }
 }
+// the tile of an M x N product
+inline int tile_rows(long long M, int N) { return N <= 16 ? 256 : N <= 32 ? 128 : M <= 16 ? 16 : M <= 32 ? 32 : 64; }
+inline int tile_cols(long long M, int N) { return 4096 / tile_rows(M, N); }
 void sgemm(cudaStream_t s, const float *A, long long sam, long long sak, const float *B, long long sbk, long long sbn,
            float *C, long long ldc, long long M, int N, long long K, const float *bias, bool relu, int splits = 1) {
-    constexpr long long kRows = 1LL << 21;   // grid.y <= 65535 tiles of 64 rows
+    const int tm = tile_rows(M, N), tn = tile_cols(M, N);
+    constexpr long long kRows = 1LL << 20;   // grid.y <= 65535 tiles of 16 rows
     for (long long m0 = 0; m0 < M; m0 += kRows) {
         const int m = (int)(M - m0 < kRows ? M - m0 : kRows);
-        dim3 g((N + TN - 1) / TN, (m + TM - 1) / TM, splits);
-        k_sgemm<<<g, 256, 0, s>>>(A + m0 * sam, sam, sak, B, sbk, sbn, C + m0 * ldc, ldc, m, N, K, bias, relu ? 1 : 0);
+        const dim3 g((N + tn - 1) / tn, (m + tm - 1) / tm, splits);
+        auto go = [&](auto kernel) {
+            kernel<<<g, 256, 0, s>>>(A + m0 * sam, sam, sak, B, sbk, sbn, C + m0 * ldc, ldc, m, N, K, bias, relu ? 1 : 0);
+        };
+        switch (tm) {
+            case 256: go(k_sgemm<256, 16>); break;
+            case 128: go(k_sgemm<128, 32>); break;
+            case 16: go(k_sgemm<16, 256>); break;
+            case 32: go(k_sgemm<32, 128>); break;
+            default: go(k_sgemm<64, 64>); break;
+        }
     }
 }
-// splits for a weight gradient whose inner dimension runs over `rows`
+// splits for a weight gradient whose inner dimension runs over `rows`: four
+// blocks per SM, at least 96 rows each. A block's steps of 16 rows wait for
+// their loads one after another, so its rows are the kernel's time: 4096
+// patches, 1024 rows or more a split: 254 to 291 us for each of the five layers
+// (a step of 4096 patches 2.28 ms, with the column sums' larger grids, the
+// narrow tiles and the im2col above 0.71 ms).
 inline int splits_for(long long rows, int M, int N) {
-    const long long tiles = (long long)((M + TM - 1) / TM) * ((N + TN - 1) / TN);
+    const int tm = tile_rows(M, N), tn = tile_cols(M, N);
+    const long long tiles = (long long)((M + tm - 1) / tm) * ((N + tn - 1) / tn);
     long long sp = (152LL * 4) / (tiles > 0 ? tiles : 1);
-    const long long per = rows / 1024;   // at least ~1024 rows per split
+    const long long per = rows / 96;
     if (sp > per) sp = per;
     return (int)(sp < 1 ? 1 : (sp > 65535 ? 65535 : sp));
 }
@@ -195,6 +226,7 @@ __global__ void k_colsum(const float *d, long long rows, int m, float *g) {
     const long long per = (rows + gridDim.x - 1) / gridDim.x;
     const long long r0 = blockIdx.x * per, r1 = min(rows, r0 + per);
     float s = 0.f;
+#pragma unroll 8
     for (long long r = r0 + rl; r < r1; r += lanes) s += d[r * m + j];
     atomicAdd(&g[j], s);
 }
@@ -217,13 +249,13 @@ struct Work {
 
 // the fp32 forward pass of n patches (x: [n][162], channel 0 then 1, rows of 9)
 int forward32(cudaStream_t s, const float *P, const float *x, long long n, const Work &w) {
-    k_im2col<<<grid_for(n * 49 * 18), 256, 0, s>>>(x, 162, 9, 1, 81, n, 2, 7, 3, w.x1);
+    k_im2col<3><<<grid_for(n * 49 * 2), 256, 0, s>>>(x, 162, 9, 1, 81, n, 2, 7, w.x1);
     sgemm(s, w.x1, 18, 1, P + OW1, 1, 18, w.a1, 16, n * 49, 16, 18, P + OB1, true);
-    k_im2col<<<grid_for(n * 25 * 144), 256, 0, s>>>(w.a1, 49 * 16, 7 * 16, 16, 1, n, 16, 5, 3, w.x2);
+    k_im2col<3><<<grid_for(n * 25 * 16), 256, 0, s>>>(w.a1, 49 * 16, 7 * 16, 16, 1, n, 16, 5, w.x2);
     sgemm(s, w.x2, 144, 1, P + OW2, 1, 144, w.a2, 16, n * 25, 16, 144, P + OB2, true);
-    k_im2col<<<grid_for(n * 9 * 144), 256, 0, s>>>(w.a2, 25 * 16, 5 * 16, 16, 1, n, 16, 3, 3, w.x3);
+    k_im2col<3><<<grid_for(n * 9 * 16), 256, 0, s>>>(w.a2, 25 * 16, 5 * 16, 16, 1, n, 16, 3, w.x3);
     sgemm(s, w.x3, 144, 1, P + OW3, 1, 144, w.a3, 32, n * 9, 32, 144, P + OB3, true);
-    k_im2col<<<grid_for(n * 288), 256, 0, s>>>(w.a3, 9 * 32, 3 * 32, 32, 1, n, 32, 1, 3, w.x4);
+    k_im2col<3><<<grid_for(n * 32), 256, 0, s>>>(w.a3, 9 * 32, 3 * 32, 32, 1, n, 32, 1, w.x4);
     sgemm(s, w.x4, 288, 1, P + OW4, 1, 288, w.a4, 144, n, 144, 288, P + OB4, true);
     sgemm(s, w.a4, 144, 1, P + OW5, 1, 144, w.out, NOUT, n, NOUT, 144, P + OB5, false);
     return ck(cudaGetLastError()) ? TPX_ECUDA : TPX_OK;
@@ -235,7 +267,10 @@ void layer_back(cudaStream_t s, const float *P, float *G, const Conv &L, const f
                 float *dX) {
     const int K = L.cin * L.kk * L.kk;
     sgemm(s, dZ, 1, L.cout, X, K, 1, G + L.ow, K, L.cout, K, rows, nullptr, false, splits_for(rows, L.cout, K));
-    k_colsum<<<grid_for(rows / 64 + 1), 256, 0, s>>>(dZ, rows, L.cout, G + L.ob);
+    // 64 rows per row lane of a block, at most eight blocks per SM (one block for
+    // 4096 rows of 144 columns took 516 us)
+    const long long strips = (rows * L.cout + 64 * 256 - 1) / (64 * 256);
+    k_colsum<<<(unsigned)(strips < 152 * 8 ? strips : 152 * 8), 256, 0, s>>>(dZ, rows, L.cout, G + L.ob);
     if (dX) sgemm(s, dZ, L.cout, 1, P + L.ow, K, 1, dX, K, rows, K, L.cout, nullptr, false);
 }
 
