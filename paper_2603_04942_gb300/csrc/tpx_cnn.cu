@@ -381,29 +381,38 @@ __global__ void k_cnn_pack(const float *P, __nv_bfloat16 *wt, float *bias) {
 // of its input grid (the rows outside the valid window are computed and
 // dropped), so the A operand of kernel tap (ky, kx) is the map itself shifted
 // by ky * W + kx rows -- a descriptor with its start moved, leading offset the
-// plane stride, stride offset one core matrix (8 rows). conv1's two channels
-// are packed with those of the two right-hand neighbours into one row
-// ([c0, c1] at x, x + 1, x + 2, then two zeros), so a k chunk is a kernel row.
-// Rows past the valid ones read stale (finite) contents of X; X starts zeroed.
-constexpr int FP = 48;                                // patches per group
-constexpr int R1 = FP * 81, T1 = (R1 + 127) / 128;    // conv1: rows of the 9 x 9 grid, MMA tiles
-constexpr int R2 = FP * 49, T2 = (R2 + 127) / 128;    // conv2: 7 x 7 grid
-constexpr int R3 = FP * 25, T3 = (R3 + 127) / 128;    // conv3: 5 x 5 grid
-constexpr int M1_ROWS = T1 * 128 + 27;                // conv1 reads up to the largest shift (18, then +9)
-constexpr int P1_ROWS = T2 * 128 + 16;                // conv2 input plane (shifts up to 2 * 7 + 2)
+// plane stride, stride offset one core matrix (8 rows). Rows past the valid
+// ones read stale (finite) contents of X; X starts zeroed.
+// The MMAs of the convolutions are bound by reading A from shared memory (45
+// cycles for 128 rows of 16, whatever N up to 32), so conv1 and conv2 compute
+// two neighbouring outputs per row: N = 2 x 16, a row per pair of positions.
+// conv1's rows hold the two channels of four positions from an even x on (a k
+// chunk is a kernel row), and each output's weights are zero at the position it
+// does not see; conv2 reads its input as one pair of planes per parity of x,
+// four taps per kernel row, again with zeros. Each output sums the same products
+// in the same order as with a row per position (equal outputs; 1,000,003 patches
+// 2245 -> 2008 us). Tried: two pipelines of 24 patches and eight warps per CTA, to
+// run one's MMAs beside the other's epilogue: 2504 us, both want shared memory.
+constexpr int FP = 44;                                // patches per group
+constexpr int C1 = 45, C2 = 28, C3 = 25;              // rows of a patch: conv1 9 x 5 pairs, conv2 7 x 4 pairs, conv3 5 x 5
+constexpr int R1 = FP * C1, T1 = (R1 + 127) / 128;    // rows, MMA tiles
+constexpr int R2 = FP * C2, T2 = (R2 + 127) / 128;
+constexpr int R3 = FP * C3, T3 = (R3 + 127) / 128;
+constexpr int M1_ROWS = T1 * 128 + 16;                // conv1 reads up to the largest shift (10, then +5)
+constexpr int P1_ROWS = T2 * 128 + 12;                // conv2 input plane (shifts up to 2 * 4 + 1)
 constexpr int P2_ROWS = T3 * 128 + 12;                // conv3 input plane (shifts up to 2 * 5 + 2)
 constexpr int PLB = FP * 16;                          // dense-layer input plane: one row per patch
 constexpr size_t cmax(size_t a, size_t b) { return a > b ? a : b; }
 constexpr size_t X_BYTES =
-    ((cmax(cmax((size_t)M1_ROWS * 16, (size_t)2 * P1_ROWS * 16),
+    ((cmax(cmax((size_t)M1_ROWS * 16, (size_t)4 * P1_ROWS * 16),
            cmax((size_t)2 * P2_ROWS * 16, cmax((size_t)(35 * FP + 128) * 16, (size_t)(17 * FP + 128) * 16))) +
       127) / 128) * 128;
-constexpr size_t W1B = 16 * 32 * 2, W2B = 16 * 144 * 2, W3B = 32 * 144 * 2, W4B = 144 * 288 * 2, W5B = 16 * 144 * 2;
+constexpr size_t W1B = 32 * 32 * 2, W2B = 32 * 192 * 2, W3B = 32 * 144 * 2, W4B = 144 * 288 * 2, W5B = 16 * 144 * 2;
 constexpr size_t W_BYTES = W1B + W2B + W3B + W4B + W5B;
 constexpr size_t RAW_BYTES = (size_t)FP * 162 * 2;    // one group of bf16 patches
 constexpr size_t BIAS_BYTES = ((Packed::bend * 4 + 127) / 128) * 128;
 constexpr size_t FUSED_SMEM = 1024 + W_BYTES + X_BYTES + 2 * RAW_BYTES + BIAS_BYTES + 64;
-static_assert(T1 * 16 <= 512 && T2 * 16 <= 512 && T3 * 32 <= 512 && FP <= 128, "tensor memory of a group");
+static_assert(T1 * 32 <= 512 && T2 * 32 <= 512 && T3 * 32 <= 512 && FP <= 128, "tensor memory of a group");
 static_assert(FUSED_SMEM <= 227 * 1024, "shared memory of the fused kernel");
 static_assert(RAW_BYTES % 16 == 0 && W_BYTES % 128 == 0, "16-byte copies");
 
@@ -504,8 +513,19 @@ __global__ void __launch_bounds__(CNN_THREADS, 1) k_cnn_fused(const __nv_bfloat1
     const int quad = warp & 3, sub = warp >> 2;   // accumulator lanes 32 * quad.., and which share of the columns
     const long long groups = (n + FP - 1) / FP;
 
-    load_weights(W1, wt + Q::w1, 16, 32);
-    load_weights(W2, wt + Q::w2, 16, 144);
+    // conv1 and conv2: output u * 16 + co is channel co at the pair's position u
+    for (int i = tid; i < 32 * 32; i += CNN_THREADS) {
+        const int r = i / 32, k = i % 32, ky = k / 8, kx = (k % 8) / 2 - r / 16, c = k & 1;
+        const bool in = ky < 3 && kx >= 0 && kx < 3;
+        *reinterpret_cast<__nv_bfloat16 *>(W1 + core_off(r, k, 32)) =
+            in ? wt[Q::w1 + (r % 16) * 32 + ky * 8 + kx * 2 + c] : __float2bfloat16_rn(0.f);
+    }
+    for (int i = tid; i < 32 * 24; i += CNN_THREADS) {   // 8 channels of a tap at a time
+        const int r = i / 24, c = i % 24, ky = c / 8, kx = (c / 2) % 4 - r / 16;
+        *reinterpret_cast<uint4 *>(W2 + core_off(r, c * 8, 192)) =
+            kx >= 0 && kx < 3 ? *reinterpret_cast<const uint4 *>(wt + Q::w2 + (r % 16) * 144 + (ky * 3 + kx) * 16 + (c & 1) * 8)
+                              : make_uint4(0, 0, 0, 0);
+    }
     load_weights(W3, wt + Q::w3, 32, 144);
     load_weights(W4, wt + Q::w4, 144, 288);
     load_weights(W5, wt + Q::w5, 16, 144);
@@ -564,23 +584,20 @@ __global__ void __launch_bounds__(CNN_THREADS, 1) k_cnn_fused(const __nv_bfloat1
         CNN_PH(0);
         // the next group's patches come in while this one runs
         if (g + gridDim.x < groups) load_group(RAW[(it + 1) & 1], x, n, g + gridDim.x);
-        // ---- conv1 input map: row (patch, y * 9 + x) = [c0, c1] at x, x + 1, x + 2, 0, 0 ----
+        // ---- conv1 input map: row (patch, y * 5 + x / 2) = [c0, c1] at x .. x + 3 (x even; zeros past the edge) ----
         {
             const __nv_bfloat16 *pr = reinterpret_cast<const __nv_bfloat16 *>(raw);
             for (int r = tid; r < R1; r += CNN_THREADS) {
-                const int pp = r / 81, pos = r % 81, xx = pos % 9;
-                const __nv_bfloat16 *c0 = pr + pp * 162 + pos, *c1 = c0 + 81;
+                const int pp = r / C1, pos = r % C1, yy = pos / 5, xx = 2 * (pos % 5);
+                const __nv_bfloat16 *c0 = pr + pp * 162 + yy * 9 + xx, *c1 = c0 + 81;
                 const __nv_bfloat16 z = __float2bfloat16_rn(0.f);
-                __nv_bfloat162 v0 = __halves2bfloat162(c0[0], c1[0]);
-                __nv_bfloat162 v1 = xx + 1 < 9 ? __halves2bfloat162(c0[1], c1[1]) : __halves2bfloat162(z, z);
-                __nv_bfloat162 v2 = xx + 2 < 9 ? __halves2bfloat162(c0[2], c1[2]) : __halves2bfloat162(z, z);
-                __nv_bfloat162 v3 = __halves2bfloat162(z, z);
-                uint4 row;
-                row.x = *reinterpret_cast<uint32_t *>(&v0);
-                row.y = *reinterpret_cast<uint32_t *>(&v1);
-                row.z = *reinterpret_cast<uint32_t *>(&v2);
-                row.w = *reinterpret_cast<uint32_t *>(&v3);
-                reinterpret_cast<uint4 *>(X)[r] = row;
+                uint32_t v[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const __nv_bfloat162 w = xx + u < 9 ? __halves2bfloat162(c0[u], c1[u]) : __halves2bfloat162(z, z);
+                    v[u] = *reinterpret_cast<const uint32_t *>(&w);
+                }
+                reinterpret_cast<uint4 *>(X)[r] = make_uint4(v[0], v[1], v[2], v[3]);
             }
         }
         CNN_PH(1);
@@ -588,61 +605,62 @@ __global__ void __launch_bounds__(CNN_THREADS, 1) k_cnn_fused(const __nv_bfloat1
         if (!run_layer([&](int q) {
                 // a descriptor's start field counts 16-byte units: one row, or
                 // 256 bytes = 16 for the next two k chunks of the weights
-                const uint32_t id = idesc_bf16(16);
-                const uint64_t da = sdesc(xs, 144, 128), db = sdesc(smem_u32(W1), 128, 512);
+                const uint32_t id = idesc_bf16(32);
+                const uint64_t da = sdesc(xs, 5 * 16, 128), db = sdesc(smem_u32(W1), 128, 512);
                 // issuer q takes tiles q, q + 4, ...; the tiles' accumulators are
                 // independent, so consecutive MMAs go to different tiles and a
                 // tile's accumulation chain does not stall the pipe
-                for (int t = q; t < T1; t += 4) mma_bf16(tmem + 16 * t, da + (uint64_t)(t * 128), db, id, false);
-                for (int t = q; t < T1; t += 4) mma_bf16(tmem + 16 * t, da + (uint64_t)(t * 128 + 18), db + 16, id, true);
+                for (int t = q; t < T1; t += 4) mma_bf16(tmem + 32 * t, da + (uint64_t)(t * 128), db, id, false);
+                for (int t = q; t < T1; t += 4) mma_bf16(tmem + 32 * t, da + (uint64_t)(t * 128 + 10), db + 16, id, true);
             })) { failed = true; break; }
         CNN_PH(2);
-        // epilogue: the 7 x 7 window -> conv2 input planes; a warp takes two
-        // tiles (32 accumulator columns) of its lane quadrant per load
-        for (int t0 = 2 * sub; t0 < T1; t0 += 8) {
+        // epilogue: the 7 x 7 window -> conv2 input planes, one pair (channels
+        // 0-7, 8-15) per parity of x; their column x = 7 is zero
+        for (int t = sub; t < T1; t += 4) {
             uint32_t v[32];
-            tmem_ld32_nowait(tmem + lane_off + 16 * t0, v);
+            tmem_ld32_nowait(tmem + lane_off + 32 * t, v);
             tmem_wait_ld();
+            const int r = t * 128 + 32 * quad + lane;
+            const int pp = r / C1, pos = r % C1, yy = pos / 5, x2 = pos % 5;
+            if (pp < FP && yy < 7 && x2 < 4) {
+                const int o = pp * C2 + yy * 4 + x2;
 #pragma unroll
-            for (int u = 0; u < 2; ++u) {
-                const int t = t0 + u;
-                const int r = t * 128 + 32 * quad + lane;
-                const int pp = r / 81, pos = r % 81, yy = pos / 9, xx = pos % 9;
-                if (t < T1 && pp < FP && yy < 7 && xx < 7) {
+                for (int u = 0; u < 2; ++u) {
                     uint4 lo, hi;
                     relu_bf16x16(v + 16 * u, SB + Q::b1, &lo, &hi);
-                    const int o = pp * 49 + yy * 7 + xx;
-                    reinterpret_cast<uint4 *>(X)[o] = lo;
-                    reinterpret_cast<uint4 *>(X + (size_t)P1_ROWS * 16)[o] = hi;
+                    if (u == 1 && x2 == 3) lo = hi = make_uint4(0, 0, 0, 0);
+                    reinterpret_cast<uint4 *>(X)[(2 * u) * P1_ROWS + o] = lo;
+                    reinterpret_cast<uint4 *>(X)[(2 * u + 1) * P1_ROWS + o] = hi;
                 }
             }
         }
         CNN_PH(3);
-        // ---- conv2: one MMA per tap (16 channels = the two planes) ----
+        // ---- conv2: per kernel row four MMAs, the positions x .. x + 3 (16 channels = a pair of planes) ----
         if (!run_layer([&](int q) {
-                const uint32_t id = idesc_bf16(16);
-                const uint64_t da = sdesc(xs, P1_ROWS * 16, 128), db = sdesc(smem_u32(W2), 128, 18 * 128);
+                const uint32_t id = idesc_bf16(32);
+                const uint64_t da = sdesc(xs, P1_ROWS * 16, 128), db = sdesc(smem_u32(W2), 128, 24 * 128);
 #pragma unroll
-                for (int k = 0; k < 9; ++k)
+                for (int k = 0; k < 12; ++k)
                     for (int t = q; t < T2; t += 4)
-                        mma_bf16(tmem + 16 * t, da + (uint64_t)(t * 128 + (k / 3) * 7 + k % 3), db + 16 * k, id, k > 0);
+                        mma_bf16(tmem + 32 * t, da + (uint64_t)((k & 1) * 2 * P1_ROWS + t * 128 + (k / 4) * 4 + (k % 4) / 2),
+                                 db + 16 * k, id, k > 0);
             })) { failed = true; break; }
         CNN_PH(4);
-        for (int t0 = 2 * sub; t0 < T2; t0 += 8) {
+        for (int t = sub; t < T2; t += 4) {
             uint32_t v[32];
-            tmem_ld32_nowait(tmem + lane_off + 16 * t0, v);
+            tmem_ld32_nowait(tmem + lane_off + 32 * t, v);
             tmem_wait_ld();
+            const int r = t * 128 + 32 * quad + lane;
+            const int pp = r / C2, pos = r % C2, yy = pos / 4, x2 = pos % 4;
+            if (pp < FP && yy < 5 && x2 < 3) {
+                const int o = pp * C3 + yy * 5 + 2 * x2;
 #pragma unroll
-            for (int u = 0; u < 2; ++u) {
-                const int t = t0 + u;
-                const int r = t * 128 + 32 * quad + lane;
-                const int pp = r / 49, pos = r % 49, yy = pos / 7, xx = pos % 7;
-                if (t < T2 && pp < FP && yy < 5 && xx < 5) {
+                for (int u = 0; u < 2; ++u) {
+                    if (2 * x2 + u >= 5) continue;
                     uint4 lo, hi;
                     relu_bf16x16(v + 16 * u, SB + Q::b2, &lo, &hi);
-                    const int o = pp * 25 + yy * 5 + xx;
-                    reinterpret_cast<uint4 *>(X)[o] = lo;
-                    reinterpret_cast<uint4 *>(X + (size_t)P2_ROWS * 16)[o] = hi;
+                    reinterpret_cast<uint4 *>(X)[o + u] = lo;
+                    reinterpret_cast<uint4 *>(X + (size_t)P2_ROWS * 16)[o + u] = hi;
                 }
             }
         }
