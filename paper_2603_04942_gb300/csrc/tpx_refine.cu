@@ -140,17 +140,23 @@ __global__ void __launch_bounds__(SELT) k_select(const uint64_t *pk, const tpx_r
         const long long i = blockIdx.x * (long long)SELB + w * (32 * SELR) + 32 * j + lane;
         const long long s = (long long)first + o + __popc(m[j] & ((1u << lane) - 1u));
         o += __popc(m[j]);
-        if (i < ncl && i > 0 && cl[i - 1].label >= cl[i].label) info->odd = 1u;
-        if (!((m[j] >> lane) & 1u)) continue;
-        const tpx_record &c = cl[i];
-        const long long r = c.label - base;
-        if (r < 0 || r >= n) info->odd = 1u;
-        if (s >= cap) continue;
-        sel[s] = i;
-        if (r >= 0 && r < n) {
-            atomicMax(&tiles[r / PT].first_inv, 0xFFFFFFFFu - (unsigned)s);
-            atomicAdd(&tiles[r / PT].count, 1u);
+        const long long label = i < ncl ? cl[i].label : 0, r = label - base;
+        if (i < ncl && i > 0 && cl[i - 1].label >= label) info->odd = 1u;
+        const bool mine = (m[j] >> lane) & 1u, in = r >= 0 && r < n;
+        if (mine && !in) info->odd = 1u;
+        // the tile's count and first slot, once per warp and tile: the warp's
+        // slots follow one another, and so do their tiles
+        const unsigned put = __ballot_sync(0xffffffffu, mine && in && s < cap);
+        if ((put >> lane) & 1u) {
+            const unsigned tile = (unsigned)(r / PT), peers = __match_any_sync(put, tile);
+            if (lane == __ffs(peers) - 1) {
+                atomicMax(&tiles[tile].first_inv, 0xFFFFFFFFu - (unsigned)s);
+                atomicAdd(&tiles[tile].count, (unsigned)__popc(peers));
+            }
         }
+        if (!mine || s >= cap) continue;
+        const tpx_record &c = cl[i];
+        sel[s] = i;
         int cx = 0, cy = 0;
         if (c.s_tot > 0) {   // the centroid rounded half up, exactly: floor((2 s_x + s_tot) / (2 s_tot))
             const long long d = 2 * c.s_tot, nx = 2 * c.s_x + c.s_tot, ny = 2 * c.s_y + c.s_tot;
