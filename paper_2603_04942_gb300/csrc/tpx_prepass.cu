@@ -222,15 +222,100 @@ __global__ void __launch_bounds__(256) k_apply(const Params p, const GAgg *bpre)
 // packets of a tile are 64 dependent steps of one warp, and three launches
 // follow (37 shots, 5 tiles: 30 + 6 + 6 + 4 us; the whole call 112 us, with
 // this kernel and two memsets and a copy fewer 69 us; 1000 shots, 117 tiles:
-// 125 -> 82 us). Here a CTA takes a tile, its 32 warps two steps each; the
-// parts are combined by one warp. The CTA that
+// 125 -> 74 us). Here a CTA takes a tile, its 32 warps two steps each; the
+// parts are combined by one warp, from picks and sums (scans of whole aggregates
+// took 18 us of 117 tiles, this 14). The CTA that
 // finishes last (a counter in the control block) scans the aggregates of all
 // tiles and writes the states; nobody waits for anybody.
+// 32 consecutive stretches of one chain, lane by lane, without a scan of whole
+// aggregates: the step into a lane's stretch follows from the last value of the
+// nearest lane below that has one, the rest are sums and picks.
+struct LaneChain {
+    unsigned mask;      // lanes with values
+    int step;           // the wrap step into this lane's stretch
+    long long prev;     // the last value before it (any_prev: there is one)
+    bool any_prev;
+    __device__ __forceinline__ void link(const GChain &c, int lane, bool has_in, long long in, long long thr) {
+        mask = __ballot_sync(0xffffffffu, c.n > 0);
+        const unsigned lower = mask & ((1u << lane) - 1u);
+        const long long v = __shfl_sync(0xffffffffu, c.last, lower ? 31 - __clz(lower) : 0);
+        any_prev = lower || has_in;
+        prev = lower ? v : in;
+        step = c.n > 0 && any_prev ? (int)jump(c.first - prev, thr) : 0;
+    }
+    // lanes below `end` as one stretch
+    __device__ __forceinline__ GChain total(const GChain &c, int lane, int end) const {
+        const unsigned m = end >= 32 ? mask : mask & ((1u << end) - 1u);
+        GChain r;
+        r.n = __reduce_add_sync(0xffffffffu, lane < end ? (int)c.n : 0);
+        r.sum = __reduce_add_sync(0xffffffffu, lane < end ? (int)c.sum + step : 0);
+        r.first = __shfl_sync(0xffffffffu, c.first, m ? __ffs(m) - 1 : 0);
+        r.last = __shfl_sync(0xffffffffu, c.last, m ? 31 - __clz(m) : 0);
+        return m ? r : chain_id();
+    }
+};
+// one chain's state before each of up to 1024 tiles, a thread per tile, from
+// the state E before the first; *step: the wrap step into the tile
+struct ScanSm { int n[32], sum[32], has[32]; long long first[32], last[32]; };
+__device__ __forceinline__ GChain chain_before(const GChain &c, const GChain &E, ScanSm &S, bool one_warp, long long thr,
+                                               int *step) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    bool has_in = E.n > 0;
+    long long in = E.last, first = E.n > 0 ? E.first : 0;
+    bool has_first = E.n > 0;
+    LaneChain l;
+    if (!one_warp) {   // the warps before this one: their last value
+        const unsigned m = __ballot_sync(0xffffffffu, c.n > 0);
+        const long long f = __shfl_sync(0xffffffffu, c.first, m ? __ffs(m) - 1 : 0);
+        const long long z = __shfl_sync(0xffffffffu, c.last, m ? 31 - __clz(m) : 0);
+        if (lane == 0) {
+            S.has[w] = m != 0;
+            S.first[w] = f;
+            S.last[w] = z;
+        }
+        __syncthreads();
+        const unsigned mw = __ballot_sync(0xffffffffu, lane < w && S.has[lane]);
+        if (mw) {
+            in = S.last[31 - __clz(mw)];
+            has_in = true;
+            if (!has_first) first = S.first[__ffs(mw) - 1];
+            has_first = true;
+        }
+    }
+    l.link(c, lane, has_in, in, thr);
+    int n = (int)c.n, x = (int)c.sum + l.step;
+    const int own_n = n, own_x = x;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int a = __shfl_up_sync(0xffffffffu, n, o), b = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) { n += a; x += b; }
+    }
+    int bn = 0, bx = 0;
+    if (!one_warp) {
+        if (lane == 31) {
+            S.n[w] = n;
+            S.sum[w] = x;
+        }
+        __syncthreads();
+        bn = __reduce_add_sync(0xffffffffu, lane < w ? S.n[lane] : 0);
+        bx = __reduce_add_sync(0xffffffffu, lane < w ? S.sum[lane] : 0);
+    }
+    const unsigned lower = l.mask & ((1u << lane) - 1u);
+    const long long wf = __shfl_sync(0xffffffffu, c.first, l.mask ? __ffs(l.mask) - 1 : 0);
+    GChain r;
+    r.n = E.n + bn + n - own_n;
+    r.sum = E.sum + bx + x - own_x;
+    r.last = l.prev;
+    r.first = has_first ? first : (lower ? wf : 0);
+    *step = l.step;
+    return l.any_prev ? r : chain_id();
+}
 __device__ __forceinline__ GChain ldcg_chain(const GChain *c) {   // written by another CTA: past L1
     GChain r;
     r.n = __ldcg(&c->n); r.first = __ldcg(&c->first); r.last = __ldcg(&c->last); r.sum = __ldcg(&c->sum);
     return r;
 }
+template <bool BATCH>
 __global__ void __launch_bounds__(SB, 1) k_prepass_small(const Params p, int T) {
     __shared__ GAgg s_a[32];
     __shared__ GChain s_h[32];
@@ -238,6 +323,7 @@ __global__ void __launch_bounds__(SB, 1) k_prepass_small(const Params p, int T) 
     __shared__ bool s_wrap[32];
     __shared__ SAgg s_w[32];
     __shared__ SAgg s_tot;
+    __shared__ ScanSm s_scan[2];
     __shared__ bool s_last;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const long long tp = p.thr_pix, tt = p.thr_tdc;
@@ -265,21 +351,24 @@ __global__ void __launch_bounds__(SB, 1) k_prepass_small(const Params p, int T) 
         __syncthreads();
         if (w == 0) {   // the 32 parts in order
             const GAgg mine = s_a[lane];
-            const GAgg incl = warp_incl_scan(mine, lane, tp, tt);
-            GAgg before = shfl_up_agg(incl, 1);
-            if (lane == 0) before = agg_id();
-            const bool step = before.pix.n && mine.pix.n && jump(mine.pix.first - before.pix.last, tp) != 0;
-            const bool wrap = __any_sync(0xffffffffu, step || s_wrap[lane]);
+            LaneChain px, td;
+            px.link(mine.pix, lane, false, 0, tp);
+            td.link(mine.tdc, lane, false, 0, tt);
+            GAgg all;
+            all.pix = px.total(mine.pix, lane, 32);
+            all.tdc = td.total(mine.tdc, lane, 32);
+            const bool wrap = __any_sync(0xffffffffu, px.step != 0 || s_wrap[lane]);
             const unsigned has = __ballot_sync(0xffffffffu, s_first[lane] >= 0);
             const int fl = has ? __ffs(has) - 1 : 0;
-            if (lane == fl) {
+            const GChain before = px.total(mine.pix, lane, fl);   // up to the part with the first TDC packet
+            if (lane == 0) {
                 TileInfo ti;
-                ti.first_tdc = has ? s_first[lane] : -1;
+                ti.first_tdc = has ? s_first[fl] : -1;
                 ti.wrap = wrap ? 1 : 0;
                 p.ts.tinfo[tile] = ti;
-                p.ts.head[tile] = has ? ccomb(before.pix, s_h[lane], tp) : chain_id();
+                p.ts.head[tile] = has ? ccomb(before, s_h[fl], tp) : chain_id();
+                p.ts.agg[tile] = all;
             }
-            if (lane == 31) p.ts.agg[tile] = incl;
             __threadfence();
             __syncwarp();
             if (lane == 0) s_last = atomicAdd(&p.ctl->prepass_done, 1u) + 1u == gridDim.x;
@@ -290,29 +379,38 @@ __global__ void __launch_bounds__(SB, 1) k_prepass_small(const Params p, int T) 
     __threadfence();
     // the state before every tile (as k_block_scan, k_top_scan and k_apply)
     const long long t = threadIdx.x;
-    if (p.n_tiles <= 32 && w > 0) return;
+    constexpr bool one = !BATCH;
+    const bool one_warp = p.n_tiles <= 32;
+    if (one_warp && w > 0) return;
     SAgg v = sid();
     if (t < p.n_tiles) {
         v.a.pix = ldcg_chain(&p.ts.agg[t].pix);
         v.a.tdc = ldcg_chain(&p.ts.agg[t].tdc);
-        v.f = run_starts_at(p, t);
+        if constexpr (BATCH) v.f = run_starts_at(p, t);
     }
-    SAgg ex;
-    if (p.n_tiles <= 32) {
-        SAgg incl = v;
+    GAgg e;
+    if constexpr (one) {
+        const GAgg E = p.E0 ? *p.E0 : agg_id();
+        int step;
+        e.tdc = chain_before(v.a.tdc, E.tdc, s_scan[0], one_warp, tt, &step);
+        e.pix = chain_before(v.a.pix, E.pix, s_scan[1], one_warp, tp, &step);
+    } else {   // a batch: segmented at the runs' first tiles
+        SAgg ex;
+        if (one_warp) {
+            SAgg incl = v;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const SAgg u = shfl_up_sagg(incl, o);
-            if (lane >= o) incl = scomb(u, incl, tp, tt);
+            for (int o = 1; o < 32; o <<= 1) {
+                const SAgg u = shfl_up_sagg(incl, o);
+                if (lane >= o) incl = scomb(u, incl, tp, tt);
+            }
+            ex = shfl_up_sagg(incl, 1);
+            if (lane == 0) ex = sid();
+        } else {
+            ex = block_excl_sagg(v, s_w, &s_tot, tp, tt);
         }
-        ex = shfl_up_sagg(incl, 1);
-        if (lane == 0) ex = sid();
-    } else {
-        ex = block_excl_sagg(v, s_w, &s_tot, tp, tt);
+        e = v.f ? agg_id() : ex.a;
     }
     if (t >= p.n_tiles) return;
-    const bool one = !p.bt.tile_run;
-    GAgg e = v.f ? agg_id() : (one && p.E0) ? acomb(*p.E0, ex.a, tp, tt) : ex.a;
     if (t == p.n_tiles - 1 && one && p.state_out) *p.state_out = acomb(e, v.a, tp, tt);
     TileInfo ti;
     ti.first_tdc = __ldcg(&p.ts.tinfo[t].first_tdc);
@@ -338,7 +436,8 @@ size_t unwrap_prepass_scratch_bytes(long long n_tiles) {
 cudaError_t launch_unwrap_prepass(const Params &p, int T, int grid, cudaStream_t s) {
     if (p.n_tiles <= 0) return cudaSuccess;
     if (p.n_tiles <= SB) {
-        k_prepass_small<<<(unsigned)p.n_tiles, SB, 0, s>>>(p, T);
+        if (p.bt.tile_run) k_prepass_small<true><<<(unsigned)p.n_tiles, SB, 0, s>>>(p, T);
+        else k_prepass_small<false><<<(unsigned)p.n_tiles, SB, 0, s>>>(p, T);
         return cudaGetLastError();
     }
     const long long nb = (p.n_tiles + SB - 1) / SB;
