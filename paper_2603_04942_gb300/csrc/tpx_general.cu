@@ -1108,26 +1108,28 @@ __global__ void __launch_bounds__(SEGW * 32, 8) k_segments(Sorted s, const long 
     }
 }
 
-// Segments of 65 to WCAP hits: one warp in shared memory, where a cell hash of
+// Segments of 65 to WCAP hits: one block in shared memory, where a cell hash of
 // the segment gives every hit the candidates of the forward half of its box
 // (same cell: later positions only), so that each adjacent pair is met once
 // even when the whole segment lies within dt; pairs set the local-maximum flags
 // and are joined by hooking rounds; then labels, peaks, root flags (emitted
-// shots only) and the root's int64 moments.
+// shots only) and the root's int64 moments. Bound by the steps that follow one
+// another in a segment: with a warp per segment 6.0e6 hits took 89 us,
+// 4e5 hits 43; with a block 53 and 22.
 __global__ void __launch_bounds__(SEGW * 32) k_segments_mid(Sorted s, const long long *seg_start, const unsigned *mid,
                                                             const SegLists *lists, int rx, int ry, int dt, int cc,
                                                             long long shot_limit, long long *labels,
                                                             unsigned char *is_peak, unsigned char *rflag, AccH *acc) {
-    __shared__ SegSm sm[SEGW];
-    const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
-    SegSm &W = sm[wi];
+    __shared__ SegSm W;
+    const int lane = threadIdx.x & 31, tid = threadIdx.x;
+    constexpr int TH = SEGW * 32;
     const long long n_mid = lists->n_mid;
-    for (long long q = blockIdx.x * (long long)SEGW + wi; q < n_mid; q += (long long)gridDim.x * SEGW) {
+    for (long long q = blockIdx.x; q < n_mid; q += gridDim.x) {
         const long long s0 = seg_start[mid[q]];
         const int L = (int)(seg_start[mid[q] + 1ll] - s0);
         const bool emit = s.emits(s0, shot_limit);
         const bool sums = cc && acc && emit;
-        for (int k = lane; k < L; k += 32) {
+        for (int k = tid; k < L; k += TH) {
             W.tofb[k] = s.tofb(s0 + k);
             W.x[k] = s.x(s0 + k);
             W.y[k] = s.y(s0 + k);
@@ -1135,12 +1137,12 @@ __global__ void __launch_bounds__(SEGW * 32) k_segments_mid(Sorted s, const long
             W.parent[k] = k;
             W.np[k] = 0;
         }
-        for (int b = lane; b < HBW; b += 32) W.hhead[b] = 0xFFFFu;
-        if (lane == 0) W.ecnt = 0;
-        __syncwarp();
-        for (int k = lane; k < L; k += 32) W.hnext[k] = (unsigned short)atomicExch(&W.hhead[wcell(W.x[k], W.y[k])], (unsigned)k);
-        __syncwarp();
-        for (int k = lane; k < L; k += 32) {
+        for (int b = tid; b < HBW; b += TH) W.hhead[b] = 0xFFFFu;
+        if (tid == 0) W.ecnt = 0;
+        __syncthreads();
+        for (int k = tid; k < L; k += TH) W.hnext[k] = (unsigned short)atomicExch(&W.hhead[wcell(W.x[k], W.y[k])], (unsigned)k);
+        __syncthreads();
+        for (int k = tid; k < L; k += TH) {
             const int tb = W.tofb[k], xk = W.x[k], yk = W.y[k], tk = W.tot[k];
             for (int dx = 0; dx <= rx; ++dx) {
                 const int cx = xk + dx;
@@ -1169,7 +1171,7 @@ __global__ void __launch_bounds__(SEGW * 32) k_segments_mid(Sorted s, const long
                 }
             }
         }
-        __syncwarp();
+        __syncthreads();
         if (cc) {
             // rounds of: pointer jumping until every hit points at its root,
             // then every recorded pair whose roots differ hooks the larger
@@ -1180,15 +1182,14 @@ __global__ void __launch_bounds__(SEGW * 32) k_segments_mid(Sorted s, const long
             for (;;) {
                 for (;;) {
                     bool moved = false;
-                    for (int k = lane; k < L; k += 32) {
+                    for (int k = tid; k < L; k += TH) {
                         const int p = W.parent[k], pp = W.parent[p];
                         if (pp != p) { W.parent[k] = pp; moved = true; }
                     }
-                    __syncwarp();
-                    if (!__any_sync(0xffffffffu, moved)) break;
+                    if (!__syncthreads_or(moved)) break;
                 }
                 bool hooked = false;
-                for (int e = lane; e < m; e += 32) {
+                for (int e = tid; e < m; e += TH) {
                     const unsigned ed = W.edge[e];
                     const int a = W.parent[ed >> 16], b = W.parent[ed & 0xFFFFu];
                     if (a != b) {
@@ -1196,28 +1197,27 @@ __global__ void __launch_bounds__(SEGW * 32) k_segments_mid(Sorted s, const long
                         hooked = true;
                     }
                 }
-                __syncwarp();
-                if (!__any_sync(0xffffffffu, hooked)) break;
+                if (!__syncthreads_or(hooked)) break;
             }
         }
-        __syncwarp();
+        __syncthreads();
         // roots of every hit (full compression; only reads after the barrier)
-        int rk[WCAP / 32];
+        int rk[WCAP / TH];
 #pragma unroll
-        for (int u = 0; u < WCAP / 32; ++u) {
-            const int k = u * 32 + lane;
+        for (int u = 0; u < WCAP / TH; ++u) {
+            const int k = u * TH + tid;
             rk[u] = (k < L && cc) ? s_find(W.parent, k) : k;
         }
-        __syncwarp();
+        __syncthreads();
 #pragma unroll
-        for (int u = 0; u < WCAP / 32; ++u) {
-            const int k = u * 32 + lane;
+        for (int u = 0; u < WCAP / TH; ++u) {
+            const int k = u * TH + tid;
             if (k < L) W.parent[k] = rk[u];
         }
-        __syncwarp();
+        __syncthreads();
 #pragma unroll
-        for (int u = 0; u < WCAP / 32; ++u) {
-            const int k = u * 32 + lane;
+        for (int u = 0; u < WCAP / TH; ++u) {
+            const int k = u * TH + tid;
             if (k >= L) break;
             const int r = rk[u];
             const unsigned hh = s.hit[s0 + k];
@@ -1231,12 +1231,12 @@ __global__ void __launch_bounds__(SEGW * 32) k_segments_mid(Sorted s, const long
             // the hash heads: 256 hits, so ToT sums times a coordinate fit 32 bits
             unsigned *q_n = W.edge, *q_tot = q_n + WCAP, *q_x = q_tot + WCAP, *q_y = q_x + WCAP;
             unsigned long long *q_t = reinterpret_cast<unsigned long long *>(W.hhead);
-            for (int k = lane; k < L; k += 32) {
+            for (int k = tid; k < L; k += TH) {
                 q_n[k] = q_tot[k] = q_x[k] = q_y[k] = 0u;
                 q_t[k] = 0ull;
             }
-            __syncwarp();
-            for (int k = lane; k < L; k += 32) {
+            __syncthreads();
+            for (int k = tid; k < L; k += TH) {
                 const int r = W.parent[k];
                 const unsigned t = W.tot[k];
                 atomicAdd(&q_n[r], 1u | (W.np[k] == 0 ? 1u << 16 : 0u));
@@ -1245,8 +1245,8 @@ __global__ void __launch_bounds__(SEGW * 32) k_segments_mid(Sorted s, const long
                 atomicAdd(&q_y[r], t * W.y[k]);
                 atomicAdd(&q_t[r], (unsigned long long)(W.tofb[k] - W.tofb[r]) * t);
             }
-            __syncwarp();
-            for (int k = lane; k < L; k += 32) {
+            __syncthreads();
+            for (int k = tid; k < L; k += TH) {
                 if (W.parent[k] != k) continue;
                 AccH a;
                 a.s_tot = q_tot[k]; a.s_x = q_x[k]; a.s_y = q_y[k]; a.s_t = (long long)q_t[k];
@@ -1254,7 +1254,7 @@ __global__ void __launch_bounds__(SEGW * 32) k_segments_mid(Sorted s, const long
                 acc[s.hit[s0 + k]] = a;
             }
         }
-        __syncwarp();
+        __syncthreads();
     }
 }
 
@@ -1475,7 +1475,7 @@ __device__ __forceinline__ long long find_index(const int64_t *index, long long 
 // (4096 hits: ToT sums times a coordinate fit; s_t for times within 1023 ticks
 // of the root, else past the table), and its entries go to global memory.
 // With six 64-bit global atomics and a 23-step search per hit, 6.0e6 hits
-// took 264 us; 92 with one hit's loads in flight per thread, fewer with four's.
+// took 264 us; 92 with one hit's loads in flight per thread, 71 with four's.
 constexpr int AH = 1024;            // hash slots: a quarter of a block's hits
 __global__ void __launch_bounds__(GT) k_accum(tpx_hits h, const long long *labels, const unsigned char *is_peak, long long n,
                                               const long long *n_rec, long long cap, const unsigned *rank,
@@ -1808,7 +1808,8 @@ int cluster_all(tpx_ctx *c, const tpx_hits &h, int64_t n, int64_t *labels, uint8
     const long long seg_max = (n + SEGW - 1) / SEGW;   // more blocks than that have no segment
     k_segments<<<(unsigned)std::min<long long>(seg_max, (long long)c->num_sms * 16), SEGW * 32, 0, s>>>(
         so, seg_start, nseg, c->cfg.rx, c->cfg.ry, dt, cc, shot_limit, lab, is_peak, rf, ac, mark, mid, lists);
-    k_segments_mid<<<(unsigned)std::min<long long>(seg_max, (long long)c->num_sms * 4), SEGW * 32, 0, s>>>(
+    // 65 hits at least per block
+    k_segments_mid<<<(unsigned)std::min<long long>(n / (WREG + 1) + 1, (long long)c->num_sms * 16), SEGW * 32, 0, s>>>(
         so, seg_start, mid, lists, c->cfg.rx, c->cfg.ry, dt, cc, shot_limit, lab, is_peak, rf, ac);
     k_long_init<<<grid_for(n), GT, 0, s>>>(so, n, lists, mark, parent, notpeak, ac, lhead, lmask);
     k_long_insert<<<grid_for(n), GT, 0, s>>>(so, n, lists, mark, lhead, lnext, lword, lmask);
