@@ -305,10 +305,10 @@ __device__ __forceinline__ GChain chain_before(const GChain &c, const GChain &E,
     GChain r;
     r.n = E.n + bn + n - own_n;
     r.sum = E.sum + bx + x - own_x;
-    r.last = l.prev;
+    r.last = l.prev;   // E's where nothing lies between
     r.first = has_first ? first : (lower ? wf : 0);
     *step = l.step;
-    return l.any_prev ? r : chain_id();
+    return r;          // E's wraps count also while there is no value yet
 }
 __device__ __forceinline__ GChain ldcg_chain(const GChain *c) {   // written by another CTA: past L1
     GChain r;
