@@ -142,91 +142,6 @@ __device__ __forceinline__ bool run_starts_at(const Params &p, long long tile) {
     return p.bt.tile_run && p.bt.run_tile0[p.bt.tile_run[tile]] == tile;
 }
 
-// per block of SB tiles: the exclusive scan inside the block (into pre[]) and
-// the block's total (into bagg[], its flag into bflag[])
-__global__ void __launch_bounds__(SB) k_block_scan(const Params p, GAgg *bagg, int *bflag) {
-    __shared__ SAgg s_w[32];
-    __shared__ SAgg s_tot;
-    const long long t = (long long)blockIdx.x * SB + threadIdx.x;
-    SAgg v = sid();
-    if (t < p.n_tiles) {
-        v.a = p.ts.agg[t];
-        v.f = run_starts_at(p, t);
-    }
-    const SAgg ex = block_excl_sagg(v, s_w, &s_tot, p.thr_pix, p.thr_tdc);
-    if (t < p.n_tiles) p.ts.pre[t] = v.f ? agg_id() : ex.a;   // a run starts from nothing
-    if (threadIdx.x == 0) {
-        bagg[blockIdx.x] = s_tot.a;
-        bflag[blockIdx.x] = s_tot.f ? 1 : 0;
-    }
-}
-
-// one block: exclusive segmented scan of the block totals, from the state
-// before the call (E0; a batch starts every run from nothing)
-__global__ void __launch_bounds__(SB) k_top_scan(const Params p, GAgg *bagg, const int *bflag, long long nb) {
-    __shared__ SAgg s_w[32];
-    __shared__ SAgg s_tot;
-    __shared__ SAgg s_carry;
-    const long long tp = p.thr_pix, tt = p.thr_tdc;
-    if (threadIdx.x == 0) {
-        s_carry.a = (!p.bt.tile_run && p.E0) ? *p.E0 : agg_id();
-        s_carry.f = false;
-    }
-    __syncthreads();
-    for (long long b0 = 0; b0 < nb; b0 += SB) {
-        const long long b = b0 + threadIdx.x;
-        SAgg v = sid();
-        if (b < nb) {
-            v.a = bagg[b];
-            v.f = bflag[b] != 0;
-        }
-        const SAgg ex = block_excl_sagg(v, s_w, &s_tot, tp, tt);
-        const SAgg carry = s_carry;
-        const SAgg r = scomb(carry, ex, tp, tt);
-        __syncthreads();
-        if (b < nb) bagg[b] = r.a;      // now: the state before block b
-        if (threadIdx.x == 0) s_carry = scomb(carry, s_tot, tp, tt);
-        __syncthreads();
-    }
-}
-
-// the state before each tile: within its block's scan, after the state before
-// the block unless its run started inside the block; the last tile also gives
-// the state after the call
-__global__ void __launch_bounds__(256) k_apply(const Params p, const GAgg *bpre) {
-    const long long t = (long long)blockIdx.x * 256 + threadIdx.x;
-    if (t >= p.n_tiles) return;
-    const long long b = t / SB, bstart = b * SB;
-    const long long tp = p.thr_pix, tt = p.thr_tdc;
-    bool fresh;   // the run of tile t starts inside block b (at or before t)
-    if (p.bt.tile_run) fresh = p.bt.run_tile0[p.bt.tile_run[t]] >= bstart;
-    else fresh = false;
-    const GAgg loc = p.ts.pre[t];
-    GAgg e = fresh ? loc : acomb(bpre[b], loc, tp, tt);
-    const GAgg g = p.ts.agg[t];
-    if (t == p.n_tiles - 1 && !p.bt.tile_run && p.state_out) *p.state_out = acomb(e, g, tp, tt);
-    TileInfo ti = p.ts.tinfo[t];
-    if (e.pix.n && g.pix.n && jump(g.pix.first - e.pix.last, tp) != 0) {   // the step into the tile's first pixel
-        ti.wrap = 1;
-        p.ts.tinfo[t] = ti;
-    }
-    // the range of a tile with triggers before it starts at its first TDC
-    // packet: the pixel chain goes on to there
-    const long long trig_base = (!p.bt.tile_run && p.E0) ? p.E0->tdc.n : 0;
-    if (e.tdc.n > trig_base && ti.first_tdc >= 0) e.pix = ccomb(e.pix, p.ts.head[t], tp);
-    p.ts.pre[t] = e;
-}
-
-// Up to SB tiles (4 M packets): the whole pre-pass in one launch. A call of a
-// few tiles is bound by latency, not by bytes: with a warp per tile the 4096
-// packets of a tile are 64 dependent steps of one warp, and three launches
-// follow (37 shots, 5 tiles: 30 + 6 + 6 + 4 us; the whole call 112 us, with
-// this kernel and two memsets and a copy fewer 69 us; 1000 shots, 117 tiles:
-// 125 -> 74 us). Here a CTA takes a tile, its 32 warps two steps each; the
-// parts are combined by one warp, from picks and sums (scans of whole aggregates
-// took 18 us of 117 tiles, this 14). The CTA that
-// finishes last (a counter in the control block) scans the aggregates of all
-// tiles and writes the states; nobody waits for anybody.
 // 32 consecutive stretches of one chain, lane by lane, without a scan of whole
 // aggregates: the step into a lane's stretch follows from the last value of the
 // nearest lane below that has one, the rest are sums and picks.
@@ -310,6 +225,116 @@ __device__ __forceinline__ GChain chain_before(const GChain &c, const GChain &E,
     *step = l.step;
     return r;          // E's wraps count also while there is no value yet
 }
+// per block of SB tiles: the exclusive scan inside the block (into pre[]) and
+// the block's total (into bagg[], its flag into bflag[])
+__global__ void __launch_bounds__(SB) k_block_scan(const Params p, GAgg *bagg, int *bflag) {
+    __shared__ SAgg s_w[32];
+    __shared__ SAgg s_tot;
+    const long long t = (long long)blockIdx.x * SB + threadIdx.x;
+    SAgg v = sid();
+    if (t < p.n_tiles) {
+        v.a = p.ts.agg[t];
+        v.f = run_starts_at(p, t);
+    }
+    if (!p.bt.tile_run) {   // one stream: no segments
+        __shared__ ScanSm s_scan[2];
+        GAgg e;
+        int step;
+        e.tdc = chain_before(v.a.tdc, chain_id(), s_scan[0], false, p.thr_tdc, &step);
+        e.pix = chain_before(v.a.pix, chain_id(), s_scan[1], false, p.thr_pix, &step);
+        if (t < p.n_tiles) p.ts.pre[t] = e;
+        if (threadIdx.x == SB - 1) {
+            bagg[blockIdx.x] = acomb(e, v.a, p.thr_pix, p.thr_tdc);
+            bflag[blockIdx.x] = 0;
+        }
+        return;
+    }
+    const SAgg ex = block_excl_sagg(v, s_w, &s_tot, p.thr_pix, p.thr_tdc);
+    if (t < p.n_tiles) p.ts.pre[t] = v.f ? agg_id() : ex.a;   // a run starts from nothing
+    if (threadIdx.x == 0) {
+        bagg[blockIdx.x] = s_tot.a;
+        bflag[blockIdx.x] = s_tot.f ? 1 : 0;
+    }
+}
+
+// one block: exclusive segmented scan of the block totals, from the state
+// before the call (E0; a batch starts every run from nothing)
+__global__ void __launch_bounds__(SB) k_top_scan(const Params p, GAgg *bagg, const int *bflag, long long nb) {
+    __shared__ SAgg s_w[32];
+    __shared__ SAgg s_tot;
+    __shared__ SAgg s_carry;
+    const long long tp = p.thr_pix, tt = p.thr_tdc;
+    if (!p.bt.tile_run && nb <= 32) {   // one warp does it (up to 1.3e8 packets: 32-bit counts)
+        if (threadIdx.x >= 32) return;
+        __shared__ ScanSm s_none;
+        const long long b = threadIdx.x;
+        const GAgg v = b < nb ? bagg[b] : agg_id(), E = p.E0 ? *p.E0 : agg_id();
+        GAgg e;
+        int step;
+        e.tdc = chain_before(v.tdc, E.tdc, s_none, true, tt, &step);
+        e.pix = chain_before(v.pix, E.pix, s_none, true, tp, &step);
+        if (b < nb) bagg[b] = e;
+        return;
+    }
+    if (threadIdx.x == 0) {
+        s_carry.a = (!p.bt.tile_run && p.E0) ? *p.E0 : agg_id();
+        s_carry.f = false;
+    }
+    __syncthreads();
+    for (long long b0 = 0; b0 < nb; b0 += SB) {
+        const long long b = b0 + threadIdx.x;
+        SAgg v = sid();
+        if (b < nb) {
+            v.a = bagg[b];
+            v.f = bflag[b] != 0;
+        }
+        const SAgg ex = block_excl_sagg(v, s_w, &s_tot, tp, tt);
+        const SAgg carry = s_carry;
+        const SAgg r = scomb(carry, ex, tp, tt);
+        __syncthreads();
+        if (b < nb) bagg[b] = r.a;      // now: the state before block b
+        if (threadIdx.x == 0) s_carry = scomb(carry, s_tot, tp, tt);
+        __syncthreads();
+    }
+}
+
+// the state before each tile: within its block's scan, after the state before
+// the block unless its run started inside the block; the last tile also gives
+// the state after the call
+__global__ void __launch_bounds__(256) k_apply(const Params p, const GAgg *bpre) {
+    const long long t = (long long)blockIdx.x * 256 + threadIdx.x;
+    if (t >= p.n_tiles) return;
+    const long long b = t / SB, bstart = b * SB;
+    const long long tp = p.thr_pix, tt = p.thr_tdc;
+    bool fresh;   // the run of tile t starts inside block b (at or before t)
+    if (p.bt.tile_run) fresh = p.bt.run_tile0[p.bt.tile_run[t]] >= bstart;
+    else fresh = false;
+    const GAgg loc = p.ts.pre[t];
+    GAgg e = fresh ? loc : acomb(bpre[b], loc, tp, tt);
+    const GAgg g = p.ts.agg[t];
+    if (t == p.n_tiles - 1 && !p.bt.tile_run && p.state_out) *p.state_out = acomb(e, g, tp, tt);
+    TileInfo ti = p.ts.tinfo[t];
+    if (e.pix.n && g.pix.n && jump(g.pix.first - e.pix.last, tp) != 0) {   // the step into the tile's first pixel
+        ti.wrap = 1;
+        p.ts.tinfo[t] = ti;
+    }
+    // the range of a tile with triggers before it starts at its first TDC
+    // packet: the pixel chain goes on to there
+    const long long trig_base = (!p.bt.tile_run && p.E0) ? p.E0->tdc.n : 0;
+    if (e.tdc.n > trig_base && ti.first_tdc >= 0) e.pix = ccomb(e.pix, p.ts.head[t], tp);
+    p.ts.pre[t] = e;
+}
+
+// Up to SB tiles (4 M packets): the whole pre-pass in one launch. A call of a
+// few tiles is bound by latency, not by bytes: with a warp per tile the 4096
+// packets of a tile are 64 dependent steps of one warp, and three launches
+// follow (37 shots, 5 tiles: 30 + 6 + 6 + 4 us; the whole call 112 us, with
+// this kernel and two memsets and a copy fewer 69 us; 1000 shots, 117 tiles:
+// 125 -> 74 us). Here a CTA takes a tile, its 32 warps two steps each; the
+// parts are combined by one warp, from picks and sums (scans of whole aggregates
+// took 18 us of 117 tiles, this 14). The CTA that
+// finishes last (a counter in the control block) scans the aggregates of all
+// tiles and writes the states; nobody waits for anybody.
 __device__ __forceinline__ GChain ldcg_chain(const GChain *c) {   // written by another CTA: past L1
     GChain r;
     r.n = __ldcg(&c->n); r.first = __ldcg(&c->first); r.last = __ldcg(&c->last); r.sum = __ldcg(&c->sum);
