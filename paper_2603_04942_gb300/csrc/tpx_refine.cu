@@ -192,9 +192,11 @@ __global__ void __launch_bounds__(SELT) k_select(const uint64_t *pk, const tpx_r
 // ToA relative to the cluster's earliest pixel, in units of 32 ticks (50 ns),
 // clamped to [-8, 8], rounded to fp16 (exact: multiples of 1/32 below 8); both
 // are exact in bf16 as well
-__device__ __forceinline__ float patch_tot(int tot) { return __bfloat162float(__float2bfloat16_rn((float)tot / 1023.f)); }
+// (the product with the rounded 1 / 1023 rounds to the same bf16 as the quotient
+// for all 1024 ToT values)
+__device__ __forceinline__ float patch_tot(int tot) { return __bfloat162float(__float2bfloat16_rn((float)tot * (1.f / 1023.f))); }
 // (the ticks already clamped to 256 = 8 units either way)
-__device__ __forceinline__ float patch_rel(int ticks) { return __half2float(__float2half_rn((float)ticks / 32.f)); }
+__device__ __forceinline__ float patch_rel(int ticks) { return __half2float(__float2half_rn((float)ticks * 0.03125f)); }
 // elements e and e + 1 of a patch row
 // (one store where the caller's buffer is aligned to the pair)
 __device__ __forceinline__ void put_pair(float *row, int e, float a, float b) {
@@ -226,7 +228,7 @@ __device__ __forceinline__ void put_pair(uint16_t *row, int e, float a, float b)
 // of a step are in flight together; the bytes are the labels (twice, mostly
 // from L2) and the patches. Before, every cell had an 8-byte key in global
 // memory, cleared, updated and read back: 300 us of the 460 of a call of
-// 440,000 patches; now 134 of 300.
+// 440,000 patches; now about 115 of 280.
 constexpr int PMAX = 96;                         // clusters a pass holds (2048 packets of 24-pixel clusters: 85)
 constexpr int PWIN = PT + 2 * PH, PU = PWIN / PTH;
 static_assert(PWIN <= 4096, "the window position has 12 bits");
@@ -254,7 +256,7 @@ __device__ __forceinline__ void write_patch(OutT *row, const unsigned *key, int 
     }
 }
 template <typename OutT>
-__global__ void __launch_bounds__(PTH, 3) k_patch_tiles(const uint64_t *pk, long long n, long long base,
+__global__ void __launch_bounds__(PTH, 4) k_patch_tiles(const uint64_t *pk, long long n, long long base,
                                                         const long long *labels, const SelRoot *roots,
                                                         const TileSel *tiles, OutT *patch, unsigned *inc,
                                                         PatchInfo *info) {
