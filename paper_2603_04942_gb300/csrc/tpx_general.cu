@@ -11,14 +11,15 @@
 //           ties keep stream order. In that order a gap larger than dt ends
 //           every cluster, so the sorted hits split into independent
 //           segments. One warp clusters a segment of up to 64 hits in
-//           registers: ballots give each hit's adjacency row (Sec. V.A box
-//           rule) and local-maximum flag (Sec. V.B); components are closures
-//           over the rows seeded at the earliest hit; the root's int64
-//           moments are warp sums. Longer segments (shots whose particles
-//           arrive within dt of each other) find their pairs through a hash
-//           of (shot, x, y) cells and join them in a global lock-free
-//           union-find whose root is the smallest position.
-// centroid: cluster ids in ascending label order (a scan over root flags in
+//           registers: a compact one from a grid of cells, any other by ballots
+//           that give each hit's adjacency row (Sec. V.A box rule) and
+//           local-maximum flag (Sec. V.B); components are closures over the
+//           rows seeded at the earliest hit; the root's int64 moments are warp
+//           sums. Up to 256 hits one block does it in shared memory. Longer
+//           segments (shots whose particles arrive within dt of each other)
+//           find their pairs through a hash of (shot, x, y) cells and join them
+//           in a global lock-free union-find whose root is the smallest position.
+// centroid: records in ascending label order (root flags counted per block in
 //           stream order), f64 final division (Sec. V.C); PAPER mode sums the
 //           box neighbourhood of each local maximum.
 // No capacity limit besides 2^31 - 1 kept pixels per call.

@@ -18,6 +18,7 @@
 //   4. k_apply: the state before each tile (its pixel chain carried on to the
 //      tile's first TDC packet, where the tile's range starts), and after the
 //      last one.
+// Up to 1024 tiles one launch does all of it (k_prepass_small).
 // Beside the aggregates, k_tile_aggs leaves what the fused kernel plans its
 // ranges from (TileInfo): each tile's first TDC packet and whether a pixel wrap
 // lies in it, so that the fused kernel neither searches for the end of a range
