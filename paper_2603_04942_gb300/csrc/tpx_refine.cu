@@ -352,7 +352,7 @@ __global__ void __launch_bounds__(PWT) k_patch_wide(const uint64_t *pk, long lon
         __syncthreads();
 #pragma unroll 8
         for (long long q = w0 + threadIdx.x; q < w1; q += PWT) {
-            if (labels[q] != c.label) continue;
+            if (labels[q] != c.label || c.label < 0) continue;   // (below 0: no cluster's, as in the tiles)
             atomicAdd(&s_cnt, 1u);
             const uint64_t w = pk[q];
             const int dx = pix_x(w) - cx + PS / 2, dy = pix_y(w) - cy + PS / 2;
