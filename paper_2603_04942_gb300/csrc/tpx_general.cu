@@ -195,24 +195,24 @@ __global__ void __launch_bounds__(GT) k_tile_agg(const uint64_t *pk, long long n
     GAgg a;
     GChain head;
     part.result(&a, &head);
+    const bool wraps = part.wraps || __any_sync(0xffffffffu, part.tdc_wraps);   // (opposite steps: a sum of 0)
     if (lane == 0) {
         s_a[w] = a;
-        s_wrap[w] = part.wraps;
+        s_wrap[w] = wraps;
     }
     __syncthreads();
     if (w == 0) {
         const GAgg mine = lane < GW ? s_a[lane] : agg_id();
         const GAgg incl = warp_incl_scan(mine, lane, tp, tt);
         const bool wrap = __any_sync(0xffffffffu, lane < GW && s_wrap[lane]);
-        if (lane == 31) {   // sums of opposite wraps cancel: `wraps` and the parts' steps tell of each
+        if (lane == 31) {
             tagg[tile] = incl;
             tcnt[tile] = incl.tdc.n;
         }
         GAgg before = shfl_up_agg(incl, 1);
         if (lane == 0) before = agg_id();
         const bool step = (before.pix.n && mine.pix.n && jump(mine.pix.first - before.pix.last, tp) != 0) ||
-                          (before.tdc.n && mine.tdc.n && jump(mine.tdc.first - before.tdc.last, tt) != 0) ||
-                          mine.tdc.sum != 0;
+                          (before.tdc.n && mine.tdc.n && jump(mine.tdc.first - before.tdc.last, tt) != 0);
         const bool any = __any_sync(0xffffffffu, step);
         if (lane == 0) twrap[tile] = wrap || any;
     }
