@@ -121,6 +121,8 @@ int grow(Tp **ptr, int64_t *cap, int64_t want) {
 namespace {
 
 constexpr size_t kCtlBytes = sizeof(tpxk::Ctl) + sizeof(unsigned);
+// its pinned copy, and behind it the two counts of a host call
+constexpr size_t kHostCountsAt = (kCtlBytes + 7) & ~size_t(7), kHostCtlBytes = kHostCountsAt + 2 * sizeof(int64_t);
 
 // A call's failure bits (a range the tiles could not hold, a batch run to
 // redo) are resolved by the tpx_sync after it. When a new call starts before
@@ -138,6 +140,13 @@ int begin_call(tpx_ctx *c) {
     c->synced = false;
     c->redone_early = 0;
     return TPX_OK;
+}
+
+// whether the fused kernel met an input it cannot hold on chip in the last call,
+// a tpx_process call (h_ctl: its control block)
+bool needs_redo(const tpx_ctx *c) {
+    return (c->h_ctl->status & (tpxk::ST_CAPACITY | tpxk::ST_EXCEPTION)) && !(c->h_ctl->status & tpxk::ST_DEVTIMEOUT) &&
+           c->last.valid;
 }
 
 // ---- tile-geometry autotuner ----
@@ -258,12 +267,12 @@ int tpx_create(tpx_ctx **out, const tpx_config *cfg, int64_t max_packets, void *
     }
     // the control block and, behind it, the sticky word: one copy brings both down
     if (cudaMalloc(&c->ctl, kCtlBytes) != cudaSuccess) { delete c; return TPX_ENOMEM; }
-    if (cudaMallocHost(&c->h_ctl, kCtlBytes) != cudaSuccess) {
+    if (cudaMallocHost(&c->h_ctl, kHostCtlBytes) != cudaSuccess) {
         cudaFree(c->ctl);
         delete c;
         return TPX_ENOMEM;
     }
-    std::memset(c->h_ctl, 0, kCtlBytes);
+    std::memset(c->h_ctl, 0, kHostCtlBytes);
     cudaMemset(c->ctl, 0, kCtlBytes);
     c->d_sticky = reinterpret_cast<unsigned *>(c->ctl + 1);
     if (cudaMalloc(&c->d_state, 2 * sizeof(tpxk::GAgg)) != cudaSuccess) {
@@ -709,8 +718,7 @@ int tpx_sync(tpx_ctx *c, tpx_counters *out) {
     if (sticky && ckr(cudaMemsetAsync(c->d_sticky, 0, 4, c->stream))) return TPX_ECUDA;
     // a checked build's index violation stays reported even when the call is redone
     const unsigned bounds = c->h_ctl->status & tpxk::ST_BOUNDS;
-    if ((c->h_ctl->status & (tpxk::ST_CAPACITY | tpxk::ST_EXCEPTION)) && !(c->h_ctl->status & tpxk::ST_DEVTIMEOUT) &&
-        c->last.valid) {
+    if (needs_redo(c)) {
         // the fused kernel met an input it cannot hold on chip: redo the call
         // exactly with the general path, then report that run
         const int rc = tpxg::redo_last(c);
@@ -1006,29 +1014,39 @@ int tpx_process_host(tpx_ctx *c, const uint64_t *h_packets, int64_t n, int64_t i
     rc = tpx_process(c, c->st_pk, n, idx_base, h_labels ? c->st_labels : nullptr, h_is_peak ? c->st_peak : nullptr,
                      c->st_cl, cl_cap, c->st_counts, c->st_trig, trig_cap, c->st_counts + 1);
     if (rc) return rc;
-    // a call that the fused kernel could not hold is redone here, before its
-    // outputs go down
-    const int rs = tpx_sync(c, nullptr);
-    int64_t counts[2] = {0, 0};
-    if (ckr(cudaMemcpyAsync(counts, c->st_counts, sizeof counts, cudaMemcpyDeviceToHost, s))) return TPX_ECUDA;
-    if (h_labels && n &&
-        cudaMemcpyAsync(h_labels, c->st_labels, ((c->cfg.flags & TPX_FLAG_LABELS32) ? 4 : 8) * (size_t)n,
-                        cudaMemcpyDeviceToHost, s) != cudaSuccess)
+    // The status, the counts and the per-packet outputs follow the kernel on the
+    // stream: one wait for them, one for the records (three, with the status
+    // read by itself first: 200 shots 99 us, so 84). A call that the fused kernel
+    // could not hold is redone after the first wait, and its outputs go down again.
+    int64_t *counts = reinterpret_cast<int64_t *>(reinterpret_cast<char *>(c->h_ctl) + kHostCountsAt);
+    auto per_packet_down = [&]() -> int {
+        if (ckr(cudaMemcpyAsync(counts, c->st_counts, 2 * sizeof(int64_t), cudaMemcpyDeviceToHost, s))) return TPX_ECUDA;
+        if (h_labels && n &&
+            ckr(cudaMemcpyAsync(h_labels, c->st_labels, ((c->cfg.flags & TPX_FLAG_LABELS32) ? 4 : 8) * (size_t)n,
+                                cudaMemcpyDeviceToHost, s)))
+            return TPX_ECUDA;
+        if (h_is_peak && n && ckr(cudaMemcpyAsync(h_is_peak, c->st_peak, n, cudaMemcpyDeviceToHost, s))) return TPX_ECUDA;
+        return TPX_OK;
+    };
+    if (ckr(cudaMemcpyAsync(c->h_ctl, c->ctl, kCtlBytes, cudaMemcpyDeviceToHost, s)) || (rc = per_packet_down()) ||
+        ckr(cudaStreamSynchronize(s)))
         return TPX_ECUDA;
-    if (h_is_peak && n && cudaMemcpyAsync(h_is_peak, c->st_peak, n, cudaMemcpyDeviceToHost, s) != cudaSuccess)
-        return TPX_ECUDA;
-    if (ckr(cudaStreamSynchronize(s))) return TPX_ECUDA;
+    const bool redo = needs_redo(c);
+    int rs = TPX_OK;
+    if (redo) {
+        rs = tpx_sync(c, nullptr);
+        if ((rc = per_packet_down()) || ckr(cudaStreamSynchronize(s))) return TPX_ECUDA;
+    }
     const int64_t ncl = counts[0] < cl_cap ? counts[0] : cl_cap;
     const int64_t ntr = counts[1] < trig_cap ? counts[1] : trig_cap;
     const size_t rsz = (c->cfg.flags & TPX_FLAG_RECORDS64) ? sizeof(tpx_record64) : sizeof(tpx_record);
-    if (ncl > 0 && cudaMemcpyAsync(h_clusters, c->st_cl, rsz * ncl, cudaMemcpyDeviceToHost, s) != cudaSuccess)
+    if (ncl > 0 && ckr(cudaMemcpyAsync(h_clusters, c->st_cl, rsz * ncl, cudaMemcpyDeviceToHost, s))) return TPX_ECUDA;
+    if (ntr > 0 && ckr(cudaMemcpyAsync(h_trig, c->st_trig, sizeof(int64_t) * ntr, cudaMemcpyDeviceToHost, s)))
         return TPX_ECUDA;
-    if (ntr > 0 && cudaMemcpyAsync(h_trig, c->st_trig, sizeof(int64_t) * ntr, cudaMemcpyDeviceToHost, s) != cudaSuccess)
-        return TPX_ECUDA;
-    if (ckr(cudaStreamSynchronize(s))) return TPX_ECUDA;
     *h_n_clusters = counts[0];
     *h_n_trig = counts[1];
-    return rs;
+    if (!redo) return tpx_sync(c, nullptr);
+    return ckr(cudaStreamSynchronize(s)) ? TPX_ECUDA : rs;
 }
 
 int tpx_debug_hold_tile(tpx_ctx *c, int64_t tile) {
