@@ -62,11 +62,16 @@ struct TileSel { unsigned first_inv, count; };   // the selected clusters whose 
 struct SelRoot { long long root, raw0; unsigned n; short cx, cy; };   // what k_patch_tiles needs of a selected cluster, in one load
 struct PatchInfo {               // read back once per call
     unsigned long long n_sel;    // selected clusters
-    unsigned n_inc;              // patches the tiles could not complete (listed)
-    unsigned n_far;              // of those, the ones that the wider search could not either
+    unsigned n_tried;            // patches that the tiles looked for
+    unsigned n_inc;              // patches not completed there (listed)
+    unsigned n_far;              // of those, the ones that the wider search could not complete either
     unsigned odd;                // labels not strictly ascending, or outside the packets, or a centre off the sensor: no tiles
-    unsigned reserved;
 };
+// The wider search reads 262 KB of labels a patch (55 ns), the kernels that look
+// anywhere all of them once (3.9 us per 10^6 packets, and 15 us of launches).
+__host__ __device__ inline bool search_wider(unsigned n_inc, long long n) {
+    return (unsigned long long)n_inc << 14 <= (unsigned long long)n + (1ull << 22);
+}
 __device__ __forceinline__ unsigned sel_flags(const tpx_record *cl, long long ncl, int min_px, unsigned (&m)[SELR],
                                               unsigned *s_c, unsigned *total) {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -178,7 +183,7 @@ __global__ void __launch_bounds__(SELT) k_select(const uint64_t *pk, const tpx_r
         v.root = r;
         v.raw0 = r >= 0 && r < n ? pix_raw(pk[r]) : 0;
         v.n = (unsigned)c.n;
-        v.cx = (short)cx;   // within the sensor: a centroid
+        v.cx = (short)cx;   // within the sensor, or the call is odd
         v.cy = (short)cy;
         roots[s] = v;
     }
@@ -222,13 +227,18 @@ __device__ __forceinline__ void put_pair(uint16_t *row, int e, float a, float b)
 // packets, with their cells in shared memory, and looks for their members
 // there and in PH packets on either side; a patch whose members all turned up
 // (the record's count) is written at once, the others are listed for the
-// kernels below. A cell's word holds all that its values follow from: ToT, the
-// packet's place in the window (the brighter pixel wins, ties go to the later)
-// and the clamped time, never zero. Bound by latency, so every thread's loads
-// of a step are in flight together; the bytes are the labels (twice, mostly
-// from L2) and the patches. Before, every cell had an 8-byte key in global
-// memory, cleared, updated and read back: 300 us of the 460 of a call of
-// 440,000 patches; now about 115 of 280.
+// kernels below. Where the shots are so long that more than half of the patches
+// tried so far went on (by whichever tiles came first), the tiles hand theirs on
+// untried: a patch is the same by any way, and the tiles' way and then the last
+// kernels' costs 11 + 4 + 25 f us per 10^6 packets with a share f of them going
+// on, the last kernels alone 27. A cell's word holds all that its values follow
+// from: ToT, the packet's place in the window (the brighter pixel wins, ties go
+// to the later) and the clamped time, never zero. Bound by latency, so every
+// thread's loads of a step are in flight together; the bytes are the labels
+// (twice, mostly from L2) and the patches. In the last kernels every cell has an
+// 8-byte key in global memory, cleared, updated and read back, as all of them
+// had before: 300 us of the 460 of a call of 440,000 patches of 20 particles a
+// shot, now about 115 of 280.
 constexpr int PMAX = 96;                         // clusters a pass holds (2048 packets of 24-pixel clusters: 85)
 constexpr int PWIN = PT + 2 * PH, PU = PWIN / PTH;
 static_assert(PWIN <= 4096, "the window position has 12 bits");
@@ -255,6 +265,25 @@ __device__ __forceinline__ void write_patch(OutT *row, const unsigned *key, int 
         put_pair(row, e, v[0], v[1]);
     }
 }
+// one warp: lists those of the patches p0 .. p0 + m that go on
+template <class F>
+__device__ __forceinline__ void list_patches(int m, F goes_on, long long p0, unsigned *inc, PatchInfo *info) {
+    const int lane = threadIdx.x & 31;
+    unsigned f[PMAX / 32], cnt = 0, at = 0;
+#pragma unroll
+    for (int u = 0; u < PMAX / 32; ++u) {
+        f[u] = __ballot_sync(0xffffffffu, 32 * u + lane < m && goes_on(32 * u + lane));
+        cnt += __popc(f[u]);
+    }
+    if (cnt == 0) return;
+    if (lane == 0) at = atomicAdd(&info->n_inc, cnt);
+    at = __shfl_sync(0xffffffffu, at, 0);
+#pragma unroll
+    for (int u = 0; u < PMAX / 32; ++u) {
+        if ((f[u] >> lane) & 1u) inc[at + __popc(f[u] & ((1u << lane) - 1u))] = (unsigned)(p0 + 32 * u + lane);
+        at += __popc(f[u]);
+    }
+}
 template <typename OutT>
 __global__ void __launch_bounds__(PTH, 4) k_patch_tiles(const uint64_t *pk, long long n, long long base,
                                                         const long long *labels, const SelRoot *roots,
@@ -265,10 +294,35 @@ __global__ void __launch_bounds__(PTH, 4) k_patch_tiles(const uint64_t *pk, long
     __shared__ int s_c[PMAX];                           // the centre, x | y << 16
     __shared__ unsigned s_cnt[PMAX], s_n[PMAX];
     __shared__ long long s_raw0[PMAX];
-    static_assert(PMAX < 255 && sizeof(s_key) + PT + 24 * PMAX < 48 * 1024, "shared memory of a pass");
+    static_assert(PMAX < 255 && PMAX % 32 == 0 && sizeof(s_key) + PT + 24 * PMAX < 48 * 1024, "shared memory of a pass");
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const long long a = blockIdx.x * (long long)PT, w0 = a - PH;
     const int tile_n = (int)min((long long)PT, n - a);
-    int L[PU];                                   // the window's labels: root - a where the root is in this tile, else -1
+    // the selected clusters of the tile: labels ascend, so they are consecutive
+    const TileSel ts = tiles[blockIdx.x];
+    const unsigned odd = info->odd;
+    unsigned tried = 0, gone = 0;
+    if (threadIdx.x == 0) {
+        tried = __ldcg(&info->n_tried);
+        gone = __ldcg(&info->n_inc);
+    }
+    if (!ts.count || odd) return;
+    const long long s0 = 0xFFFFFFFFu - ts.first_inv, s1 = s0 + ts.count;
+    if (__syncthreads_or(tried >= 4096u && gone > tried / 2)) {
+        if (warp == 0)
+            for (long long p0 = s0; p0 < s1; p0 += PMAX)
+                list_patches((int)min((long long)PMAX, s1 - p0), [](int) { return true; }, p0, inc, info);
+        return;
+    }
+    auto root_of = [&](long long p0, int m) -> SelRoot { return threadIdx.x < m ? roots[p0 + threadIdx.x] : SelRoot{}; };
+    auto clear = [&](int m) {
+        for (int k = threadIdx.x; k < PT / 4; k += PTH) reinterpret_cast<unsigned *>(s_slot)[k] = 0u;
+        for (int k = threadIdx.x; k < m * PC; k += PTH) s_key[k] = 0u;
+    };
+    int m = (int)min((long long)PMAX, s1 - s0);
+    SelRoot v = root_of(s0, m);
+    clear(m);
+    int L[PU];
 #pragma unroll
     for (int u = 0; u < PU; ++u) {
         const long long q = w0 + u * PTH + threadIdx.x;
@@ -276,17 +330,7 @@ __global__ void __launch_bounds__(PTH, 4) k_patch_tiles(const uint64_t *pk, long
         const long long r = lab - base - a;
         L[u] = lab >= 0 && r >= 0 && r < tile_n ? (int)r : -1;
     }
-    // the selected clusters of the tile: labels ascend, so they are consecutive
-    const TileSel ts = tiles[blockIdx.x];
-    if (!ts.count || info->odd) return;
-    const long long s0 = 0xFFFFFFFFu - ts.first_inv, s1 = s0 + ts.count;
-    for (long long p0 = s0; p0 < s1; p0 += PMAX) {
-        const int m = (int)min((long long)PMAX, s1 - p0);
-        SelRoot v;
-        if (threadIdx.x < m) v = roots[p0 + threadIdx.x];
-        __syncthreads();
-        for (int k = threadIdx.x; k < PT / 4; k += PTH) reinterpret_cast<unsigned *>(s_slot)[k] = 0u;
-        for (int k = threadIdx.x; k < m * PC; k += PTH) s_key[k] = 0u;
+    for (long long p0 = s0;;) {
         __syncthreads();
         if (threadIdx.x < m) {
             s_slot[v.root - a] = (unsigned char)(threadIdx.x + 1);
@@ -317,20 +361,27 @@ __global__ void __launch_bounds__(PTH, 4) k_patch_tiles(const uint64_t *pk, long
             }
         }
         __syncthreads();
-        const int lane = threadIdx.x & 31;
-        for (int j = threadIdx.x >> 5; j < m; j += PTH / 32) {
-            if (s_cnt[j] != s_n[j]) {
-                if (lane == 0) inc[atomicAdd(&info->n_inc, 1u)] = (unsigned)(p0 + j);
-                continue;
-            }
-            write_patch(patch + (p0 + j) * (long long)NIN, s_key + j * PC, lane);
+        if (warp == 0) {
+            list_patches(m, [&](int j) { return s_cnt[j] != s_n[j]; }, p0, inc, info);
+            if (lane == 0) atomicAdd(&info->n_tried, (unsigned)m);
         }
+        for (int j = warp; j < m; j += PTH / 32)
+            if (s_cnt[j] == s_n[j]) write_patch(patch + (p0 + j) * (long long)NIN, s_key + j * PC, lane);
+        p0 += PMAX;
+        if (p0 >= s1) break;
+        m = (int)min((long long)PMAX, s1 - p0);
+        v = root_of(p0, m);
+        __syncthreads();
+        clear(m);
     }
 }
 
-// The listed patches with a wider search, a CTA each: PW packets on either side
-// of the root. (50 particles a shot: a shot's readout is longer than PH.) What
-// is still incomplete goes on to the second list.
+// The listed patches, when they are few, with a wider search, a CTA each: PW
+// packets on either side of the root. (Of 25 particles a shot one in a few
+// thousand leaves the window, of 110 one in four.) What is still incomplete goes
+// on to the second list. Tried: a CTA for all listed patches of a tile, going on
+// from its window until every member turned up; it costs 15 us per 10^6 packets
+// at 110 particles a shot and 43 at 500, more than the last kernels.
 constexpr int PW = 16384, PWT = 256;
 template <typename OutT>
 __global__ void __launch_bounds__(PWT) k_patch_wide(const uint64_t *pk, long long n, long long base, const long long *labels,
@@ -340,6 +391,7 @@ __global__ void __launch_bounds__(PWT) k_patch_wide(const uint64_t *pk, long lon
     __shared__ unsigned s_word[PC];
     __shared__ unsigned s_cnt;
     const unsigned ni = info->n_inc;
+    if (!search_wider(ni, n)) return;
     for (unsigned j = blockIdx.x; j < ni; j += gridDim.x) {
         const long long s = inc[j];
         const tpx_record &c = cl[sel[s]];
@@ -380,51 +432,56 @@ __global__ void k_list_all(unsigned *inc, long long ns) {
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < ns; i += (long long)gridDim.x * blockDim.x) inc[i] = (unsigned)i;
 }
 // the listed patch of each root packet
-__global__ void k_roots(const tpx_record *cl, const long long *sel, const unsigned *inc, long long ni, long long base,
-                        long long n, int *slot_of_root) {
+__global__ void k_roots(const SelRoot *roots, const unsigned *list, long long ni, long long n, int *slot_of_root) {
     for (long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x; j < ni; j += (long long)gridDim.x * blockDim.x) {
-        const long long r = cl[sel[inc[j]]].label - base;
+        const long long r = roots[list[j]].root;
         if (r >= 0 && r < n) slot_of_root[r] = (int)j;   // else not a record of these packets: an empty patch
     }
 }
-__global__ void k_fill_i32(int *p, long long n, int v) {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) p[i] = v;
+// no root is listed, no cell hit
+__global__ void k_clear(int *slot_of_root, long long n, unsigned long long *key, long long cells) {
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < max(n, cells); i += (long long)gridDim.x * blockDim.x) {
+        if (i < n) slot_of_root[i] = -1;
+        if (i < cells) key[i] = 0ull;
+    }
 }
-// the brighter pixel of a shared cell wins (ties: the later one)
+// The brighter pixel of a shared cell wins (ties: the later one). As cell_word,
+// the key holds all that the cell's values follow from, the packet's place in 40
+// bits: the patches are then written from the keys alone (631,000 patches: 246
+// -> 134 us, against reading the winner's packet again for every cell).
 __global__ void k_patch_keys(const uint64_t *pk, long long n, long long base, const long long *labels,
-                             const int *slot_of_root, const unsigned *inc, const int *centre, unsigned long long *key) {
+                             const int *slot_of_root, const unsigned *list, const SelRoot *roots, const int *centre,
+                             unsigned long long *key) {
     for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < n; q += (long long)gridDim.x * blockDim.x) {
         const long long L = labels[q] - base;
         if (labels[q] < 0 || L < 0 || L >= n) continue;
         const int j = slot_of_root[L];
         if (j < 0) continue;
-        const long long s = inc[j];
+        const unsigned s = list[j];
+        const SelRoot v = roots[s];
+        const int cx = centre ? centre[2ll * s] : v.cx, cy = centre ? centre[2ll * s + 1] : v.cy;
         const uint64_t w = pk[q];
-        const int dx = pix_x(w) - centre[2 * s] + PS / 2, dy = pix_y(w) - centre[2 * s + 1] + PS / 2;
+        const int dx = pix_x(w) - cx + PS / 2, dy = pix_y(w) - cy + PS / 2;
         if (dx < 0 || dx >= PS || dy < 0 || dy >= PS) continue;
-        const unsigned long long k = ((unsigned long long)(pix_tot(w) + 1) << 40) | (unsigned long long)q;
-        atomicMax(&key[(long long)j * PC + dy * PS + dx], k);
+        atomicMax(&key[(long long)j * PC + dy * PS + dx], ((unsigned long long)(pix_tot(w) + 1) << 50) | ((unsigned long long)q << 10) |
+                                                              (unsigned long long)(rel_ticks(pix_raw(w), v.raw0) + kRelMax + 1));
     }
 }
-// empty cells 0
+// a thread per cell; empty cells 0
 template <typename OutT>
-__global__ void k_patch_fill(const uint64_t *pk, long long base, const tpx_record *cl, const long long *sel,
-                             const unsigned *inc, const unsigned long long *key, long long ni, OutT *patch) {
+__global__ void k_patch_fill(const unsigned *list, const unsigned long long *key, long long ni, OutT *patch) {
     for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < ni * PC; c += (long long)gridDim.x * blockDim.x) {
-        const long long j = c / PC, s = inc[j];
-        const int e = 2 * (int)(c - j * PC);   // elements e, e + 1 of the row
-        float v[2];
-#pragma unroll
-        for (int u = 0; u < 2; ++u) {
-            const bool t = e + u < PC;
-            const unsigned long long k = key[j * PC + (t ? e + u : e + u - PC)];
-            v[u] = 0.f;
-            if (k == 0) continue;
-            const long long q = (long long)(k & ((1ull << 40) - 1));
-            // the root packet is in range: the key came from this cluster
-            v[u] = t ? patch_tot(pix_tot(pk[q])) : patch_rel(rel_ticks(pix_raw(pk[q]), pix_raw(pk[cl[sel[s]].label - base])));
+        const long long j = c / PC;
+        const unsigned long long k = key[c];
+        const float tot = k ? patch_tot((int)(k >> 50) - 1) : 0.f, rel = k ? patch_rel((int)(k & 1023u) - kRelMax - 1) : 0.f;
+        OutT *row = patch + list[j] * (long long)NIN + (c - j * PC);
+        if constexpr (sizeof(OutT) == 4) {
+            row[0] = tot;
+            row[PC] = rel;
+        } else {
+            reinterpret_cast<__nv_bfloat16 *>(row)[0] = __float2bfloat16_rn(tot);
+            reinterpret_cast<__nv_bfloat16 *>(row)[PC] = __float2bfloat16_rn(rel);
         }
-        put_pair(patch + s * NIN, e, v[0], v[1]);
     }
 }
 
@@ -908,14 +965,16 @@ static int refine_patches(tpx_ctx *c, const uint64_t *d_packets, int64_t n, int6
     PatchInfo h{};
     if (ck(cudaMemcpyAsync(&h, info, sizeof h, cudaMemcpyDeviceToHost, s)) || ck(cudaStreamSynchronize(s))) return TPX_ECUDA;
     const long long np = (long long)h.n_sel, ns = np < capacity ? np : capacity;
-    const long long ni = h.odd ? ns : (long long)h.n_far;
+    const bool wider = search_wider(h.n_inc, n);
+    const long long ni = h.odd ? ns : (long long)(wider ? h.n_far : h.n_inc);
+    const unsigned *list = h.odd || wider ? far : inc;
     if (ni > 0) {
         if (h.odd) k_list_all<<<grid_for(ns), 256, 0, s>>>(far, ns);
-        k_fill_i32<<<grid_for(n), 256, 0, s>>>(slot, n, -1);
-        k_roots<<<grid_for(ni), 256, 0, s>>>(d_clusters, sel, far, ni, base, n, slot);
-        if (ck(cudaMemsetAsync(key, 0, 8 * (size_t)ni * PC, s))) return TPX_ECUDA;
-        k_patch_keys<<<grid_for(n), 256, 0, s>>>(d_packets, n, base, lab, slot, far, d_centre, key);
-        k_patch_fill<OutT><<<grid_for(ni * PC), 256, 0, s>>>(d_packets, base, d_clusters, sel, far, key, ni, d_patches);
+        k_clear<<<grid_for(std::max<long long>(n, ni * PC)), 256, 0, s>>>(slot, n, key, ni * PC);
+        k_roots<<<grid_for(ni), 256, 0, s>>>(roots, list, ni, n, slot);
+        k_patch_keys<<<grid_for(n), 256, 0, s>>>(d_packets, n, base, lab, slot, list, roots,
+                                                 h.odd ? d_centre : nullptr, key);
+        k_patch_fill<OutT><<<grid_for(ni * PC), 256, 0, s>>>(list, key, ni, d_patches);
     }
     if (ck(cudaGetLastError())) return TPX_ECUDA;
     return np > capacity ? TPX_EOVERFLOW : TPX_OK;
