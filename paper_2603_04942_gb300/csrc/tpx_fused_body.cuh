@@ -214,6 +214,7 @@ struct __align__(16) Smem {
     // (most tiles of a run whose shots span several) takes none.
     struct Pend {
         long long tile, ntr;      // the tile; its trigger total (single streams)
+        long long at;             // STAGED_ONLY: where its records are staged
         int ncl, ntdc, run;       // its records and triggers; its run
         bool first, big;          // the run's first tile; records in the big-range slot
     } pend[4];
@@ -570,7 +571,8 @@ __device__ bool copy_out(Smem &S, const Params &p, unsigned seq, int slot, bool 
     const long long O = Ow.x;
     const long long keep = min((long long)nc, max(0LL, p.cl_cap - O));
     const unsigned long long *src = reinterpret_cast<const unsigned long long *>(
-        (BATCH && big) ? br_stage(p, slot) : p.stage + ((long long)blockIdx.x * NP + slot) * C);
+        (BATCH && big) ? br_stage(p, slot)
+                       : p.stage + (STAGED_ONLY ? S.pend[slot].at : ((long long)blockIdx.x * NP + slot) * C));
     if (p.rec64) {   // 64-byte records: the first 8 words of each staged record
         unsigned long long *d64 = reinterpret_cast<unsigned long long *>(p.clusters) + O * 8;
         const long long nw = keep * 8;
@@ -2119,7 +2121,12 @@ __global__ void __launch_bounds__(NT, MINB) fused_kernel(const Params p) {
         // first tile nor the call's last) needs no offset: its count is
         // published, and the successors' look-backs add it up
         const bool any = STAGED && (ncl != 0 || S.cnt[C_TDCS] != 0 || (BATCH && tile == tile0) || tile == p.n_tiles - 1);
-        tpx_record *const stage = STAGED ? p.stage + ((long long)blockIdx.x * NP + ent % NP) * C : nullptr;
+        // STAGED_ONLY: at the range's position in the stream (the tiles' ranges do
+        // not overlap, and a range has no more records than packets), so that the
+        // staging holds a call's packets, not a whole range for each of its small
+        // tiles (a context of 155,648 packets: 113 -> 38 MB)
+        tpx_record *const stage = STAGED_ONLY ? p.stage + gbase
+                                  : STAGED ? p.stage + ((long long)blockIdx.x * NP + ent % NP) * C : nullptr;
         if (STAGED) {   // the slot's previous records are out (checked before the next barrier)
             if (tid == 0) wait_count(&S.consumed, ent - NP, p);
         } else if (wid == 0) {   // unstaged: the records' offset now, by an inline look-back
@@ -2283,6 +2290,7 @@ __global__ void __launch_bounds__(NT, MINB) fused_kernel(const Params p) {
             if (any) {
                 Smem::Pend &e = S.pend[ent % NP];
                 e.tile = tile;
+                if constexpr (STAGED_ONLY) e.at = gbase;
                 e.ncl = ncl;
                 e.ntr = ntr_here;
                 e.ntdc = (int)(ntr_here - (E.tdc.n - trig_base));

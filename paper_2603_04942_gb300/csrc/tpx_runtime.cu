@@ -68,9 +68,10 @@ int alloc_scratch(tpx_ctx *c, int64_t max_packets) {
     const size_t b_flags = al(sizeof(unsigned) * tiles), b_agg = al(sizeof(tpxk::GAgg) * tiles),
                  b_head = al(sizeof(tpxk::GChain) * tiles), b_info = al(sizeof(tpxk::TileInfo) * tiles),
                  b_cnt = al(sizeof(long long) * tiles), b_blk = al(tpxk::unwrap_prepass_scratch_bytes(tiles));
-    // record staging of the fused kernel: one range's records per CTA
-    size_t stage_records = 0;   // the largest grid of a call times its range capacity
-    for (int geo : {(int)tpxk::GEO_T4096, (int)tpxk::GEO_T2048, (int)tpxk::GEO_SMALL}) {
+    // record staging of the fused kernel: one range's records per CTA (the largest
+    // grid of a call times its range capacity); the small tiles stage theirs by position
+    size_t stage_records = (size_t)std::min<int64_t>(max_packets, c->num_sms * Ts);
+    for (int geo : {(int)tpxk::GEO_T4096, (int)tpxk::GEO_T2048}) {
         const int64_t tg = (max_packets + tpxk::fused_tile_packets(geo) - 1) / tpxk::fused_tile_packets(geo);
         int64_t ctas = (int64_t)c->num_sms * tpxk::fused_ctas_per_sm(geo);
         if (tg < ctas) ctas = tg < 1 ? 1 : tg;
