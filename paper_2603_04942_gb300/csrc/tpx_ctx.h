@@ -43,6 +43,7 @@ struct tpx_ctx {
     int64_t stage_records;    // its capacity
     tpxk::Ctl *ctl;           // device control block
     tpxk::Ctl *h_ctl;         // pinned host copy
+    int64_t *h_words;         // behind it: four words that a call brings down and reads before it returns
     unsigned *d_sticky;       // failure bits of calls that were not synchronised
     bool synced;              // tpx_sync ran after the last call
     int64_t redone_early;     // the last call was already redone (autotuner sample)

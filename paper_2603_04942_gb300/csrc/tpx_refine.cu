@@ -62,10 +62,10 @@ struct TileSel { unsigned first_inv, count; };   // the selected clusters whose 
 struct SelRoot { long long root, raw0; unsigned n; short cx, cy; };   // what k_patch_tiles needs of a selected cluster, in one load
 struct PatchInfo {               // read back once per call
     unsigned long long n_sel;    // selected clusters
-    unsigned n_tried;            // patches that the tiles looked for
-    unsigned n_inc;              // patches not completed there (listed)
+    unsigned n_inc;              // patches not completed by the tiles (listed)
     unsigned n_far;              // of those, the ones that the wider search could not complete either
     unsigned odd;                // labels not strictly ascending, or outside the packets, or a centre off the sensor: no tiles
+    unsigned reserved;
 };
 // The wider search reads 262 KB of labels a patch (55 ns), the kernels that look
 // anywhere all of them once (3.9 us per 10^6 packets, and 15 us of launches).
@@ -228,7 +228,7 @@ __device__ __forceinline__ void put_pair(uint16_t *row, int e, float a, float b)
 // there and in PH packets on either side; a patch whose members all turned up
 // (the record's count) is written at once, the others are listed for the
 // kernels below. Where the shots are so long that more than half of the patches
-// tried so far went on (by whichever tiles came first), the tiles hand theirs on
+// before a tile's have gone on (by when it starts), the tile hands its own on
 // untried: a patch is the same by any way, and the tiles' way and then the last
 // kernels' costs 11 + 4 + 25 f us per 10^6 packets with a share f of them going
 // on, the last kernels alone 27. A cell's word holds all that its values follow
@@ -267,7 +267,7 @@ __device__ __forceinline__ void write_patch(OutT *row, const unsigned *key, int 
 }
 // one warp: lists those of the patches p0 .. p0 + m that go on
 template <class F>
-__device__ __forceinline__ void list_patches(int m, F goes_on, long long p0, unsigned *inc, PatchInfo *info) {
+__device__ __forceinline__ void list_patches(int m, F goes_on, unsigned p0, unsigned *inc, PatchInfo *info) {
     const int lane = threadIdx.x & 31;
     unsigned f[PMAX / 32], cnt = 0, at = 0;
 #pragma unroll
@@ -280,7 +280,7 @@ __device__ __forceinline__ void list_patches(int m, F goes_on, long long p0, uns
     at = __shfl_sync(0xffffffffu, at, 0);
 #pragma unroll
     for (int u = 0; u < PMAX / 32; ++u) {
-        if ((f[u] >> lane) & 1u) inc[at + __popc(f[u] & ((1u << lane) - 1u))] = (unsigned)(p0 + 32 * u + lane);
+        if ((f[u] >> lane) & 1u) inc[at + __popc(f[u] & ((1u << lane) - 1u))] = p0 + 32 * u + lane;
         at += __popc(f[u]);
     }
 }
@@ -301,25 +301,21 @@ __global__ void __launch_bounds__(PTH, 4) k_patch_tiles(const uint64_t *pk, long
     // the selected clusters of the tile: labels ascend, so they are consecutive
     const TileSel ts = tiles[blockIdx.x];
     const unsigned odd = info->odd;
-    unsigned tried = 0, gone = 0;
-    if (threadIdx.x == 0) {
-        tried = __ldcg(&info->n_tried);
-        gone = __ldcg(&info->n_inc);
-    }
+    const unsigned gone = threadIdx.x == 0 ? __ldcg(&info->n_inc) : 0u;
     if (!ts.count || odd) return;
-    const long long s0 = 0xFFFFFFFFu - ts.first_inv, s1 = s0 + ts.count;
-    if (__syncthreads_or(tried >= 4096u && gone > tried / 2)) {
+    const unsigned s0 = 0xFFFFFFFFu - ts.first_inv, s1 = s0 + ts.count;
+    if (__syncthreads_or(gone > 2048u && gone > s0 / 2)) {
         if (warp == 0)
-            for (long long p0 = s0; p0 < s1; p0 += PMAX)
-                list_patches((int)min((long long)PMAX, s1 - p0), [](int) { return true; }, p0, inc, info);
+            for (unsigned p0 = s0; p0 < s1; p0 += PMAX)
+                list_patches((int)min((unsigned)PMAX, s1 - p0), [](int) { return true; }, p0, inc, info);
         return;
     }
-    auto root_of = [&](long long p0, int m) -> SelRoot { return threadIdx.x < m ? roots[p0 + threadIdx.x] : SelRoot{}; };
+    auto root_of = [&](unsigned p0, int m) -> SelRoot { return threadIdx.x < m ? roots[p0 + threadIdx.x] : SelRoot{}; };
     auto clear = [&](int m) {
         for (int k = threadIdx.x; k < PT / 4; k += PTH) reinterpret_cast<unsigned *>(s_slot)[k] = 0u;
         for (int k = threadIdx.x; k < m * PC; k += PTH) s_key[k] = 0u;
     };
-    int m = (int)min((long long)PMAX, s1 - s0);
+    int m = (int)min((unsigned)PMAX, ts.count);
     SelRoot v = root_of(s0, m);
     clear(m);
     int L[PU];
@@ -327,10 +323,10 @@ __global__ void __launch_bounds__(PTH, 4) k_patch_tiles(const uint64_t *pk, long
     for (int u = 0; u < PU; ++u) {
         const long long q = w0 + u * PTH + threadIdx.x;
         const long long lab = q >= 0 && q < n ? labels[q] : -1ll;
-        const long long r = lab - base - a;
-        L[u] = lab >= 0 && r >= 0 && r < tile_n ? (int)r : -1;
+        const unsigned long long r = (unsigned long long)(lab - base - a);
+        L[u] = lab >= 0 && r < (unsigned)tile_n ? (int)r : -1;
     }
-    for (long long p0 = s0;;) {
+    for (unsigned p0 = s0;;) {
         __syncthreads();
         if (threadIdx.x < m) {
             s_slot[v.root - a] = (unsigned char)(threadIdx.x + 1);
@@ -361,15 +357,12 @@ __global__ void __launch_bounds__(PTH, 4) k_patch_tiles(const uint64_t *pk, long
             }
         }
         __syncthreads();
-        if (warp == 0) {
-            list_patches(m, [&](int j) { return s_cnt[j] != s_n[j]; }, p0, inc, info);
-            if (lane == 0) atomicAdd(&info->n_tried, (unsigned)m);
-        }
+        if (warp == PTH / 32 - 1) list_patches(m, [&](int j) { return s_cnt[j] != s_n[j]; }, p0, inc, info);
         for (int j = warp; j < m; j += PTH / 32)
             if (s_cnt[j] == s_n[j]) write_patch(patch + (p0 + j) * (long long)NIN, s_key + j * PC, lane);
         p0 += PMAX;
         if (p0 >= s1) break;
-        m = (int)min((long long)PMAX, s1 - p0);
+        m = (int)min((unsigned)PMAX, s1 - p0);
         v = root_of(p0, m);
         __syncthreads();
         clear(m);
@@ -962,8 +955,9 @@ static int refine_patches(tpx_ctx *c, const uint64_t *d_packets, int64_t n, int6
         k_patch_wide<OutT><<<c->num_sms * 4, PWT, 0, s>>>(d_packets, n, base, lab, d_clusters, sel, d_centre, inc, d_patches,
                                                           far, info);
     }
-    PatchInfo h{};
-    if (ck(cudaMemcpyAsync(&h, info, sizeof h, cudaMemcpyDeviceToHost, s)) || ck(cudaStreamSynchronize(s))) return TPX_ECUDA;
+    static_assert(sizeof(PatchInfo) <= 4 * sizeof(int64_t), "h_words");
+    if (ck(cudaMemcpyAsync(c->h_words, info, sizeof(PatchInfo), cudaMemcpyDeviceToHost, s)) || ck(cudaStreamSynchronize(s))) return TPX_ECUDA;
+    const PatchInfo &h = *reinterpret_cast<const PatchInfo *>(c->h_words);
     const long long np = (long long)h.n_sel, ns = np < capacity ? np : capacity;
     const bool wider = search_wider(h.n_inc, n);
     const long long ni = h.odd ? ns : (long long)(wider ? h.n_far : h.n_inc);

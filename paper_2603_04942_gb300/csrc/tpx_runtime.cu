@@ -122,8 +122,8 @@ int grow(Tp **ptr, int64_t *cap, int64_t want) {
 namespace {
 
 constexpr size_t kCtlBytes = sizeof(tpxk::Ctl) + sizeof(unsigned);
-// its pinned copy, and behind it the two counts of a host call
-constexpr size_t kHostCountsAt = (kCtlBytes + 7) & ~size_t(7), kHostCtlBytes = kHostCountsAt + 2 * sizeof(int64_t);
+// its pinned copy, and behind it h_words
+constexpr size_t kHostWordsAt = (kCtlBytes + 7) & ~size_t(7), kHostCtlBytes = kHostWordsAt + 4 * sizeof(int64_t);
 
 // A call's failure bits (a range the tiles could not hold, a batch run to
 // redo) are resolved by the tpx_sync after it. When a new call starts before
@@ -274,6 +274,7 @@ int tpx_create(tpx_ctx **out, const tpx_config *cfg, int64_t max_packets, void *
         return TPX_ENOMEM;
     }
     std::memset(c->h_ctl, 0, kHostCtlBytes);
+    c->h_words = reinterpret_cast<int64_t *>(reinterpret_cast<char *>(c->h_ctl) + kHostWordsAt);
     cudaMemset(c->ctl, 0, kCtlBytes);
     c->d_sticky = reinterpret_cast<unsigned *>(c->ctl + 1);
     if (cudaMalloc(&c->d_state, 2 * sizeof(tpxk::GAgg)) != cudaSuccess) {
@@ -1019,7 +1020,7 @@ int tpx_process_host(tpx_ctx *c, const uint64_t *h_packets, int64_t n, int64_t i
     // stream: one wait for them, one for the records (three, with the status
     // read by itself first: 200 shots 99 us, so 84). A call that the fused kernel
     // could not hold is redone after the first wait, and its outputs go down again.
-    int64_t *counts = reinterpret_cast<int64_t *>(reinterpret_cast<char *>(c->h_ctl) + kHostCountsAt);
+    int64_t *counts = c->h_words;
     auto per_packet_down = [&]() -> int {
         if (ckr(cudaMemcpyAsync(counts, c->st_counts, 2 * sizeof(int64_t), cudaMemcpyDeviceToHost, s))) return TPX_ECUDA;
         if (h_labels && n &&
