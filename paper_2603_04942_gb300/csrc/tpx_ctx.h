@@ -137,6 +137,10 @@ struct tpx_ctx {
 // ping-pong; tpx_runtime.cu)
 void take_state(tpx_ctx *c, const tpxk::GAgg **E0, tpxk::GAgg **out);
 
+// device memory (not mapped host or managed memory): a kernel may prefetch from
+// it into L2 with the bulk-copy engine (tpx_runtime.cu)
+bool device_memory(const void *ptr);
+
 // general (global-memory) path, tpx_general.cu
 namespace tpxg {
 // grow the context's general scratch to at least `bytes` (synchronises)

@@ -716,7 +716,7 @@ __device__ __forceinline__ void load_b2(uint32_t addr, uint32_t (&b)[4]) {
 template <int H, int MT>
 __global__ void __launch_bounds__(256, 1) k_mlp_bf16(const float *__restrict__ x, long long n,
                                                       const uint16_t *__restrict__ wt, const float *__restrict__ bias,
-                                                      float *__restrict__ out) {
+                                                      float *__restrict__ out, bool l2) {
     using G = MlpGeo<H>;
     constexpr int NT = G::NT, S2 = G::S2, NH = NT / 2, ROWS = 128 * MT, K1 = K1P / 16;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -725,9 +725,9 @@ __global__ void __launch_bounds__(256, 1) k_mlp_bf16(const float *__restrict__ x
     uint16_t *W3s = W2s + H * S2;
     float *Bs = reinterpret_cast<float *>(W3s + 8 * S2);
     const long long n_tiles = (n + ROWS - 1) / ROWS;
-    // the whole 16-byte words of tile t's rows, into L2
+    // the whole 16-byte words of tile t's rows, into L2 (l2: they lie in device memory)
     auto prefetch = [&](long long t) {
-        if (threadIdx.x != 0 || t >= n_tiles) return;
+        if (threadIdx.x != 0 || t >= n_tiles || !l2) return;
         const char *a = reinterpret_cast<const char *>(x + t * ROWS * NIN);
         const char *b = reinterpret_cast<const char *>(x + min(n, (t + 1) * (long long)ROWS) * NIN);
         a += (16 - (reinterpret_cast<uintptr_t>(a) & 15)) & 15;
@@ -883,8 +883,9 @@ int infer_h(tpx_ctx *c, const void *packed, const float *x, long long n, float *
     const float *bias = reinterpret_cast<const float *>(static_cast<const char *>(packed) + packed_bias_off(G::wend));
     // one tile of 128 rows per SM is the shortest way for few rows; beyond that 256 rows a tile
     const long long tiles = (n + 127) / 128;
-    if (tiles <= sms) k_mlp_bf16<H, 1><<<(unsigned)tiles, 256, G::smem, c->stream>>>(x, n, wt, bias, out);
-    else k_mlp_bf16<H, 2><<<(unsigned)std::min<long long>((n + 255) / 256, sms), 256, G::smem, c->stream>>>(x, n, wt, bias, out);
+    const bool l2 = device_memory(x);
+    if (tiles <= sms) k_mlp_bf16<H, 1><<<(unsigned)tiles, 256, G::smem, c->stream>>>(x, n, wt, bias, out, l2);
+    else k_mlp_bf16<H, 2><<<(unsigned)std::min<long long>((n + 255) / 256, sms), 256, G::smem, c->stream>>>(x, n, wt, bias, out, l2);
     return ck(cudaGetLastError()) ? TPX_ECUDA : TPX_OK;
 }
 template <int H>

@@ -14,6 +14,16 @@
 #include "tpx_fused.cuh"
 
 
+bool device_memory(const void *ptr) {
+    if (!ptr) return false;
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, ptr) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return a.type == cudaMemoryTypeDevice;
+}
+
 void take_state(tpx_ctx *c, const tpxk::GAgg **E0, tpxk::GAgg **out) {
     *E0 = (c->cfg.chain || c->state_once) ? &c->d_state[c->cur] : nullptr;
     *out = &c->d_state[c->cur ^ 1];
@@ -161,18 +171,6 @@ int tune_pick(const tpx_ctx *c, int64_t n) {
         return n <= (int64_t)c->num_sms * tpxk::fused_tile_packets(tpxk::GEO_SMALL) ? tpxk::GEO_SMALL : tpxk::GEO_T4096;
     // alternate, the smaller tiles first
     return c->tune.issued[tpxk::GEO_T2048 - 1] <= c->tune.issued[tpxk::GEO_T4096 - 1] ? tpxk::GEO_T2048 : tpxk::GEO_T4096;
-}
-
-// device memory (not mapped host or managed memory): the fused kernel may
-// prefetch such packets into L2 with the bulk-copy engine
-bool device_memory(const void *ptr) {
-    if (!ptr) return false;
-    cudaPointerAttributes a;
-    if (cudaPointerGetAttributes(&a, ptr) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
-    return a.type == cudaMemoryTypeDevice;
 }
 
 // kernel timing: add the oldest recorded launch's pre-pass and fused-kernel
