@@ -309,18 +309,6 @@ __device__ __forceinline__ uint32_t core_off(int r, int k, int kp) {
 
 constexpr long long kSpin = 1LL << 24;   // bounded mbarrier wait (then an error flag)
 
-// asynchronous global -> shared copies (16 or 4 bytes; 0 source bytes fill zeros)
-__device__ __forceinline__ void cp16(void *dst, const void *src, bool valid) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(valid ? 16 : 0)
-                 : "memory");
-}
-__device__ __forceinline__ void cp4(void *dst, const void *src) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_wait_all() {
-    asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
-}
-
 // packed inference weights: per layer [N][KP] bf16 with column k = tap * cin +
 // ci (8 channels of a tap per 16-byte chunk; conv1: ky * 8 + kx * 2 + ci, one
 // chunk per kernel row), zero padded; then the biases (fp32, padded to N)

@@ -96,20 +96,6 @@ __device__ __forceinline__ unsigned ld_relaxed(const unsigned *p) {
 __device__ __forceinline__ void st_release(unsigned *p, unsigned v) {
     asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
-__device__ __forceinline__ void st_agg(GAgg *dst, const GAgg &a) {
-    long long *d = reinterpret_cast<long long *>(dst);
-    const long long *s = reinterpret_cast<const long long *>(&a);
-#pragma unroll
-    for (int i = 0; i < 8; i++) __stcg(d + i, s[i]);
-}
-__device__ __forceinline__ GAgg ld_agg(const GAgg *src) {
-    GAgg a;
-    const long long *s = reinterpret_cast<const long long *>(src);
-    long long *d = reinterpret_cast<long long *>(&a);
-#pragma unroll
-    for (int i = 0; i < 8; i++) d[i] = __ldcg(s + i);
-    return a;
-}
 
 // A (segment, y, x) cell's bit of the cell table: TR rows of 256 columns, the
 // rows of a shot shifted by its number, so that a row of cells is a run of bits
@@ -346,15 +332,6 @@ __device__ __forceinline__ unsigned long long warp_sum(unsigned long long v) {
 // chain costs one bounded wait, not one per tile
 __device__ __forceinline__ bool timed_out(const Params &p) {
     return (*reinterpret_cast<volatile unsigned *>(&p.ctl->status) & ST_DEVTIMEOUT) != 0;
-}
-
-__device__ __forceinline__ GChain shfl_down_chain(const GChain &v, int o) {
-    GChain u;
-    u.n = __shfl_down_sync(0xffffffffu, v.n, o);
-    u.first = __shfl_down_sync(0xffffffffu, v.first, o);
-    u.last = __shfl_down_sync(0xffffffffu, v.last, o);
-    u.sum = __shfl_down_sync(0xffffffffu, v.sum, o);
-    return u;
 }
 
 // Bounded decoupled look-back, one warp. Each trip reads the flags of

@@ -1460,15 +1460,6 @@ __global__ void __launch_bounds__(GT) k_root_place(RootFlag f, tpx_hits h, long 
     if (blockIdx.x == nb - 1 && threadIdx.x == 0) latch_count(first + total, cap, n_rec, status, counter);
 }
 
-__device__ __forceinline__ long long find_index(const int64_t *index, long long n, long long v) {
-    long long lo = 0, hi = n;
-    while (lo < hi) {
-        const long long mid = lo + ((hi - lo) >> 1);
-        if (index[mid] < v) lo = mid + 1; else hi = mid;
-    }
-    return lo;
-}
-
 // Every hit adds to its record's sums. The record comes from the rank table
 // (4 bytes per stream index; a binary search over the roots where the indices
 // span more). A block's 4096 hits in stream order belong to a few hundred
