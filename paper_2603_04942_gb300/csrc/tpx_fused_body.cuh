@@ -758,6 +758,11 @@ __device__ __forceinline__ unsigned br_find(uint32_t pb, unsigned x) {
         x = g;
     }
 }
+__device__ __forceinline__ unsigned br_root(uint32_t pb, unsigned x) {   // changes nothing
+    unsigned px;
+    while ((px = br_ld(pb, x)) != x) x = px;
+    return x;
+}
 // The root of a big-range cluster need not be any particular pixel (its
 // label comes from its moments), so roots are linked by a hashed priority,
 // the lower under the higher: the sorted order puts a cluster's pixels on
@@ -1256,8 +1261,10 @@ __device__ __noinline__ int big_range(Smem &S, const Params &p, long long base, 
     cta_sync();
     for (int w = tid; w < BR_LW; w += NTW) lbits[w] = 0u;
     BR_PH(23);
-    // compress: every pixel points to its root
-    for (int i = tid; i < N; i += NTW) br_st(pb, (unsigned)i, br_find(pb, (unsigned)i));
+    // compress: every pixel points to its root. Each pointer is changed by its own
+    // thread alone: a find that halves paths on the way could put an ancestor back
+    // over a root that the pixel's thread has just stored
+    for (int i = tid; i < N; i += NTW) br_st(pb, (unsigned)i, br_root(pb, (unsigned)i));
     cta_sync();
     // roots: their moment records cleared, counted
     {
