@@ -243,8 +243,11 @@ constexpr int BR_REGION = (int)offsetof(Smem, tdc_t);
 static_assert(BR_REGION >= BIG_REGION, "the big-range scratch");
 // the neighbour pass chains the pixels by cell: heads in place of the sort's
 // bins, and the chains of the first BR_NX pixels in shared memory (the others'
-// in the scratch)
+// in the scratch); the window pass reads the sorted records through the same
+// place, BR_CH pixels at a time with those before them
 constexpr int BR_NX = 16 * NT;
+constexpr int BR_CH = 2 * NT, BR_SB = 4 * NT;
+static_assert(8 * BR_SB <= 2 * BR_NX, "the window's records in the chains' place");
 constexpr int BR_FIXED = 4 * (BR_BINS + 4) + 4 * BR_LW + 2 * BR_LW + 4 * 5 * BR_S + 4 * 16 + 2 * BR_NX;
 // kept pixels: a 16-bit parent and a local-maximum bit each
 constexpr int BR_N0 = ((BR_REGION - BR_FIXED) * 8 / 17) & ~63;
@@ -720,8 +723,8 @@ __device__ __forceinline__ void scan_label_bits(Smem &S) {
 // pixel walks the chains of the forward half of its box (in its own cell only
 // the pixels before it in the sorted order), so every adjacent pair (Sec. V.A:
 // same shot, box neighbours, |dt| within the radius) is seen once. (Comparing
-// each pixel with all of the time bins and stripes around it cost 134 of the
-// path's 179 warp instructions per packet.) Union-find over the sorted order
+// each pixel with all of the time bins and stripes around it, as wide boxes
+// still do, cost 134 of 179 warp instructions per packet.) Union-find over the sorted order
 // runs in shared
 // memory (16-bit parents, roots linked by a hashed priority). The
 // exact integer moments of each cluster (Sec. V.C) are gathered with
@@ -797,6 +800,101 @@ __device__ __forceinline__ void br_unite(uint32_t pb, unsigned a, unsigned b) {
 #else
 #define BR_PH(k) do {} while (0)
 #endif
+// What the window pass needs of a big range: its sorted pixels, the ends of
+// their keys (bins), the shots' first bins, times and bin widths.
+struct BrSorted {
+    const uint64_t *srec;
+    const uint16_t *spos;
+    const unsigned *bins;
+    const int *lo, *b0, *w;
+    uint64_t *sbuf;
+    int *task;
+    uint32_t pb, nb_sh;
+    int N, NS, SW;
+};
+// The earlier pixels that can neighbour pixel i: two runs of consecutive slots,
+// the previous time bin's stripes around its own, and its own bin's left stripe
+// with its own key up to itself.
+__device__ __forceinline__ void br_candidates(const BrSorted &V, int i, uint64_t r, int *a0, int *la, int *b0, int *lb) {
+    const int s = r_seg(r), st = r_x(r) / V.SW;
+    const int bin = V.b0[s] + (r_tof(r) - V.lo[s]) / V.w[s];
+    auto first = [&](int k) -> int { return k > 0 ? (int)V.bins[k - 1] : 0; };   // a key's first slot
+    *a0 = *la = 0;
+    if (bin > V.b0[s]) {
+        *a0 = first((bin - 1) * V.NS + max(st - 1, 0));
+        *la = (int)V.bins[(bin - 1) * V.NS + min(st + 1, V.NS - 1)] - *a0;
+    }
+    *b0 = first(bin * V.NS + max(st - 1, 0));
+    *lb = i - *b0;
+}
+// The neighbour pass of wide boxes: every pixel is compared with the pixels of
+// its window, whatever the radii; an adjacent pair clears the loser's
+// local-maximum flag and unites. A warp takes 32 consecutive pixels at a time,
+// the next task from the chunk's counter, and spreads all their (pixel,
+// candidate) pairs evenly over its lanes: a prefix of the pixels' counts, and
+// each lane finds the pixel of its pair by a search over the lanes.
+__device__ __noinline__ void br_window(const Params &p, const BrSorted V) {
+    const int tid = threadIdx.x, lane = tid & 31, rx = p.rx, ry = p.ry, dt = p.dt;
+    for (int a = 0; a < V.N; a += BR_CH) {
+        const int e = min(V.N, a + BR_CH);
+        int lo;   // the chunk's pixels look no further back than the start of the first one's previous bin
+        {
+            const uint64_t ra = V.srec[a];
+            const int s = r_seg(ra), bin = V.b0[s] + (r_tof(ra) - V.lo[s]) / V.w[s];
+            const int k0 = (bin > V.b0[s] ? bin - 1 : bin) * V.NS;
+            lo = k0 > 0 ? (int)V.bins[k0 - 1] : 0;
+        }
+        const bool fits = e - lo <= BR_SB;
+        if (tid == 0) *V.task = 0;
+        if (fits)
+            for (int j = lo + tid; j < e; j += NTW) V.sbuf[j - lo] = V.srec[j];
+        cta_sync();
+        auto rec_at = [&](int j) -> uint64_t { return fits ? V.sbuf[j - lo] : V.srec[j]; };
+        const int ntask = (e - a + 31) >> 5;
+        for (;;) {
+            int task = 0;
+            if (lane == 0) task = atomicAdd(V.task, 1);
+            task = __shfl_sync(0xffffffffu, task, 0);
+            if (task >= ntask) break;
+            const int i0 = a + 32 * task, i = i0 + lane;
+            int a0 = 0, na = 0, c0 = 0, nc = 0;
+            if (i < e) br_candidates(V, i, rec_at(i), &a0, &na, &c0, &nc);
+            const int n = na + nc;
+            int incl = n;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int u = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += u;
+            }
+            const int off = incl - n;
+            const int W = __shfl_sync(0xffffffffu, incl, 31);
+            for (int wb = 0; wb < W; wb += 32) {
+                const int w = wb + lane;
+                int q = 0;   // the last lane whose pairs start at or before w
+#pragma unroll
+                for (int step = 16; step > 0; step >>= 1) {
+                    const int o = __shfl_sync(0xffffffffu, off, q + step);
+                    if (o <= w) q += step;
+                }
+                const int qa0 = __shfl_sync(0xffffffffu, a0, q), qna = __shfl_sync(0xffffffffu, na, q);
+                const int qc0 = __shfl_sync(0xffffffffu, c0, q), qoff = __shfl_sync(0xffffffffu, off, q);
+                if (w >= W) continue;
+                const int c = w - qoff, ip = i0 + q, j = c < qna ? qa0 + c : qc0 + (c - qna);
+                if (!TPX_IN(j, V.N) || !TPX_IN(ip, V.N)) continue;
+                const uint64_t rp = rec_at(ip), rj = rec_at(j);
+                const int dx = r_x(rj) - r_x(rp), dy = r_y(rj) - r_y(rp);
+                if (dx < -rx || dx > rx || dy < -ry || dy > ry || !within(r_tof(rj) - r_tof(rp), dt)) continue;
+                const int tj = r_tot(rj), ti = r_tot(rp);
+                const bool j_wins = tj > ti || (tj == ti && V.spos[j] > V.spos[ip]);
+                const int loser = j_wins ? ip : j;
+                br_or(V.nb_sh + 4 * (loser >> 5), 1u << (loser & 31));
+                br_unite(V.pb, (unsigned)ip, (unsigned)j);
+            }
+        }
+        cta_sync();
+    }
+}
+
 template <bool BATCH>
 __device__ __noinline__ int big_range(Smem &S, const Params &p, long long base, long long rend, int f, int from,
                                       bool prev_global, const GAgg &E, int slot) {
@@ -1112,150 +1210,174 @@ __device__ __noinline__ int big_range(Smem &S, const Params &p, long long base, 
     }
     for (int i = tid; i < N; i += NTW) par[i] = (uint16_t)i;
     for (int w = tid; w < BR_N / 32; w += NTW) npk[w] = 0u;
-    // the neighbour pass's flags, a byte each in what the parents leave free:
-    // plain stores (as bits, 32 lanes of one cluster met in the same word's
-    // atomics: a third of the path's cycles)
-    uint8_t *lost = 3 * N + 3 <= 2 * BR_N ? reinterpret_cast<uint8_t *>(par + N) : nullptr;
-    if (lost)
-        for (int i = tid; i < N; i += NTW) lost[i] = 0;
-    // Behind them, and on in the label bitmap's place, a byte hashed from each
-    // pixel's cell, as far as that goes (18,592 pixels with 4096-packet tiles):
-    // the other cells of a bucket cost no read of their record, which come from
-    // L2 (14% hits in L1)
-    constexpr int TAG2 = 6 * BR_LW;                              // bytes of lbits and lpre
-    const int tag1 = lost ? 2 * (BR_N - N) - N : 0;
-    uint8_t *tags1 = reinterpret_cast<uint8_t *>(par + N) + N, *tags2 = reinterpret_cast<uint8_t *>(lbits);
-    auto tag_of = [&](uint32_t cell) -> unsigned { return (cell * 0x85EBCA6Bu) >> 24; };
     cta_sync();
-    // ---- the cell chains: the last pixel of a bucket first ----
-    constexpr unsigned NONE = 0xFFFFu;
-    auto bucket = [&](uint32_t cell) -> unsigned { return __umulhi(cell * 0x9E3779B1u, (unsigned)BR_BINS); };
-    for (int b = tid; b < BR_BINS; b += NTW) bins[b] = NONE;
-    cta_sync();
-    for (int i = tid; i < N; i += NTW) {
-        const uint32_t cell = r_cell(g_srec[i]);
-        const unsigned prev = atomicExch(&bins[bucket(cell)], (unsigned)i);
-        if (i < BR_NX) nx_sh[i] = (uint16_t)prev; else nx_g[i] = (uint16_t)prev;
-        if (i < tag1) tags1[i] = (uint8_t)tag_of(cell);
-        else if (i - tag1 < TAG2) tags2[i - tag1] = (uint8_t)tag_of(cell);
-    }
-    cta_sync();
-
-    BR_PH(22);
-    // ---- neighbour pass: every pixel against the chains of the cells that can
-    // hold its neighbours (the box rule, Sec. V.A); an adjacent pair clears the
-    // loser's local-maximum flag (Sec. V.B: the larger ToT wins, equal ToT goes
-    // to the later pixel). A pixel points to the first neighbour it finds: its
-    // own entry only, and pointers go forward in a strict order (cell, then
-    // slot), so they form a forest without a single compare-and-swap. The next
-    // three neighbours are kept aside. Consecutive slots are mostly one
-    // cluster, so a warp's chains are near each other and its records in L1 ----
-    // the first pixel from j on along its chain that may be of the cell (own:
-    // only those before pixel i), NONE at the end
-    auto next_of = [&](int i, uint32_t cell, unsigned j, bool own) -> unsigned {
-        const unsigned tag = tag_of(cell);
-        while (j != NONE) {
-            if (!TPX_IN(j, N)) return NONE;
-            const int k = (int)j - tag1;
-            const unsigned t = k < 0 ? tags1[j] : k < TAG2 ? tags2[k] : tag;
-            if (t == tag && !(own && j >= (unsigned)i)) return j;
-            j = j < (unsigned)BR_NX ? nx_sh[j] : nx_g[j];
+    // Boxes of more than the eight neighbours: the cells of the forward half (13
+    // at radius 2, 113 at 7) or the candidates of a window, whichever is less
+    // work (a cell costs about as much as eight candidates). 66 shots of 9000
+    // pixels: chains 836, 1318, 5187 us at radius 2, 3, 7, windows 495, 526, 545;
+    // with a time radius over the whole shot chains 945 at radius 2, windows 2780.
+    const int cells = (rx + 1) * (2 * ry + 1) - ry;
+    bool window = false;
+    if (cells > 5) {
+        const BrSorted V{g_srec, g_spos, bins, sg_lo, sg_b0, sg_w, reinterpret_cast<uint64_t *>(nx_sh), &misc[12], pb, nb_sh, N, NS, SW};
+        unsigned cand = 0;   // N^2 in all at most
+        for (int i = tid; i < N; i += NTW) {
+            int a0, la, b0, lb;
+            br_candidates(V, i, g_srec[i], &a0, &la, &b0, &lb);
+            cand += (unsigned)(la + lb);
         }
-        return NONE;
-    };
-    auto link = [&](unsigned j) -> unsigned { return j < (unsigned)BR_NX ? nx_sh[j] : nx_g[j]; };
-    // every neighbour of pixel i among the forward half of its box
-    auto walk_all = [&](int i, uint64_t ri, auto pair) {
-        const int x = r_x(ri), y = r_y(ri), tb = r_tof(ri);
-        const uint32_t seg = r_cell(ri) & ~0xFFFFu;
-        auto cell_at = [&](int cx, int cy) -> uint32_t { return seg | ((uint32_t)cy << 8) | (uint32_t)cx; };
-        auto first_of = [&](int cx, int cy, bool own) -> unsigned {
-            if (cx > 255 || cy < 0 || cy > 255) return NONE;
-            return next_of(i, cell_at(cx, cy), bins[bucket(cell_at(cx, cy))], own);
-        };
-        // the chain from its first candidate j on, whose record is r
-        auto walk = [&](uint32_t cell, unsigned j, uint64_t r, bool own) {
+        cand = __reduce_add_sync(0xffffffffu, cand);
+        if (lane == 0) atomicAdd(reinterpret_cast<unsigned *>(&misc[13]), cand);
+        cta_sync();
+        window = (unsigned)misc[13] <= 8u * (unsigned)cells * (unsigned)N;
+        if (window) br_window(p, V);
+    }
+    if (!window) {
+        // the neighbour pass's flags, a byte each in what the parents leave free:
+        // plain stores (as bits, 32 lanes of one cluster met in the same word's
+        // atomics: a third of the path's cycles)
+        uint8_t *lost = 3 * N + 3 <= 2 * BR_N ? reinterpret_cast<uint8_t *>(par + N) : nullptr;
+        if (lost)
+            for (int i = tid; i < N; i += NTW) lost[i] = 0;
+        // Behind them, and on in the label bitmap's place, a byte hashed from each
+        // pixel's cell, as far as that goes (18,592 pixels with 4096-packet tiles):
+        // the other cells of a bucket cost no read of their record, which come from
+        // L2 (14% hits in L1)
+        constexpr int TAG2 = 6 * BR_LW;                              // bytes of lbits and lpre
+        const int tag1 = lost ? 2 * (BR_N - N) - N : 0;
+        uint8_t *tags1 = reinterpret_cast<uint8_t *>(par + N) + N, *tags2 = reinterpret_cast<uint8_t *>(lbits);
+        auto tag_of = [&](uint32_t cell) -> unsigned { return (cell * 0x85EBCA6Bu) >> 24; };
+        cta_sync();
+        // ---- the cell chains: the last pixel of a bucket first ----
+        constexpr unsigned NONE = 0xFFFFu;
+        auto bucket = [&](uint32_t cell) -> unsigned { return __umulhi(cell * 0x9E3779B1u, (unsigned)BR_BINS); };
+        for (int b = tid; b < BR_BINS; b += NTW) bins[b] = NONE;
+        cta_sync();
+        for (int i = tid; i < N; i += NTW) {
+            const uint32_t cell = r_cell(g_srec[i]);
+            const unsigned prev = atomicExch(&bins[bucket(cell)], (unsigned)i);
+            if (i < BR_NX) nx_sh[i] = (uint16_t)prev; else nx_g[i] = (uint16_t)prev;
+            if (i < tag1) tags1[i] = (uint8_t)tag_of(cell);
+            else if (i - tag1 < TAG2) tags2[i - tag1] = (uint8_t)tag_of(cell);
+        }
+        cta_sync();
+
+        BR_PH(22);
+        // ---- neighbour pass: every pixel against the chains of the cells that can
+        // hold its neighbours (the box rule, Sec. V.A); an adjacent pair clears the
+        // loser's local-maximum flag (Sec. V.B: the larger ToT wins, equal ToT goes
+        // to the later pixel). A pixel points to the first neighbour it finds: its
+        // own entry only, and pointers go forward in a strict order (cell, then
+        // slot), so they form a forest without a single compare-and-swap. The next
+        // three neighbours are kept aside. Consecutive slots are mostly one
+        // cluster, so a warp's chains are near each other and its records in L1 ----
+        // the first pixel from j on along its chain that may be of the cell (own:
+        // only those before pixel i), NONE at the end
+        auto next_of = [&](int i, uint32_t cell, unsigned j, bool own) -> unsigned {
+            const unsigned tag = tag_of(cell);
             while (j != NONE) {
-                if (r_cell(r) == cell && within(r_tof(r) - tb, dtr)) pair(j, r);
-                j = next_of(i, cell, link(j), own);
-                if (j != NONE) r = g_srec[j];
+                if (!TPX_IN(j, N)) return NONE;
+                const int k = (int)j - tag1;
+                const unsigned t = k < 0 ? tags1[j] : k < TAG2 ? tags2[k] : tag;
+                if (t == tag && !(own && j >= (unsigned)i)) return j;
+                j = j < (unsigned)BR_NX ? nx_sh[j] : nx_g[j];
+            }
+            return NONE;
+        };
+        auto link = [&](unsigned j) -> unsigned { return j < (unsigned)BR_NX ? nx_sh[j] : nx_g[j]; };
+        // every neighbour of pixel i among the forward half of its box
+        auto walk_all = [&](int i, uint64_t ri, auto pair) {
+            const int x = r_x(ri), y = r_y(ri), tb = r_tof(ri);
+            const uint32_t seg = r_cell(ri) & ~0xFFFFu;
+            auto cell_at = [&](int cx, int cy) -> uint32_t { return seg | ((uint32_t)cy << 8) | (uint32_t)cx; };
+            auto first_of = [&](int cx, int cy, bool own) -> unsigned {
+                if (cx > 255 || cy < 0 || cy > 255) return NONE;
+                return next_of(i, cell_at(cx, cy), bins[bucket(cell_at(cx, cy))], own);
+            };
+            // the chain from its first candidate j on, whose record is r
+            auto walk = [&](uint32_t cell, unsigned j, uint64_t r, bool own) {
+                while (j != NONE) {
+                    if (r_cell(r) == cell && within(r_tof(r) - tb, dtr)) pair(j, r);
+                    j = next_of(i, cell, link(j), own);
+                    if (j != NONE) r = g_srec[j];
+                }
+            };
+            if (rx == 1 && ry == 1) {   // the five cells' first candidates, then their records together
+                unsigned j[5];
+                uint64_t r[5];
+                j[0] = first_of(x, y, true);
+                j[1] = first_of(x, y + 1, false);
+                j[2] = first_of(x + 1, y, false);
+                j[3] = first_of(x + 1, y - 1, false);
+                j[4] = first_of(x + 1, y + 1, false);
+#pragma unroll
+                for (int k = 0; k < 5; ++k) r[k] = j[k] != NONE ? g_srec[j[k]] : 0ull;
+                walk(cell_at(x, y), j[0], r[0], true);
+                walk(cell_at(x, y + 1), j[1], r[1], false);
+                walk(cell_at(x + 1, y), j[2], r[2], false);
+                walk(cell_at(x + 1, y - 1), j[3], r[3], false);
+                walk(cell_at(x + 1, y + 1), j[4], r[4], false);
+            } else {
+                for (int dx = 0; dx <= rx; ++dx)
+                    for (int dy = dx == 0 ? 0 : -ry; dy <= ry; ++dy) {
+                        const bool own = dx == 0 && dy == 0;
+                        const unsigned j = first_of(x + dx, y + dy, own);
+                        if (j != NONE) walk(cell_at(x + dx, y + dy), j, g_srec[j], own);
+                    }
             }
         };
-        if (rx == 1 && ry == 1) {   // the five cells' first candidates, then their records together
-            unsigned j[5];
-            uint64_t r[5];
-            j[0] = first_of(x, y, true);
-            j[1] = first_of(x, y + 1, false);
-            j[2] = first_of(x + 1, y, false);
-            j[3] = first_of(x + 1, y - 1, false);
-            j[4] = first_of(x + 1, y + 1, false);
-#pragma unroll
-            for (int k = 0; k < 5; ++k) r[k] = j[k] != NONE ? g_srec[j[k]] : 0ull;
-            walk(cell_at(x, y), j[0], r[0], true);
-            walk(cell_at(x, y + 1), j[1], r[1], false);
-            walk(cell_at(x + 1, y), j[2], r[2], false);
-            walk(cell_at(x + 1, y - 1), j[3], r[3], false);
-            walk(cell_at(x + 1, y + 1), j[4], r[4], false);
-        } else {
-            for (int dx = 0; dx <= rx; ++dx)
-                for (int dy = dx == 0 ? 0 : -ry; dy <= ry; ++dy) {
-                    const bool own = dx == 0 && dy == 0;
-                    const unsigned j = first_of(x + dx, y + dy, own);
-                    if (j != NONE) walk(cell_at(x + dx, y + dy), j, g_srec[j], own);
-                }
-        }
-    };
-    for (int i0 = wid * 32; i0 < N; i0 += NTW) {
-        const int i = i0 + lane;
-        bool own_lost = false;
-        if (i < N) {
-            const uint64_t ri = g_srec[i];
-            const int ti = r_tot(ri);
-            unsigned n = 0;
-            uint64_t more = 0;
-            walk_all(i, ri, [&](unsigned j, uint64_t rj) {
-                const int tj = r_tot(rj);
-                const bool j_wins = tj > ti || (tj == ti && g_spos[j] > g_spos[i]);
-                if (j_wins) own_lost = true;
-                else if (lost) lost[j] = 1;
-                else br_or(nb_sh + 4 * (j >> 5), 1u << (j & 31));
-                if (n == 0) br_st(pb, (unsigned)i, j);
-                else if (n <= 3) more |= (uint64_t)j << (16 * (n - 1));
-                n = min(n + 1, 5u);
-            });
-            g_more[i] = more | ((uint64_t)n << 48);
-        }
-        const unsigned w = __ballot_sync(0xffffffffu, own_lost);   // 32 consecutive slots: one word
-        if (lane == 0 && w) br_or(nb_sh + 4 * (i0 >> 5), w);
-    }
-    cta_sync();
-    // every pixel to its root, then the pairs that the pointers left out: the
-    // two ends have one root already, nearly always (with a union for each of
-    // the 4 pairs per pixel, lanes of one cluster met in the same
-    // compare-and-swaps and flag words: this pass took 1.1e6 cycles of the
-    // path's 1.5e6 per shot of 15,500 pixels, now 0.33e6 of 0.73e6; 600 such
-    // shots 4.1 -> 2.35 ms)
-    for (int i = tid; i < N; i += NTW) {
-        unsigned r = br_ld(pb, (unsigned)i);
-        for (unsigned up = br_ld(pb, r); up != r; up = br_ld(pb, r)) r = up;
-        br_st(pb, (unsigned)i, r);
-    }
-    if (lost)
         for (int i0 = wid * 32; i0 < N; i0 += NTW) {
-            const unsigned w = __ballot_sync(0xffffffffu, i0 + lane < N && lost[i0 + lane]);
+            const int i = i0 + lane;
+            bool own_lost = false;
+            if (i < N) {
+                const uint64_t ri = g_srec[i];
+                const int ti = r_tot(ri);
+                unsigned n = 0;
+                uint64_t more = 0;
+                walk_all(i, ri, [&](unsigned j, uint64_t rj) {
+                    const int tj = r_tot(rj);
+                    const bool j_wins = tj > ti || (tj == ti && g_spos[j] > g_spos[i]);
+                    if (j_wins) own_lost = true;
+                    else if (lost) lost[j] = 1;
+                    else br_or(nb_sh + 4 * (j >> 5), 1u << (j & 31));
+                    if (n == 0) br_st(pb, (unsigned)i, j);
+                    else if (n <= 3) more |= (uint64_t)j << (16 * (n - 1));
+                    n = min(n + 1, 5u);
+                });
+                g_more[i] = more | ((uint64_t)n << 48);
+            }
+            const unsigned w = __ballot_sync(0xffffffffu, own_lost);   // 32 consecutive slots: one word
             if (lane == 0 && w) br_or(nb_sh + 4 * (i0 >> 5), w);
         }
-    cta_sync();
-    for (int i = tid; i < N; i += NTW) {
-        const uint64_t more = g_more[i];
-        const unsigned n = (unsigned)(more >> 48);
-        auto join = [&](unsigned j) {
-            if (TPX_IN(j, N) && br_ld(pb, (unsigned)i) != br_ld(pb, j)) br_unite(pb, (unsigned)i, j);
-        };
-        if (n <= 4) {
-            for (unsigned k = 1; k < n; ++k) join((unsigned)(more >> (16 * (k - 1))) & 0xFFFFu);
-        } else {
-            walk_all(i, g_srec[i], [&](unsigned j, uint64_t) { join(j); });
+        cta_sync();
+        // every pixel to its root, then the pairs that the pointers left out: the
+        // two ends have one root already, nearly always (with a union for each of
+        // the 4 pairs per pixel, lanes of one cluster met in the same
+        // compare-and-swaps and flag words: this pass took 1.1e6 cycles of the
+        // path's 1.5e6 per shot of 15,500 pixels, now 0.33e6 of 0.73e6; 600 such
+        // shots 4.1 -> 2.35 ms)
+        for (int i = tid; i < N; i += NTW) {
+            unsigned r = br_ld(pb, (unsigned)i);
+            for (unsigned up = br_ld(pb, r); up != r; up = br_ld(pb, r)) r = up;
+            br_st(pb, (unsigned)i, r);
+        }
+        if (lost)
+            for (int i0 = wid * 32; i0 < N; i0 += NTW) {
+                const unsigned w = __ballot_sync(0xffffffffu, i0 + lane < N && lost[i0 + lane]);
+                if (lane == 0 && w) br_or(nb_sh + 4 * (i0 >> 5), w);
+            }
+        cta_sync();
+        for (int i = tid; i < N; i += NTW) {
+            const uint64_t more = g_more[i];
+            const unsigned n = (unsigned)(more >> 48);
+            auto join = [&](unsigned j) {
+                if (TPX_IN(j, N) && br_ld(pb, (unsigned)i) != br_ld(pb, j)) br_unite(pb, (unsigned)i, j);
+            };
+            if (n <= 4) {
+                for (unsigned k = 1; k < n; ++k) join((unsigned)(more >> (16 * (k - 1))) & 0xFFFFu);
+            } else {
+                walk_all(i, g_srec[i], [&](unsigned j, uint64_t) { join(j); });
+            }
         }
     }
     cta_sync();
