@@ -27,6 +27,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 #include <cstdio>
@@ -452,11 +453,11 @@ __device__ __forceinline__ void load_weights(unsigned char *dst, const __nv_bflo
     }
 }
 
-// the bf16 patches of group g (zero past the last patch), 16-byte copies
-__device__ __forceinline__ void load_group(unsigned char *raw, const __nv_bfloat16 *x, long long n, long long g) {
-    const long long b0 = g * (long long)RAW_BYTES, bend = n * 324;
+// the bf16 patches of group g, fp of them (zero past the last patch), 16-byte copies
+__device__ __forceinline__ void load_group(unsigned char *raw, const __nv_bfloat16 *x, long long n, long long g, int fp) {
+    const long long b0 = g * fp * 324, bend = n * 324;
     const unsigned char *src = reinterpret_cast<const unsigned char *>(x);
-    for (int i = threadIdx.x; i < (int)(RAW_BYTES / 16); i += blockDim.x) {
+    for (int i = threadIdx.x; i < fp * 324 / 16; i += blockDim.x) {
         const long long o = b0 + 16LL * i;
         const long long rem = bend - o;
         const int bytes = rem >= 16 ? 16 : (rem > 0 ? (int)rem : 0);
@@ -484,11 +485,17 @@ __device__ unsigned long long g_cnn_phase[16];
 #define CNN_PH(k) do {} while (0)
 #endif
 
-__global__ void __launch_bounds__(CNN_THREADS, 1) k_cnn_fused(const __nv_bfloat16 *__restrict__ x, long long n,
+// FULL: groups of FP patches; else of fp (a multiple of 4, so that a group starts
+// on 16 bytes), with the layers' rows and tiles of those alone
+template <bool FULL>
+__global__ void __launch_bounds__(CNN_THREADS, 1) k_cnn_fused(const __nv_bfloat16 *__restrict__ x, long long n, int group,
                                                       const __nv_bfloat16 *__restrict__ wt,
                                                       const float *__restrict__ bias, float *__restrict__ out,
                                                       unsigned *status) {
     using Q = Packed;
+    const int fp = FULL ? FP : group;
+    const int r1 = fp * C1, t1 = FULL ? T1 : (r1 + 127) / 128;
+    const int t2 = FULL ? T2 : (fp * C2 + 127) / 128, t3 = FULL ? T3 : (fp * C3 + 127) / 128;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char *base = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     unsigned char *W1 = base, *W2 = W1 + W1B, *W3 = W2 + W2B, *W4 = W3 + W3B, *W5 = W4 + W4B;
@@ -499,7 +506,7 @@ __global__ void __launch_bounds__(CNN_THREADS, 1) k_cnn_fused(const __nv_bfloat1
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bar + 1);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int quad = warp & 3, sub = warp >> 2;   // accumulator lanes 32 * quad.., and which share of the columns
-    const long long groups = (n + FP - 1) / FP;
+    const long long groups = (n + fp - 1) / fp;
 
     // conv1 and conv2: output u * 16 + co is channel co at the pair's position u
     for (int i = tid; i < 32 * 32; i += CNN_THREADS) {
@@ -526,7 +533,7 @@ __global__ void __launch_bounds__(CNN_THREADS, 1) k_cnn_fused(const __nv_bfloat1
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     long long g = blockIdx.x;
-    if (g < groups) load_group(RAW[0], x, n, g);
+    if (g < groups) load_group(RAW[0], x, n, g, fp);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
@@ -571,11 +578,11 @@ __global__ void __launch_bounds__(CNN_THREADS, 1) k_cnn_fused(const __nv_bfloat1
         __syncthreads();
         CNN_PH(0);
         // the next group's patches come in while this one runs
-        if (g + gridDim.x < groups) load_group(RAW[(it + 1) & 1], x, n, g + gridDim.x);
+        if (g + gridDim.x < groups) load_group(RAW[(it + 1) & 1], x, n, g + gridDim.x, fp);
         // ---- conv1 input map: row (patch, y * 5 + x / 2) = [c0, c1] at x .. x + 3 (x even; zeros past the edge) ----
         {
             const __nv_bfloat16 *pr = reinterpret_cast<const __nv_bfloat16 *>(raw);
-            for (int r = tid; r < R1; r += CNN_THREADS) {
+            for (int r = tid; r < r1; r += CNN_THREADS) {
                 const int pp = r / C1, pos = r % C1, yy = pos / 5, xx = 2 * (pos % 5);
                 const __nv_bfloat16 *c0 = pr + pp * 162 + yy * 9 + xx, *c1 = c0 + 81;
                 const __nv_bfloat16 z = __float2bfloat16_rn(0.f);
@@ -598,19 +605,19 @@ __global__ void __launch_bounds__(CNN_THREADS, 1) k_cnn_fused(const __nv_bfloat1
                 // issuer q takes tiles q, q + 4, ...; the tiles' accumulators are
                 // independent, so consecutive MMAs go to different tiles and a
                 // tile's accumulation chain does not stall the pipe
-                for (int t = q; t < T1; t += 4) mma_bf16(tmem + 32 * t, da + (uint64_t)(t * 128), db, id, false);
-                for (int t = q; t < T1; t += 4) mma_bf16(tmem + 32 * t, da + (uint64_t)(t * 128 + 10), db + 16, id, true);
+                for (int t = q; t < t1; t += 4) mma_bf16(tmem + 32 * t, da + (uint64_t)(t * 128), db, id, false);
+                for (int t = q; t < t1; t += 4) mma_bf16(tmem + 32 * t, da + (uint64_t)(t * 128 + 10), db + 16, id, true);
             })) { failed = true; break; }
         CNN_PH(2);
         // epilogue: the 7 x 7 window -> conv2 input planes, one pair (channels
         // 0-7, 8-15) per parity of x; their column x = 7 is zero
-        for (int t = sub; t < T1; t += 4) {
+        for (int t = sub; t < t1; t += 4) {
             uint32_t v[32];
             tmem_ld32_nowait(tmem + lane_off + 32 * t, v);
             tmem_wait_ld();
             const int r = t * 128 + 32 * quad + lane;
             const int pp = r / C1, pos = r % C1, yy = pos / 5, x2 = pos % 5;
-            if (pp < FP && yy < 7 && x2 < 4) {
+            if (pp < fp && yy < 7 && x2 < 4) {
                 const int o = pp * C2 + yy * 4 + x2;
 #pragma unroll
                 for (int u = 0; u < 2; ++u) {
@@ -629,18 +636,18 @@ __global__ void __launch_bounds__(CNN_THREADS, 1) k_cnn_fused(const __nv_bfloat1
                 const uint64_t da = sdesc(xs, P1_ROWS * 16, 128), db = sdesc(smem_u32(W2), 128, 24 * 128);
 #pragma unroll
                 for (int k = 0; k < 12; ++k)
-                    for (int t = q; t < T2; t += 4)
+                    for (int t = q; t < t2; t += 4)
                         mma_bf16(tmem + 32 * t, da + (uint64_t)((k & 1) * 2 * P1_ROWS + t * 128 + (k / 4) * 4 + (k % 4) / 2),
                                  db + 16 * k, id, k > 0);
             })) { failed = true; break; }
         CNN_PH(4);
-        for (int t = sub; t < T2; t += 4) {
+        for (int t = sub; t < t2; t += 4) {
             uint32_t v[32];
             tmem_ld32_nowait(tmem + lane_off + 32 * t, v);
             tmem_wait_ld();
             const int r = t * 128 + 32 * quad + lane;
             const int pp = r / C2, pos = r % C2, yy = pos / 4, x2 = pos % 4;
-            if (pp < FP && yy < 5 && x2 < 3) {
+            if (pp < fp && yy < 5 && x2 < 3) {
                 const int o = pp * C3 + yy * 5 + 2 * x2;
 #pragma unroll
                 for (int u = 0; u < 2; ++u) {
@@ -659,18 +666,18 @@ __global__ void __launch_bounds__(CNN_THREADS, 1) k_cnn_fused(const __nv_bfloat1
                 const uint64_t da = sdesc(xs, P2_ROWS * 16, 128), db = sdesc(smem_u32(W3), 128, 18 * 128);
 #pragma unroll
                 for (int k = 0; k < 9; ++k)
-                    for (int t = q; t < T3; t += 4)
+                    for (int t = q; t < t3; t += 4)
                         mma_bf16(tmem + 32 * t, da + (uint64_t)(t * 128 + (k / 3) * 5 + k % 3), db + 16 * k, id, k > 0);
             })) { failed = true; break; }
         CNN_PH(6);
         // epilogue: the 3 x 3 window -> fc1 input, one row per patch, plane (pos * 4 + channel / 8)
-        for (int t = sub; t < T3; t += 4) {
+        for (int t = sub; t < t3; t += 4) {
             uint32_t v[32];
             tmem_ld32_nowait(tmem + lane_off + 32 * t, v);
             tmem_wait_ld();
             const int r = t * 128 + 32 * quad + lane;
             const int pp = r / 25, pos = r % 25, yy = pos / 5, xx = pos % 5;
-            if (pp < FP && yy < 3 && xx < 3) {
+            if (pp < fp && yy < 3 && xx < 3) {
                 uint4 a0, a1, a2, a3;
                 relu_bf16x16(v, SB + Q::b3, &a0, &a1);
                 relu_bf16x16(v + 16, SB + Q::b3 + 16, &a2, &a3);
@@ -710,7 +717,7 @@ __global__ void __launch_bounds__(CNN_THREADS, 1) k_cnn_fused(const __nv_bfloat1
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     const int c = c0 + 16 * h;
-                    if (c < 144 && pp < FP) {
+                    if (c < 144 && pp < fp) {
                         uint4 lo, hi;
                         relu_bf16x16(v + 16 * h, SB + Q::b4 + c, &lo, &hi);
                         *reinterpret_cast<uint4 *>(X + (size_t)(c / 8) * PLB + 16 * pp) = lo;
@@ -735,8 +742,8 @@ __global__ void __launch_bounds__(CNN_THREADS, 1) k_cnn_fused(const __nv_bfloat1
             tmem_ld32_nowait(tmem + lane_off, v);        // accumulators 0 and 1
             tmem_ld16(tmem + lane_off + 32, u);          // accumulator 2 (and the wait)
             const int pp = 32 * quad + lane;
-            const long long row = g * FP + pp;
-            if (pp < FP && row < n) {
+            const long long row = g * fp + pp;
+            if (pp < fp && row < n) {
 #pragma unroll
                 for (int j = 0; j < NOUT; ++j)
                     out[row * NOUT + j] = __uint_as_float(v[j]) + __uint_as_float(v[16 + j]) + __uint_as_float(u[j]) +
@@ -754,13 +761,21 @@ __global__ void __launch_bounds__(CNN_THREADS, 1) k_cnn_fused(const __nv_bfloat1
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem) : "memory");
 }
 
+constexpr long long kEvenRounds = 8;   // beyond, a round more or less is little
 int launch_fused_cnn(tpx_ctx *c, const __nv_bfloat16 *x, long long n, const __nv_bfloat16 *wt, const float *bias,
                      float *out) {
-    if (ck(cudaFuncSetAttribute(k_cnn_fused, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FUSED_SMEM))) return TPX_ECUDA;
-    const long long groups = (n + FP - 1) / FP;
-    long long grid = c->num_sms;   // one CTA per SM: its shared memory and all of tensor memory
-    if (grid > groups) grid = groups;
-    k_cnn_fused<<<(unsigned)grid, CNN_THREADS, FUSED_SMEM, c->stream>>>(x, n, wt, bias, out, &c->ctl->status);
+    // one CTA per SM: its shared memory and all of tensor memory. Few patches are
+    // shared out evenly over the fewest rounds that full groups take (1000 patches
+    // 47 -> 38 us; 7296, one round of the 48-patch groups before: 45, with two of
+    // full groups 60, with two of 24 51)
+    const long long sms = c->num_sms, rounds = (n + sms * FP - 1) / (sms * FP);
+    const long long even = ((n + sms * rounds - 1) / (sms * rounds) + 3) / 4 * 4;
+    const bool full = rounds > kEvenRounds || even >= FP;
+    const int fp = full ? FP : (int)even;
+    const unsigned grid = (unsigned)std::min<long long>(sms, (n + fp - 1) / fp);
+    const auto kernel = full ? k_cnn_fused<true> : k_cnn_fused<false>;
+    if (ck(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FUSED_SMEM))) return TPX_ECUDA;
+    kernel<<<grid, CNN_THREADS, FUSED_SMEM, c->stream>>>(x, n, fp, wt, bias, out, &c->ctl->status);
     return ck(cudaGetLastError()) ? TPX_ECUDA : TPX_OK;
 }
 
