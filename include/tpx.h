@@ -80,9 +80,13 @@ typedef struct tpx_config {
     int32_t tile_geometry;      /* fused kernel tiles: TPX_TILE_4096 (1024-
                                    thread CTAs, one per SM, ranges of up to
                                    8192 positions), TPX_TILE_2048 (512-thread
-                                   CTAs, two per SM, up to 4096 positions),
-                                   or TPX_TILE_DEFAULT (the library's choice,
-                                   TPX_TILE_4096).  Not a paper parameter:
+                                   CTAs, two per SM, up to 5120 positions),
+                                   or TPX_TILE_DEFAULT (the library's choice:
+                                   tiles of 1024 packets with ranges of up to
+                                   8192 positions while there is an SM for
+                                   each, else TPX_TILE_4096, from 2^20 packets
+                                   on the faster of both, see tpx_tuning).
+                                   Not a paper parameter:
                                    results are identical, only speed and the
                                    range limit differ.                        */
     int32_t flags;              /* TPX_FLAG_* bits, 0 by default              */
@@ -310,11 +314,11 @@ int tpx_kernel_times(tpx_ctx *ctx, double *prepass_ms, double *fused_ms, int64_t
    it).  This call synchronises the device and copies the 32 counters of one
    tile geometry (TPX_TILE_4096 or TPX_TILE_2048) to h_cycles[32], zeroing
    them when `clear` is nonzero.  Phases: 0 tile start, 1 tile load,
-   2 look-ahead, 3 walk 2 and its scan, 4 trigger times, 5 walk 4 (records),
-   6 hash insert, 7 neighbour pass, 8 compression, 9 unions, 10 roots,
-   11 member lists, 12 member-list walks (and the previous tile's copy-out),
-   13 label ranks and staged stores, 14 labels and offsets, 15 tail,
-   16 the CTA's end.  The normal build returns TPX_EUNSUPPORTED (zeros);
+   2 records into slots, 3 pixel wraps, 4 trigger times, 5 walk 4 (records),
+   6 cell table ranks, 7 neighbour pass, 9 unions, 10 roots, 11 member lists,
+   12 member-list walks, 13 records and label entries, 14 labels, 15 tail,
+   16 the CTA's end, 17 big ranges (batches), 19 label ranks, 20 to 26 the
+   steps of a big range.  The normal build returns TPX_EUNSUPPORTED (zeros);
    TPX_EINVAL for another geometry or a NULL pointer. */
 int tpx_debug_phase_times(int tile_geometry, uint64_t *h_cycles, int clear);
 
@@ -328,7 +332,7 @@ int tpx_debug_phase_times(int tile_geometry, uint64_t *h_cycles, int clear);
    that fix the library's memory up front).  Same inputs and outputs as
    tpx_process, but no context: the configuration and the CUDA stream are
    passed directly, and the look-back scratch is one fixed array in device
-   memory that is part of the library (about 2.4 MB per device that loads it,
+   memory that is part of the library (about 3 MB per device that loads it,
    held until exit).  The first call on each device, with that device current,
    looks up the array's device address (cudaGetSymbolAddress).  All calls on a
    device share the array and it keeps the last call's contents (the per-call
@@ -477,7 +481,7 @@ int tpx_cnn_train_step(tpx_ctx *ctx, float *d_params, float *d_adam_m, float *d_
    to d_packed (tpx_cnn_packed_bytes() bytes, 256-byte aligned);
    tpx_cnn_infer runs the five layers over n <= 2^30 patches d_x [n x 162]
    bf16 (16-byte aligned; tpx_refine_patches_bf16) in one kernel: groups of
-   48 patches per CTA, the layers as implicit GEMMs whose activations stay in
+   up to 44 patches per CTA, the layers as implicit GEMMs whose activations stay in
    shared memory, each hidden activation rounded to bf16 after its ReLU, into
    d_out [n x 6] floats.  d_work is not used (tpx_cnn_infer_work_bytes is
    kept for the interface: 256 bytes for n > 0); it may be NULL.
@@ -514,15 +518,16 @@ int tpx_refine_patches_bf16(tpx_ctx *ctx, const uint64_t *d_packets, int64_t n_p
    range (its shots up to the next trigger packet) is longer than the tile
    can hold on chip clusters it in the same launch with the big-range path:
    the whole range decoded into the CTA's global scratch, its kept pixels
-   sorted by (shot, time bin), each pixel compared with its own and the
+   sorted by (shot, time bin, columns), their neighbours found through a hash
+   of the cells or, for wide boxes, among the pixels of the same and the
    previous bin (the same results as the tile's path).  A range even that
    cannot hold (more than 65,535 packets, more kept pixels than its shared
-   scratch: 31,040, or 24,960 with 2048-packet tiles, more than 256 trigger
+   scratch: 34,880, or 27,392 with 2048-packet tiles, more than 256 trigger
    packets), any range in PAPER mode, and a pixel whose trigger lies
    outside its range send the run to the general path: such runs are redone
    exactly at tpx_sync (counters.redone = the number of such runs) and
-   spliced into the outputs.  The big-range scratch takes 13.3 MB per CTA of
-   the grid (10.8 MB with 2048-packet tiles) of the batch scratch.
+   spliced into the outputs.  The big-range scratch takes 14.9 MB per CTA of
+   the grid (11.8 MB with 2048-packet tiles) of the batch scratch.
      h_run_offsets   host [n_runs + 1], h_run_offsets[0] = 0, non-decreasing
      d_labels, d_is_peak  per packet of the whole buffer, or NULL; labels are
                      positions in the whole buffer

@@ -183,7 +183,7 @@ inline int tile_cols(long long M, int N) { return 4096 / tile_rows(M, N); }
 void sgemm(cudaStream_t s, const float *A, long long sam, long long sak, const float *B, long long sbk, long long sbn,
            float *C, long long ldc, long long M, int N, long long K, const float *bias, bool relu, int splits = 1) {
     const int tm = tile_rows(M, N), tn = tile_cols(M, N);
-    constexpr long long kRows = 1LL << 20;   // grid.y <= 65535 tiles of 16 rows
+    constexpr long long kRows = 1LL << 20;   // grid.y <= 65535: more than 32 rows are in tiles of 64 at least
     for (long long m0 = 0; m0 < M; m0 += kRows) {
         const int m = (int)(M - m0 < kRows ? M - m0 : kRows);
         const dim3 g((N + tn - 1) / tn, (m + tm - 1) / tm, splits);

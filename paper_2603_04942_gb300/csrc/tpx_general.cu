@@ -784,9 +784,9 @@ __global__ void __launch_bounds__(GT) k_seg_starts(Sorted s, long long n, int dt
 struct AccH { long long s_tot, s_x, s_y, s_t; unsigned n, npk; };
 
 constexpr int WREG = 64;            // hits of a segment held in registers (two per lane)
-constexpr int WCAP = 256;           // hits of a segment held by one warp in shared memory
+constexpr int WCAP = 256;           // hits of a segment held by one block in shared memory
 constexpr int ECAP = 1024;          // adjacent pairs of a segment kept for the hooking rounds
-constexpr int HBW = 512;            // cell-hash buckets of a warp's segment
+constexpr int HBW = 512;            // cell-hash buckets of a block's segment
 constexpr int SEGW = 4;             // warps per block
 struct SmallSm {                    // a segment of up to WREG hits
     int tofb[WREG];

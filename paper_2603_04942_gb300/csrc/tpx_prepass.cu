@@ -360,7 +360,7 @@ __global__ void __launch_bounds__(SB, 1) k_prepass_small(const Params p, int T) 
     {
         const long long tile = blockIdx.x;
         const TileSpan sp = tile_span(p, tile, T);
-        const int per = T / 32;   // 64 or 128 packets: one or two steps
+        const int per = T / 32;   // 32, 64 or 128 packets: half a step, one or two
         const int qb = w * per, qe = min(sp.cnt, qb + per);
         WarpPart<2> part;
         if (qb < qe) part.run(p.pk + sp.base, (sp.base & 1) == 0, qb, qe, tp, tt, lane);
