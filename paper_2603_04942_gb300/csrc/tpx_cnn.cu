@@ -372,15 +372,16 @@ __global__ void k_cnn_pack(const float *P, __nv_bfloat16 *wt, float *bias) {
 // by ky * W + kx rows -- a descriptor with its start moved, leading offset the
 // plane stride, stride offset one core matrix (8 rows). Rows past the valid
 // ones read stale (finite) contents of X; X starts zeroed.
-// The MMAs of the convolutions are bound by reading A from shared memory (45
-// cycles for 128 rows of 16, whatever N up to 32), so conv1 and conv2 compute
-// two neighbouring outputs per row: N = 2 x 16, a row per pair of positions.
+// The MMAs of the convolutions are bound by reading A from shared memory (128
+// rows of 16 take 41 cycles with N = 16 and 48 with N = 32, conv2's phase in the
+// instrumented build), so conv1 and conv2 compute two neighbouring outputs per
+// row: N = 2 x 16, a row per pair of positions.
 // conv1's rows hold the two channels of four positions from an even x on (a k
 // chunk is a kernel row), and each output's weights are zero at the position it
 // does not see; conv2 reads its input as one pair of planes per parity of x,
 // four taps per kernel row, again with zeros. Each output sums the same products
-// in the same order as with a row per position (equal outputs; 1,000,003 patches
-// 2245 -> 2008 us). Tried: two pipelines of 24 patches and eight warps per CTA, to
+// in the same order as with a row per position (equal outputs for finite
+// activations; 1,000,003 patches 2245 -> 2008 us). Tried: two pipelines of 24 patches and eight warps per CTA, to
 // run one's MMAs beside the other's epilogue: 2504 us, both want shared memory.
 constexpr int FP = 44;                                // patches per group
 constexpr int C1 = 45, C2 = 28, C3 = 25;              // rows of a patch: conv1 9 x 5 pairs, conv2 7 x 4 pairs, conv3 5 x 5

@@ -233,9 +233,10 @@ __device__ __forceinline__ void put_pair(uint16_t *row, int e, float a, float b)
 // kernels' costs 11 + 4 + 25 f us per 10^6 packets with a share f of them going
 // on, the last kernels alone 27. A cell's word holds all that its values follow
 // from: ToT, the packet's place in the window (the brighter pixel wins, ties go
-// to the later) and the clamped time, never zero. Bound by latency, so every
-// thread's loads of a step are in flight together; the bytes are the labels
-// (twice, mostly from L2) and the patches. In the last kernels every cell has an
+// to the later) and the clamped time, never zero. Bound by instruction issue
+// (77% of the slots) and by the latency of its steps, so every thread's loads of
+// a step are in flight together; the bytes are the labels (twice, half of them
+// from L2) and the patches, 31% of the copy rate. In the last kernels every cell has an
 // 8-byte key in global memory, cleared, updated and read back, as all of them
 // had before: 300 us of the 460 of a call of 440,000 patches of 20 particles a
 // shot, now about 115 of 280.
@@ -711,7 +712,7 @@ __device__ __forceinline__ void load_b2(uint32_t addr, uint32_t (&b)[4]) {
 // weight fragment serves 32 rows; layer 2 runs in two halves of its outputs,
 // each at once taken into layer 3, so that the accumulators fit the registers;
 // a CTA's next rows are prefetched into L2 a tile ahead. 1,000,003 rows of width
-// 160: 326 -> 272 us (2.9 cycles per m16n8k16 and SM). Every accumulator sees
+// 160: 326 -> 272 us (the tensor pipe at 66% of an SM's active cycles). Every accumulator sees
 // the same products in the same order as with MT = 1, so the outputs are equal.
 template <int H, int MT>
 __global__ void __launch_bounds__(256, 1) k_mlp_bf16(const float *__restrict__ x, long long n,
