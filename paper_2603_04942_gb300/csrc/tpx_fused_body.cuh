@@ -8,7 +8,7 @@
 // Bound by instruction issue and by the barriers between its phases, not by
 // bytes (18 B per packet, 5% of the copy bandwidth). Measured on 2.46e8 packets
 // of the large recipe, 2048-packet tiles: 61.9 -> 41.7 us per 10^6 packets,
-// 45.4 -> 29.5 warp instructions per packet, against the form with a chained
+// 45.4 -> 29.8 warp instructions per packet, against the form with a chained
 // hash of the pixels in arrival order, a walk for the unwrap chains and the
 // copy-out as a phase of the workers.
 //
